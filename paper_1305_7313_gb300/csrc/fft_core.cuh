@@ -372,6 +372,8 @@ template <int SIGN, class T> struct Dft {
     else if constexpr (R == 6) prime_factor<2, 3, true>(x, w);
     else if constexpr (R == 9) composite<3, 3, true>(x, w);
     else if constexpr (R == 12) prime_factor<4, 3, true>(x, w);
+    else if constexpr (R == 18) prime_factor<9, 2, true>(x, w);
+    else if constexpr (R == 24) prime_factor<8, 3, true>(x, w);
     else composite<4, 4, true>(x, w);  // R == 16
   }
 
@@ -497,6 +499,8 @@ template <int SIGN, class T> struct Dft {
     else if constexpr (R == 6) prime_factor<2, 3>(x);
     else if constexpr (R == 9) composite<3, 3>(x);
     else if constexpr (R == 12) prime_factor<4, 3>(x);
+    else if constexpr (R == 18) prime_factor<9, 2>(x);
+    else if constexpr (R == 24) prime_factor<8, 3>(x);
     else composite<4, 4>(x);  // R == 16
   }
 };
@@ -651,6 +655,182 @@ __device__ __forceinline__ void fft_lines(cplx<T>* buf, const cplx<T>* tw) {
   const int t = tid / NLINES;
   const bool active = t < TL;
   fft_stages<T, N, SIGN, TL, ES, 0, 1, MAXT, EMAX, OMAP>(buf + line * LS, t, active, tw);
+}
+
+// ------------------------------------------------ two-factor transforms in place
+//
+// The pair passes transform lines of N = A B points as
+//
+//   n = b + B r  (r < A, b < B),   k = q + A s  (q < A, s < B):
+//   X[k] = sum_b w_B^(b s) w_N^(b q) sum_r x[b + B r] w_A^(r q)
+//
+// A-stage (item (line, b)): the A-point DFT over r, output q left at position
+// b + B q, where the inputs came from.  B-stage (item (line, q)): the B values
+// at positions B q .. B q + B - 1, twiddles w_N^(b q) on the inputs, B-point
+// DFT, output s left at B q + s.  Every item reads and writes the same B or A
+// positions, so a stage needs one barrier after it and none between its reads
+// and writes, an item's registers are free before the next item's loads, and a
+// thread holds one item (max(A, B) values) instead of all its elements of the
+// line.  The frequency k ends at position spec_pos(k) = k / A + B (k mod A).
+// The inverse of a spectrum in that order runs the stages backwards (B-point
+// DFT over s, twiddles on the A-stage's inputs, A-point DFT over q) and leaves
+// natural order.
+//
+// Factors: A is a multiple of 4, so that four consecutive points 4c .. 4c + 3
+// of a spectrum-ordered line sit B apart (the accumulator updates read them as
+// one group), and consecutive k fall on distinct shared-memory banks except at
+// N = 64 (at 96, 12 x 8 would put them 8 values apart: six-way conflicts).
+struct TwoFactor {
+  int a, b;
+};
+template <int N, int TILE = 0> constexpr TwoFactor two_factor() {
+  static_assert(N == 8 || N == 12 || N == 16 || N == 24 || N == 32 || N == 36 || N == 48 || N == 64 || N == 72 ||
+                    N == 96,
+                "no factors chosen for this line length");
+  return N == 8    ? TwoFactor{4, 2}
+         : N == 12 ? TwoFactor{4, 3}
+         : N == 16 ? TwoFactor{4, 4}
+         : N == 24 ? TwoFactor{4, 6}
+         : N == 32 ? TwoFactor{8, 4}
+         : N == 36 ? TwoFactor{12, 3}
+         : N == 48 ? TwoFactor{4, 12}
+         : N == 64 ? TwoFactor{8, 8}
+         : N == 72 ? TwoFactor{12, 6}
+         : TILE == 1 ? TwoFactor{12, 8}
+                     : TwoFactor{8, 12};
+}
+template <int A, int B> FFT_HD constexpr int spec_pos(int k) { return k / A + B * (k % A); }
+
+// DFT of x_0, w[1] x_1, ..., w[R-1] x_{R-1} (w: R consecutive twiddles in shared
+// memory, two to a 16-byte load in FP32).
+template <class T, int R, int SIGN>
+__device__ __forceinline__ void dft_twiddled(cplx<T>* x, const cplx<T>* wp) {
+  cplx<T> w[R];
+  if constexpr (sizeof(cplx<T>) == 8 && R % 2 == 0) {
+    const float4* w4 = reinterpret_cast<const float4*>(wp);
+#pragma unroll
+    for (int r = 0; r < R; r += 2) {
+      const float4 t = w4[r / 2];
+      w[r] = cmake<T>(t.x, t.y);
+      w[r + 1] = cmake<T>(t.z, t.w);
+    }
+  } else {
+#pragma unroll
+    for (int r = 1; r < R; ++r) w[r] = wp[r];
+    w[0] = w[1];  // not read: x_0 carries no twiddle
+  }
+  if constexpr (FftTraits<T>::fused) {
+    Dft<SIGN, T>::template run_tw<R, false>(x, w);
+  } else {
+#pragma unroll
+    for (int r = 1; r < R; ++r) x[r] = cmul(x[r], w[r]);
+    Dft<SIGN, T>::template run<R>(x);
+  }
+}
+
+// item / n and item % n for a run-time 1 <= n <= 1024 and item < 65536 (one
+// multiplication by a reciprocal computed once per kernel).
+struct RtDiv {
+  unsigned n, mag;
+  __device__ __forceinline__ explicit RtDiv(int n_) : n((unsigned)n_), mag(n_ > 1 ? 0xffffffffu / (unsigned)n_ + 1u : 0u) {}
+  __device__ __forceinline__ int div(int item) const { return mag ? (int)__umulhi((unsigned)item, mag) : item; }
+};
+
+// A-stage (or, with the roles of A and B exchanged by the caller, any stage) on
+// lines in shared memory: item (line l, j), j < NJ, takes the R elements at
+// buf + off(l) + j JS + r STEP in place.  TW: twiddles tw[j R + r].  Threads
+// take items line-fast, so a warp's items are consecutive lines.
+template <class T, int R, int SIGN, int NJ, int JS, int STEP, bool TW, int THR, class Off>
+__device__ __forceinline__ void stage_rt(cplx<T>* buf, const cplx<T>* tw, int nlines, const RtDiv& by, const Off& off) {
+  for (int item = threadIdx.x; item < nlines * NJ; item += THR) {
+    const int j = by.div(item), l = item - j * nlines;
+    cplx<T>* p = buf + off(l) + j * JS;
+    cplx<T> x[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r) x[r] = p[r * STEP];
+    if constexpr (TW) dft_twiddled<T, R, SIGN>(x, tw + j * R);
+    else Dft<SIGN, T>::template run<R>(x);
+#pragma unroll
+    for (int r = 0; r < R; ++r) p[r * STEP] = x[r];
+  }
+  __syncthreads();
+}
+// Items of a stage unrolled together: all of a thread's in FP32 and FP64; one
+// in double-float, whose items are over a thousand instructions each.
+template <class T> constexpr int kItemUnroll = FftTraits<T>::fused ? 16 : 1;
+
+// The same with a compile-time line count and line stride LS.
+template <class T, int R, int SIGN, int NJ, int JS, int STEP, bool TW, int THR, int NLINES, int LS>
+__device__ __forceinline__ void stage_ct(cplx<T>* buf, const cplx<T>* tw) {
+#pragma unroll(kItemUnroll<T>)
+  for (int item0 = 0; item0 < NLINES * NJ; item0 += THR) {
+    const int item = item0 + threadIdx.x;
+    if ((NLINES * NJ) % THR == 0 || item < NLINES * NJ) {
+      const int j = item / NLINES, l = item - j * NLINES;
+      cplx<T>* p = buf + l * LS + j * JS;
+      cplx<T> x[R];
+#pragma unroll
+      for (int r = 0; r < R; ++r) x[r] = p[r * STEP];
+      if constexpr (TW) dft_twiddled<T, R, SIGN>(x, tw + j * R);
+      else Dft<SIGN, T>::template run<R>(x);
+#pragma unroll
+      for (int r = 0; r < R; ++r) p[r * STEP] = x[r];
+    }
+  }
+  __syncthreads();
+}
+
+// ------------------------------------------------ a plane in three passes
+//
+// With N = 4 M a plane takes three trips through registers instead of four: the
+// columns' M-point stage (its input read from global memory), then one item per
+// M x M that does the columns' 4-point stage and the rows' first 4-point stage
+// on a 4 x 4 block, then the rows' M-point stage.  For lines n = b + 4 r, k = q
+// + M s along the columns (place b + 4 q after the first stage, 4 q + s after
+// the second) and n = b + M r, k = q + 4 s along the rows (place b + M q, then
+// M q + s).
+template <int M> FFT_HD constexpr int plane_row_place(int k) { return 4 * (k % M) + k / M; }
+template <int M> FFT_HD constexpr int plane_col_place(int k) { return M * (k % 4) + k / 4; }
+
+// The middle pass: block item (x, y), x, y < M, rows 4x .. 4x + 3, columns y + M j.
+// 4-point DFTs with twiddles tw[4 x + b] down the columns, then 4-point DFTs
+// along the rows, in place.  Where M is a multiple of 4 a half warp takes 4 y
+// of 4 consecutive x: 4 RP = 4 modulo 16 values, so its accesses fall on
+// distinct banks.
+template <class T, int M, int SIGN, int THR, int RP>
+__device__ __forceinline__ void plane_block_pass(cplx<T>* P, const cplx<T>* tw) {
+#pragma unroll(kItemUnroll<T>)
+  for (int item0 = 0; item0 < M * M; item0 += THR) {
+    const int item = item0 + threadIdx.x;
+    if ((M * M) % THR != 0 && item >= M * M) break;
+    int x, y;
+    if constexpr (M % 4 == 0) {
+      const int h = item >> 4, g = h / (M / 4);
+      x = 4 * g + ((item >> 2) & 3);
+      y = 4 * (h - g * (M / 4)) + (item & 3);
+    } else {
+      x = item / M;
+      y = item - x * M;
+    }
+    cplx<T>* p = P + 4 * x * RP + y;
+    cplx<T> v[4][4];  // [row along r][column j]
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      cplx<T> c[4];
+#pragma unroll
+      for (int b = 0; b < 4; ++b) c[b] = p[b * RP + j * M];
+      dft_twiddled<T, 4, SIGN>(c, tw + 4 * x);
+#pragma unroll
+      for (int b = 0; b < 4; ++b) v[b][j] = c[b];
+    }
+#pragma unroll
+    for (int b = 0; b < 4; ++b) {
+      Dft<SIGN, T>::r4(v[b]);
+#pragma unroll
+      for (int j = 0; j < 4; ++j) p[b * RP + j * M] = v[b][j];
+    }
+  }
+  __syncthreads();
 }
 
 }  // namespace fockx

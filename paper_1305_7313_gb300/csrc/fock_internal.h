@@ -28,7 +28,7 @@ struct DevPlan {
   int n;            // cubic grid N
   int k3h;          // N/2 + 1: stored half of the last axis
   int64_t ntot;     // N^3
-  int64_t hsize;    // elements of one half-spectrum pair buffer: N * N * 2 * k3h
+  int64_t hsize;    // elements reserved per pair-transform buffer (at least N^3: [i1][k2][k3])
   int npw;
   const int* gidx;     // [npw] grid offset of G
   const int* gidxneg;  // [npw] grid offset of -G
@@ -41,17 +41,22 @@ struct DevPlan {
   double psi_scale;    // 1 / sqrt(Omega)
   double out_scale;    // sqrt(Omega) / Ntot
   int msmall2;         // |m|^2 at or below which kernel terms are done in FP64 (mixed form)
-  // Columns of the stored half that pair densities reach (Gamma point): row k2
-  // keeps k3 < ncol[k2]; the column pass takes them NC = 2 (N/2 + 1) lines per
-  // CTA from colmap (ncta_col * NC entries, (k2 << 16) | (s << 15) | k3, -1: none)
+  // Columns (k2, k3) that pair densities reach (Gamma point), a set closed under
+  // (k2, k3) -> (-k2, -k3): column k3 (0 .. N-1) keeps k2 < (ncol[k3] & 0xffff)
+  // and k2 >= N - (ncol[k3] >> 16).  The column pass takes them as pairs of a
+  // line and its mirror image, col_lines pairs per CTA, from colmap (ncta_col *
+  // col_lines entries, (k2 << 16) | (self << 15) | k3 of the line with k3 <= N/2,
+  // self: the line is its own mirror image; -1: none)
   const int* ncol;
   const int* colmap;
   int ncta_col;
-  // rows k2 that have kept columns are [0, row_lo) and [N - row_hi, N) (a
-  // ball centred on G = 0 reaches a symmetric range of m2; row_lo = N,
-  // row_hi = 0 when every row is kept); col_max = the largest ncol[k2]
+  // rows k2 that have kept columns are [0, row_lo) and [N - row_hi, N); kept
+  // k3 are below col_max or mirror images of such
   int row_lo, row_hi, col_max;
-  // the kept columns (k2 << 16) | k3 in row order (nkept entries)
+  // the kept rows' places in a plane transformed along i2, ascending: [2][N],
+  // per tiling (the factors fix the order)
+  const int* rowpos;
+  // the kept columns (k2 << 16) | k3, rows outer (nkept entries)
   const int* kept;
   int nkept;
   // radix-plan variant ("tiling", 0 or 1) of the forward plane, column and
@@ -94,7 +99,7 @@ struct KernelOps {
   int real_bytes;  // sizeof of the working real type
   int prec;        // 0 FP64, 1 mixed FP32, 2 double-float (fock_precision)
   int n;           // grid size these kernels are compiled for
-  int col_lines;   // lines of the column map a column-pass CTA takes
+  int col_lines;   // line pairs of the column map a column-pass CTA takes
   size_t smem;     // largest dynamic shared memory of its kernels
   cudaError_t (*configure)(const DevPlan&);
   // c(G) of bands [band0, band0 + nbat) to psi(r); X is scratch of >= ceil(nbat/2) grids.
@@ -116,6 +121,8 @@ struct KernelOps {
   // radices[nst], threads per line, threads per CTA; returns the number of
   // distinct tilings (1 or 2)
   int (*tile_plan)(int pass, int tile, int* radices, int* nst, int* threads_per_line, int* threads);
+  // row of the transformed plane that holds frequency k2 in the forward plane pass
+  int (*row_place)(int tile, int k2);
 };
 
 // Kernels for grid size n and precision (0: FP64, 1: mixed); NULL if not built.

@@ -38,10 +38,6 @@ namespace fockx {
 
 __device__ __forceinline__ int freq_of(int k, int n) { return k < (n + 1) / 2 ? k : k - n; }
 
-// Rounds of global loads each thread issues before storing them to shared
-// memory in the pass prologues (memory-level parallelism).
-constexpr int kLoadUnroll = 4;
-
 // Per working type: the precision code of the plan (0 FP64, 1 mixed FP32,
 // 2 double-float) and the type of the accumulators W.
 template <class T> struct RealTraits;
@@ -84,6 +80,16 @@ template <> __device__ __forceinline__ double2 ldcg_hint<double2>(const double2*
   double2 v;
   asm volatile("ld.global.cg.L2::cache_hint.v2.f64 {%0, %1}, [%2], %3;" : "=d"(v.x), "=d"(v.y) : "l"(p), "l"(pol));
   return v;
+}
+template <> __device__ __forceinline__ cdf64 ldcg_hint<cdf64>(const cdf64* p, unsigned long long pol) {
+  float4 v;
+  asm volatile("ld.global.cg.L2::cache_hint.v4.f32 {%0, %1, %2, %3}, [%4], %5;"
+               : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+               : "l"(p), "l"(pol));
+  cdf64 r;
+  r.x = df64(v.x, v.y);
+  r.y = df64(v.z, v.w);
+  return r;
 }
 // Four floats with an L2 eviction policy (16-byte aligned).
 __device__ __forceinline__ float4 ld_f4_hint(const float* p, unsigned long long pol) {
@@ -280,39 +286,6 @@ __device__ inline void block_sum4_ff(const float v[4], float hi[4], float lo[4],
   }
 }
 
-// One kernel term of the smallest |m| (|m|^2 <= msmall2: 27 points per pair)
-// of the mixed-form column pass, in FP64: element e of the CTA's lines, at
-// (k1, k2, k3) of pair s.  Adds its energy terms to the pair slot itself.
-// Kept out of line so the FP64 instructions are not predicated into every
-// warp of the kernel.
-template <class T, int N>
-__device__ __noinline__ void small_g_term_fp64(const DevPlan& g, cplx<T>* S, int e, int k1, int k2, int k3,
-                                               int s, const Chain& ch, double* epair, double* dpair) {
-  constexpr int KH = N / 2 + 1;
-  const int64_t vi = ((int64_t)k1 * N + k2) * KH + k3;
-  const double wgt = (k3 == 0 || 2 * k3 == N) ? 1.0 : 2.0;
-  cplx<T> z = S[e];
-  double zx = z.x, zy = z.y;
-  if (g.ovl != nullptr && k1 == 0 && k2 == 0 && k3 == 0) {
-    // G = 0: the sum of the pair density over the grid, from the FP64 overlap
-    // of the pair's coefficients instead of the FP32 transform (real)
-    const int i = s ? ch.bi : ch.ai, j = s ? ch.bj : ch.aj;
-    zx = g.ovl_scale * g.ovl[(int64_t)i * g.ovl_ld + (j - g.ovl_j0)];
-    zy = 0.0;
-  }
-  const double a2 = zx * zx + zy * zy;
-  const double v = g.vtab64[vi];
-  const int slot = s ? ch.pb : ch.pa;
-  if (slot >= 0) {
-    atomicAdd(&epair[slot], wgt * v * a2);
-    if (g.dvtab64) atomicAdd(&dpair[slot], wgt * g.dvtab64[vi] * a2);
-  }
-  const double vs = v * g.inv_ntot;
-  z.x = T(zx * vs);
-  z.y = T(zy * vs);
-  S[e] = z;
-}
-
 // Stage the twiddle table in shared memory: tw[t] = e^{-2 pi i t/N} for the
 // forward transforms, tw[N + t] = its conjugate for the inverse ones, so no
 // transform negates a twiddle where it uses it.
@@ -431,71 +404,178 @@ __global__ void k_gather(DevPlan g, const cplx<T>* __restrict__ X, int nb, int b
 
 // ------------------------------------------------------------------ pair passes
 
+// Compile-time geometry of the pair passes for grid size N and tiling TILE
+// (the factors of the two-factor transforms and the threads that share them).
+template <class T, int N, int TILE = 0>
+struct PairGeo {
+  using C = cplx<T>;
+  static constexpr TwoFactor f = two_factor<N, TILE>();
+  static constexpr int A = f.a, B = f.b;
+  static_assert(A * B == N && A % 4 == 0, "factors of the line length, the first a multiple of 4");
+  static constexpr int RP = N + 1;  // odd row stride of a plane: rows on distinct banks
+  // FP32 plane passes transform all N rows or columns in shared memory, kept
+  // or not (85 of 96 at 96^3, L 27): packing the kept ones leaves gaps and
+  // wraps inside a half warp, and each costs it one more shared-memory
+  // wavefront, of the unit that bounds these passes (96^3 forward pass with
+  // two-factor stages: 27.2 M wavefronts a 38-chain launch packed, 20.5 M this
+  // way).  FP64 and double-float are bound by arithmetic and transform the kept
+  // ones only.
+  static constexpr bool ALL_LINES = sizeof(C) == 8;
+  // FP32 plane passes take three trips through registers (N = 4 M): shared
+  // memory bounds them, and a trip fewer takes 20.5 -> 15.1 M wavefronts a
+  // 38-chain launch at 96^3 (forward; 3.44 -> 3.06 us a chain, inverse 4.29 ->
+  // 3.65).  FP64 and double-float are bound by arithmetic: the two-factor
+  // stages' items are smaller and share out more evenly (FP64 24^3 forward 0.85
+  // against 1.05 us, 48^3 6.39 against 6.49, 96^3 even)
+  static constexpr bool BLOCK = RealTraits<T>::prec == 1 && TILE == 0;
+  static constexpr int M = N / 4;
+  // threads per line: an M-point item each, or whole two-factor items
+  static constexpr int TPL = TILE == 1 ? 8 : (!BLOCK && (N == 72 || N == 36) ? 3 : 4);
+  static constexpr int THR_PLANE = (N * TPL + 31) / 32 * 32;
+  // where a plane's passes leave frequency k of the columns and of the rows
+  static __host__ __device__ constexpr int row_place(int k) {
+    return BLOCK ? plane_row_place<M>(k) : spec_pos<A, B>(k);
+  }
+  static __host__ __device__ constexpr int col_place(int k) {
+    return BLOCK ? plane_col_place<M>(k) : spec_pos<A, B>(k);
+  }
+  // elements 4c .. 4c + 3 of a transformed row: quad_place(c) + u QUAD
+  static constexpr int QUAD = BLOCK ? M : B;
+  static __host__ __device__ constexpr int quad_place(int c) { return col_place(4 * c); }
+  // the row i2 that the inverse pass leaves at place p
+  static __host__ __device__ constexpr int row_of(int p) { return BLOCK ? p / 4 + M * (p % 4) : p; }
+  static __host__ __device__ constexpr int place_of_row(int i2) { return BLOCK ? plane_row_place<M>(i2) : i2; }
+  // column pass: NP lines and their mirror images a CTA, so that a warp's
+  // loads and stores are runs of NP consecutive columns
+  static constexpr int NP = 16, NL = 2 * NP;
+  // its factors: N/4 and 4 in FP32 and FP64 (fewest operations, and the values
+  // of a line pair that the middle stage holds are 8, so twice the warps fit:
+  // 96^3 2.39 -> 2.32 us a chain in FP32, 43.7 -> 42.4 in FP64, 48^3 5.62 ->
+  // 5.05 in FP64) except at 64 and 72, where the two-factor ones are 2-6% faster
+  static constexpr bool COL4 = TILE == 0 && RealTraits<T>::prec != 2 && N != 64 && N != 72;
+  static constexpr int CA = COL4 ? M : A, CB = N / CA;
+  static constexpr int THR_COL = TILE == 1 ? 256 : COL4 ? 128
+                                 : N == 96 || N == 64 || N == 32 || N == 16 ? 128
+                                 : N == 72                                  ? 192
+                                 : N == 36                                  ? 96
+                                                                            : 64;
+  static_assert(THR_PLANE <= 1024 && THR_COL % NL == 0, "CTA sizes");
+  // the plane, the twiddles of two stages, the forward pass's row list
+  static constexpr size_t SMEM_PLANE = sizeof(C) * (size_t)(N * RP + 2 * N) + (ALL_LINES ? 0 : N * sizeof(int));
+  static constexpr size_t SMEM_COL =
+      sizeof(C) * (size_t)(N * NL + 2 * N) + 32 * 4 * sizeof(double) + NL * sizeof(int);
+  // CTAs per SM the kernels are register-budgeted for: as many as the shared
+  // memory holds at the registers an item takes (56 in FP32 plane passes: 12
+  // complex values and their addresses; twice that in FP64 and double-float;
+  // the column pass holds the B values of a line and of its mirror image)
+  static constexpr int fit(size_t smem, int thr, int regs) {
+    const int by_smem = (int)(kSmemPerSM / (smem + 1024)), by_regs = 65536 / (thr * regs), by_thr = 2048 / thr;
+    const int m = by_smem < by_regs ? by_smem : by_regs;
+    const int k = m < by_thr ? m : by_thr;
+    return k < 1 ? 1 : (k > 32 ? 32 : k);
+  }
+  static constexpr int WIDE = sizeof(C) == 8 ? 1 : 2;
+  static constexpr int MIN_PLANE =
+      fit(SMEM_PLANE, THR_PLANE, !BLOCK ? 104 / (3 - WIDE) : WIDE * (M >= 24 ? 80 : M >= 16 ? 64 : M >= 12 ? 56 : 48));
+  static constexpr int MIN_COL = fit(SMEM_COL, THR_COL, RealTraits<T>::prec == 2 ? 104 : WIDE * (CB >= 12 ? 88 : CB >= 8 || CA >= 24 ? 72 : CA >= 16 ? 64 : 56));
+};
+
+// Stage the twiddles of a stage of NJ items of R values a line (NJ R = N):
+// tw[j R + r] = e^{SIGN 2 pi i j r / N}, an item's R of them side by side.
+template <class T, int SIGN, int R, int N, int THR>
+__device__ __forceinline__ void load_stage_twiddles(cplx<T>* tw, const DevPlan& g) {
+  const cplx<T>* src = static_cast<const cplx<T>*>(g.tw);
+  for (int t = threadIdx.x; t < N; t += THR) {
+    const cplx<T> w = src[(t / R) * (t % R)];
+    tw[t] = SIGN < 0 ? w : cmake<T>(w.x, -w.y);
+  }
+}
+
 // One task of the forward plane pass: plane i1 of chain `ch`, whose transform
-// buffer is Hc.  Shared memory: Geo::SMEM_PLANE bytes at smem_raw.
-template <class T, int N, int MAXT, int EMAX = 0>
+// buffer is Hc.  Shared memory: PairGeo::SMEM_PLANE bytes at smem_raw.
+template <class T, int N, int THR, int TILE = 0>
 __device__ __forceinline__ void pair_fwd_task(const DevPlan& g, const T* __restrict__ psi,
                                               const Chain& ch, cplx<T>* __restrict__ Hc, int i1,
                                               unsigned char* smem_raw) {
   using C = cplx<T>;
-  using G = Geo<T, N, MAXT, EMAX>;
-  constexpr int RP = G::RP, KH = G::KH, NC = G::NC;
+  using G = PairGeo<T, N, TILE>;
+  constexpr int RP = G::RP, A = G::A, B = G::B;
   C* P = reinterpret_cast<C*>(smem_raw);
   C* tw = P + N * RP;
-  load_twiddles<T>(tw, g);
+  constexpr int M = G::M;
+  load_stage_twiddles<T, -1, G::BLOCK ? 4 : B, N, THR>(tw, g);
+  if constexpr (G::BLOCK) load_stage_twiddles<T, -1, M, N, THR>(tw + N, g);
   const int64_t plane0 = (int64_t)i1 * N * N;
   const bool hb = ch.bi >= 0;
   const T* pai = psi + (int64_t)ch.ai * g.ntot + plane0;
   const T* paj = psi + (int64_t)ch.aj * g.ntot + plane0;
   const T* pbi = psi + (int64_t)(hb ? ch.bi : 0) * g.ntot + plane0;
   const T* pbj = psi + (int64_t)(hb ? ch.bj : 0) * g.ntot + plane0;
-  // Columns first: the first stage along i2 reads the pair product straight
-  // from the orbital planes (a warp's lines are consecutive columns i3, so the
-  // loads coalesce) and leaves its outputs in shared memory; then the rows.
-  // this thread's column i3 (line-fast mapping of the transform along i2)
-  const int c3 = threadIdx.x % N;
-  const T* qai = pai + c3;
-  const T* qaj = paj + c3;
-  const T* qbi = pbi + c3;
-  const T* qbj = pbj + c3;
+  // Columns (along i2) first: the first stage reads the pair product straight
+  // from the orbital planes (a warp's items are consecutive columns i3, so the
+  // loads coalesce); only its outputs enter shared memory.
+  constexpr int R0 = G::BLOCK ? M : A, J0 = N / R0;
+  const auto columns = [&](const auto& product) {
+#pragma unroll(kItemUnroll<T>)
+    for (int item0 = 0; item0 < N * J0; item0 += THR) {
+      const int item = item0 + threadIdx.x;
+      if ((N * J0) % THR == 0 || item < N * J0) {
+        const int b = item / N, l = item - b * N;
+        C x[R0];
+#pragma unroll
+        for (int r = 0; r < R0; ++r) x[r] = product(item + r * (J0 * N));  // element i2 = b + J0 r of column l
+        Dft<-1, T>::template run<R0>(x);
+#pragma unroll
+        for (int q = 0; q < R0; ++q) P[(b + J0 * q) * RP + l] = x[q];
+      }
+    }
+  };
   if (hb && ch.ai == ch.bi) {
     // the usual chain, pairs (i, j) and (i, j'): psi_i is read once
-    const auto product = [&](int, int i2) {
-      const T x = qai[i2 * N];
-      return cmake<T>(x * qaj[i2 * N], x * qbj[i2 * N]);
-    };
-    fft_lines_from<T, N, -1, N, G::TLP, 1, RP, MAXT, EMAX>(P, tw, product);  // along i2
+    columns([&](int e) {
+      const T x = pai[e];
+      return cmake<T>(x * paj[e], x * pbj[e]);
+    });
   } else {
-    const auto product = [&](int, int i2) {
-      return cmake<T>(qai[i2 * N] * qaj[i2 * N], hb ? qbi[i2 * N] * qbj[i2 * N] : T(0));
-    };
-    fft_lines_from<T, N, -1, N, G::TLP, 1, RP, MAXT, EMAX>(P, tw, product);  // along i2
+    columns([&](int e) { return cmake<T>(pai[e] * paj[e], hb ? pbi[e] * pbj[e] : T(0)); });
   }
-  // along i3: only the rows k2 that hold kept columns, [0, row_lo) and
-  // [N - row_hi, N) (the split below reads row k2 and its mirror N - k2, both in)
-  const int rlo = g.row_lo, nrows = g.row_lo + g.row_hi;
-  const auto row_off = [&](int l) { return (l < rlo ? l : l + (N - nrows)) * RP; };
-  fft_lines_rt<T, N, -1, G::TLP, 1, MAXT, EMAX>(P, tw, nrows, row_off);
-  C* Hp = Hc + (int64_t)i1 * N * NC;
-  // split by Hermitian symmetry over the list of kept columns (k2, k3): every
-  // lane busy, consecutive threads on consecutive k3 of a row
-  for (int e = threadIdx.x; e < g.nkept; e += blockDim.x) {
+  __syncthreads();
+  if constexpr (G::BLOCK) plane_block_pass<T, M, -1, THR, RP>(P, tw);
+  else stage_ct<T, B, -1, A, B * RP, RP, true, THR, N, 1>(P, tw);
+  // k2 is now at row G::row_place(k2); the rest of the transforms along i3
+  if constexpr (G::ALL_LINES) {
+    if constexpr (!G::BLOCK) stage_ct<T, A, -1, B, 1, B, false, THR, N, RP>(P, tw);
+    constexpr int R1 = G::BLOCK ? M : B;
+    stage_ct<T, R1, -1, N / R1, R1, 1, true, THR, N, RP>(P, G::BLOCK ? tw + N : tw);
+  } else {
+    // only the rows k2 that hold kept columns, in order of their places
+    int* rows = reinterpret_cast<int*>(tw + 2 * N);
+    const int nrows = g.row_lo + g.row_hi;
+    const RtDiv by(nrows);
+    for (int r = threadIdx.x; r < nrows; r += THR) rows[r] = __ldg(g.rowpos + TILE * N + r) * RP;
+    __syncthreads();
+    const auto row_off = [&](int l) { return rows[l]; };
+    if constexpr (!G::BLOCK) stage_rt<T, A, -1, B, 1, B, false, THR>(P, tw, nrows, by, row_off);
+    constexpr int R1 = G::BLOCK ? M : B;
+    stage_rt<T, R1, -1, N / R1, R1, 1, true, THR>(P, G::BLOCK ? tw + N : tw, nrows, by, row_off);
+  }
+  C* Hp = Hc + (int64_t)i1 * N * N;
+  // the kept columns (k2, k3), consecutive threads on consecutive k3 of a row
+  for (int e = threadIdx.x; e < g.nkept; e += THR) {
     const int code = __ldg(g.kept + e);
     const int k2 = code >> 16, k3 = code & 0xffff;
-    const int m2 = k2 == 0 ? 0 : N - k2, m3 = k3 == 0 ? 0 : N - k3;
-    const C z = P[k2 * RP + k3], zm = P[m2 * RP + m3];
-    Hp[k2 * NC + k3] = cmake<T>(half_of(z.x + zm.x), half_of(z.y - zm.y));
-    Hp[k2 * NC + KH + k3] = cmake<T>(half_of(z.y + zm.y), half_of(zm.x - z.x));
+    Hp[k2 * N + k3] = P[G::row_place(k2) * RP + G::col_place(k3)];
   }
 }
 
-template <class T, int N, int EMAX = 0>
-__global__ void __launch_bounds__(Geo<T, N, kMaxThreads, EMAX>::THR_PLANE)
+template <class T, int N, int TILE = 0>
+__global__ void __launch_bounds__(PairGeo<T, N, TILE>::THR_PLANE, PairGeo<T, N, TILE>::MIN_PLANE)
     k_pair_fwd(DevPlan g, const T* __restrict__ psi, const Chain* __restrict__ chains,
                cplx<T>* __restrict__ H) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const Chain ch = chains[blockIdx.y];
-  pair_fwd_task<T, N, kMaxThreads, EMAX>(g, psi, ch, H + (int64_t)blockIdx.y * g.hsize, blockIdx.x, smem_raw);
+  pair_fwd_task<T, N, PairGeo<T, N, TILE>::THR_PLANE, TILE>(g, psi, ch, H + (int64_t)blockIdx.y * g.hsize,
+                                                            blockIdx.x, smem_raw);
 }
 
 // Publish a CTA's energy partials (thread 0): atomically into the pair slots,
@@ -533,433 +613,373 @@ __device__ __forceinline__ void det_add(double* p, df64 v, double scale) {
 }
 __device__ __forceinline__ void det_add(float*, float, double) {}  // not offered for the mixed form
 
-// Line code of the column pass: (k2 << 16) | (s << 15) | k3, or -1 (no line).
+// Column code: (k2 << 16) | (self << 15) | k3 of a line pair's first line, or
+// -1 (no line); self: the line is its own mirror image (k2 and k3 both 0 or N/2).
 __device__ __forceinline__ int line_k2(int code) { return code >> 16; }
-__device__ __forceinline__ int line_s(int code) { return (code >> 15) & 1; }
+__device__ __forceinline__ int line_self(int code) { return (code >> 15) & 1; }
 __device__ __forceinline__ int line_k3(int code) { return code & 0x7fff; }
 
-// Asynchronous global-to-shared copies (cp.async) for the double-float
-// inverse plane pass of the stand-alone kernels: every element of a thread is
-// in flight at once, no register holds it.  Inside the persistent kernel the
-// loads stay ld.global.cg (the buffer was written earlier by the same launch,
-// so L1 must not serve it).
-constexpr bool kColAsync = true;
-// The column and inverse passes read their first transform stage straight from
-// the transform buffer (no staging pass through shared memory).  Measured at
-// 96^3: column pass -2..-6% in every form, inverse pass -13% (mixed) and -3%
-// (FP64) but +9% in double-float, whose inverse pass keeps the cp.async staging.
-constexpr bool kFirstStageDirect = true;
-template <class T> __host__ __device__ constexpr bool inv_first_stage_direct() {
-  return kFirstStageDirect && RealTraits<T>::prec != 2;
+// One kernel term of the smallest |m| (|m|^2 <= msmall2: 27 points per pair)
+// of the mixed-form column pass, in FP64: the values z at (k1, k2, k3) and y at
+// the mirror point.  Adds its energy terms (weight wgt) to the pair slots
+// itself and scales both values.  Kept out of line so the FP64 instructions are
+// not predicated into every warp of the kernel.
+template <class T, int N>
+__device__ __noinline__ void small_g_term_fp64(const DevPlan& g, cplx<T>* z, cplx<T>* y, int k1, int k2, int k3,
+                                               double wgt, const Chain& ch, double* epair, double* dpair) {
+  const int64_t vi = ((int64_t)k1 * N + k2) * (N / 2 + 1) + k3;
+  double zx = z->x, zy = z->y, yx = y->x, yy = y->y;
+  if (g.ovl != nullptr && k1 == 0 && k2 == 0 && k3 == 0) {
+    // G = 0: the sums of the two pair densities over the grid, from the FP64
+    // overlaps of the pairs' coefficients instead of the FP32 transform (real)
+    zx = g.ovl_scale * g.ovl[(int64_t)ch.ai * g.ovl_ld + (ch.aj - g.ovl_j0)];
+    zy = ch.bi >= 0 ? g.ovl_scale * g.ovl[(int64_t)ch.bi * g.ovl_ld + (ch.bj - g.ovl_j0)] : 0.0;
+    yx = zx;
+    yy = zy;
+  }
+  const double ax = zx + yx, ay = zy - yy, bx = zy + yy, by = yx - zx;  // 2 A and 2 B of the two densities
+  const double a2 = 0.25 * (ax * ax + ay * ay), b2 = 0.25 * (bx * bx + by * by);
+  const double v = g.vtab64[vi];
+  if (ch.pa >= 0) atomicAdd(&epair[ch.pa], wgt * v * a2);
+  if (ch.pb >= 0) atomicAdd(&epair[ch.pb], wgt * v * b2);
+  if (g.dvtab64) {
+    const double dv = g.dvtab64[vi];
+    if (ch.pa >= 0) atomicAdd(&dpair[ch.pa], wgt * dv * a2);
+    if (ch.pb >= 0) atomicAdd(&dpair[ch.pb], wgt * dv * b2);
+  }
+  const double vs = v * g.inv_ntot;
+  *z = cmake<T>(T(zx * vs), T(zy * vs));
+  *y = cmake<T>(T(yx * vs), T(yy * vs));
 }
 
-// Stage the column pass's line codes (NL a CTA) in shared memory.
-template <int NL>
-__device__ __forceinline__ void col_codes(const DevPlan& g, int cta, int* codes) {
-  for (int l = threadIdx.x; l < NL; l += blockDim.x) codes[l] = __ldg(g.colmap + cta * NL + l);
-  __syncthreads();
-}
-
-// The column of Hc (NC stored columns a row) that this thread's line of the
-// column pass reads and writes (the line-fast thread mapping of the
-// transforms: line tid mod NL), or NULL for a line without a code.  codes
-// must be staged.
-template <class C, int N, int NC, int NL>
-__device__ __forceinline__ C* col_line_ptr(C* Hc, const int* codes) {
-  constexpr int KH = NC / 2;
-  const int code = codes[threadIdx.x % NL];
-  return code >= 0 ? Hc + line_k2(code) * NC + line_s(code) * KH + line_k3(code) : nullptr;
-}
-
-// Store the transformed lines: thread (line l, sub-thread t) writes elements
-// i1 = t, t + TL, ... of its own line (consecutive lanes hold consecutive
-// lines, so both the shared reads and the global writes are contiguous).
-template <class C, int N, int NC, int NL, int TL>
-__device__ __forceinline__ void col_store_lines(C* lp, const C* S) {
-  const int l = threadIdx.x % NL, t = threadIdx.x / NL;
-  if (lp != nullptr && t < TL) {
-#pragma unroll 4
-    for (int i1 = t; i1 < N; i1 += TL) lp[(int64_t)i1 * N * NC] = S[i1 * NL + l];
+// Kernel multiply and energy partials of one item of the column pass: the B
+// frequencies k1 = q + A s of a line (z) and of its mirror image (y, block
+// (A - q) mod A, where -k1 is element (B - 1 - s), or (B - s) mod B for q = 0).
+// With Z = FFT(rho_a + i rho_b), 2 A = Z(k) + Z(-k)* and 2 B = -i (Z(k) -
+// Z(-k)*) are the transforms of the two real densities: e_a += v |2A|^2,
+// e_b += v |2B|^2 (acc 0 and 1; 2 and 3 with dv/domega), both without
+// cancellation.  v: kernel values the energies take, vs: the ones that scale.
+template <class T, int B, bool Q0, class V>
+__device__ __forceinline__ void mirror_multiply(cplx<T>* z, cplx<T>* y, const V& kernel, T acc[4]) {
+#pragma unroll
+  for (int s = 0; s < B; ++s) {
+    cplx<T>& Z = z[s];
+    cplx<T>& Y = y[Q0 ? (B - s) % B : B - 1 - s];
+    const T ax = Z.x + Y.x, ay = Z.y - Y.y, bx = Z.y + Y.y, by = Y.x - Z.x;
+    const T a2 = ax * ax + ay * ay, b2 = bx * bx + by * by;
+    kernel(s, Z, Y, a2, b2, acc);
   }
 }
 
-// The column pass in double-float arithmetic: the df64 tables of v / Ntot and
-// dv/domega, per-thread double-float energy sums that are reduced (in FP64)
-// before the inverse transform, so they hold no registers across it.
-template <int N, int MAXT, int EMAX = 0>
-__device__ __forceinline__ void pair_col_task_df(const DevPlan& g, cdf64* __restrict__ Hc, const Chain& ch,
-                                                 int cta, double* __restrict__ epair, double* __restrict__ dpair,
-                                                 unsigned char* smem_raw) {
-  using C = cdf64;
-  using G = Geo<df64, N, MAXT, EMAX>;
-  constexpr int KH = G::KH, NC = G::NC, NL = G::NLC;
-  C* S = reinterpret_cast<C*>(smem_raw);
-  C* tw = S + N * NL;
-  double* red = reinterpret_cast<double*>(tw + G::TWN);
-  int* codes = reinterpret_cast<int*>(red + 32 * 4);
-  load_twiddles<df64>(tw, g);
-  const bool want_d = g.dvtab64 != nullptr;
-  const df64* vt = static_cast<const df64*>(g.vtab);  // v / Ntot
-  const df64* dvt = static_cast<const df64*>(g.dvtab);  // dv/domega
-  col_codes<NL>(g, cta, codes);
-  {
-    const C* lp = col_line_ptr<C, N, NC, NL>(Hc, codes);
-    const auto val = [&](int, int i1) {
-      C v;
-      if (lp != nullptr) {
-        v = ldcg_c(lp + (int64_t)i1 * N * NC);
-      } else {
-        v.x = df64(0.f);
-        v.y = df64(0.f);
-      }
-      return v;
-    };
-    fft_lines_from<df64, N, -1, NL, G::TLC, 1, NL, MAXT, EMAX>(S, tw, val);  // along i1
-  }
-  {
-    df64 accd[4] = {df64(0.f), df64(0.f), df64(0.f), df64(0.f)};
-    // one line per thread (decoded once), walking k1
-    const int l = threadIdx.x % NL, kstep = blockDim.x / NL;
-    const int code = threadIdx.x < kstep * NL ? codes[l] : -1;
-    if (code >= 0) {
-      const int k2 = line_k2(code), s = line_s(code), k3 = line_k3(code);
-      const float wgt = (k3 == 0 || 2 * k3 == N) ? 1.0f : 2.0f;
-      df64 e_sum(0.f), d_sum(0.f);
-      for (int k1 = threadIdx.x / NL; k1 < N; k1 += kstep) {
-        const int e = k1 * NL + l;
-        const int vi = (k1 * N + k2) * KH + k3;
-        C z = S[e];
-        const df64 a2 = z.x * z.x + z.y * z.y;
-        const df64 v = vt[vi];
-        e_sum += v * a2;
-        if (want_d) d_sum += dvt[vi] * a2;
-        z.x *= v;
-        z.y *= v;
-        S[e] = z;
-      }
-      e_sum = ldexp_pow2(e_sum, wgt);
-      d_sum = ldexp_pow2(d_sum, wgt);
-      if (s) {
-        accd[1] = e_sum;
-        accd[3] = d_sum;
-      } else {
-        accd[0] = e_sum;
-        accd[2] = d_sum;
-      }
-    }
-    block_sum4_df(accd, reinterpret_cast<float*>(red));  // synchronises the CTA
-    if (threadIdx.x == 0) {
-      const double ntot = double(g.ntot);  // the energy table holds v / Ntot
-      const double acc[4] = {to_double(accd[0]) * ntot, to_double(accd[1]) * ntot, to_double(accd[2]),
-                             to_double(accd[3])};
-      put_energies(g, ch, cta, acc, want_d, epair, dpair);
-    }
-  }
-  fft_lines<df64, N, +1, NL, G::TLC, 1, NL, MAXT, EMAX>(S, tw);  // inverse along k1
-  col_store_lines<C, N, NC, NL, G::TLC>(col_line_ptr<C, N, NC, NL>(Hc, codes), S);
-}
-
-// The column pass in FP64 or in the mixed form.
-template <class T, int N, int MAXT, int EMAX = 0>
-__device__ __forceinline__ void pair_col_task_std(const DevPlan& g, cplx<T>* __restrict__ Hc,
-                                                  const Chain& ch, int cta, double* __restrict__ epair,
-                                                  double* __restrict__ dpair, unsigned char* smem_raw) {
+// One task of the column pass: the NP line pairs `cta` of the column map for
+// chain `ch` (transform buffer Hc).  The forward transform's B-stage, the
+// kernel multiply and the inverse transform's B-stage work on the same B
+// values of a line and of its mirror image, so they run in registers: a line
+// passes through shared memory twice (after the forward A-stage, which reads
+// global memory, and before the inverse one, which writes it).  Shared memory:
+// PairGeo::SMEM_COL bytes at smem_raw.
+template <class T, int N, int THR, int TILE = 0>
+__device__ __forceinline__ void pair_col_task(const DevPlan& g, cplx<T>* __restrict__ Hc, const Chain& ch, int cta,
+                                              double* __restrict__ epair, double* __restrict__ dpair,
+                                              unsigned char* smem_raw) {
   using C = cplx<T>;
-  using G = Geo<T, N, MAXT, EMAX>;
-  constexpr int KH = G::KH, NC = G::NC, NL = G::NLC;
+  using G = PairGeo<T, N, TILE>;
+  constexpr int A = G::CA, B = G::CB, NP = G::NP, NL = G::NL, KH = N / 2 + 1;
+  static_assert(THR % NL == 0, "a thread keeps one line of the A-stages");
+  constexpr int PREC = RealTraits<T>::prec;
   C* S = reinterpret_cast<C*>(smem_raw);
   C* tw = S + N * NL;
-  double* red = reinterpret_cast<double*>(tw + G::TWN);
-  int* codes = reinterpret_cast<int*>(red + 32 * 4);
-  load_twiddles<T>(tw, g);
-  col_codes<NL>(g, cta, codes);
-  {
-    // the first stage reads this thread's line straight from the transform
-    // buffer: one base pointer per thread, compile-time offsets per element
-    const C* lp = col_line_ptr<C, N, NC, NL>(Hc, codes);
-    const auto val = [&](int, int i1) {
-      C v;
-      if (lp != nullptr) {
-        v = ldcg_c(lp + (int64_t)i1 * N * NC);
-      } else {
-        v.x = 0;
-        v.y = 0;
-      }
-      return v;
-    };
-    fft_lines_from<T, N, -1, NL, G::TLC, 1, NL, MAXT, EMAX>(S, tw, val);  // along i1
+  double* red = reinterpret_cast<double*>(tw + 2 * N);
+  load_stage_twiddles<T, -1, B, N, THR>(tw, g);
+  load_stage_twiddles<T, +1, A, N, THR>(tw + N, g);
+  // this thread's line of the A-stages: l < NP a pair's first line, else its mirror image
+  const int l = threadIdx.x % NL;
+  const int lcode = __ldg(g.colmap + cta * NP + l % NP);
+  C* lp = nullptr;
+  if (lcode >= 0) {
+    const int k2 = line_k2(lcode), k3 = line_k3(lcode);
+    lp = Hc + (l < NP ? k2 * N + k3 : (k2 == 0 ? 0 : N - k2) * N + (k3 == 0 ? 0 : N - k3));
   }
-
-  // kernel multiply and energy partials
-  const bool want_d = g.dvtab64 != nullptr;
-  double acc[4] = {0.0, 0.0, 0.0, 0.0};  // e_a, e_b, d_a, d_b (FP64 terms)
-  float acc_f32[4] = {0.f, 0.f, 0.f, 0.f};  // the same from the FP32 terms (mixed form)
-  // one line per thread (decoded once), walking k1
-  const int l = threadIdx.x % NL, kstep = blockDim.x / NL;
-  const int code = threadIdx.x < kstep * NL ? codes[l] : -1;
-  if constexpr (RealTraits<T>::prec == 0) {
-    if (code >= 0) {
-      const int k2 = line_k2(code), s = line_s(code), k3 = line_k3(code);
-      const double wgt = (k3 == 0 || 2 * k3 == N) ? 1.0 : 2.0;
-      const double* v64 = g.vtab64 + k2 * KH + k3;
-      const double* dv64 = g.dvtab64 ? g.dvtab64 + k2 * KH + k3 : nullptr;
-      // v / Ntot, or -f0 v / Ntot when the occupations are uniform (vtab_f set)
-      const double* vs64 = static_cast<const double*>(g.vtab) + k2 * KH + k3;
-      double e_sum = 0.0, d_sum = 0.0;
-      for (int k1 = threadIdx.x / NL; k1 < N; k1 += kstep) {
-        const int e = k1 * NL + l;
-        const int vo = k1 * N * KH;
-        C z = S[e];
-        const double a2 = z.x * z.x + z.y * z.y;
-        e_sum += v64[vo] * a2;
-        if (want_d) d_sum += dv64[vo] * a2;
-        const double vs = vs64[vo];
-        z.x *= vs;
-        z.y *= vs;
-        S[e] = z;
+#pragma unroll(kItemUnroll<T>)
+  for (int b0 = 0; b0 < B; b0 += THR / NL) {
+    const int b = b0 + threadIdx.x / NL;
+    if (B % (THR / NL) == 0 || b < B) {
+      C x[A];
+#pragma unroll
+      for (int r = 0; r < A; ++r) {
+        if (lp != nullptr) x[r] = ldcg_c(lp + (int64_t)(b + B * r) * (N * N));
+        else x[r] = cmake<T>(T(0), T(0));
       }
-      if (s) {  // explicit selects: a runtime index would put acc in local memory
-        acc[1] = wgt * e_sum;
-        acc[3] = wgt * d_sum;
-      } else {
-        acc[0] = wgt * e_sum;
-        acc[2] = wgt * d_sum;
-      }
+      Dft<-1, T>::template run<A>(x);
+#pragma unroll
+      for (int q = 0; q < A; ++q) S[(b + B * q) * NL + l] = x[q];
     }
-  } else {
-    const T* vt = static_cast<const T*>(g.vtab);    // v / Ntot
-    const T* dvt = static_cast<const T*>(g.dvtab);  // dv/domega
-    T accf[4] = {T(0), T(0), T(0), T(0)};
-    if (code >= 0) {
-      const int k2 = line_k2(code), s = line_s(code), k3 = line_k3(code);
+  }
+  // this thread's line pair of the B-stages
+  const int p = threadIdx.x % NP;
+  const int code = __ldg(g.colmap + cta * NP + p);
+  const int k2 = code >= 0 ? line_k2(code) : 0, k3 = code >= 0 ? line_k3(code) : 0;
+  const int vo = k2 * KH + k3;
+  const bool want_d = g.dvtab64 != nullptr;
+  const T* vt = static_cast<const T*>(g.vtab) + vo;    // v / Ntot (or -f0 v / Ntot, FP64)
+  const T* dvt = static_cast<const T*>(g.dvtab) + vo;  // dv/domega
+  T acc[4] = {T(0), T(0), T(0), T(0)};
+  __syncthreads();
+  if constexpr (PREC == 2) {
+    // double-float: the same steps through shared memory.  Done in registers
+    // they are 10,000 unrolled instructions (11 an addition), beyond the
+    // instruction cache: 28.2 us a chain at 96^3 against 12.7 this way
+    stage_ct<T, B, -1, A, B * NL, NL, true, THR, NL, 1>(S, tw);
+    for (int e = threadIdx.x; e < NP * N; e += THR) {  // a thread keeps its pair: THR is a multiple of NP
+      const int k1 = e / NP, m1 = k1 == 0 ? 0 : N - k1;
+      C* pz = S + spec_pos<A, B>(k1) * NL + p;
+      C* py = S + spec_pos<A, B>(m1) * NL + NP + p;
+      C Z = *pz, Y = *py;
+      const T ax = Z.x + Y.x, ay = Z.y - Y.y, bx = Z.y + Y.y, by = Y.x - Z.x;
+      const T a2 = ax * ax + ay * ay, b2 = bx * bx + by * by;
+      const T v = vt[k1 * (N * KH)];
+      acc[0] += v * a2;
+      acc[1] += v * b2;
+      if (want_d) {
+        const T dv = dvt[k1 * (N * KH)];
+        acc[2] += dv * a2;
+        acc[3] += dv * b2;
+      }
+      Z.x *= v;
+      Z.y *= v;
+      Y.x *= v;
+      Y.y *= v;
+      *pz = Z;
+      *py = Y;
+    }
+    __syncthreads();
+    stage_ct<T, B, +1, A, B * NL, NL, false, THR, NL, 1>(S, tw);
+  } else
+  for (int item = threadIdx.x; item < NP * A; item += THR) {
+    const int q = item / NP, qm = q == 0 ? 0 : A - q;
+    C z[B], y[B];
+    T v[B];
+#pragma unroll
+    for (int s = 0; s < B; ++s) v[s] = vt[(q + A * s) * (N * KH)];
+#pragma unroll
+    for (int b = 0; b < B; ++b) {
+      z[b] = S[(B * q + b) * NL + p];
+      y[b] = S[(B * qm + b) * NL + NP + p];
+    }
+    dft_twiddled<T, B, -1>(z, tw + q * B);
+    dft_twiddled<T, B, -1>(y, tw + qm * B);
+    if constexpr (PREC == 0) {
+      const double* v64 = g.vtab64 + vo;
+      const double* dv64 = want_d ? g.dvtab64 + vo : nullptr;
+      const auto kernel = [&](int s, C& Z, C& Y, double a2, double b2, double* e) {
+        const int o = (q + A * s) * (N * KH);
+        const double ve = v64[o];
+        e[0] += ve * a2;
+        e[1] += ve * b2;
+        if (want_d) {
+          const double dv = dv64[o];
+          e[2] += dv * a2;
+          e[3] += dv * b2;
+        }
+        Z.x *= v[s];
+        Z.y *= v[s];
+        Y.x *= v[s];
+        Y.y *= v[s];
+      };
+      if (q == 0) mirror_multiply<T, B, true>(z, y, kernel, acc);
+      else mirror_multiply<T, B, false>(z, y, kernel, acc);
+    } else {
+      // the table holds v / Ntot, undone in FP64 after the CTA reduction
+      const auto kernel = [&](int s, C& Z, C& Y, T a2, T b2, T* e) {
+        e[0] += v[s] * a2;
+        e[1] += v[s] * b2;
+        if (want_d) {
+          const T dv = dvt[(q + A * s) * (N * KH)];
+          e[2] += dv * a2;
+          e[3] += dv * b2;
+        }
+        Z.x *= v[s];
+        Z.y *= v[s];
+        Y.x *= v[s];
+        Y.y *= v[s];
+      };
       const int m2 = freq_of(k2, N), m3 = freq_of(k3, N);
       const int r23 = m2 * m2 + m3 * m3;
-      const T wgt = (k3 == 0 || 2 * k3 == N) ? T(1) : T(2);
-      const T* vl = vt + k2 * KH + k3;
-      const T* dvl = dvt + k2 * KH + k3;
-      T e_sum = T(0), d_sum = T(0);
-      if (r23 > g.msmall2) {  // no term of this line is a small-|G| one
-        const int k10 = threadIdx.x / NL;
-        const T* vp = vl + k10 * N * KH;
-        const T* dvp = dvl + k10 * N * KH;
-        C* sp = S + k10 * NL + l;
-        const int vstep = kstep * N * KH, sstep = kstep * NL;
-        // batches of U elements: the U table loads are in flight together
-        constexpr int U = 8;
-        int k1 = k10;
-        for (; k1 + (U - 1) * kstep < N; k1 += U * kstep, vp += U * vstep, dvp += U * vstep, sp += U * sstep) {
-          T v[U], dv[U];
-          C z[U];
-#pragma unroll
-          for (int u = 0; u < U; ++u) {
-            v[u] = vp[u * vstep];
-            dv[u] = want_d ? dvp[u * vstep] : T(0);
-            z[u] = sp[u * sstep];
+      bool small = false;
+      {
+        // terms with |m|^2 <= msmall2 (at most 3, so |m1| <= 1: k1 = 0 and 1
+        // in element 0 of blocks 0 and 1, N - 1 in the last of block A - 1) in FP64
+        small = code >= 0 && r23 <= g.msmall2 && (q <= 1 || q == A - 1);
+        if (small) {
+          const double wgt = line_self(code) ? 1.0 : 2.0;
+          const bool first = q <= 1 && q * q + r23 <= g.msmall2;
+          const bool last = q == A - 1 && 1 + r23 <= g.msmall2;
+          const C zero = cmake<T>(T(0), T(0));
+          // the FP64 terms' values leave the arrays while the FP32 loop runs
+          C z0 = z[0], y0 = q == 0 ? y[0] : y[B - 1], z1 = z[B - 1], y1 = q == 0 ? y[1 % B] : y[0];
+          if (first) {
+            small_g_term_fp64<T, N>(g, &z0, &y0, q, k2, k3, wgt, ch, epair, dpair);
+            z[0] = zero;
+            if (q == 0) y[0] = zero;
+            else y[B - 1] = zero;
           }
-#pragma unroll
-          for (int u = 0; u < U; ++u) {
-            const T a2 = z[u].x * z[u].x + z[u].y * z[u].y;
-            e_sum += v[u] * a2;
-            d_sum += dv[u] * a2;
-            sp[u * sstep] = cmake<T>(z[u].x * v[u], z[u].y * v[u]);
+          if (last) {  // q = A - 1 > 0
+            small_g_term_fp64<T, N>(g, &z1, &y1, N - 1, k2, k3, wgt, ch, epair, dpair);
+            z[B - 1] = zero;
+            y[0] = zero;
           }
-        }
-        for (; k1 < N; k1 += kstep, vp += vstep, dvp += vstep, sp += sstep) {
-          C z = *sp;
-          const T a2 = z.x * z.x + z.y * z.y;
-          const T v = *vp;
-          e_sum += v * a2;
-          if (want_d) d_sum += *dvp * a2;
-          z.x *= v;
-          z.y *= v;
-          *sp = z;
-        }
-      } else {
-        for (int k1 = threadIdx.x / NL; k1 < N; k1 += kstep) {
-          const int e = k1 * NL + l;
-          const int m1 = freq_of(k1, N);
-          if (m1 * m1 + r23 <= g.msmall2) {
-            if (s == 0 || ch.bi >= 0) small_g_term_fp64<T, N>(g, S, e, k1, k2, k3, s, ch, epair, dpair);
-            continue;
+          if (q == 0) mirror_multiply<T, B, true>(z, y, kernel, acc);
+          else mirror_multiply<T, B, false>(z, y, kernel, acc);
+          if (first) {
+            z[0] = z0;
+            if (q == 0) y[0] = y0;
+            else y[B - 1] = y0;
           }
-          const int vo = k1 * N * KH;
-          C z = S[e];
-          const T a2 = z.x * z.x + z.y * z.y;
-          const T v = vl[vo];
-          e_sum += v * a2;
-          if (want_d) d_sum += dvl[vo] * a2;
-          z.x *= v;
-          z.y *= v;
-          S[e] = z;
+          if (last) {
+            z[B - 1] = z1;
+            y[0] = y1;
+          }
         }
       }
-      if (s) {
-        accf[1] = wgt * e_sum;
-        accf[3] = wgt * d_sum;
-      } else {
-        accf[0] = wgt * e_sum;
-        accf[2] = wgt * d_sum;
+      if (!small) {
+        if (q == 0) mirror_multiply<T, B, true>(z, y, kernel, acc);
+        else mirror_multiply<T, B, false>(z, y, kernel, acc);
       }
     }
-    // per-thread FP32 sums of at most N (N+2) / blockDim non-negative terms;
-    // the table holds v / Ntot, undone in FP64 after the CTA reduction
-    acc_f32[0] = accf[0];
-    acc_f32[1] = accf[1];
-    acc_f32[2] = accf[2];
-    acc_f32[3] = accf[3];
-  }
-  __syncthreads();
-  fft_lines<T, N, +1, NL, G::TLC, 1, NL, MAXT, EMAX>(S, tw);  // inverse along k1
-  col_store_lines<C, N, NC, NL, G::TLC>(col_line_ptr<C, N, NC, NL>(Hc, codes), S);
-  if constexpr (RealTraits<T>::prec != 1) {
-    block_sum4(acc, red);
-  } else {
-    float hi[4], lo[4];
-    block_sum4_ff(acc_f32, hi, lo, reinterpret_cast<float*>(red));
-    if (threadIdx.x == 0) {
-      const double ntot = double(g.ntot);  // the FP32 table holds v / Ntot
-      for (int k = 0; k < 4; ++k) acc[k] = ((double)hi[k] + (double)lo[k]) * (k < 2 ? ntot : 1.0);
+    Dft<+1, T>::template run<B>(z);
+    Dft<+1, T>::template run<B>(y);
+#pragma unroll
+    for (int b = 0; b < B; ++b) {
+      S[(B * q + b) * NL + p] = z[b];
+      S[(B * qm + b) * NL + NP + p] = y[b];
     }
   }
-  if (threadIdx.x == 0) put_energies(g, ch, cta, acc, want_d, epair, dpair);
-}
-
-// One task of the column pass: the NLC lines `cta` of the column map for chain
-// `ch` (transform buffer Hc).  Shared memory: Geo::SMEM_COLH bytes at smem_raw.
-template <class T, int N, int MAXT, int EMAX = 0>
-__device__ __forceinline__ void pair_col_task(const DevPlan& g, cplx<T>* __restrict__ Hc,
-                                              const Chain& ch, int cta, double* __restrict__ epair,
-                                              double* __restrict__ dpair, unsigned char* smem_raw) {
-  if constexpr (RealTraits<T>::prec == 2) {
-    pair_col_task_df<N, MAXT, EMAX>(g, Hc, ch, cta, epair, dpair, smem_raw);
+  // energies: each point and its mirror image counted once here (weight 2, a
+  // self-mirrored line 1), |2A|^2 = 4 |A|^2; the reduction's barrier is the one
+  // between the inverse transform's stages
+  const double wgt = code < 0 ? 0.0 : (line_self(code) ? 0.25 : 0.5);
+  double e4[4];
+  if constexpr (PREC == 0) {
+#pragma unroll
+    for (int k = 0; k < 4; ++k) e4[k] = wgt * acc[k];
+    block_sum4(e4, red);
+  } else if constexpr (PREC == 2) {
+    df64 a[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) a[k] = ldexp_pow2(acc[k], (float)wgt);
+    block_sum4_df(a, reinterpret_cast<float*>(red));
+    if (threadIdx.x == 0)
+      for (int k = 0; k < 4; ++k) e4[k] = to_double(a[k]) * (k < 2 ? double(g.ntot) : 1.0);
   } else {
-    pair_col_task_std<T, N, MAXT, EMAX>(g, Hc, ch, cta, epair, dpair, smem_raw);
+    float a[4], hi[4], lo[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) a[k] = (float)wgt * acc[k];
+    block_sum4_ff(a, hi, lo, reinterpret_cast<float*>(red));
+    if (threadIdx.x == 0)
+      for (int k = 0; k < 4; ++k) e4[k] = ((double)hi[k] + (double)lo[k]) * (k < 2 ? double(g.ntot) : 1.0);
+  }
+  if (threadIdx.x == 0) put_energies(g, ch, cta, e4, want_d, epair, dpair);
+  // inverse A-stage, straight to the transform buffer (a self-mirrored line's
+  // second copy is dropped)
+  if (lp != nullptr && !(l >= NP && line_self(lcode))) {
+#pragma unroll(kItemUnroll<T>)
+    for (int b0 = 0; b0 < B; b0 += THR / NL) {
+      const int b = b0 + threadIdx.x / NL;
+      if (B % (THR / NL) == 0 || b < B) {
+        C x[A];
+#pragma unroll
+        for (int q = 0; q < A; ++q) x[q] = S[(b + B * q) * NL + l];
+        dft_twiddled<T, A, +1>(x, tw + N + b * A);
+#pragma unroll
+        for (int r = 0; r < A; ++r) lp[(int64_t)(b + B * r) * (N * N)] = x[r];
+      }
+    }
   }
 }
 
-template <class T, int N, int EMAX = 0>
-__global__ void __launch_bounds__(Geo<T, N, kMaxThreads, EMAX>::THR_COL, Geo<T, N, kMaxThreads, EMAX>::MIN_CTAS_COL)
+template <class T, int N, int TILE = 0>
+__global__ void __launch_bounds__(PairGeo<T, N, TILE>::THR_COL, PairGeo<T, N, TILE>::MIN_COL)
     k_pair_col(DevPlan g, cplx<T>* __restrict__ H, const Chain* __restrict__ chains,
                double* __restrict__ epair, double* __restrict__ dpair) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const Chain ch = chains[blockIdx.y];
-  pair_col_task<T, N, kMaxThreads, EMAX>(g, H + (int64_t)blockIdx.y * g.hsize, ch, blockIdx.x, epair, dpair,
-                                         smem_raw);
+  pair_col_task<T, N, PairGeo<T, N, TILE>::THR_COL, TILE>(g, H + (int64_t)blockIdx.y * g.hsize, ch, blockIdx.x,
+                                                          epair, dpair, smem_raw);
 }
 
 // One task of the inverse plane pass: plane i1 of chain `ch` (transform buffer
-// Hc), accumulating into W.  Shared memory: Geo::SMEM_PLANE bytes at smem_raw.
-template <class T, int N, int MAXT, int EMAX = 0>
+// Hc), accumulating into W.  Shared memory: PairGeo::SMEM_PLANE bytes at
+// smem_raw.
+template <class T, int N, int THR, int TILE = 0>
 __device__ __forceinline__ void pair_inv_task(const DevPlan& g, const T* __restrict__ psi,
                                               acc_t<T>* __restrict__ W, const T* __restrict__ occ,
                                               const Chain& ch, const cplx<T>* __restrict__ Hc, int i1,
                                               unsigned char* smem_raw) {
   using C = cplx<T>;
-  using G = Geo<T, N, MAXT, EMAX>;
-  constexpr int KH = G::KH, NC = G::NC, NCP = G::NCP;
+  using G = PairGeo<T, N, TILE>;
+  constexpr int RP = G::RP, A = G::A, B = G::B;
   C* Q = reinterpret_cast<C*>(smem_raw);
-  C* tw = Q + N * NCP;
-  int* ncol = reinterpret_cast<int*>(tw + G::TWN);
-  load_twiddles<T>(tw, g);
-  for (int r = threadIdx.x; r < N; r += blockDim.x) ncol[r] = __ldg(g.ncol + r);
-  __syncthreads();
-  const C* Hp = Hc + (int64_t)i1 * N * NC;
-  // 1-2. the stored half plane, row k2 = [A(k2, 0..N/2) | B(k2, 0..N/2)],
-  //    columns no pair density reaches (never written) read as zero, and its
-  //    inverse transform along k2 into Q[k2][c] (odd row stride NCP).  Only
-  //    the columns k3 < col_max of A and B hold anything: 2 col_max lines are
-  //    transformed, line l being column l (A) or KH + l - col_max (B).
-  const int cm = g.col_max;
-  const auto col_of = [&](int l) { return l < cm ? l : KH + (l - cm); };
-  if constexpr (inv_first_stage_direct<T>()) {
-    const unsigned long long last_use = l2_policy_evict_first();  // H is dead after this read
-    const auto val = [&](int l, int k2) {
-      C v;
-      if ((l < cm ? l : l - cm) < ncol[k2]) {
-        v = ldcg_hint(Hp + k2 * NC + col_of(l), last_use);
-      } else {
-        v.x = 0;
-        v.y = 0;
-      }
-      return v;
-    };
-    fft_lines_from_rt<T, N, +1, G::TLC, NCP, MAXT, EMAX>(Q, tw, 2 * cm, val, col_of);
+  C* tw = Q + N * RP;
+  constexpr int M = G::M;
+  // first transform along k2: DFTs of RB values k2 = q + NA s, s < RB
+  constexpr int RB = G::BLOCK ? M : B, NA = N / RB;
+  load_stage_twiddles<T, +1, G::BLOCK ? 4 : A, N, THR>(tw, g);
+  load_stage_twiddles<T, +1, RB, N, THR>(tw + N, g);
+  const C* Hp = Hc + (int64_t)i1 * N * N;
+  // 1. inverse transform along k2 of the columns that hold something: k3 in
+  //    [0, col_max) and its mirror images.  Its first stage reads the transform
+  //    buffer (last use of it); a column's elements outside its kept rows
+  //    [0, up) and [N - dn, N) were never written and count as zero.
+  const unsigned long long last_use = l2_policy_evict_first();
+  const auto column = [&](int q, int k3) {
+    const int ud = __ldg(g.ncol + k3);
+    const int up = ud & 0xffff, dn = N - (ud >> 16);
+    C x[RB];
+#pragma unroll
+    for (int s = 0; s < RB; ++s) {
+      const int k2 = q + NA * s;
+      if (k2 < up || k2 >= dn) x[s] = ldcg_hint(Hp + k2 * N + k3, last_use);
+      else x[s] = cmake<T>(T(0), T(0));
+    }
+    Dft<+1, T>::template run<RB>(x);
+#pragma unroll
+    for (int b = 0; b < RB; ++b) Q[(G::BLOCK ? 4 * b + q : RB * q + b) * RP + k3] = x[b];
+  };
+  if constexpr (G::ALL_LINES) {
+#pragma unroll(kItemUnroll<T>)
+    for (int item0 = 0; item0 < N * NA; item0 += THR) {
+      const int item = item0 + threadIdx.x, q = item / N;
+      if ((N * NA) % THR == 0 || item < N * NA) column(q, item - q * N);
+    }
+    __syncthreads();
+    if constexpr (!G::BLOCK) stage_ct<T, A, +1, B, RP, B * RP, true, THR, N, 1>(Q, tw);
   } else {
-  if constexpr (kColAsync && MAXT == kMaxThreads) {
-    for (int e = threadIdx.x; e < N * NC; e += blockDim.x) {
-      const int k2 = e / NC, c = e - k2 * NC;
-      const int keep = (c < KH ? c : c - KH) < ncol[k2];
-      const unsigned dst = (unsigned)__cvta_generic_to_shared(Q + k2 * NCP + c);
-      asm volatile("cp.async.ca.shared.global [%0], [%1], %2, %3;" ::"r"(dst), "l"(Hp + e), "n"((int)sizeof(C)),
-                   "r"(keep ? (int)sizeof(C) : 0)
-                   : "memory");
+    const int cm = g.col_max;
+    const int nl = 2 * cm - 1 < N ? 2 * cm - 1 : N;
+    const auto k3_of = [&](int l) { return l < cm ? l : l + (N - nl); };
+    const RtDiv by(nl);
+    for (int item = threadIdx.x; item < nl * NA; item += THR) {
+      const int q = by.div(item);
+      column(q, k3_of(item - q * nl));
     }
-    asm volatile("cp.async.wait_all;" ::: "memory");
+    // the columns in between hold nothing
+    const int nz = N - nl;
+    for (int e = threadIdx.x; e < N * nz; e += THR) {
+      const int r = e / nz;
+      Q[r * RP + cm + (e - r * nz)] = cmake<T>(T(0), T(0));
+    }
+    __syncthreads();
+    if constexpr (!G::BLOCK) stage_rt<T, A, +1, B, RP, B * RP, true, THR>(Q, tw, nl, by, k3_of);
+  }
+  // 2. the rest along k2 and the rows: row i2 at place G::BLOCK ? 4 b + r for
+  //    i2 = b + M r : i2, Q[.][G::col_place(i3)] = phi_a + i phi_b
+  if constexpr (G::BLOCK) {
+    plane_block_pass<T, M, +1, THR, RP>(Q, tw);
+    stage_ct<T, M, +1, 4, M, 1, true, THR, N, RP>(Q, tw + N);
   } else {
-    for (int e0 = threadIdx.x; e0 < N * NC; e0 += kLoadUnroll * blockDim.x) {
-      C v[kLoadUnroll];
-#pragma unroll
-      for (int u = 0; u < kLoadUnroll; ++u) {
-        const int e = e0 + u * blockDim.x;
-        if (e < N * NC) {
-          const int k2 = e / NC, c = e - k2 * NC;
-          v[u] = ldcg_c(Hp + e);
-          if (!((c < KH ? c : c - KH) < ncol[k2])) v[u] = cmake<T>(T(0), T(0));
-        }
-      }
-#pragma unroll
-      for (int u = 0; u < kLoadUnroll; ++u) {
-        const int e = e0 + u * blockDim.x;
-        if (e < N * NC) {
-          const int k2 = e / NC, c = e - k2 * NC;
-          Q[k2 * NCP + c] = v[u];
-        }
-      }
-    }
+    stage_ct<T, A, +1, B, 1, B, false, THR, N, RP>(Q, tw);
+    stage_ct<T, B, +1, A, B, 1, true, THR, N, RP>(Q, tw + N);
   }
-  __syncthreads();
-  fft_lines_rt<T, N, +1, G::TLC, NCP, MAXT, EMAX>(Q, tw, 2 * cm, col_of);  // inverse transform along k2
-  }
-  // 3. rows: z(k3) = A^(k3) + i B^(k3) for k3 <= N/2 and, from the Hermitian
-  //    symmetry of the transforms of the real planes, z(N - k3) =
-  //    conj(A^(k3)) + i conj(B^(k3)); one warp per row (reads, then writes);
-  //    columns k3 >= col_max were not transformed and hold nothing
-  {
-    const int lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-    static_assert(N / 2 + 1 <= 64, "two stored columns per lane");
-    for (int i2 = threadIdx.x >> 5; i2 < N; i2 += nw) {
-      C* row = Q + i2 * NCP;
-      C av[2], bv[2];
-#pragma unroll
-      for (int t = 0; t < 2; ++t) {
-        const int k = lane + 32 * t;
-        if (k < cm) {
-          av[t] = row[k];
-          bv[t] = row[KH + k];
-        } else {
-          av[t] = cmake<T>(T(0), T(0));
-          bv[t] = av[t];
-        }
-      }
-      __syncwarp();
-#pragma unroll
-      for (int t = 0; t < 2; ++t) {
-        const int k = lane + 32 * t;
-        if (k < KH) {
-          row[k] = cmake<T>(av[t].x - bv[t].y, av[t].y + bv[t].x);
-          if (k > 0 && 2 * k < N) row[N - k] = cmake<T>(av[t].x + bv[t].y, bv[t].x - av[t].y);
-        }
-      }
-      __syncwarp();
-    }
-  }
-  __syncthreads();
-  // 4. inverse transform along k3 of the N rows: Q[i2][i3] = phi_a + i phi_b,
-  //    in FP32 with each row left in quad phases (element 4c + u of row i2 at
-  //    i2 NCP + u N/4 + c): the four-point groups of the accumulator update
-  //    are then read with consecutive lanes on consecutive addresses
-  constexpr int OMAP = (RealTraits<T>::prec == 1 && N % 4 == 0) ? 1 : 0;
-  fft_lines<T, N, +1, N, G::TLP, NCP, 1, MAXT, EMAX, OMAP>(Q, tw);
   const int64_t plane0 = (int64_t)i1 * N * N;
   const bool hb = ch.bi >= 0;
   // Up to four updates k, W[tgt_k] -= f[src_k] psi[src_k] phi:
@@ -1003,11 +1023,11 @@ __device__ __forceinline__ void pair_inv_task(const DevPlan& g, const T* __restr
       float* wj = wt[0];
       float* wj2 = wt[2];
       float* wi = wt[1];
-      for (int e4 = threadIdx.x; e4 < N * N / 4; e4 += blockDim.x) {
-        const int e = 4 * e4;
-        const int i2 = e4 / (N / 4), c = e4 - i2 * (N / 4);
-        const C* q = Q + i2 * NCP + c;  // quad phases: element 4c + u at u N/4 + c
-        const C z0 = q[0], z1 = q[N / 4], z2 = q[2 * (N / 4)], z3 = q[3 * (N / 4)];
+      for (int e4 = threadIdx.x; e4 < N * N / 4; e4 += THR) {
+        const int row = e4 / (N / 4), c = e4 - row * (N / 4);
+        const int e = G::row_of(row) * N + 4 * c;
+        const C* q = Q + row * RP + G::quad_place(c);
+        const C z0 = q[0], z1 = q[G::QUAD], z2 = q[2 * G::QUAD], z3 = q[3 * G::QUAD];
         const float4 vi = ld_f4_hint(pi + e, keep);
         const float4 vj = ld_f4_hint(pj + e, keep);
         const float4 vj2 = ld_f4_hint(pj2 + e, keep);
@@ -1027,13 +1047,13 @@ __device__ __forceinline__ void pair_inv_task(const DevPlan& g, const T* __restr
       }
       return;
     }
-    for (int e4 = threadIdx.x; e4 < N * N / 4; e4 += blockDim.x) {
-      const int e = 4 * e4;
-      const int i2 = e4 / (N / 4), cq = e4 - i2 * (N / 4);
+    for (int e4 = threadIdx.x; e4 < N * N / 4; e4 += THR) {
+      const int row = e4 / (N / 4), cq = e4 - row * (N / 4);
+      const int e = G::row_of(row) * N + 4 * cq;
       float4 phia, phib;
       {
-        const C* q = Q + i2 * NCP + cq;  // quad phases
-        const C z0 = q[0], z1 = q[N / 4], z2 = q[2 * (N / 4)], z3 = q[3 * (N / 4)];
+        const C* q = Q + row * RP + G::quad_place(cq);
+        const C z0 = q[0], z1 = q[G::QUAD], z2 = q[2 * G::QUAD], z3 = q[3 * G::QUAD];
         phia = make_float4(z0.x, z1.x, z2.x, z3.x);
         phib = make_float4(z0.y, z1.y, z2.y, z3.y);
       }
@@ -1074,9 +1094,27 @@ __device__ __forceinline__ void pair_inv_task(const DevPlan& g, const T* __restr
     const bool same_f = f[0] == f[1] && f[2] == f[3];
     // FP64: phi carries -f0 already (uniform occupations)
     const bool prescaled = RealTraits<T>::prec == 0 && g.vtab_f != nullptr;
-    for (int e = threadIdx.x; e < N * N; e += blockDim.x) {
+    // the usual chain, pairs (i, j) and (i, j') with i, j, j' distinct, both
+    // updates wanted, one occupation: four multiplications or multiply-adds a
+    // point (and one for -f each where phi does not carry it)
+    if (hb && !det && ch.ai == ch.bi && ch.ai != ch.aj && ch.ai != ch.bj && ch.aj != ch.bj &&
+        !(ch.flags & (kChainOneSidedA | kChainOneSidedB)) && (prescaled || (f[0] == f[1] && f[0] == f[3]))) {
+      const T m = -f[0];
+#pragma unroll 4
+      for (int e = threadIdx.x; e < N * N; e += THR) {
+        const int i2 = e / N, i3 = e - i2 * N;
+        C z = Q[G::place_of_row(i2) * RP + G::col_place(i3)];
+        if (!prescaled) z = cmake<T>(m * z.x, m * z.y);
+        const T xi = ps[0][e], xj = ps[1][e], xj2 = ps[3][e];
+        atomic_add_real(wt[0] + e, xi * z.x);
+        atomic_add_real(wt[2] + e, xi * z.y);
+        atomic_add_real(wt[1] + e, xj * z.x + xj2 * z.y);
+      }
+      return;
+    }
+    for (int e = threadIdx.x; e < N * N; e += THR) {
       const int i2 = e / N, i3 = e - i2 * N;
-      const C z = Q[i2 * NCP + i3];
+      const C z = Q[G::place_of_row(i2) * RP + G::col_place(i3)];
       T c[4];
       if (RealTraits<T>::prec == 0 && prescaled) {
 #pragma unroll
@@ -1103,14 +1141,14 @@ __device__ __forceinline__ void pair_inv_task(const DevPlan& g, const T* __restr
   }
 }
 
-template <class T, int N, int EMAX = 0>
-__global__ void __launch_bounds__(Geo<T, N, kMaxThreads, EMAX>::THR_COLH, Geo<T, N, kMaxThreads, EMAX>::MIN_CTAS)
+template <class T, int N, int TILE = 0>
+__global__ void __launch_bounds__(PairGeo<T, N, TILE>::THR_PLANE, PairGeo<T, N, TILE>::MIN_PLANE)
     k_pair_inv(DevPlan g, const T* __restrict__ psi, acc_t<T>* __restrict__ W, const T* __restrict__ occ,
                const Chain* __restrict__ chains, const cplx<T>* __restrict__ H) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const Chain ch = chains[blockIdx.y];
-  pair_inv_task<T, N, kMaxThreads, EMAX>(g, psi, W, occ, ch, H + (int64_t)blockIdx.y * g.hsize, blockIdx.x,
-                                         smem_raw);
+  pair_inv_task<T, N, PairGeo<T, N, TILE>::THR_PLANE, TILE>(g, psi, W, occ, ch, H + (int64_t)blockIdx.y * g.hsize,
+                                                            blockIdx.x, smem_raw);
 }
 
 // ------------------------------------------------------------ FFT tilings
@@ -1144,43 +1182,45 @@ template <class T, int N>
 struct Launch {
   using C = cplx<T>;
   using G = Geo<T, N>;
-  static constexpr int E1 = tile1_emax<T, N>();  // EMAX of tile 1 (0: tile 1 is tile 0)
-  using G1 = Geo<T, N, kMaxThreads, E1>;
+  using P0 = PairGeo<T, N, 0>;
+  // the second tiling of the pair passes, where one is compiled
+  static constexpr int T1 = (N == 96 && RealTraits<T>::prec != 2) ? 1 : 0;
+  using P1 = PairGeo<T, N, T1>;
 
   static cudaError_t configure(const DevPlan&) {
-    const void* fns[] = {(const void*)k_col_full<T, N, +1>, (const void*)k_col_full<T, N, -1>,
-                         (const void*)k_plane_full<T, N, +1, 0, 1>,
-                         (const void*)k_plane_full<T, N, -1, 1, 0>, (const void*)k_pair_fwd<T, N>,
-                         (const void*)k_pair_fwd<T, N, E1>};
-    for (const void* f : fns) {
-      cudaError_t err = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)G::SMEM_PLANE);
-      if (err != cudaSuccess) return err;
+    const auto smem = [](const void* f, size_t bytes) {
+      return cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    };
+    cudaError_t err = cudaSuccess;
+    for (const void* f : {(const void*)k_col_full<T, N, +1>, (const void*)k_col_full<T, N, -1>,
+                          (const void*)k_plane_full<T, N, +1, 0, 1>, (const void*)k_plane_full<T, N, -1, 1, 0>})
+      if (err == cudaSuccess) err = smem(f, G::SMEM_PLANE);
+    for (const void* f : {(const void*)k_pair_fwd<T, N>, (const void*)k_pair_inv<T, N>})
+      if (err == cudaSuccess) err = smem(f, P0::SMEM_PLANE);
+    if (err == cudaSuccess) err = smem((const void*)k_pair_col<T, N>, P0::SMEM_COL);
+    if constexpr (T1 == 1) {
+      for (const void* f : {(const void*)k_pair_fwd<T, N, T1>, (const void*)k_pair_inv<T, N, T1>})
+        if (err == cudaSuccess) err = smem(f, P1::SMEM_PLANE);
+      if (err == cudaSuccess) err = smem((const void*)k_pair_col<T, N, T1>, P1::SMEM_COL);
     }
-    for (const void* f : {(const void*)k_pair_inv<T, N>, (const void*)k_pair_inv<T, N, E1>}) {
-      cudaError_t err = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)G::SMEM_INV);
-      if (err != cudaSuccess) return err;
-    }
-    for (const void* f : {(const void*)k_pair_col<T, N>, (const void*)k_pair_col<T, N, E1>}) {
-      cudaError_t err = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)G::SMEM_COLH);
-      if (err != cudaSuccess) return err;
-    }
-    return cudaSuccess;
+    return err;
   }
 
-  // Radix plan of tile `tile` (0 or 1) of pass `pass` (0 forward plane, 1
-  // column, 2 inverse plane): stage radices, stage count, threads per line of
-  // the pass's first transform and threads per CTA.
+  // Tiling `tile` (0 or 1) of pass `pass` (0 forward plane, 1 column, 2 inverse
+  // plane): factors of a line, threads per line of the pass's first transform
+  // and threads per CTA.
   static int tile_plan(int pass, int tile, int* radices, int* nst, int* threads_per_line, int* threads) {
-    const RadixPlan pl = tile == 1 ? G1::pl : G::pl;
-    *nst = pl.nst;
-    for (int k = 0; k < pl.nst; ++k) radices[k] = pl.r[k];
-    const bool plane = pass == 0;
-    *threads_per_line = plane ? pl.tl_plane : pl.tl_colh;
-    const int thr_col = pass == 1 ? G::THR_COL : G::THR_COLH, thr_col1 = pass == 1 ? G1::THR_COL : G1::THR_COLH;
-    *threads = tile == 1 ? (plane ? G1::THR_PLANE : thr_col1) : (plane ? G::THR_PLANE : thr_col);
-    return E1 != 0 ? 2 : 1;
+    const bool plane = pass != 1, block = plane && (tile == 1 ? P1::BLOCK : P0::BLOCK);
+    const TwoFactor f = block ? TwoFactor{N / 4, 4} : plane ? (tile == 1 ? P1::f : P0::f)
+                                 : (tile == 1 ? TwoFactor{P1::CA, P1::CB} : TwoFactor{P0::CA, P0::CB});
+    *nst = 2;
+    radices[0] = f.a;
+    radices[1] = f.b;
+    *threads = plane ? (tile == 1 ? P1::THR_PLANE : P0::THR_PLANE) : (tile == 1 ? P1::THR_COL : P0::THR_COL);
+    *threads_per_line = *threads / (plane ? N : P0::NL);
+    return T1 + 1;
   }
+  static int row_place(int tile, int k2) { return tile == 1 ? P1::row_place(k2) : P0::row_place(k2); }
 
   static cudaError_t to_real(const DevPlan& g, const double2* psiG, int nb, int band0, int nbat,
                              void* Xv, void* psiv, cudaStream_t s) {
@@ -1195,39 +1235,43 @@ struct Launch {
     return cudaGetLastError();
   }
 
+  template <int TILE>
+  static cudaError_t fwd_tile(const DevPlan& g, const void* psi, const Chain* ch, int nch, void* H, cudaStream_t s) {
+    using P = PairGeo<T, N, TILE>;
+    k_pair_fwd<T, N, TILE><<<dim3(N, nch), P::THR_PLANE, P::SMEM_PLANE, s>>>(g, static_cast<const T*>(psi), ch,
+                                                                             static_cast<C*>(H));
+    return cudaGetLastError();
+  }
   static cudaError_t pair_fwd(const DevPlan& g, const void* psi, const Chain* ch, int nch, void* H,
                               cudaStream_t s) {
-    if (E1 != 0 && g.tile[0] == 1)
-      k_pair_fwd<T, N, E1><<<dim3(N, nch), G1::THR_PLANE, G::SMEM_PLANE, s>>>(
-          g, static_cast<const T*>(psi), ch, static_cast<C*>(H));
-    else
-      k_pair_fwd<T, N><<<dim3(N, nch), G::THR_PLANE, G::SMEM_PLANE, s>>>(
-          g, static_cast<const T*>(psi), ch, static_cast<C*>(H));
-    return cudaGetLastError();
+    return T1 == 1 && g.tile[0] == 1 ? fwd_tile<T1>(g, psi, ch, nch, H, s) : fwd_tile<0>(g, psi, ch, nch, H, s);
   }
 
+  template <int TILE>
+  static cudaError_t col_tile(const DevPlan& g, void* H, const Chain* ch, int nch, double* ep, double* dp,
+                              cudaStream_t s) {
+    using P = PairGeo<T, N, TILE>;
+    k_pair_col<T, N, TILE><<<dim3(g.ncta_col, nch), P::THR_COL, P::SMEM_COL, s>>>(g, static_cast<C*>(H), ch, ep, dp);
+    return cudaGetLastError();
+  }
   static cudaError_t pair_col(const DevPlan& g, void* H, const Chain* ch, int nch, double* ep,
                               double* dp, cudaStream_t s) {
-    if (E1 != 0 && g.tile[1] == 1)
-      k_pair_col<T, N, E1><<<dim3(g.ncta_col, nch), G1::THR_COL, G::SMEM_COLH, s>>>(
-          g, static_cast<C*>(H), ch, ep, dp);
-    else
-      k_pair_col<T, N><<<dim3(g.ncta_col, nch), G::THR_COL, G::SMEM_COLH, s>>>(
-          g, static_cast<C*>(H), ch, ep, dp);
-    return cudaGetLastError();
+    return T1 == 1 && g.tile[1] == 1 ? col_tile<T1>(g, H, ch, nch, ep, dp, s) : col_tile<0>(g, H, ch, nch, ep, dp, s);
   }
 
+  template <int TILE>
+  static cudaError_t inv_tile(const DevPlan& g, const void* psi, void* W, const void* occ, const Chain* ch, int nch,
+                              const void* H, cudaStream_t s) {
+    using P = PairGeo<T, N, TILE>;
+    k_pair_inv<T, N, TILE><<<dim3(N, nch), P::THR_PLANE, P::SMEM_PLANE, s>>>(
+        g, static_cast<const T*>(psi), static_cast<acc_t<T>*>(W), static_cast<const T*>(occ), ch,
+        static_cast<const C*>(H));
+    return cudaGetLastError();
+  }
   static cudaError_t pair_inv(const DevPlan& g, const void* psi, void* W, const void* occ,
                               const Chain* ch, int nch, const void* H, cudaStream_t s) {
-    if (E1 != 0 && g.tile[2] == 1)
-      k_pair_inv<T, N, E1><<<dim3(N, nch), G1::THR_COLH, G::SMEM_INV, s>>>(
-          g, static_cast<const T*>(psi), static_cast<acc_t<T>*>(W), static_cast<const T*>(occ), ch,
-          static_cast<const C*>(H));
-    else
-      k_pair_inv<T, N><<<dim3(N, nch), G::THR_COLH, G::SMEM_INV, s>>>(
-          g, static_cast<const T*>(psi), static_cast<acc_t<T>*>(W), static_cast<const T*>(occ), ch,
-          static_cast<const C*>(H));
-    return cudaGetLastError();
+    return T1 == 1 && g.tile[2] == 1 ? inv_tile<T1>(g, psi, W, occ, ch, nch, H, s)
+                                     : inv_tile<0>(g, psi, W, occ, ch, nch, H, s);
   }
 
   static cudaError_t to_sphere(const DevPlan& g, const void* W, int nb, int band0, int nbat,
@@ -1242,9 +1286,9 @@ struct Launch {
   }
 
   static constexpr KernelOps ops() {
-    return KernelOps{(int)sizeof(T), RealTraits<T>::prec, N, G::NLC,
-                     smem_max(smem_max(G::SMEM_COLH, G::SMEM_PLANE), G::SMEM_INV),
-                     configure, to_real, pair_fwd, pair_col, pair_inv, to_sphere, tile_plan};
+    return KernelOps{(int)sizeof(T), RealTraits<T>::prec, N, P0::NP,
+                     smem_max(smem_max(P0::SMEM_COL, P0::SMEM_PLANE), G::SMEM_PLANE),
+                     configure, to_real, pair_fwd, pair_col, pair_inv, to_sphere, tile_plan, row_place};
   }
 };
 

@@ -27,17 +27,14 @@
 
 namespace fockx {
 
-// CTA size: enough for the 96^3 column pass (4 threads per line in FP32, 8 in FP64)
-template <class T> constexpr int kPersistMaxT = sizeof(T) == 8 ? 800 : 416;
+// CTA size: four threads a line of the 96^3 plane passes
+template <class T> constexpr int kPersistMaxT = 384;
 
 template <class T>
 struct PersistGeo {
   // largest dynamic shared memory over the grid sizes the persistent kernel runs
   static constexpr size_t smem_of(size_t a, size_t b) { return a > b ? a : b; }
-  static constexpr size_t SMEM = smem_of(
-      smem_of(smem_of(Geo<T, 96, kPersistMaxT<T>>::SMEM_PLANE, Geo<T, 96, kPersistMaxT<T>>::SMEM_COLH),
-              smem_of(Geo<T, 72, kPersistMaxT<T>>::SMEM_PLANE, Geo<T, 72, kPersistMaxT<T>>::SMEM_COLH)),
-      smem_of(Geo<T, 96, kPersistMaxT<T>>::SMEM_INV, Geo<T, 72, kPersistMaxT<T>>::SMEM_INV));
+  static constexpr size_t SMEM = smem_of(PairGeo<T, 96>::SMEM_PLANE, PairGeo<T, 96>::SMEM_COL);
   static constexpr int MIN_CTAS = sizeof(T) == 4 ? 2 : 1;  // shared memory allows 2 in FP32
 };
 

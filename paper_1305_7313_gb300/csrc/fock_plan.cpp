@@ -89,6 +89,7 @@ struct fock_plan {
   int* d_ncol = nullptr;
   int* d_colmap = nullptr;
   int* d_kept = nullptr;
+  int* d_rowpos = nullptr;
   // deterministic accumulation (fock_plan_set_deterministic)
   bool det = false;
   double vnorm = 0.0;          // ||v||_2 over the whole grid
@@ -445,6 +446,90 @@ fock_status prepare_prescaled(fock_plan* p, const double* occ, int nb, DevPlan* 
   dp->vtab_f = p->d_vtab_f;
   dp->vtab_f_factor = -f0;
   return FOCK_OK;
+}
+
+// The columns (k2, k3) of the pair densities' spectra that the pair passes keep.
+struct PairColumns {
+  std::vector<int> ncol;   // [N] per k3: k2 < (ncol & 0xffff) or k2 >= N - (ncol >> 16)
+  std::vector<int> kept;   // (k2 << 16) | k3, rows outer
+  std::vector<int> rowpos;  // [2][N] places of the kept rows in a transformed plane, ascending, per tiling
+  std::vector<int> pairs;  // (k2 << 16) | (self << 15) | k3 of one line of each mirror pair, rows outer
+  int64_t half_lines = 0;  // lines of the two densities' half spectra (k3 <= N/2) the ball marks
+  int row_lo = 0, row_hi = 0, col_max = 1;
+};
+
+void pair_columns(const fock_plan* p, PairColumns& out) {
+  const int n = p->n, kh = n / 2 + 1;
+  std::vector<unsigned char> mark((size_t)n * n, 0);
+  {
+    const double r2 = 8.0 * p->ecut * (1.0 + 1e-9);
+    int mb[3];
+    for (int a = 0; a < 3; ++a) {
+      const double* c = p->cell + 3 * a;
+      const double len = std::sqrt(c[0] * c[0] + c[1] * c[1] + c[2] * c[2]);
+      mb[a] = (int)std::floor(std::sqrt(r2) * len / (2.0 * kPi)) + 1;
+    }
+    for (int m1 = -mb[0]; m1 <= mb[0]; ++m1)
+      for (int m2 = -mb[1]; m2 <= mb[1]; ++m2)
+        for (int m3 = -mb[2]; m3 <= mb[2]; ++m3)
+          if (g2_of(p->recip, m1, m2, m3) <= r2)
+            mark[(size_t)(((m2 % n) + n) % n) * n + (((m3 % n) + n) % n)] = 1;
+  }
+  for (int k2 = 0; k2 < n; ++k2) {
+    int c = 0;
+    for (int k3 = 0; k3 < kh; ++k3)
+      if (mark[(size_t)k2 * n + k3]) c = k3 + 1;
+    out.half_lines += 2 * c;
+  }
+  // per column k3 <= N/2 the smallest runs k2 < up and k2 >= n - dn that cover
+  // the marked k2; the mirror column n - k3 keeps the mirror images.  Columns
+  // 0 and N/2 are their own mirror images: up = dn + 1 (k2 = 0 has no partner)
+  out.ncol.assign(n, 0);
+  for (int k3 = 0; k3 < kh; ++k3) {
+    int up = 0, dn = 0;
+    for (int k2 = 0; k2 < n; ++k2)
+      if (mark[(size_t)k2 * n + k3]) {
+        if (2 * k2 <= n) up = std::max(up, k2 + 1);
+        else dn = std::max(dn, n - k2);
+      }
+    if (up == 0 && dn == 0) continue;
+    up = std::max(up, 1);
+    if (k3 == 0 || 2 * k3 == n) {
+      up = std::max(up, dn + 1);
+      dn = up - 1;
+    }
+    out.ncol[k3] = up | (dn << 16);
+    if (k3 > 0 && 2 * k3 < n) out.ncol[n - k3] = (dn + 1) | ((up - 1) << 16);
+    out.col_max = std::max(out.col_max, k3 + 1);
+  }
+  const auto keeps = [&](int k2, int k3) {
+    return k2 < (out.ncol[k3] & 0xffff) || k2 >= n - (out.ncol[k3] >> 16);
+  };
+  for (int k3 = 0; k3 < n; ++k3) {
+    out.row_lo = std::max(out.row_lo, out.ncol[k3] & 0xffff);
+    out.row_hi = std::max(out.row_hi, out.ncol[k3] >> 16);
+  }
+  if (out.row_lo + out.row_hi >= n) {
+    out.row_lo = n;
+    out.row_hi = 0;
+  }
+  for (int t = 0; t < 2; ++t) {
+    std::vector<int> rows;
+    for (int k2 = 0; k2 < n; ++k2)
+      if (k2 < out.row_lo || k2 >= n - out.row_hi) rows.push_back(p->ops->row_place(t, k2));
+    std::sort(rows.begin(), rows.end());
+    rows.resize(n, 0);
+    out.rowpos.insert(out.rowpos.end(), rows.begin(), rows.end());
+  }
+  for (int k2 = 0; k2 < n; ++k2)
+    for (int k3 = 0; k3 < n; ++k3) {
+      if (!keeps(k2, k3)) continue;
+      out.kept.push_back((k2 << 16) | k3);
+      const int m2 = (n - k2) % n, m3 = (n - k3) % n;
+      const bool self = m2 == k2 && m3 == k3;
+      // the line with 0 < k3 < N/2, or of the two with k3 = 0 (N/2) the one with k2 <= N/2
+      if (k3 < m3 || (k3 == m3 && k2 <= m2)) out.pairs.push_back((k2 << 16) | (self ? 1 << 15 : 0) | k3);
+    }
 }
 
 int bands_per_grid_batch(const fock_plan* p) {
@@ -819,39 +904,17 @@ fock_status fock_plan_create(fock_plan_t* out, const int grid[3], const double c
         }
     p->vnorm = std::sqrt(s2);
   }
-  // Columns (k2, k3 <= N/2) of the half spectrum a pair density can reach.
-  // The product of two sphere orbitals has components only at |G| <= 2 Gmax,
-  // so the columns that the ball |G|^2 <= 8 Ecut hits (indices modulo N, so a
-  // grid that aliases the pair densities keeps what the aliases reach) are
-  // kept; the others hold rounding noise only and are never stored,
-  // transformed or read.  Row k2 keeps the prefix k3 < ncol[k2].
-  std::vector<int> ncol(n, 0);
-  {
-    const double r2 = 8.0 * ecut_ha * (1.0 + 1e-9);
-    int mb[3];
-    for (int a = 0; a < 3; ++a) {
-      const double len = std::sqrt(cell[3 * a] * cell[3 * a] + cell[3 * a + 1] * cell[3 * a + 1] +
-                                   cell[3 * a + 2] * cell[3 * a + 2]);
-      mb[a] = (int)std::floor(std::sqrt(r2) * len / (2.0 * kPi)) + 1;
-    }
-    std::vector<unsigned char> mark((size_t)n * n, 0);
-    for (int m1 = -mb[0]; m1 <= mb[0]; ++m1)
-      for (int m2 = -mb[1]; m2 <= mb[1]; ++m2)
-        for (int m3 = -mb[2]; m3 <= mb[2]; ++m3)
-          if (g2_of(p->recip, m1, m2, m3) <= r2)
-            mark[(size_t)(((m2 % n) + n) % n) * n + (((m3 % n) + n) % n)] = 1;
-    for (int k2 = 0; k2 < n; ++k2)
-      for (int k3 = 0; k3 < kh; ++k3)
-        if (mark[(size_t)k2 * n + k3]) ncol[k2] = k3 + 1;
-  }
-  std::vector<int> colmap, kept;
-  for (int k2 = 0; k2 < n; ++k2)
-    for (int s = 0; s < 2; ++s)
-      for (int k3 = 0; k3 < ncol[k2]; ++k3) colmap.push_back((k2 << 16) | (s << 15) | k3);
-  for (int k2 = 0; k2 < n; ++k2)
-    for (int k3 = 0; k3 < ncol[k2]; ++k3) kept.push_back((k2 << 16) | k3);
+  // Columns (k2, k3) a pair density can reach.  The product of two sphere
+  // orbitals has components only at |G| <= 2 Gmax, so the columns that the ball
+  // |G|^2 <= 8 Ecut hits (indices modulo N, so a grid that aliases the pair
+  // densities keeps what the aliases reach) are kept; the others hold rounding
+  // noise only and are never stored, transformed or read.
+  PairColumns cols;
+  pair_columns(p, cols);
+  p->kept_columns = cols.half_lines;
+  const std::vector<int>&ncol = cols.ncol, &kept = cols.kept;
+  std::vector<int>& colmap = cols.pairs;
   const int nlines = ops->col_lines;
-  p->kept_columns = (int64_t)colmap.size();
   const int ncta_col = std::max(1, (int)((colmap.size() + nlines - 1) / nlines));
   colmap.resize((size_t)ncta_col * nlines, -1);
 
@@ -888,6 +951,7 @@ fock_status fock_plan_create(fock_plan_t* out, const int grid[3], const double c
   if (ok)
     ok = upload((void**)&p->d_ncol, ncol.data(), sizeof(int) * ncol.size()) &&
          upload((void**)&p->d_colmap, colmap.data(), sizeof(int) * colmap.size()) &&
+         upload((void**)&p->d_rowpos, cols.rowpos.data(), sizeof(int) * cols.rowpos.size()) &&
          upload((void**)&p->d_kept, kept.data(), sizeof(int) * kept.size());
   if (ok) {
     if (fp64) {
@@ -953,23 +1017,11 @@ fock_status fock_plan_create(fock_plan_t* out, const int grid[3], const double c
   d.colmap = p->d_colmap;
   d.ncta_col = ncta_col;
   d.kept = p->d_kept;
+  d.rowpos = p->d_rowpos;
   d.nkept = (int)kept.size();
-  {
-    // kept rows as two runs [0, lo) and [n - hi, n); any other pattern keeps all rows
-    int lo = 0, hi = 0, cmax = 0;
-    while (lo < n && ncol[lo] > 0) ++lo;
-    while (hi < n - lo && ncol[n - 1 - hi] > 0) ++hi;
-    bool runs = true;
-    for (int k2 = lo; k2 < n - hi; ++k2) runs = runs && ncol[k2] == 0;
-    if (!runs) {
-      lo = n;
-      hi = 0;
-    }
-    for (int k2 = 0; k2 < n; ++k2) cmax = std::max(cmax, ncol[k2]);
-    d.row_lo = lo;
-    d.row_hi = hi;
-    d.col_max = std::max(1, cmax);
-  }
+  d.row_lo = cols.row_lo;
+  d.row_hi = cols.row_hi;
+  d.col_max = cols.col_max;
   d.det = 0;  // set per call on a copy when the plan is deterministic
   d.tile[0] = d.tile[1] = d.tile[2] = 0;
   d.det_scale = nullptr;
@@ -1544,6 +1596,7 @@ fock_status fock_destroy(fock_plan_t plan) {
   cudaFree(plan->d_ncol);
   cudaFree(plan->d_colmap);
   cudaFree(plan->d_kept);
+  cudaFree(plan->d_rowpos);
   cudaFree(plan->d_stats);
   cudaFree(plan->d_scale);
   cudaFree(plan->d_epart);
