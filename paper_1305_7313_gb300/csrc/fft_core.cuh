@@ -1,34 +1,22 @@
-// fft_core.cuh — batched mixed-radix (2, 3, 4, 8) Stockham FFT on lines held in
-// shared memory, specialised at compile time for one line length N.
+// fft_core.cuh — the transforms of the Fock apply: in-register DFTs of radix 2,
+// 3, 4 and 8 and of the composites 6, 9, 12, 16, 18 and 24, and the stages that
+// put them together on lines and planes held in shared memory, specialised at
+// compile time for one line length N.
 //
 // The 3D FFTs of the Fock apply (orbitals to real space, pair densities to G
 // space and back, V_x psi back to G space; §4 of the paper computes all of
 // them "via Fast Fourier Transform") are done as one pass over planes and one
-// pass over columns.  Inside a pass, every CTA owns whole lines in shared
-// memory and runs the Stockham autosort recursion on them:
-//
-//   stage (radix R, P = product of the radices of the earlier stages):
-//     for every butterfly b in [0, N/R):  k = b mod P
-//       x_r = in[b + r N/R] * w_N^(SIGN r k N/(PR)),   r = 0..R-1
-//       y   = DFT_R(x)                                  (exp(SIGN 2 pi i r q / R))
-//       out[(b - k) R + k + q P] = y_q,                 q = 0..R-1
-//
-// which leaves the result in natural order after the last stage.  A stage is
-// done in place: each thread loads all its butterfly inputs into registers,
-// the CTA synchronises, then the outputs are written back.  In float and
-// double the products x_r w are not rounded on their own but folded into the
+// pass over columns.  A line of N = A B points takes two stages, A-point DFTs
+// and B-point DFTs with twiddles on their inputs, each in place; the twiddle
+// products are not rounded on their own in float and double but folded into the
 // first butterfly sums as fused multiply-adds (Dft::run_tw).
 //
-// Thread mapping: thread `tid` works on line (tid mod NLINES) as sub-thread
-// (tid / NLINES) of TL sub-threads per line; consecutive threads therefore
-// touch consecutive lines, which keeps shared-memory accesses conflict-free
-// when lines are contiguous (column FFTs) or when the line stride is odd
-// (row FFTs with a padded stride).  Sub-thread t owns butterflies t, t + TL, ...
-// of every stage, so it holds N / TL elements between the two barriers.
+// Thread mapping: consecutive threads take consecutive lines, which keeps
+// shared-memory accesses conflict-free when lines are contiguous (columns) or
+// when the line stride is odd (rows with a padded stride).
 //
 // Twiddles come from a table w[t] = exp(-2 pi i t / N), t < N, computed on the
-// host in FP64 and staged in shared memory together with its conjugate
-// (tw[N + t]), which the SIGN = +1 transforms read.
+// host in FP64; a kernel stages the N products a stage reads in shared memory.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -44,9 +32,7 @@
 namespace fockx {
 
 constexpr int kMaxStages = 8;
-// The shared-memory twiddle table holds the forward table e^{-2 pi i t/N}
-// (t < N) followed by its conjugate for the inverse transforms.
-constexpr int kTwiddleTable = 2;
+constexpr int kTwiddleTable = 2;  // forward and inverse twiddles
 constexpr int kMaxThreads = 1024;
 constexpr int kEmax = 24;  // elements a thread may hold across a stage
 
@@ -504,158 +490,6 @@ template <int SIGN, class T> struct Dft {
     else composite<4, 4>(x);  // R == 16
   }
 };
-
-// Position of output element k of a line in shared memory: OMAP 0 natural
-// order; OMAP 1 "quad phases": the line is stored as four runs of N/4, run
-// k mod 4 holding elements k mod 4, k mod 4 + 4, ... (so that element 4c + u
-// sits at u N/4 + c).  Only the last stage of a transform applies a map.
-template <int N, int OMAP> FFT_HD constexpr int out_pos(int k) {
-  if constexpr (OMAP == 1) return (k & 3) * (N / 4) + (k >> 2);
-  else return k;
-}
-
-// One Stockham stage on one line (base, element stride ES) for sub-thread t of TL.
-template <class T, int N, int R, int P, int TL, int ES, int SIGN, int OMAP = 0>
-__device__ __forceinline__ void fft_stage(cplx<T>* base, int t, bool active, const cplx<T>* tw) {
-  using C = cplx<T>;
-  constexpr int NB = N / R;
-  constexpr int PER = NB / TL;
-  constexpr int TWS = N / (P * R);
-  const C* twt = SIGN > 0 ? tw + N : tw;  // the conjugate table for inverse transforms
-  C x[PER][R];
-  if (active) {
-#pragma unroll
-    for (int k = 0; k < PER; ++k) {
-      const int b = t + TL * k;
-#pragma unroll
-      for (int r = 0; r < R; ++r) x[k][r] = base[(b + r * NB) * ES];
-    }
-  }
-  __syncthreads();
-  if (active) {
-#pragma unroll
-    for (int k = 0; k < PER; ++k) {
-      const int b = t + TL * k;
-      const int kk = b % P;
-      if constexpr (P > 1 && FftTraits<T>::fused) {
-        C w[R];
-#pragma unroll
-        for (int r = 1; r < R; ++r) w[r] = twt[r * kk * TWS];
-        w[0] = w[1];  // not read: x_0 carries no twiddle
-        Dft<SIGN, T>::template run_tw<R, false>(x[k], w);
-      } else {
-        if constexpr (P > 1) {
-#pragma unroll
-          for (int r = 1; r < R; ++r) x[k][r] = cmul(x[k][r], twt[r * kk * TWS]);
-        }
-        Dft<SIGN, T>::template run<R>(x[k]);
-      }
-      const int j = (b - kk) * R + kk;
-#pragma unroll
-      for (int q = 0; q < R; ++q) base[out_pos<N, OMAP>(j + q * P) * ES] = x[k][q];
-    }
-  }
-  __syncthreads();
-}
-
-// The first stage (P = 1, no twiddles) with its inputs taken from a loader
-// (element m of line `line`: load(line, m)) instead of shared memory: the
-// caller's data never pass through shared memory before the transform.
-template <class T, int N, int R, int TL, int ES, int SIGN, class Load>
-__device__ __forceinline__ void fft_stage_first(cplx<T>* base, int t, bool active, int line, const Load& load) {
-  using C = cplx<T>;
-  constexpr int NB = N / R;
-  constexpr int PER = NB / TL;
-  C x[PER][R];
-  if (active) {
-#pragma unroll
-    for (int k = 0; k < PER; ++k) {
-      const int b = t + TL * k;
-#pragma unroll
-      for (int r = 0; r < R; ++r) x[k][r] = load(line, b + r * NB);
-    }
-  }
-  if (active) {
-#pragma unroll
-    for (int k = 0; k < PER; ++k) {
-      const int b = t + TL * k;
-      Dft<SIGN, T>::template run<R>(x[k]);
-#pragma unroll
-      for (int q = 0; q < R; ++q) base[(b * R + q) * ES] = x[k][q];
-    }
-  }
-  __syncthreads();
-}
-
-template <class T, int N, int SIGN, int TL, int ES, int S, int P, int MAXT, int EMAX = 0, int OMAP = 0>
-__device__ __forceinline__ void fft_stages(cplx<T>* base, int t, bool active, const cplx<T>* tw) {
-  constexpr RadixPlan pl = make_radix_plan(N, MAXT, plan_emax<T, EMAX>());
-  if constexpr (S < pl.nst) {
-    constexpr int R = pl.r[S];
-    fft_stage<T, N, R, P, TL, ES, SIGN, (S + 1 == pl.nst) ? OMAP : 0>(base, t, active, tw);
-    fft_stages<T, N, SIGN, TL, ES, S + 1, P * R, MAXT, EMAX, OMAP>(base, t, active, tw);
-  }
-}
-
-// FFT of NLINES lines of length N whose input comes from load(line, m) and
-// whose output lands in shared memory (line l at buf + l*LS, stride ES).
-template <class T, int N, int SIGN, int NLINES, int TL, int LS, int ES, int MAXT, int EMAX = 0, class Load>
-__device__ __forceinline__ void fft_lines_from(cplx<T>* buf, const cplx<T>* tw, const Load& load) {
-  constexpr RadixPlan pl = make_radix_plan(N, MAXT, plan_emax<T, EMAX>());
-  constexpr int R0 = pl.r[0];
-  const int tid = threadIdx.x;
-  const int line = tid % NLINES;
-  const int t = tid / NLINES;
-  const bool active = t < TL;
-  fft_stage_first<T, N, R0, TL, ES, SIGN>(buf + line * LS, t, active, line, load);
-  fft_stages<T, N, SIGN, TL, ES, 1, R0, MAXT, EMAX>(buf + line * LS, t, active, tw);
-}
-
-// FFT of `nlines` lines (a run-time count) whose input comes from
-// load(line, m) and whose output lands in shared memory at buf + off(line)
-// (elements ES apart).  Consecutive threads take consecutive lines, as in
-// fft_lines_from; threads beyond nlines * TL idle, so whole warps drop out when
-// fewer lines are transformed.
-template <class T, int N, int SIGN, int TL, int ES, int MAXT, int EMAX = 0, class Load, class Off>
-__device__ __forceinline__ void fft_lines_from_rt(cplx<T>* buf, const cplx<T>* tw, int nlines, const Load& load,
-                                                  const Off& off) {
-  constexpr RadixPlan pl = make_radix_plan(N, MAXT, plan_emax<T, EMAX>());
-  constexpr int R0 = pl.r[0];
-  const int tid = threadIdx.x;
-  const int line = tid % nlines;
-  const int t = tid / nlines;
-  const bool active = t < TL;
-  cplx<T>* base = buf + off(line);
-  fft_stage_first<T, N, R0, TL, ES, SIGN>(base, t, active, line, load);
-  fft_stages<T, N, SIGN, TL, ES, 1, R0, MAXT, EMAX>(base, t, active, tw);
-}
-
-// FFT in place of `nlines` lines (a run-time count) in shared memory, line l
-// at buf + off(l), elements ES apart; as fft_lines otherwise.
-template <class T, int N, int SIGN, int TL, int ES, int MAXT, int EMAX = 0, class Off>
-__device__ __forceinline__ void fft_lines_rt(cplx<T>* buf, const cplx<T>* tw, int nlines, const Off& off) {
-  const int tid = threadIdx.x;
-  const int line = tid % nlines;
-  const int t = tid / nlines;
-  const bool active = t < TL;
-  fft_stages<T, N, SIGN, TL, ES, 0, 1, MAXT, EMAX>(buf + off(line), t, active, tw);
-}
-
-// FFT of NLINES lines of length N in shared memory: line l starts at buf + l*LS,
-// its elements are ES apart.  Every thread of the CTA must call this (it
-// synchronises); threads with tid >= NLINES*TL idle.
-// MAXT and EMAX name the radix plan (make_radix_plan(N, MAXT, plan_emax<T,
-// EMAX>())) that TL was chosen for.
-// OMAP: the order the last stage leaves the elements of a line in (out_pos).
-template <class T, int N, int SIGN, int NLINES, int TL, int LS, int ES, int MAXT = kMaxThreads, int EMAX = 0,
-          int OMAP = 0>
-__device__ __forceinline__ void fft_lines(cplx<T>* buf, const cplx<T>* tw) {
-  const int tid = threadIdx.x;
-  const int line = tid % NLINES;
-  const int t = tid / NLINES;
-  const bool active = t < TL;
-  fft_stages<T, N, SIGN, TL, ES, 0, 1, MAXT, EMAX, OMAP>(buf + line * LS, t, active, tw);
-}
 
 // ------------------------------------------------ two-factor transforms in place
 //

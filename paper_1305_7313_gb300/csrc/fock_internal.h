@@ -23,6 +23,32 @@ struct Chain {
 constexpr int kChainOneSidedA = 1;
 constexpr int kChainOneSidedB = 2;
 
+// The columns (k2, k3) of a spectrum that hold something (device pointers).
+// Column k3 (0 .. N-1) keeps k2 < (ncol[k3] & 0xffff) and k2 >= N - (ncol[k3]
+// >> 16); columns no line of which is kept, and the other k2, are never stored,
+// transformed or read.
+struct ColumnSet {
+  const int* ncol;
+  // the column passes' lines, ncta CTAs of them: (k2 << 16) | (self << 15) | k3,
+  // or -1 (none).  Gamma point: the set is closed under (k2, k3) -> (-k2, -k3)
+  // and an entry stands for a line (k3 <= N/2) and its mirror image (self: the
+  // line is its own); k points: an entry is one line.
+  const int* lines;
+  int ncta;
+  // kept rows k2 lie in [0, row_lo) and [N - row_hi, N), kept columns k3 in
+  // [0, col_lo) and [N - col_hi, N)
+  int row_lo, row_hi, col_lo, col_hi;
+  // the kept rows' places in a plane transformed along i2, ascending: [2][N],
+  // per tiling (the factors fix the order)
+  const int* rowpos;
+  // the kept columns (k2 << 16) | k3, rows outer (nkept entries)
+  const int* kept;
+  int nkept;
+  // sphere sets: position of the coefficient at (k1, line) in the sphere, or
+  // -1, at (cta N + k1) slots + slot (slots: lines a CTA holds in shared memory)
+  const int* coef;
+};
+
 // Everything a kernel needs to know about a plan (device pointers included).
 struct DevPlan {
   int n;            // cubic grid N
@@ -30,8 +56,6 @@ struct DevPlan {
   int64_t ntot;     // N^3
   int64_t hsize;    // elements reserved per pair-transform buffer (at least N^3: [i1][k2][k3])
   int npw;
-  const int* gidx;     // [npw] grid offset of G
-  const int* gidxneg;  // [npw] grid offset of -G
   const void* tw;      // [N] exp(-2 pi i t / N) in the working precision
   const void* vtab;    // [N][N][k3h] v(G) / Ntot in the working precision
   const double* vtab64;   // [N][N][k3h] v(G) in FP64
@@ -41,29 +65,13 @@ struct DevPlan {
   double psi_scale;    // 1 / sqrt(Omega)
   double out_scale;    // sqrt(Omega) / Ntot
   int msmall2;         // |m|^2 at or below which kernel terms are done in FP64 (mixed form)
-  // Columns (k2, k3) that pair densities reach (Gamma point), a set closed under
-  // (k2, k3) -> (-k2, -k3): column k3 (0 .. N-1) keeps k2 < (ncol[k3] & 0xffff)
-  // and k2 >= N - (ncol[k3] >> 16).  The column pass takes them as pairs of a
-  // line and its mirror image, col_lines pairs per CTA, from colmap (ncta_col *
-  // col_lines entries, (k2 << 16) | (self << 15) | k3 of the line with k3 <= N/2,
-  // self: the line is its own mirror image; -1: none)
-  const int* ncol;
-  const int* colmap;
-  int ncta_col;
-  // rows k2 that have kept columns are [0, row_lo) and [N - row_hi, N); kept
-  // k3 are below col_max or mirror images of such
-  int row_lo, row_hi, col_max;
-  // the kept rows' places in a plane transformed along i2, ascending: [2][N],
-  // per tiling (the factors fix the order)
-  const int* rowpos;
-  // the kept columns (k2 << 16) | k3, rows outer (nkept entries)
-  const int* kept;
-  int nkept;
+  ColumnSet cols;  // columns the pair densities reach
+  ColumnSet orb;   // columns of the orbitals' sphere (Gamma point)
   // radix-plan variant ("tiling", 0 or 1) of the forward plane, column and
   // inverse plane passes
   int tile[3];
   // deterministic accumulation: W holds 64-bit fixed point scaled by det_scale[0]
-  // (= 2^s), the column pass stores per-CTA energy partials at [pair * ncta_col + cta]
+  // (= 2^s), the column pass stores per-CTA energy partials at [pair * cols.ncta + cta]
   int det;
   const double* det_scale;
   // Brillouin-zone sampling: full-grid tables [nq][N][N][N] of v(G + q)
@@ -99,7 +107,7 @@ struct KernelOps {
   int real_bytes;  // sizeof of the working real type
   int prec;        // 0 FP64, 1 mixed FP32, 2 double-float (fock_precision)
   int n;           // grid size these kernels are compiled for
-  int col_lines;   // line pairs of the column map a column-pass CTA takes
+  int col_pairs;   // line pairs a column-pass CTA takes
   size_t smem;     // largest dynamic shared memory of its kernels
   cudaError_t (*configure)(const DevPlan&);
   // c(G) of bands [band0, band0 + nbat) to psi(r); X is scratch of >= ceil(nbat/2) grids.
@@ -123,6 +131,10 @@ struct KernelOps {
   int (*tile_plan)(int pass, int tile, int* radices, int* nst, int* threads_per_line, int* threads);
   // row of the transformed plane that holds frequency k2 in the forward plane pass
   int (*row_place)(int tile, int k2);
+  // FP64: out(G) = FFT[vloc(r) IFFT c](G) on the sphere for bands [band0, band0 +
+  // nbat) of psiG (vloc real, [N][N][N]); NULL in the other forms
+  cudaError_t (*vloc)(const DevPlan&, const double2* psiG, int nb, int band0, int nbat, const double* vloc, void* X,
+                      double2* out, cudaStream_t);
 };
 
 // Kernels for grid size n and precision (0: FP64, 1: mixed); NULL if not built.
@@ -132,15 +144,17 @@ const KernelOps* find_kernel_ops(int prec, int n);
 // per transform; band0 is a global state index, psiG / vpsiG point at the
 // first band of the batch).
 struct KOps {
+  int col_lines;  // lines a column-pass CTA takes
   cudaError_t (*configure)();
-  cudaError_t (*to_real)(const DevPlan&, const double2* psiG, int npw, const int* gidx, int band0, int nbat,
+  // orb, npw: the columns and the size of one k point's sphere
+  cudaError_t (*to_real)(const DevPlan&, const ColumnSet& orb, const double2* psiG, int npw, int band0, int nbat,
                          void* X, void* u, cudaStream_t);
   cudaError_t (*pair_fwd)(const DevPlan&, const void* u, const Chain* ch, int nch, void* H, cudaStream_t);
   cudaError_t (*pair_col)(const DevPlan&, void* H, const Chain* ch, int nch, double* epair, cudaStream_t);
   cudaError_t (*pair_inv)(const DevPlan&, const void* u, void* W, const void* occw, const Chain* ch, int nch,
                           const void* H, cudaStream_t);
-  cudaError_t (*to_sphere)(const DevPlan&, const void* W, int band0, int nbat, int npw, const int* gidx,
-                           void* X, double2* vpsiG, cudaStream_t);
+  cudaError_t (*to_sphere)(const DevPlan&, const ColumnSet& orb, const void* W, int band0, int nbat, int npw, void* X,
+                           double2* vpsiG, cudaStream_t);
 };
 const KOps* find_kops(int prec, int n);
 
@@ -165,7 +179,7 @@ struct Segment {
   int dep;     // segment that must be complete first (-1: none)
   int dep2;    // second such segment (-1: none)
   int task0;   // first ticket
-  int ntasks;  // (N, or ncta_col for the column pass) * nch
+  int ntasks;  // (N, or cols.ncta for the column pass) * nch
   int pad;
 };
 
@@ -210,17 +224,18 @@ cudaError_t launch_det_to_double(void* w, int64_t n, const double* scale, cudaSt
 cudaError_t launch_det_pair_sums(const double* part, int npairs, int ncta, double* out, cudaStream_t s);
 
 // Sternheimer CG (fock_sternheimer.cu): kets are complex128 [m][npw], FP64.
-cudaError_t st_vmul(const double* v, const double* psi, double* w, int m, int64_t ntot, cudaStream_t s);
-cudaError_t st_dots(const double2* a, const double2* b, int m, int npw, double* out, cudaStream_t s);
+// part buffers: partial sums, at most st_chunks(npw) a band; c: [m][nocc].
+int st_chunks(int npw);
 cudaError_t st_proj_coef(const double2* u, int nocc, const double2* x, int m, int npw, double* c, cudaStream_t s);
+// b = -Q w, rr[n] = <b_n|b_n>
 cudaError_t st_rhs(const double2* w, const double2* u, const double* c, int nocc, int m, int npw, double2* b,
-                   cudaStream_t s);
+                   double* part, double* rr, cudaStream_t s);
 cudaError_t st_finish(double2* ap, const double2* p, const double* kin, const double* eps, const double2* u,
-                      const double* c, int nocc, double alpha, int m, int npw, cudaStream_t s);
-cudaError_t st_step(double2* x, double2* r, const double2* p, const double2* ap, const double* rr, const double* pap,
-                    int m, int npw, cudaStream_t s);
-cudaError_t st_dir(double2* p, const double2* r, const double* rr_new, const double* rr, int m, int npw,
-                   cudaStream_t s);
+                      const double* c, int nocc, double alpha, int m, int npw, double* part, cudaStream_t s);
+cudaError_t st_step(double2* x, double2* r, const double2* p, const double2* ap, const double* rr,
+                    const double* part_pap, int m, int npw, double* part_rr, cudaStream_t s);
+cudaError_t st_dir(double2* p, const double2* r, const double* part_rr, const double* rr, int m, int npw,
+                   double* rr_new, cudaStream_t s);
 cudaError_t st_gather_rows(const double2* src, double2* dst, const int* perm, int m, int npw, cudaStream_t s);
 cudaError_t st_gather_scalars(const double* src, double* dst, const int* perm, int m, cudaStream_t s);
 

@@ -6,29 +6,23 @@
 //   psi  [nb][N][N][N]  real T      orbitals in real space, psi(r) of §4
 //   W    [nb][N][N][N]  real A      accumulators of V_x psi_j(r) (A = T, or
 //                                   double for df64)
-//   H    [chain][N][N][2][N/2+1]    complex T: per plane i1 and row k2, the
-//        stored half (k3 <= N/2) of the 2D transforms of the two pair densities
-//        of a chain (index 0: pair a, 1: pair b)
-//   X    [q][N][N][N]   complex T   full grids for the O(nb) transforms
+//   H    [chain][N][N][N]    complex T: per plane i1 the kept columns (k2, k3)
+//        of the 2D transform of a chain's two pair densities
+//   X    [q][N][N][N]   complex T   the same for the O(nb) transforms
 //
 // Hot path per chain of two pairs (a = (ai, aj), b = (bi, bj)):
 //   pair_fwd  (plane i1):  z = psi_ai psi_aj + i psi_bi psi_bj, 2D FFT over
-//             (i2, i3) (columns first; the first stage forms z from the orbital
-//             planes in global memory), split z = A + iB by Hermitian symmetry
-//             (A, B are the transforms of real planes), store the kept columns
-//             of the k3 <= N/2 half of A and B.
-//   Every pass reads the first stage of its first transform straight from
-//   global memory (fft_lines_from), so no input is staged in shared memory
-//   (the double-float inverse pass stages its plane with cp.async instead).
-//   pair_col  (NC columns): FFT along i1 of the stored columns a pair density
-//             reaches (DevPlan::colmap: NC = 2 (N/2+1) lines per CTA), energy partials
-//             sum w(k3) v |A|^2 and sum w(k3) v |B|^2 (w = 1 on the k3 = 0, N/2
-//             planes, 2 elsewhere: the k3 > N/2 half is the mirror image), times
-//             v/Ntot, inverse FFT along k1.
-//   pair_inv  (plane i1):  inverse FFT along k2 of the stored half plane (A and B
-//             columns), rebuild each row z = A + iB over all k3 (the k3 > N/2
-//             half from the conjugates), inverse FFT along k3 -> phi_a + i phi_b, then
-//             W_aj -= f_ai psi_ai phi_a, W_ai -= f_aj psi_aj phi_a (i != j), same for b.
+//             (i2, i3), its first stage forming z from the orbital planes in
+//             global memory; the kept columns of the result go to H.
+//   pair_col  (column pairs):  FFT along i1 of a column and of its mirror image
+//             (-k2, -k3), which together hold the transforms of both real
+//             densities at k and -k: energy partials sum v |A|^2 and sum v
+//             |B|^2, times v/Ntot, inverse FFT along k1.
+//   pair_inv  (plane i1):  inverse 2D FFT of the kept columns -> phi_a + i phi_b,
+//             then W_aj -= f_ai psi_ai phi_a, W_ai -= f_aj psi_aj phi_a (i != j),
+//             same for b.
+// Every pass reads the first stage of its first transform straight from global
+// memory, so no input is staged in shared memory.
 #pragma once
 
 #include "fft_core.cuh"
@@ -168,7 +162,9 @@ __device__ inline void block_sum4_df(df64 v[4], float* red) {
 // Shared memory of one SM on sm_103 (228 KB; each resident CTA also reserves 1 KB).
 constexpr size_t kSmemPerSM = 233472;
 
-// Compile-time geometry of the passes for grid size N and radix-plan variant
+// Compile-time geometry of line transforms by radix plans (make_radix_plan; the
+// host checks print it; the passes' own geometry is PairGeo below) for grid size
+// N and radix-plan variant
 // EMAX (elements a thread holds across a stage; 0: the type's own).
 template <class T, int N, int MAXT = kMaxThreads, int EMAX = 0>
 struct Geo {
@@ -286,125 +282,9 @@ __device__ inline void block_sum4_ff(const float v[4], float hi[4], float lo[4],
   }
 }
 
-// Stage the twiddle table in shared memory: tw[t] = e^{-2 pi i t/N} for the
-// forward transforms, tw[N + t] = its conjugate for the inverse ones, so no
-// transform negates a twiddle where it uses it.
-template <class T>
-__device__ __forceinline__ void load_twiddles(cplx<T>* tw, const DevPlan& g) {
-  const cplx<T>* src = static_cast<const cplx<T>*>(g.tw);
-  for (int t = threadIdx.x; t < g.n; t += blockDim.x) {
-    const cplx<T> w = src[t];
-    tw[t] = w;
-    tw[g.n + t] = cmake<T>(w.x, -w.y);
-  }
-}
+// ------------------------------------------------------------------- geometry
 
-// ---------------------------------------------------------------- O(nb) passes
-
-// X[q] = scatter(c_{b0} + i c_{b0+1}) for band pairs q of the batch (X zeroed before).
-template <class T>
-__global__ void k_scatter(DevPlan g, const double2* __restrict__ psiG, int nb, int band0, int nbat,
-                          cplx<T>* __restrict__ X) {
-  const int q = blockIdx.y;
-  const int b0 = band0 + 2 * q;
-  const bool has1 = (2 * q + 1 < nbat) && (b0 + 1 < nb);
-  cplx<T>* Xq = X + (int64_t)q * g.ntot;
-  for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < g.npw; k += gridDim.x * blockDim.x) {
-    const double2 c0 = psiG[(int64_t)b0 * g.npw + k];
-    const double2 c1 = has1 ? psiG[(int64_t)(b0 + 1) * g.npw + k] : make_double2(0.0, 0.0);
-    Xq[g.gidx[k]] = cmake<T>(T(c0.x - c1.y), T(c0.y + c1.x));
-  }
-}
-
-// FFT along i1 of the slab X[q][:, i2, :] (all N columns).
-template <class T, int N, int SIGN>
-__global__ void __launch_bounds__(Geo<T, N>::THR_COLF) k_col_full(DevPlan g, cplx<T>* __restrict__ X) {
-  using C = cplx<T>;
-  using G = Geo<T, N>;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  C* S = reinterpret_cast<C*>(smem_raw);
-  C* tw = S + N * N;
-  const int i2 = blockIdx.x;
-  C* Xq = X + (int64_t)blockIdx.y * g.ntot;
-  load_twiddles<T>(tw, g);
-  for (int e = threadIdx.x; e < N * N; e += blockDim.x) {
-    const int i1 = e / N, i3 = e - i1 * N;
-    S[e] = Xq[((int64_t)i1 * N + i2) * N + i3];
-  }
-  __syncthreads();
-  fft_lines<T, N, SIGN, N, G::TLP, 1, N>(S, tw);
-  for (int e = threadIdx.x; e < N * N; e += blockDim.x) {
-    const int i1 = e / N, i3 = e - i1 * N;
-    Xq[((int64_t)i1 * N + i2) * N + i3] = S[e];
-  }
-}
-
-// 2D FFT over (i2, i3) of plane i1 of X[q].  PRO 0: load from X; PRO 1: z = W_b0 + i W_b0+1.
-// EPI 0: store to X; EPI 1: psi_b0 = Re z * psi_scale, psi_b0+1 = Im z * psi_scale.
-template <class T, int N, int SIGN, int PRO, int EPI>
-__global__ void __launch_bounds__(Geo<T, N>::THR_PLANE)
-    k_plane_full(DevPlan g, cplx<T>* __restrict__ X, const acc_t<T>* __restrict__ W, T* __restrict__ psi,
-                 int band0, int nb, int nbat) {
-  using C = cplx<T>;
-  using G = Geo<T, N>;
-  constexpr int RP = G::RP;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  C* P = reinterpret_cast<C*>(smem_raw);
-  C* tw = P + N * RP;
-  const int i1 = blockIdx.x, q = blockIdx.y;
-  const int b0 = band0 + 2 * q;
-  const bool has1 = (2 * q + 1 < nbat) && (b0 + 1 < nb);
-  C* Xq = X + (int64_t)q * g.ntot + (int64_t)i1 * N * N;
-  const int64_t plane0 = (int64_t)i1 * N * N;
-  load_twiddles<T>(tw, g);
-  for (int e = threadIdx.x; e < N * N; e += blockDim.x) {
-    const int i2 = e / N, i3 = e - i2 * N;
-    C z;
-    if (PRO == 0) {
-      z = Xq[e];
-    } else {
-      z.x = T(W[(int64_t)b0 * g.ntot + plane0 + e]);
-      z.y = has1 ? T(W[(int64_t)(b0 + 1) * g.ntot + plane0 + e]) : T(0);
-    }
-    P[i2 * RP + i3] = z;
-  }
-  __syncthreads();
-  fft_lines<T, N, SIGN, N, G::TLP, RP, 1>(P, tw);  // along i3
-  fft_lines<T, N, SIGN, N, G::TLP, 1, RP>(P, tw);  // along i2
-  const T s = T(g.psi_scale);
-  for (int e = threadIdx.x; e < N * N; e += blockDim.x) {
-    const int i2 = e / N, i3 = e - i2 * N;
-    const C z = P[i2 * RP + i3];
-    if (EPI == 0) {
-      Xq[e] = z;
-    } else {
-      psi[(int64_t)b0 * g.ntot + plane0 + e] = z.x * s;
-      if (has1) psi[(int64_t)(b0 + 1) * g.ntot + plane0 + e] = z.y * s;
-    }
-  }
-}
-
-// (V_x psi)(G) of the band pair q: Y = fft(W_b0 + i W_b0+1); X_b0(G) = (Y(G) + Y(-G)*)/2,
-// X_b0+1(G) = (Y(G) - Y(-G)*)/(2i); both scaled by sqrt(Omega)/Ntot.
-template <class T>
-__global__ void k_gather(DevPlan g, const cplx<T>* __restrict__ X, int nb, int band0, int nbat,
-                         double2* __restrict__ vpsiG) {
-  const int q = blockIdx.y;
-  const int b0 = band0 + 2 * q;
-  const bool has1 = (2 * q + 1 < nbat) && (b0 + 1 < nb);
-  const cplx<T>* Xq = X + (int64_t)q * g.ntot;
-  const double s = 0.5 * g.out_scale;
-  for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < g.npw; k += gridDim.x * blockDim.x) {
-    const cplx<T> y = Xq[g.gidx[k]], ym = Xq[g.gidxneg[k]];
-    const double yx = to_double(y.x), yy = to_double(y.y), mx = to_double(ym.x), my = to_double(ym.y);
-    vpsiG[(int64_t)b0 * g.npw + k] = make_double2(s * (yx + mx), s * (yy - my));
-    if (has1) vpsiG[(int64_t)(b0 + 1) * g.npw + k] = make_double2(s * (yy + my), s * (mx - yx));
-  }
-}
-
-// ------------------------------------------------------------------ pair passes
-
-// Compile-time geometry of the pair passes for grid size N and tiling TILE
+// Compile-time geometry of the passes for grid size N and tiling TILE
 // (the factors of the two-factor transforms and the threads that share them).
 template <class T, int N, int TILE = 0>
 struct PairGeo {
@@ -491,80 +371,433 @@ __device__ __forceinline__ void load_stage_twiddles(cplx<T>* tw, const DevPlan& 
   }
 }
 
+// Column code: (k2 << 16) | (self << 15) | k3 of a line pair's first line, or
+// -1 (no line); self: the line is its own mirror image (k2 and k3 both 0 or N/2).
+__device__ __forceinline__ int line_k2(int code) { return code >> 16; }
+__device__ __forceinline__ int line_self(int code) { return (code >> 15) & 1; }
+__device__ __forceinline__ int line_k3(int code) { return code & 0x7fff; }
+
+// ------------------------------------------------------------ plane transforms
+
+// Forward 2D transform of one plane, from load(e), e = i2 N + i3, to the kept
+// columns of its N x N block Hp of a transform buffer.
+template <class T, int N, int THR, int TILE, class Load>
+__device__ __forceinline__ void plane_forward(const DevPlan& g, const ColumnSet& cs, cplx<T>* __restrict__ Hp,
+                                              unsigned char* smem_raw, const Load& load) {
+  using C = cplx<T>;
+  using G = PairGeo<T, N, TILE>;
+  constexpr int RP = G::RP, A = G::A, B = G::B, M = G::M;
+  C* P = reinterpret_cast<C*>(smem_raw);
+  C* tw = P + N * RP;
+  load_stage_twiddles<T, -1, G::BLOCK ? 4 : B, N, THR>(tw, g);
+  if constexpr (G::BLOCK) load_stage_twiddles<T, -1, M, N, THR>(tw + N, g);
+  // Columns (along i2) first: the first stage reads its input through load (a
+  // warp's items are consecutive columns i3, so the loads coalesce); only its
+  // outputs enter shared memory.
+  constexpr int R0 = G::BLOCK ? M : A, J0 = N / R0;
+#pragma unroll(kItemUnroll<T>)
+  for (int item0 = 0; item0 < N * J0; item0 += THR) {
+    const int item = item0 + threadIdx.x;
+    if ((N * J0) % THR == 0 || item < N * J0) {
+      const int b = item / N, l = item - b * N;
+      C x[R0];
+#pragma unroll
+      for (int r = 0; r < R0; ++r) x[r] = load(item + r * (J0 * N));  // element i2 = b + J0 r of column l
+      Dft<-1, T>::template run<R0>(x);
+#pragma unroll
+      for (int q = 0; q < R0; ++q) P[(b + J0 * q) * RP + l] = x[q];
+    }
+  }
+  __syncthreads();
+  if constexpr (G::BLOCK) plane_block_pass<T, M, -1, THR, RP>(P, tw);
+  else stage_ct<T, B, -1, A, B * RP, RP, true, THR, N, 1>(P, tw);
+  // k2 is now at row G::row_place(k2); the rest of the transforms along i3
+  constexpr int R1 = G::BLOCK ? M : B;
+  const C* tw1 = G::BLOCK ? tw + N : tw;
+  if constexpr (G::ALL_LINES) {
+    if constexpr (!G::BLOCK) stage_ct<T, A, -1, B, 1, B, false, THR, N, RP>(P, tw);
+    stage_ct<T, R1, -1, N / R1, R1, 1, true, THR, N, RP>(P, tw1);
+  } else {
+    // only the rows k2 that hold kept columns, in order of their places
+    int* rows = reinterpret_cast<int*>(tw + 2 * N);
+    const int nrows = cs.row_lo + cs.row_hi;
+    const RtDiv by(nrows);
+    for (int r = threadIdx.x; r < nrows; r += THR) rows[r] = __ldg(cs.rowpos + TILE * N + r) * RP;
+    __syncthreads();
+    const auto row_off = [&](int l) { return rows[l]; };
+    if constexpr (!G::BLOCK) stage_rt<T, A, -1, B, 1, B, false, THR>(P, tw, nrows, by, row_off);
+    stage_rt<T, R1, -1, N / R1, R1, 1, true, THR>(P, tw1, nrows, by, row_off);
+  }
+  // the kept columns (k2, k3), consecutive threads on consecutive k3 of a row
+  for (int e = threadIdx.x; e < cs.nkept; e += THR) {
+    const int code = __ldg(cs.kept + e);
+    const int k2 = code >> 16, k3 = code & 0xffff;
+    Hp[k2 * N + k3] = P[G::row_place(k2) * RP + G::col_place(k3)];
+  }
+}
+
+// Inverse 2D transform of one plane from the kept columns of its block Hp (read
+// for the last time) into shared memory: point (i2, i3) at Q +
+// G::place_of_row(i2) RP + G::col_place(i3).
+template <class T, int N, int THR, int TILE>
+__device__ __forceinline__ void plane_inverse(const DevPlan& g, const ColumnSet& cs, const cplx<T>* __restrict__ Hp,
+                                              unsigned char* smem_raw) {
+  using C = cplx<T>;
+  using G = PairGeo<T, N, TILE>;
+  constexpr int RP = G::RP, A = G::A, B = G::B, M = G::M;
+  C* Q = reinterpret_cast<C*>(smem_raw);
+  C* tw = Q + N * RP;
+  // first transform along k2: DFTs of RB values k2 = q + NA s, s < RB
+  constexpr int RB = G::BLOCK ? M : B, NA = N / RB;
+  load_stage_twiddles<T, +1, G::BLOCK ? 4 : A, N, THR>(tw, g);
+  load_stage_twiddles<T, +1, RB, N, THR>(tw + N, g);
+  // 1. along k2, the columns that hold something.  The first stage reads the
+  //    transform buffer; a column's elements outside its kept rows [0, up) and
+  //    [N - dn, N) were never written and count as zero.
+  const unsigned long long last_use = l2_policy_evict_first();
+  const auto column = [&](int q, int k3) {
+    const int ud = __ldg(cs.ncol + k3);
+    const int up = ud & 0xffff, dn = N - (ud >> 16);
+    C x[RB];
+#pragma unroll
+    for (int s = 0; s < RB; ++s) {
+      const int k2 = q + NA * s;
+      if (k2 < up || k2 >= dn) x[s] = ldcg_hint(Hp + k2 * N + k3, last_use);
+      else x[s] = cmake<T>(T(0), T(0));
+    }
+    Dft<+1, T>::template run<RB>(x);
+#pragma unroll
+    for (int b = 0; b < RB; ++b) Q[(G::BLOCK ? 4 * b + q : RB * q + b) * RP + k3] = x[b];
+  };
+  if constexpr (G::ALL_LINES) {
+#pragma unroll(kItemUnroll<T>)
+    for (int item0 = 0; item0 < N * NA; item0 += THR) {
+      const int item = item0 + threadIdx.x, q = item / N;
+      if ((N * NA) % THR == 0 || item < N * NA) column(q, item - q * N);
+    }
+    __syncthreads();
+    if constexpr (!G::BLOCK) stage_ct<T, A, +1, B, RP, B * RP, true, THR, N, 1>(Q, tw);
+  } else {
+    const int lo = cs.col_lo, nl = cs.col_lo + cs.col_hi;
+    const auto k3_of = [&](int l) { return l < lo ? l : l + (N - nl); };
+    const RtDiv by(nl);
+    for (int item = threadIdx.x; item < nl * NA; item += THR) {
+      const int q = by.div(item);
+      column(q, k3_of(item - q * nl));
+    }
+    // the columns in between hold nothing
+    const int nz = N - nl;
+    for (int e = threadIdx.x; e < N * nz; e += THR) {
+      const int r = e / nz;
+      Q[r * RP + lo + (e - r * nz)] = cmake<T>(T(0), T(0));
+    }
+    __syncthreads();
+    if constexpr (!G::BLOCK) stage_rt<T, A, +1, B, RP, B * RP, true, THR>(Q, tw, nl, by, k3_of);
+  }
+  // 2. the rest along k2 and the rows
+  if constexpr (G::BLOCK) {
+    plane_block_pass<T, M, +1, THR, RP>(Q, tw);
+    stage_ct<T, M, +1, 4, M, 1, true, THR, N, RP>(Q, tw + N);
+  } else {
+    stage_ct<T, A, +1, B, 1, B, false, THR, N, RP>(Q, tw);
+    stage_ct<T, B, +1, A, B, 1, true, THR, N, RP>(Q, tw + N);
+  }
+}
+
+// ---------------------------------------------------------------- O(nb) passes
+//
+// The sphere reaches a fraction of the columns (15% at 96^3, L 27, Ecut 12), so
+// the transforms between the sphere and real space run over those columns only:
+// a column pass that gathers its input from the coefficients (or leaves its
+// output there) and a plane pass over the kept columns.  X holds one N^3 block
+// per band pair (Gamma point: z = psi_b0 + i psi_b1) or band (k points), of
+// which only the kept columns are written and read.
+
+// A CTA's line slot l of a column map: its first element in a transform buffer
+// (slots from NP on: the mirror image), or NULL.
+template <class C, int N, int NP>
+__device__ __forceinline__ C* line_ptr(C* H, const int* lines, int cta, int l) {
+  const int code = __ldg(lines + cta * NP + l % NP);
+  if (code < 0) return nullptr;
+  const int k2 = line_k2(code), k3 = line_k3(code);
+  return H + (l < NP ? k2 * N + k3 : (k2 == 0 ? 0 : N - k2) * N + (k3 == 0 ? 0 : N - k3));
+}
+
+// Inverse transform along k1 of the sphere's columns, from the coefficients of
+// bands b0 and b0 + 1 (z = c0 + i c1) or, KP, of band b0 alone.
+template <class T, int N, bool KP>
+__global__ void __launch_bounds__(PairGeo<T, N>::THR_COL)
+    k_orb_col_inv(DevPlan g, ColumnSet cs, const double2* __restrict__ psiG, int npw, int nb, int band0, int nbat,
+                  cplx<T>* __restrict__ X) {
+  using C = cplx<T>;
+  using G = PairGeo<T, N>;
+  constexpr int A = G::CA, B = G::CB, NL = G::NL, NP = KP ? NL : G::NP, THR = G::THR_COL;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  C* S = reinterpret_cast<C*>(smem_raw);
+  C* tw = S + N * NL;
+  load_stage_twiddles<T, +1, B, N, THR>(tw, g);
+  const int q0 = blockIdx.y, cta = blockIdx.x;
+  const int b0 = band0 + (KP ? q0 : 2 * q0);
+  const bool has1 = !KP && (2 * q0 + 1 < nbat) && (b0 + 1 < nb);
+  const double2* c0 = psiG + (int64_t)b0 * npw;
+  const double2* c1 = c0 + (has1 ? npw : 0);
+  const int l = threadIdx.x % NL;
+  const int* coef = cs.coef + (int64_t)cta * N * NL + l;
+  C* lp = line_ptr<C, N, NP>(X + (int64_t)q0 * g.ntot, cs.lines, cta, l);
+  const bool twin = !KP && l >= NP && lp != nullptr && line_self(__ldg(cs.lines + cta * NP + l % NP));
+#pragma unroll(kItemUnroll<T>)
+  for (int j0 = 0; j0 < B; j0 += THR / NL) {
+    const int b = j0 + threadIdx.x / NL;
+    if (B % (THR / NL) == 0 || b < B) {
+      C x[A];
+#pragma unroll
+      for (int r = 0; r < A; ++r) {
+        const int at = __ldg(coef + (b + B * r) * NL);
+        C z = cmake<T>(T(0), T(0));
+        if (at >= 0) {
+          const double2 u = c0[at];
+          if (has1) {
+            const double2 w = c1[at];
+            z = cmake<T>(T(u.x - w.y), T(u.y + w.x));
+          } else {
+            z = cmake<T>(T(u.x), T(u.y));
+          }
+        }
+        x[r] = z;
+      }
+      Dft<+1, T>::template run<A>(x);
+#pragma unroll
+      for (int q = 0; q < A; ++q) S[(b + B * q) * NL + l] = x[q];
+    }
+  }
+  __syncthreads();
+  if (lp != nullptr && !twin) {
+#pragma unroll(kItemUnroll<T>)
+    for (int j0 = 0; j0 < A; j0 += THR / NL) {
+      const int q = j0 + threadIdx.x / NL;
+      if (A % (THR / NL) == 0 || q < A) {
+        C x[B];
+#pragma unroll
+        for (int b = 0; b < B; ++b) x[b] = S[(B * q + b) * NL + l];
+        dft_twiddled<T, B, +1>(x, tw + q * B);
+#pragma unroll
+        for (int s = 0; s < B; ++s) lp[(int64_t)(q + A * s) * (N * N)] = x[s];
+      }
+    }
+  }
+}
+
+// Forward transform along i1 of the sphere's columns, to the coefficients out
+// of bands b0 and b0 + 1, the transforms of Re and Im of the block: with Y its
+// transform, (Y(G) + Y(-G)*) / 2 and (Y(G) - Y(-G)*) / 2i, times scale; KP: of
+// band b0 alone.
+template <class T, int N, bool KP>
+__global__ void __launch_bounds__(PairGeo<T, N>::THR_COL)
+    k_orb_col_fwd(DevPlan g, ColumnSet cs, const cplx<T>* __restrict__ X, double scale, int npw, int nb, int band0,
+                  int nbat, double2* __restrict__ out) {
+  using C = cplx<T>;
+  using G = PairGeo<T, N>;
+  constexpr int A = G::CA, B = G::CB, NL = G::NL, NP = KP ? NL : G::NP, THR = G::THR_COL;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  C* S = reinterpret_cast<C*>(smem_raw);
+  C* tw = S + N * NL;
+  load_stage_twiddles<T, -1, B, N, THR>(tw, g);
+  const int q0 = blockIdx.y, cta = blockIdx.x;
+  const int b0 = band0 + (KP ? q0 : 2 * q0);
+  const bool has1 = !KP && (2 * q0 + 1 < nbat) && (b0 + 1 < nb);
+  const int l = threadIdx.x % NL;
+  const C* lp = line_ptr<const C, N, NP>(X + (int64_t)q0 * g.ntot, cs.lines, cta, l);
+#pragma unroll(kItemUnroll<T>)
+  for (int j0 = 0; j0 < B; j0 += THR / NL) {
+    const int b = j0 + threadIdx.x / NL;
+    if (B % (THR / NL) == 0 || b < B) {
+      C x[A];
+#pragma unroll
+      for (int r = 0; r < A; ++r) {
+        if (lp != nullptr) x[r] = ldcg_c(lp + (int64_t)(b + B * r) * (N * N));
+        else x[r] = cmake<T>(T(0), T(0));
+      }
+      Dft<-1, T>::template run<A>(x);
+#pragma unroll
+      for (int q = 0; q < A; ++q) S[(b + B * q) * NL + l] = x[q];
+    }
+  }
+  __syncthreads();
+  double2* o0 = out + (int64_t)b0 * npw;
+  const int* coef = cs.coef + (int64_t)cta * N * NL;
+  if constexpr (KP) {
+    for (int item = threadIdx.x; item < NL * A; item += THR) {
+      const int q = item / NL;
+      C z[B];
+#pragma unroll
+      for (int b = 0; b < B; ++b) z[b] = S[(B * q + b) * NL + l];
+      dft_twiddled<T, B, -1>(z, tw + q * B);
+#pragma unroll
+      for (int s = 0; s < B; ++s) {
+        const int at = __ldg(coef + (q + A * s) * NL + l);
+        if (at >= 0) o0[at] = make_double2(scale * to_double(z[s].x), scale * to_double(z[s].y));
+      }
+    }
+  } else {
+    const double h = 0.5 * scale;
+    const int p = threadIdx.x % NP;
+    for (int item = threadIdx.x; item < NP * A; item += THR) {
+      const int q = item / NP, qm = q == 0 ? 0 : A - q;
+      C z[B], y[B];
+#pragma unroll
+      for (int b = 0; b < B; ++b) {
+        z[b] = S[(B * q + b) * NL + p];
+        y[b] = S[(B * qm + b) * NL + NP + p];
+      }
+      dft_twiddled<T, B, -1>(z, tw + q * B);
+      dft_twiddled<T, B, -1>(y, tw + qm * B);
+      const auto put = [&](int s, C Z, C Y) {
+        const int at = __ldg(coef + (q + A * s) * NL + p);
+        if (at < 0) return;
+        const int k1 = q + A * s;
+        const int am = __ldg(coef + (k1 == 0 ? 0 : N - k1) * NL + NP + p);  // -G: the sphere is closed under it
+        const double yx = to_double(Z.x), yy = to_double(Z.y), mx = to_double(Y.x), my = to_double(Y.y);
+        const double ax = h * (yx + mx), ay = h * (yy - my);
+        o0[at] = make_double2(ax, ay);
+        o0[am] = make_double2(ax, -ay);
+        if (has1) {
+          const double bx = h * (yy + my), by = h * (mx - yx);
+          o0[npw + at] = make_double2(bx, by);
+          o0[npw + am] = make_double2(bx, -by);
+        }
+      };
+#pragma unroll
+      for (int s = 0; s < B; ++s) {
+        const C ya = y[(B - s) % B], yb = y[B - 1 - s];
+        put(s, z[s], cmake<T>(q == 0 ? ya.x : yb.x, q == 0 ? ya.y : yb.y));
+      }
+    }
+  }
+}
+
+// Inverse plane pass: psi_b0 = Re z psi_scale, psi_b0+1 = Im z psi_scale (KP: u
+// = z psi_scale, complex).
+template <class T, int N, bool KP>
+__global__ void __launch_bounds__(PairGeo<T, N>::THR_PLANE, PairGeo<T, N>::MIN_PLANE)
+    k_orb_plane_inv(DevPlan g, ColumnSet cs, const cplx<T>* __restrict__ X, void* __restrict__ psiv, int band0, int nb,
+                    int nbat) {
+  using C = cplx<T>;
+  using G = PairGeo<T, N>;
+  constexpr int THR = G::THR_PLANE, RP = G::RP;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const C* Q = reinterpret_cast<const C*>(smem_raw);
+  const int i1 = blockIdx.x, q = blockIdx.y;
+  plane_inverse<T, N, THR, 0>(g, cs, X + (int64_t)q * g.ntot + (int64_t)i1 * N * N, smem_raw);
+  const int64_t plane0 = (int64_t)i1 * N * N;
+  const T s = T(g.psi_scale);
+  const int b0 = band0 + (KP ? q : 2 * q);
+  const bool has1 = !KP && (2 * q + 1 < nbat) && (b0 + 1 < nb);
+  for (int e = threadIdx.x; e < N * N; e += THR) {
+    const int i2 = e / N, i3 = e - i2 * N;
+    const C z = Q[G::place_of_row(i2) * RP + G::col_place(i3)];
+    if constexpr (KP) {
+      static_cast<C*>(psiv)[(int64_t)b0 * g.ntot + plane0 + e] = cmake<T>(z.x * s, z.y * s);
+    } else {
+      T* psi = static_cast<T*>(psiv) + (int64_t)b0 * g.ntot + plane0 + e;
+      *psi = z.x * s;
+      if (has1) psi[g.ntot] = z.y * s;
+    }
+  }
+}
+
+// Forward plane pass of z = W_b0 + i W_b0+1 (KP: of the complex W_b0).
+template <class T, int N, bool KP>
+__global__ void __launch_bounds__(PairGeo<T, N>::THR_PLANE, PairGeo<T, N>::MIN_PLANE)
+    k_orb_plane_fwd(DevPlan g, ColumnSet cs, const void* __restrict__ Wv, cplx<T>* __restrict__ X, int band0, int nb,
+                    int nbat) {
+  using C = cplx<T>;
+  using G = PairGeo<T, N>;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int i1 = blockIdx.x, q = blockIdx.y;
+  const int b0 = band0 + (KP ? q : 2 * q);
+  const int64_t at = (int64_t)b0 * g.ntot + (int64_t)i1 * N * N;
+  C* Hp = X + (int64_t)q * g.ntot + (int64_t)i1 * N * N;
+  if constexpr (KP) {
+    const C* W = static_cast<const C*>(Wv) + at;
+    plane_forward<T, N, G::THR_PLANE, 0>(g, cs, Hp, smem_raw, [&](int e) { return W[e]; });
+  } else {
+    const acc_t<T>* W = static_cast<const acc_t<T>*>(Wv) + at;
+    const bool has1 = (2 * q + 1 < nbat) && (b0 + 1 < nb);
+    plane_forward<T, N, G::THR_PLANE, 0>(g, cs, Hp, smem_raw, [&](int e) {
+      return cmake<T>(T(W[e]), has1 ? T(W[g.ntot + e]) : T(0));
+    });
+  }
+}
+
+// A local potential applied in real space, plane i1 of X[q] in place: inverse
+// plane pass, times vloc(r) (real, so the two bands of z stay apart), forward
+// plane pass, all in shared memory.  FP64 (two-factor stages): the rows leave
+// the inverse in spectrum order along i3 and the forward transform runs its
+// stages from that order back to natural order.
+template <class T, int N>
+__global__ void __launch_bounds__(PairGeo<T, N>::THR_PLANE, PairGeo<T, N>::MIN_PLANE)
+    k_orb_plane_vloc(DevPlan g, ColumnSet cs, const T* __restrict__ vloc, cplx<T>* __restrict__ X) {
+  using C = cplx<T>;
+  using G = PairGeo<T, N>;
+  static_assert(!G::BLOCK && !G::ALL_LINES, "written for the two-factor stages");
+  constexpr int RP = G::RP, A = G::A, B = G::B, THR = G::THR_PLANE;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  C* P = reinterpret_cast<C*>(smem_raw);
+  C* tw = P + N * RP;
+  const int i1 = blockIdx.x;
+  C* Hp = X + (int64_t)blockIdx.y * g.ntot + (int64_t)i1 * N * N;
+  plane_inverse<T, N, THR, 0>(g, cs, Hp, smem_raw);
+  const T* v = vloc + (int64_t)i1 * N * N;
+  for (int e = threadIdx.x; e < N * N; e += THR) {
+    const int i2 = e / N, i3 = e - i2 * N;
+    C& z = P[i2 * RP + spec_pos<A, B>(i3)];
+    const T w = v[e];
+    z = cmake<T>(z.x * w, z.y * w);
+  }
+  load_stage_twiddles<T, -1, B, N, THR>(tw, g);      // columns' B-stage
+  load_stage_twiddles<T, -1, A, N, THR>(tw + N, g);  // rows' A-stage
+  int* rows = reinterpret_cast<int*>(tw + 2 * N);
+  const int nrows = cs.row_lo + cs.row_hi;
+  const RtDiv by(nrows);
+  for (int r = threadIdx.x; r < nrows; r += THR) rows[r] = __ldg(cs.rowpos + r) * RP;
+  __syncthreads();
+  stage_ct<T, A, -1, B, RP, B * RP, false, THR, N, 1>(P, tw);
+  stage_ct<T, B, -1, A, B * RP, RP, true, THR, N, 1>(P, tw);
+  const auto row_off = [&](int l) { return rows[l]; };
+  stage_rt<T, B, -1, A, B, 1, false, THR>(P, tw, nrows, by, row_off);
+  stage_rt<T, A, -1, B, 1, B, true, THR>(P, tw + N, nrows, by, row_off);  // k3 at its place
+  for (int e = threadIdx.x; e < cs.nkept; e += THR) {
+    const int code = __ldg(cs.kept + e);
+    const int k2 = code >> 16, k3 = code & 0xffff;
+    Hp[k2 * N + k3] = P[G::row_place(k2) * RP + k3];
+  }
+}
+
+// ------------------------------------------------------------------ pair passes
+
 // One task of the forward plane pass: plane i1 of chain `ch`, whose transform
 // buffer is Hc.  Shared memory: PairGeo::SMEM_PLANE bytes at smem_raw.
 template <class T, int N, int THR, int TILE = 0>
 __device__ __forceinline__ void pair_fwd_task(const DevPlan& g, const T* __restrict__ psi,
                                               const Chain& ch, cplx<T>* __restrict__ Hc, int i1,
                                               unsigned char* smem_raw) {
-  using C = cplx<T>;
-  using G = PairGeo<T, N, TILE>;
-  constexpr int RP = G::RP, A = G::A, B = G::B;
-  C* P = reinterpret_cast<C*>(smem_raw);
-  C* tw = P + N * RP;
-  constexpr int M = G::M;
-  load_stage_twiddles<T, -1, G::BLOCK ? 4 : B, N, THR>(tw, g);
-  if constexpr (G::BLOCK) load_stage_twiddles<T, -1, M, N, THR>(tw + N, g);
   const int64_t plane0 = (int64_t)i1 * N * N;
   const bool hb = ch.bi >= 0;
   const T* pai = psi + (int64_t)ch.ai * g.ntot + plane0;
   const T* paj = psi + (int64_t)ch.aj * g.ntot + plane0;
   const T* pbi = psi + (int64_t)(hb ? ch.bi : 0) * g.ntot + plane0;
   const T* pbj = psi + (int64_t)(hb ? ch.bj : 0) * g.ntot + plane0;
-  // Columns (along i2) first: the first stage reads the pair product straight
-  // from the orbital planes (a warp's items are consecutive columns i3, so the
-  // loads coalesce); only its outputs enter shared memory.
-  constexpr int R0 = G::BLOCK ? M : A, J0 = N / R0;
-  const auto columns = [&](const auto& product) {
-#pragma unroll(kItemUnroll<T>)
-    for (int item0 = 0; item0 < N * J0; item0 += THR) {
-      const int item = item0 + threadIdx.x;
-      if ((N * J0) % THR == 0 || item < N * J0) {
-        const int b = item / N, l = item - b * N;
-        C x[R0];
-#pragma unroll
-        for (int r = 0; r < R0; ++r) x[r] = product(item + r * (J0 * N));  // element i2 = b + J0 r of column l
-        Dft<-1, T>::template run<R0>(x);
-#pragma unroll
-        for (int q = 0; q < R0; ++q) P[(b + J0 * q) * RP + l] = x[q];
-      }
-    }
-  };
+  cplx<T>* Hp = Hc + (int64_t)i1 * N * N;
   if (hb && ch.ai == ch.bi) {
     // the usual chain, pairs (i, j) and (i, j'): psi_i is read once
-    columns([&](int e) {
+    plane_forward<T, N, THR, TILE>(g, g.cols, Hp, smem_raw, [&](int e) {
       const T x = pai[e];
       return cmake<T>(x * paj[e], x * pbj[e]);
     });
   } else {
-    columns([&](int e) { return cmake<T>(pai[e] * paj[e], hb ? pbi[e] * pbj[e] : T(0)); });
-  }
-  __syncthreads();
-  if constexpr (G::BLOCK) plane_block_pass<T, M, -1, THR, RP>(P, tw);
-  else stage_ct<T, B, -1, A, B * RP, RP, true, THR, N, 1>(P, tw);
-  // k2 is now at row G::row_place(k2); the rest of the transforms along i3
-  if constexpr (G::ALL_LINES) {
-    if constexpr (!G::BLOCK) stage_ct<T, A, -1, B, 1, B, false, THR, N, RP>(P, tw);
-    constexpr int R1 = G::BLOCK ? M : B;
-    stage_ct<T, R1, -1, N / R1, R1, 1, true, THR, N, RP>(P, G::BLOCK ? tw + N : tw);
-  } else {
-    // only the rows k2 that hold kept columns, in order of their places
-    int* rows = reinterpret_cast<int*>(tw + 2 * N);
-    const int nrows = g.row_lo + g.row_hi;
-    const RtDiv by(nrows);
-    for (int r = threadIdx.x; r < nrows; r += THR) rows[r] = __ldg(g.rowpos + TILE * N + r) * RP;
-    __syncthreads();
-    const auto row_off = [&](int l) { return rows[l]; };
-    if constexpr (!G::BLOCK) stage_rt<T, A, -1, B, 1, B, false, THR>(P, tw, nrows, by, row_off);
-    constexpr int R1 = G::BLOCK ? M : B;
-    stage_rt<T, R1, -1, N / R1, R1, 1, true, THR>(P, G::BLOCK ? tw + N : tw, nrows, by, row_off);
-  }
-  C* Hp = Hc + (int64_t)i1 * N * N;
-  // the kept columns (k2, k3), consecutive threads on consecutive k3 of a row
-  for (int e = threadIdx.x; e < g.nkept; e += THR) {
-    const int code = __ldg(g.kept + e);
-    const int k2 = code >> 16, k3 = code & 0xffff;
-    Hp[k2 * N + k3] = P[G::row_place(k2) * RP + G::col_place(k3)];
+    plane_forward<T, N, THR, TILE>(g, g.cols, Hp, smem_raw, [&](int e) {
+      return cmake<T>(pai[e] * paj[e], hb ? pbi[e] * pbj[e] : T(0));
+    });
   }
 }
 
@@ -584,7 +817,7 @@ __global__ void __launch_bounds__(PairGeo<T, N, TILE>::THR_PLANE, PairGeo<T, N, 
 __device__ __forceinline__ void put_energies(const DevPlan& g, const Chain& ch, int cta, const double acc[4],
                                              bool want_d, double* epair, double* dpair) {
   if (g.det) {
-    const int64_t nc = g.ncta_col;
+    const int64_t nc = g.cols.ncta;
     if (ch.pa >= 0) epair[ch.pa * nc + cta] = acc[0];
     if (ch.pb >= 0) epair[ch.pb * nc + cta] = acc[1];
     if (want_d) {
@@ -612,12 +845,6 @@ __device__ __forceinline__ void det_add(double* p, df64 v, double scale) {
   atomicAdd(reinterpret_cast<unsigned long long*>(p), (unsigned long long)q);
 }
 __device__ __forceinline__ void det_add(float*, float, double) {}  // not offered for the mixed form
-
-// Column code: (k2 << 16) | (self << 15) | k3 of a line pair's first line, or
-// -1 (no line); self: the line is its own mirror image (k2 and k3 both 0 or N/2).
-__device__ __forceinline__ int line_k2(int code) { return code >> 16; }
-__device__ __forceinline__ int line_self(int code) { return (code >> 15) & 1; }
-__device__ __forceinline__ int line_k3(int code) { return code & 0x7fff; }
 
 // One kernel term of the smallest |m| (|m|^2 <= msmall2: 27 points per pair)
 // of the mixed-form column pass, in FP64: the values z at (k1, k2, k3) and y at
@@ -694,12 +921,7 @@ __device__ __forceinline__ void pair_col_task(const DevPlan& g, cplx<T>* __restr
   load_stage_twiddles<T, +1, A, N, THR>(tw + N, g);
   // this thread's line of the A-stages: l < NP a pair's first line, else its mirror image
   const int l = threadIdx.x % NL;
-  const int lcode = __ldg(g.colmap + cta * NP + l % NP);
-  C* lp = nullptr;
-  if (lcode >= 0) {
-    const int k2 = line_k2(lcode), k3 = line_k3(lcode);
-    lp = Hc + (l < NP ? k2 * N + k3 : (k2 == 0 ? 0 : N - k2) * N + (k3 == 0 ? 0 : N - k3));
-  }
+  C* lp = line_ptr<C, N, NP>(Hc, g.cols.lines, cta, l);
 #pragma unroll(kItemUnroll<T>)
   for (int b0 = 0; b0 < B; b0 += THR / NL) {
     const int b = b0 + threadIdx.x / NL;
@@ -717,7 +939,7 @@ __device__ __forceinline__ void pair_col_task(const DevPlan& g, cplx<T>* __restr
   }
   // this thread's line pair of the B-stages
   const int p = threadIdx.x % NP;
-  const int code = __ldg(g.colmap + cta * NP + p);
+  const int code = __ldg(g.cols.lines + cta * NP + p);
   const int k2 = code >= 0 ? line_k2(code) : 0, k3 = code >= 0 ? line_k3(code) : 0;
   const int vo = k2 * KH + k3;
   const bool want_d = g.dvtab64 != nullptr;
@@ -881,7 +1103,7 @@ __device__ __forceinline__ void pair_col_task(const DevPlan& g, cplx<T>* __restr
   if (threadIdx.x == 0) put_energies(g, ch, cta, e4, want_d, epair, dpair);
   // inverse A-stage, straight to the transform buffer (a self-mirrored line's
   // second copy is dropped)
-  if (lp != nullptr && !(l >= NP && line_self(lcode))) {
+  if (lp != nullptr && !(l >= NP && line_self(__ldg(g.cols.lines + cta * NP + l % NP)))) {
 #pragma unroll(kItemUnroll<T>)
     for (int b0 = 0; b0 < B; b0 += THR / NL) {
       const int b = b0 + threadIdx.x / NL;
@@ -917,69 +1139,9 @@ __device__ __forceinline__ void pair_inv_task(const DevPlan& g, const T* __restr
                                               unsigned char* smem_raw) {
   using C = cplx<T>;
   using G = PairGeo<T, N, TILE>;
-  constexpr int RP = G::RP, A = G::A, B = G::B;
-  C* Q = reinterpret_cast<C*>(smem_raw);
-  C* tw = Q + N * RP;
-  constexpr int M = G::M;
-  // first transform along k2: DFTs of RB values k2 = q + NA s, s < RB
-  constexpr int RB = G::BLOCK ? M : B, NA = N / RB;
-  load_stage_twiddles<T, +1, G::BLOCK ? 4 : A, N, THR>(tw, g);
-  load_stage_twiddles<T, +1, RB, N, THR>(tw + N, g);
-  const C* Hp = Hc + (int64_t)i1 * N * N;
-  // 1. inverse transform along k2 of the columns that hold something: k3 in
-  //    [0, col_max) and its mirror images.  Its first stage reads the transform
-  //    buffer (last use of it); a column's elements outside its kept rows
-  //    [0, up) and [N - dn, N) were never written and count as zero.
-  const unsigned long long last_use = l2_policy_evict_first();
-  const auto column = [&](int q, int k3) {
-    const int ud = __ldg(g.ncol + k3);
-    const int up = ud & 0xffff, dn = N - (ud >> 16);
-    C x[RB];
-#pragma unroll
-    for (int s = 0; s < RB; ++s) {
-      const int k2 = q + NA * s;
-      if (k2 < up || k2 >= dn) x[s] = ldcg_hint(Hp + k2 * N + k3, last_use);
-      else x[s] = cmake<T>(T(0), T(0));
-    }
-    Dft<+1, T>::template run<RB>(x);
-#pragma unroll
-    for (int b = 0; b < RB; ++b) Q[(G::BLOCK ? 4 * b + q : RB * q + b) * RP + k3] = x[b];
-  };
-  if constexpr (G::ALL_LINES) {
-#pragma unroll(kItemUnroll<T>)
-    for (int item0 = 0; item0 < N * NA; item0 += THR) {
-      const int item = item0 + threadIdx.x, q = item / N;
-      if ((N * NA) % THR == 0 || item < N * NA) column(q, item - q * N);
-    }
-    __syncthreads();
-    if constexpr (!G::BLOCK) stage_ct<T, A, +1, B, RP, B * RP, true, THR, N, 1>(Q, tw);
-  } else {
-    const int cm = g.col_max;
-    const int nl = 2 * cm - 1 < N ? 2 * cm - 1 : N;
-    const auto k3_of = [&](int l) { return l < cm ? l : l + (N - nl); };
-    const RtDiv by(nl);
-    for (int item = threadIdx.x; item < nl * NA; item += THR) {
-      const int q = by.div(item);
-      column(q, k3_of(item - q * nl));
-    }
-    // the columns in between hold nothing
-    const int nz = N - nl;
-    for (int e = threadIdx.x; e < N * nz; e += THR) {
-      const int r = e / nz;
-      Q[r * RP + cm + (e - r * nz)] = cmake<T>(T(0), T(0));
-    }
-    __syncthreads();
-    if constexpr (!G::BLOCK) stage_rt<T, A, +1, B, RP, B * RP, true, THR>(Q, tw, nl, by, k3_of);
-  }
-  // 2. the rest along k2 and the rows: row i2 at place G::BLOCK ? 4 b + r for
-  //    i2 = b + M r : i2, Q[.][G::col_place(i3)] = phi_a + i phi_b
-  if constexpr (G::BLOCK) {
-    plane_block_pass<T, M, +1, THR, RP>(Q, tw);
-    stage_ct<T, M, +1, 4, M, 1, true, THR, N, RP>(Q, tw + N);
-  } else {
-    stage_ct<T, A, +1, B, 1, B, false, THR, N, RP>(Q, tw);
-    stage_ct<T, B, +1, A, B, 1, true, THR, N, RP>(Q, tw + N);
-  }
+  constexpr int RP = G::RP;
+  const C* Q = reinterpret_cast<const C*>(smem_raw);
+  plane_inverse<T, N, THR, TILE>(g, g.cols, Hc + (int64_t)i1 * N * N, smem_raw);  // phi_a + i phi_b
   const int64_t plane0 = (int64_t)i1 * N * N;
   const bool hb = ch.bi >= 0;
   // Up to four updates k, W[tgt_k] -= f[src_k] psi[src_k] phi:
@@ -1181,7 +1343,6 @@ constexpr size_t smem_max(size_t a, size_t b) { return a > b ? a : b; }
 template <class T, int N>
 struct Launch {
   using C = cplx<T>;
-  using G = Geo<T, N>;
   using P0 = PairGeo<T, N, 0>;
   // the second tiling of the pair passes, where one is compiled
   static constexpr int T1 = (N == 96 && RealTraits<T>::prec != 2) ? 1 : 0;
@@ -1192,9 +1353,12 @@ struct Launch {
       return cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
     };
     cudaError_t err = cudaSuccess;
-    for (const void* f : {(const void*)k_col_full<T, N, +1>, (const void*)k_col_full<T, N, -1>,
-                          (const void*)k_plane_full<T, N, +1, 0, 1>, (const void*)k_plane_full<T, N, -1, 1, 0>})
-      if (err == cudaSuccess) err = smem(f, G::SMEM_PLANE);
+    for (const void* f : {(const void*)k_orb_col_inv<T, N, false>, (const void*)k_orb_col_fwd<T, N, false>})
+      if (err == cudaSuccess) err = smem(f, P0::SMEM_COL);
+    for (const void* f : {(const void*)k_orb_plane_inv<T, N, false>, (const void*)k_orb_plane_fwd<T, N, false>})
+      if (err == cudaSuccess) err = smem(f, P0::SMEM_PLANE);
+    if constexpr (RealTraits<T>::prec == 0)
+      if (err == cudaSuccess) err = smem((const void*)k_orb_plane_vloc<T, N>, P0::SMEM_PLANE);
     for (const void* f : {(const void*)k_pair_fwd<T, N>, (const void*)k_pair_inv<T, N>})
       if (err == cudaSuccess) err = smem(f, P0::SMEM_PLANE);
     if (err == cudaSuccess) err = smem((const void*)k_pair_col<T, N>, P0::SMEM_COL);
@@ -1226,13 +1390,27 @@ struct Launch {
                              void* Xv, void* psiv, cudaStream_t s) {
     C* X = static_cast<C*>(Xv);
     const int nq = (nbat + 1) / 2;
-    cudaError_t err = cudaMemsetAsync(X, 0, sizeof(C) * (size_t)g.ntot * nq, s);
-    if (err != cudaSuccess) return err;
-    k_scatter<T><<<dim3((g.npw + 255) / 256, nq), 256, 0, s>>>(g, psiG, nb, band0, nbat, X);
-    k_col_full<T, N, +1><<<dim3(N, nq), G::THR_COLF, G::SMEM_COLF, s>>>(g, X);
-    k_plane_full<T, N, +1, 0, 1><<<dim3(N, nq), G::THR_PLANE, G::SMEM_PLANE, s>>>(
-        g, X, nullptr, static_cast<T*>(psiv), band0, nb, nbat);
+    k_orb_col_inv<T, N, false><<<dim3(g.orb.ncta, nq), P0::THR_COL, P0::SMEM_COL, s>>>(g, g.orb, psiG, g.npw, nb, band0,
+                                                                                     nbat, X);
+    k_orb_plane_inv<T, N, false><<<dim3(N, nq), P0::THR_PLANE, P0::SMEM_PLANE, s>>>(g, g.orb, X, psiv, band0, nb,
+                                                                                    nbat);
     return cudaGetLastError();
+  }
+
+  static cudaError_t apply_vloc(const DevPlan& g, const double2* psiG, int nb, int band0, int nbat, const double* vloc,
+                                void* Xv, double2* out, cudaStream_t s) {
+    if constexpr (RealTraits<T>::prec == 0) {
+      C* X = static_cast<C*>(Xv);
+      const int nq = (nbat + 1) / 2;
+      k_orb_col_inv<T, N, false><<<dim3(g.orb.ncta, nq), P0::THR_COL, P0::SMEM_COL, s>>>(g, g.orb, psiG, g.npw, nb,
+                                                                                       band0, nbat, X);
+      k_orb_plane_vloc<T, N><<<dim3(N, nq), P0::THR_PLANE, P0::SMEM_PLANE, s>>>(g, g.orb, vloc, X);
+      k_orb_col_fwd<T, N, false><<<dim3(g.orb.ncta, nq), P0::THR_COL, P0::SMEM_COL, s>>>(
+          g, g.orb, X, g.inv_ntot, g.npw, nb, band0, nbat, out);
+      return cudaGetLastError();
+    } else {
+      return cudaErrorNotSupported;
+    }
   }
 
   template <int TILE>
@@ -1251,7 +1429,7 @@ struct Launch {
   static cudaError_t col_tile(const DevPlan& g, void* H, const Chain* ch, int nch, double* ep, double* dp,
                               cudaStream_t s) {
     using P = PairGeo<T, N, TILE>;
-    k_pair_col<T, N, TILE><<<dim3(g.ncta_col, nch), P::THR_COL, P::SMEM_COL, s>>>(g, static_cast<C*>(H), ch, ep, dp);
+    k_pair_col<T, N, TILE><<<dim3(g.cols.ncta, nch), P::THR_COL, P::SMEM_COL, s>>>(g, static_cast<C*>(H), ch, ep, dp);
     return cudaGetLastError();
   }
   static cudaError_t pair_col(const DevPlan& g, void* H, const Chain* ch, int nch, double* ep,
@@ -1278,17 +1456,17 @@ struct Launch {
                                void* Xv, double2* vpsiG, cudaStream_t s) {
     C* X = static_cast<C*>(Xv);
     const int nq = (nbat + 1) / 2;
-    k_plane_full<T, N, -1, 1, 0><<<dim3(N, nq), G::THR_PLANE, G::SMEM_PLANE, s>>>(
-        g, X, static_cast<const acc_t<T>*>(W), nullptr, band0, nb, nbat);
-    k_col_full<T, N, -1><<<dim3(N, nq), G::THR_COLF, G::SMEM_COLF, s>>>(g, X);
-    k_gather<T><<<dim3((g.npw + 255) / 256, nq), 256, 0, s>>>(g, X, nb, band0, nbat, vpsiG);
+    k_orb_plane_fwd<T, N, false><<<dim3(N, nq), P0::THR_PLANE, P0::SMEM_PLANE, s>>>(g, g.orb, W, X, band0, nb, nbat);
+    k_orb_col_fwd<T, N, false><<<dim3(g.orb.ncta, nq), P0::THR_COL, P0::SMEM_COL, s>>>(
+        g, g.orb, X, g.out_scale, g.npw, nb, band0, nbat, vpsiG);
     return cudaGetLastError();
   }
 
   static constexpr KernelOps ops() {
     return KernelOps{(int)sizeof(T), RealTraits<T>::prec, N, P0::NP,
-                     smem_max(smem_max(P0::SMEM_COL, P0::SMEM_PLANE), G::SMEM_PLANE),
-                     configure, to_real, pair_fwd, pair_col, pair_inv, to_sphere, tile_plan, row_place};
+                     smem_max(P0::SMEM_COL, P0::SMEM_PLANE),
+                     configure, to_real, pair_fwd, pair_col, pair_inv, to_sphere, tile_plan, row_place,
+                     RealTraits<T>::prec == 0 ? apply_vloc : nullptr};
   }
 };
 

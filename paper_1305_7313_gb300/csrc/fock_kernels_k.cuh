@@ -22,236 +22,185 @@
 
 namespace fockx {
 
-// X[q] = scatter(c_{band0 + q}) on the sphere of one k point (X zeroed before).
-template <class T>
-__global__ void k_scatter_k(int npw, const int* __restrict__ gidx, int64_t ntot,
-                            const double2* __restrict__ psiG, int band0, cplx<T>* __restrict__ X) {
-  const int q = blockIdx.y;
-  cplx<T>* Xq = X + (int64_t)q * ntot;
-  for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < npw; k += gridDim.x * blockDim.x) {
-    const double2 c = psiG[(int64_t)(band0 + q) * npw + k];
-    Xq[gidx[k]] = cmake<T>(T(c.x), T(c.y));
-  }
-}
-
-// 2D FFT of plane i1 of X[q].  MODE 0: X -> u[band0 + q] * psi_scale (inverse
-// transform of the orbitals); MODE 1: W[band0 + q] -> X (forward transform of V_x psi).
-template <class T, int N, int SIGN, int MODE>
-__global__ void __launch_bounds__(Geo<T, N>::THR_PLANE)
-    k_plane_k(DevPlan g, cplx<T>* __restrict__ X, cplx<T>* __restrict__ U, int band0) {
-  using C = cplx<T>;
-  using G = Geo<T, N>;
-  constexpr int RP = G::RP;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  C* P = reinterpret_cast<C*>(smem_raw);
-  C* tw = P + N * RP;
-  const int i1 = blockIdx.x, q = blockIdx.y;
-  const int64_t plane0 = (int64_t)i1 * N * N;
-  C* Xq = X + (int64_t)q * g.ntot + plane0;
-  C* Ub = U + (int64_t)(band0 + q) * g.ntot + plane0;
-  load_twiddles<T>(tw, g);
-  for (int e = threadIdx.x; e < N * N; e += blockDim.x) {
-    const int i2 = e / N, i3 = e - i2 * N;
-    P[i2 * RP + i3] = MODE == 0 ? Xq[e] : Ub[e];
-  }
-  __syncthreads();
-  fft_lines<T, N, SIGN, N, G::TLP, RP, 1>(P, tw);  // along i3
-  fft_lines<T, N, SIGN, N, G::TLP, 1, RP>(P, tw);  // along i2
-  const T s = T(g.psi_scale);
-  for (int e = threadIdx.x; e < N * N; e += blockDim.x) {
-    const int i2 = e / N, i3 = e - i2 * N;
-    const C z = P[i2 * RP + i3];
-    if (MODE == 0) Ub[e] = cmake<T>(z.x * s, z.y * s);
-    else Xq[e] = z;
-  }
-}
-
-// (V_x psi)(G) of band band0 + q on the sphere of one k point.
-template <class T>
-__global__ void k_gather_k(int npw, const int* __restrict__ gidx, int64_t ntot, double scale,
-                           const cplx<T>* __restrict__ X, int band0, double2* __restrict__ vpsiG) {
-  const int q = blockIdx.y;
-  const cplx<T>* Xq = X + (int64_t)q * ntot;
-  for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < npw; k += gridDim.x * blockDim.x) {
-    const cplx<T> y = Xq[gidx[k]];
-    vpsiG[(int64_t)(band0 + q) * npw + k] = make_double2(scale * double(y.x), scale * double(y.y));
-  }
-}
-
-// Forward plane pass of a pair: plane i1 of u_a* u_b, 2D FFT, whole plane to H.
+// Forward plane pass of a pair: plane i1 of u_a* u_b to the kept columns of H.
 template <class T, int N>
-__global__ void __launch_bounds__(Geo<T, N>::THR_PLANE)
+__global__ void __launch_bounds__(PairGeo<T, N>::THR_PLANE, PairGeo<T, N>::MIN_PLANE)
     k_kpair_fwd(DevPlan g, const cplx<T>* __restrict__ u, const Chain* __restrict__ chains,
                 cplx<T>* __restrict__ H) {
   using C = cplx<T>;
-  using G = Geo<T, N>;
-  constexpr int RP = G::RP;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  C* P = reinterpret_cast<C*>(smem_raw);
-  C* tw = P + N * RP;
   const int i1 = blockIdx.x;
   const Chain ch = chains[blockIdx.y];
-  load_twiddles<T>(tw, g);
   const int64_t plane0 = (int64_t)i1 * N * N;
   const C* ua = u + (int64_t)ch.ai * g.ntot + plane0;
   const C* ub = u + (int64_t)ch.aj * g.ntot + plane0;
-  // columns first, the first stage reading conj(u_a) u_b straight from global
-  // memory (consecutive columns per warp: coalesced), then the rows
-  const auto product = [&](int i3, int i2) {
-    const int e = i2 * N + i3;
-    const C a = ua[e], b = ub[e];
-    return cmake<T>(a.x * b.x + a.y * b.y, a.x * b.y - a.y * b.x);  // conj(a) b
-  };
-  fft_lines_from<T, N, -1, N, G::TLP, 1, RP, kMaxThreads>(P, tw, product);  // along i2
-  fft_lines<T, N, -1, N, G::TLP, RP, 1>(P, tw);                            // along i3
-  C* Hp = H + (int64_t)blockIdx.y * g.ntot + plane0;
-  for (int e = threadIdx.x; e < N * N; e += blockDim.x) {
-    const int i2 = e / N, i3 = e - i2 * N;
-    Hp[e] = P[i2 * RP + i3];
-  }
+  plane_forward<T, N, PairGeo<T, N>::THR_PLANE, 0>(g, g.cols, H + (int64_t)blockIdx.y * g.ntot + plane0, smem_raw,
+                                                   [&](int e) {
+                                                     const C a = ua[e], b = ub[e];
+                                                     return cmake<T>(a.x * b.x + a.y * b.y, a.x * b.y - a.y * b.x);
+                                                   });
 }
 
-// Column pass of a pair: row k2, FFT along i1, times v(G + q) / Ntot, energy
-// partial sum_G v(G + q) |rho(G)|^2, inverse FFT along k1.
+// One kernel term with |m + q|^2 <= msmall2 (reduced coordinates) of the
+// mixed-form column pass in FP64, from the FP64 table; the one with m + q = 0
+// (q = 0 pairs) from the FP64 overlap of the pair's coefficients when the plan
+// provides it.  Kept out of line so the FP64 instructions are not predicated
+// into every warp of the kernel.
 template <class T, int N>
-__global__ void __launch_bounds__(Geo<T, N>::THR_COLF, Geo<T, N>::MIN_CTAS)
+__device__ __noinline__ void small_gq_term_fp64(const DevPlan& g, cplx<T>* z, int k1, int k2, int k3, const Chain& ch,
+                                                double* epair) {
+  double zx = z->x, zy = z->y;
+  if (g.kovl_re != nullptr && ch.pad1 == g.q0 && k1 == 0 && k2 == 0 && k3 == 0 && ch.ai / g.kovl_nb == ch.aj / g.kovl_nb) {
+    // q = 0 pair (a, b) of one k point: sum over the grid of conj(u_a) u_b
+    const int nb = g.kovl_nb, kk = ch.ai / nb;
+    const int64_t oi = ((int64_t)kk * nb + ch.ai % nb) * nb + ch.aj % nb;
+    zx = g.ovl_scale * g.kovl_re[oi];
+    zy = g.ovl_scale * g.kovl_im[oi];
+  }
+  const double v = g.vtabq64[(int64_t)ch.pad1 * g.ntot + ((int64_t)k1 * N + k2) * N + k3];
+  if (ch.pa >= 0) atomicAdd(&epair[ch.pa], v * (zx * zx + zy * zy));
+  const double vs = v * g.inv_ntot;
+  *z = cmake<T>(T(zx * vs), T(zy * vs));
+}
+
+// Column pass of a pair: the NL lines `cta` of the column map, FFT along i1,
+// times v(G + q) / Ntot, energy partial sum_G v(G + q) |rho(G)|^2, inverse FFT
+// along k1.  As the Gamma-point column pass: the forward B-stage, the multiply
+// and the inverse B-stage run in registers.
+template <class T, int N>
+__global__ void __launch_bounds__(PairGeo<T, N>::THR_COL, PairGeo<T, N>::MIN_COL)
     k_kpair_col(DevPlan g, cplx<T>* __restrict__ H, const Chain* __restrict__ chains,
                 double* __restrict__ epair) {
   using C = cplx<T>;
-  using G = Geo<T, N>;
+  using G = PairGeo<T, N>;
+  constexpr int A = G::CA, B = G::CB, NL = G::NL, THR = G::THR_COL;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C* S = reinterpret_cast<C*>(smem_raw);
-  C* tw = S + N * N;
-  double* red = reinterpret_cast<double*>(tw + G::TWN);
-  const int k2 = blockIdx.x;
+  C* tw = S + N * NL;
+  double* red = reinterpret_cast<double*>(tw + 2 * N);
   const Chain ch = chains[blockIdx.y];
-  C* Hc = H + (int64_t)blockIdx.y * g.ntot;
-  load_twiddles<T>(tw, g);
-  // the row k2 of every plane i1, read by the first stage of the transform
-  // along i1 straight from global memory
-  const auto val = [&](int i3, int i1) { return Hc[((int64_t)i1 * N + k2) * N + i3]; };
-  fft_lines_from<T, N, -1, N, G::TLP, 1, N, kMaxThreads>(S, tw, val);  // along i1
-  const int64_t qoff = (int64_t)ch.pad1 * g.ntot;
-  double acc[4] = {0.0, 0.0, 0.0, 0.0};
-  if constexpr (sizeof(T) == 8) {
-    const double* v64 = g.vtabq64 + qoff;
-    for (int e = threadIdx.x; e < N * N; e += blockDim.x) {
-      const int k1 = e / N, k3 = e - k1 * N;
-      const double v = v64[((int64_t)k1 * N + k2) * N + k3];
-      C z = S[e];
-      acc[0] += v * (z.x * z.x + z.y * z.y);
-      const double vs = v * g.inv_ntot;
-      z.x *= vs;
-      z.y *= vs;
-      S[e] = z;
+  load_stage_twiddles<T, -1, B, N, THR>(tw, g);
+  load_stage_twiddles<T, +1, A, N, THR>(tw + N, g);
+  const int l = threadIdx.x % NL;
+  const int code = __ldg(g.cols.lines + blockIdx.x * NL + l);
+  const int k2 = code >= 0 ? line_k2(code) : 0, k3 = code >= 0 ? line_k3(code) : 0;
+  C* lp = code >= 0 ? H + (int64_t)blockIdx.y * g.ntot + k2 * N + k3 : nullptr;
+#pragma unroll(kItemUnroll<T>)
+  for (int b0 = 0; b0 < B; b0 += THR / NL) {
+    const int b = b0 + threadIdx.x / NL;
+    if (B % (THR / NL) == 0 || b < B) {
+      C x[A];
+#pragma unroll
+      for (int r = 0; r < A; ++r) {
+        if (lp != nullptr) x[r] = ldcg_c(lp + (int64_t)(b + B * r) * (N * N));
+        else x[r] = cmake<T>(T(0), T(0));
+      }
+      Dft<-1, T>::template run<A>(x);
+#pragma unroll
+      for (int q = 0; q < A; ++q) S[(b + B * q) * NL + l] = x[q];
     }
-  } else {
-    const T* vt = static_cast<const T*>(g.vtabq) + qoff;  // v / Ntot
-    float accf[4] = {0.f, 0.f, 0.f, 0.f};
-    // the terms with |m + q|^2 <= msmall2 (reduced coordinates) in FP64 from
-    // the FP64 table; the one with m + q = 0 (q = 0 pairs) from the FP64
-    // overlap of the pair's coefficients when the plan provides it
-    bool row_small = false;
-    float q1 = 0.f, q3 = 0.f, r2 = 0.f;
-    if (g.qfrac != nullptr && g.msmall2 >= 0) {
-      q1 = g.qfrac[3 * ch.pad1];
-      q3 = g.qfrac[3 * ch.pad1 + 2];
-      const float m2 = float(freq_of(k2, N)) + g.qfrac[3 * ch.pad1 + 1];
-      r2 = m2 * m2;
-      row_small = r2 <= float(g.msmall2);
+  }
+  const int64_t vo = (int64_t)ch.pad1 * g.ntot + k2 * N + k3;
+  const T* vt = static_cast<const T*>(g.vtabq) + vo;  // v / Ntot
+  // whether this line holds terms with |m + q|^2 <= msmall2 (mixed form)
+  bool small = false;
+  float q1 = 0.f, r23 = 0.f;
+  if constexpr (sizeof(T) == 4) {
+    if (g.qfrac != nullptr && g.msmall2 >= 0 && code >= 0) {
+      const float* qf = g.qfrac + 3 * ch.pad1;
+      q1 = qf[0];
+      const float m2 = float(freq_of(k2, N)) + qf[1], m3 = float(freq_of(k3, N)) + qf[2];
+      r23 = m2 * m2 + m3 * m3;
+      small = r23 <= float(g.msmall2);
     }
-    if (!row_small) {
-      for (int e = threadIdx.x; e < N * N; e += blockDim.x) {
-        const int k1 = e / N, k3 = e - k1 * N;
-        const T v = vt[((int64_t)k1 * N + k2) * N + k3];
-        C z = S[e];
-        accf[0] += v * (z.x * z.x + z.y * z.y);
-        z.x *= v;
-        z.y *= v;
-        S[e] = z;
+  }
+  T acc = T(0);
+  __syncthreads();
+  for (int item = threadIdx.x; item < NL * A; item += THR) {
+    const int q = item / NL;
+    C z[B];
+    T v[B];
+#pragma unroll
+    for (int s = 0; s < B; ++s) v[s] = vt[(q + A * s) * (N * N)];
+#pragma unroll
+    for (int b = 0; b < B; ++b) z[b] = S[(B * q + b) * NL + l];
+    dft_twiddled<T, B, -1>(z, tw + q * B);
+    if constexpr (sizeof(T) == 8) {
+      const double* v64 = g.vtabq64 + vo;
+#pragma unroll
+      for (int s = 0; s < B; ++s) {
+        acc += v64[(q + A * s) * (N * N)] * (z[s].x * z[s].x + z[s].y * z[s].y);
+        z[s] = cmake<T>(z[s].x * v[s], z[s].y * v[s]);
       }
     } else {
-      const double* v64 = g.vtabq64 + qoff;
-      double e64 = 0.0;
-      // |m1 + q1|^2 <= msmall2 - m2q^2 bounds |m1| by b1 (and m3 by b3): an
-      // integer box test first, the exact one inside it; k3 is the same for
-      // all of a thread's elements when the CTA's threads are a multiple of N
-      const float lim = sqrtf(float(g.msmall2) - r2);
-      const int b1 = min(N / 2 - 1, (int)floorf(lim + fabsf(q1))), b3 = min(N / 2 - 1, (int)floorf(lim + fabsf(q3)));
-      const bool k3_fixed = blockDim.x % N == 0;
-      const int k3t = threadIdx.x % N;
-      const bool box3_t = (k3t + b3 < N ? k3t + b3 : k3t + b3 - N) <= 2 * b3;
-      for (int e = threadIdx.x; e < N * N; e += blockDim.x) {
-        const int k1 = e / N, k3 = e - k1 * N;
-        const int64_t vi = ((int64_t)k1 * N + k2) * N + k3;
-        C z = S[e];
-        const int w1 = k1 + b1 < N ? k1 + b1 : k1 + b1 - N;
-        const bool box3 = k3_fixed ? box3_t : (k3 + b3 < N ? k3 + b3 : k3 + b3 - N) <= 2 * b3;
-        bool small = false;
-        if (box3 && w1 <= 2 * b1) {
-          const float m1 = float(freq_of(k1, N)) + q1, m3 = float(freq_of(k3, N)) + q3;
-          small = m1 * m1 + r2 + m3 * m3 <= float(g.msmall2);
+      // FP64 terms leave the array while the FP32 loop runs; at most five k1 of
+      // a line hold one (|m1 + q1| < 2, |q1| < 1)
+      if (!small) {
+#pragma unroll
+        for (int s = 0; s < B; ++s) {
+          acc += v[s] * (z[s].x * z[s].x + z[s].y * z[s].y);
+          z[s] = cmake<T>(z[s].x * v[s], z[s].y * v[s]);
         }
-        if (small) {
-          double zx = z.x, zy = z.y;
-          if (g.kovl_re != nullptr && ch.pad1 == g.q0 && k1 == 0 && k2 == 0 && k3 == 0 &&
-              ch.ai / g.kovl_nb == ch.aj / g.kovl_nb) {
-            // q = 0 pair (a, b) of one k point: sum over the grid of conj(u_a) u_b
-            const int nb = g.kovl_nb, kk = ch.ai / nb;
-            const int64_t oi = ((int64_t)kk * nb + ch.ai % nb) * nb + ch.aj % nb;
-            zx = g.ovl_scale * g.kovl_re[oi];
-            zy = g.ovl_scale * g.kovl_im[oi];
+      } else {
+#pragma unroll
+        for (int s = 0; s < B; ++s) {
+          const float m1 = float(freq_of(q + A * s, N)) + q1;
+          if (m1 * m1 + r23 <= float(g.msmall2)) {
+            C t = z[s];
+            small_gq_term_fp64<T, N>(g, &t, q + A * s, k2, k3, ch, epair);
+            z[s] = t;
+          } else {
+            acc += v[s] * (z[s].x * z[s].x + z[s].y * z[s].y);
+            z[s] = cmake<T>(z[s].x * v[s], z[s].y * v[s]);
           }
-          const double v = v64[vi];
-          e64 += v * (zx * zx + zy * zy);
-          const double vs = v * g.inv_ntot;
-          z.x = T(zx * vs);
-          z.y = T(zy * vs);
-        } else {
-          const T v = vt[vi];
-          accf[0] += v * (z.x * z.x + z.y * z.y);
-          z.x *= v;
-          z.y *= v;
         }
-        S[e] = z;
       }
-      if (e64 != 0.0 && ch.pa >= 0) atomicAdd(&epair[ch.pa], e64);
     }
-    float hi[4], lo[4];
-    block_sum4_ff(accf, hi, lo, reinterpret_cast<float*>(red));
-    if (threadIdx.x == 0) acc[0] = ((double)hi[0] + (double)lo[0]) * double(g.ntot);
+    Dft<+1, T>::template run<B>(z);
+#pragma unroll
+    for (int b = 0; b < B; ++b) S[(B * q + b) * NL + l] = z[b];
   }
-  __syncthreads();
-  fft_lines<T, N, +1, N, G::TLP, 1, N>(S, tw);  // inverse along k1
-  for (int e = threadIdx.x; e < N * N; e += blockDim.x) {
-    const int i1 = e / N, i3 = e - i1 * N;
-    Hc[((int64_t)i1 * N + k2) * N + i3] = S[e];
+  double e = 0.0;
+  if constexpr (sizeof(T) == 8) {
+    double e4[4] = {code >= 0 ? acc : 0.0, 0.0, 0.0, 0.0};
+    block_sum4(e4, red);
+    e = e4[0];
+  } else {
+    float a[4] = {code >= 0 ? acc : 0.f, 0.f, 0.f, 0.f}, hi[4], lo[4];
+    block_sum4_ff(a, hi, lo, reinterpret_cast<float*>(red));
+    if (threadIdx.x == 0) e = ((double)hi[0] + (double)lo[0]) * double(g.ntot);
   }
-  if constexpr (sizeof(T) == 8) block_sum4(acc, red);
-  if (threadIdx.x == 0 && ch.pa >= 0) atomicAdd(&epair[ch.pa], acc[0]);
+  if (threadIdx.x == 0 && ch.pa >= 0) atomicAdd(&epair[ch.pa], e);
+  if (lp != nullptr) {
+#pragma unroll(kItemUnroll<T>)
+    for (int b0 = 0; b0 < B; b0 += THR / NL) {
+      const int b = b0 + threadIdx.x / NL;
+      if (B % (THR / NL) == 0 || b < B) {
+        C x[A];
+#pragma unroll
+        for (int q = 0; q < A; ++q) x[q] = S[(b + B * q) * NL + l];
+        dft_twiddled<T, A, +1>(x, tw + N + b * A);
+#pragma unroll
+        for (int r = 0; r < A; ++r) lp[(int64_t)(b + B * r) * (N * N)] = x[r];
+      }
+    }
+  }
 }
 
 // Inverse plane pass of a pair and the W updates.
 template <class T, int N>
-__global__ void __launch_bounds__(Geo<T, N>::THR_PLANE, Geo<T, N>::MIN_CTAS_KINV)
+__global__ void __launch_bounds__(PairGeo<T, N>::THR_PLANE, PairGeo<T, N>::MIN_PLANE)
     k_kpair_inv(DevPlan g, const cplx<T>* __restrict__ u, cplx<T>* __restrict__ W,
                 const T* __restrict__ occw, const Chain* __restrict__ chains, const cplx<T>* __restrict__ H) {
   using C = cplx<T>;
-  using G = Geo<T, N>;
-  constexpr int RP = G::RP;
+  using G = PairGeo<T, N>;
+  constexpr int RP = G::RP, THR = G::THR_PLANE;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  C* P = reinterpret_cast<C*>(smem_raw);
-  C* tw = P + N * RP;
+  const C* P = reinterpret_cast<const C*>(smem_raw);
   const int i1 = blockIdx.x;
   const Chain ch = chains[blockIdx.y];
-  load_twiddles<T>(tw, g);
   const int64_t plane0 = (int64_t)i1 * N * N;
-  const C* Hp = H + (int64_t)blockIdx.y * g.ntot + plane0;
-  // the plane, read by the first stage of the transform along k2 straight from
-  // global memory (consecutive columns k3 per warp), then the rows
-  const auto val = [&](int k3, int k2) { return Hp[k2 * N + k3]; };
-  fft_lines_from<T, N, +1, N, G::TLP, 1, RP, kMaxThreads>(P, tw, val);  // along k2
-  fft_lines<T, N, +1, N, G::TLP, RP, 1>(P, tw);                        // along k3
+  plane_inverse<T, N, THR, 0>(g, g.cols, H + (int64_t)blockIdx.y * g.ntot + plane0, smem_raw);
   const int a = ch.ai, b = ch.aj;
   const bool both = a != b;
   const T fa = occw[a], fb = occw[b];
@@ -260,12 +209,12 @@ __global__ void __launch_bounds__(Geo<T, N>::THR_PLANE, Geo<T, N>::MIN_CTAS_KINV
   C* wa = W + (int64_t)a * g.ntot + plane0;
   C* wb = W + (int64_t)b * g.ntot + plane0;
   if constexpr (sizeof(T) == 4) {
-    static_assert(N % 2 == 0, "pairwise vector updates need even N");
     // two complex points per thread: one 16-byte vector atomic per target
-    for (int e2 = threadIdx.x; e2 < N * N / 2; e2 += blockDim.x) {
-      const int e = 2 * e2;
-      const int i2 = e / N, i3 = e - i2 * N;
-      const C p0 = P[i2 * RP + i3], p1 = P[i2 * RP + i3 + 1];
+    for (int e2 = threadIdx.x; e2 < N * N / 2; e2 += THR) {
+      const int row = e2 / (N / 2), c = e2 - row * (N / 2);
+      const int e = G::row_of(row) * N + 2 * c;
+      const C* p = P + row * RP;
+      const C p0 = p[G::col_place(2 * c)], p1 = p[G::col_place(2 * c + 1)];
       const float4 va = *reinterpret_cast<const float4*>(ua + e);
       float4 d;  // -fa * ua * phi
       d.x = -fa * (va.x * p0.x - va.y * p0.y);
@@ -288,9 +237,9 @@ __global__ void __launch_bounds__(Geo<T, N>::THR_PLANE, Geo<T, N>::MIN_CTAS_KINV
       }
     }
   } else {
-    for (int e = threadIdx.x; e < N * N; e += blockDim.x) {
+    for (int e = threadIdx.x; e < N * N; e += THR) {
       const int i2 = e / N, i3 = e - i2 * N;
-      const C p = P[i2 * RP + i3];
+      const C p = P[G::place_of_row(i2) * RP + G::col_place(i3)];
       const C x = ua[e];
       atomicAdd(&wb[e].x, -fa * (x.x * p.x - x.y * p.y));
       atomicAdd(&wb[e].y, -fa * (x.x * p.y + x.y * p.x));
@@ -306,31 +255,27 @@ __global__ void __launch_bounds__(Geo<T, N>::THR_PLANE, Geo<T, N>::MIN_CTAS_KINV
 template <class T, int N>
 struct LaunchK {
   using C = cplx<T>;
-  using G = Geo<T, N>;
+  using G = PairGeo<T, N>;
 
   static cudaError_t configure() {
-    const void* fns[] = {(const void*)k_plane_k<T, N, +1, 0>, (const void*)k_plane_k<T, N, -1, 1>,
-                         (const void*)k_kpair_fwd<T, N>, (const void*)k_kpair_inv<T, N>,
-                         (const void*)k_col_full<T, N, +1>, (const void*)k_col_full<T, N, -1>};
-    for (const void* f : fns) {
-      cudaError_t err = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)G::SMEM_PLANE);
+    for (const void* f : {(const void*)k_orb_plane_inv<T, N, true>, (const void*)k_orb_plane_fwd<T, N, true>,
+                          (const void*)k_kpair_fwd<T, N>, (const void*)k_kpair_inv<T, N>}) {
+      cudaError_t err = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)G::SMEM_PLANE);
       if (err != cudaSuccess) return err;
     }
-    return cudaFuncSetAttribute((const void*)k_kpair_col<T, N>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)smem_colk());
+    for (const void* f : {(const void*)k_orb_col_inv<T, N, true>, (const void*)k_orb_col_fwd<T, N, true>,
+                          (const void*)k_kpair_col<T, N>}) {
+      cudaError_t err = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)G::SMEM_COL);
+      if (err != cudaSuccess) return err;
+    }
+    return cudaSuccess;
   }
 
-  static constexpr size_t smem_colk() { return sizeof(C) * (size_t)(N * N + G::TWN) + 32 * 4 * sizeof(double); }
-
-  static cudaError_t to_real(const DevPlan& g, const double2* psiG, int npw, const int* gidx, int band0,
-                             int nbat, void* Xv, void* u, cudaStream_t s) {
+  static cudaError_t to_real(const DevPlan& g, const ColumnSet& orb, const double2* psiG, int npw, int band0, int nbat,
+                             void* Xv, void* u, cudaStream_t s) {
     C* X = static_cast<C*>(Xv);
-    cudaError_t err = cudaMemsetAsync(X, 0, sizeof(C) * (size_t)g.ntot * nbat, s);
-    if (err != cudaSuccess) return err;
-    k_scatter_k<T><<<dim3((npw + 255) / 256, nbat), 256, 0, s>>>(npw, gidx, g.ntot, psiG, 0, X);
-    k_col_full<T, N, +1><<<dim3(N, nbat), G::THR_COLF, G::SMEM_COLF, s>>>(g, X);
-    k_plane_k<T, N, +1, 0><<<dim3(N, nbat), G::THR_PLANE, G::SMEM_PLANE, s>>>(g, X, static_cast<C*>(u), band0);
+    k_orb_col_inv<T, N, true><<<dim3(orb.ncta, nbat), G::THR_COL, G::SMEM_COL, s>>>(g, orb, psiG, npw, nbat, 0, nbat, X);
+    k_orb_plane_inv<T, N, true><<<dim3(N, nbat), G::THR_PLANE, G::SMEM_PLANE, s>>>(g, orb, X, u, band0, nbat, nbat);
     return cudaGetLastError();
   }
 
@@ -343,7 +288,7 @@ struct LaunchK {
 
   static cudaError_t pair_col(const DevPlan& g, void* H, const Chain* ch, int nch, double* ep,
                               cudaStream_t s) {
-    k_kpair_col<T, N><<<dim3(N, nch), G::THR_COLF, smem_colk(), s>>>(g, static_cast<C*>(H), ch, ep);
+    k_kpair_col<T, N><<<dim3(g.cols.ncta, nch), G::THR_COL, G::SMEM_COL, s>>>(g, static_cast<C*>(H), ch, ep);
     return cudaGetLastError();
   }
 
@@ -355,18 +300,17 @@ struct LaunchK {
     return cudaGetLastError();
   }
 
-  static cudaError_t to_sphere(const DevPlan& g, const void* W, int band0, int nbat, int npw, const int* gidx,
+  static cudaError_t to_sphere(const DevPlan& g, const ColumnSet& orb, const void* W, int band0, int nbat, int npw,
                                void* Xv, double2* vpsiG, cudaStream_t s) {
     C* X = static_cast<C*>(Xv);
-    k_plane_k<T, N, -1, 1><<<dim3(N, nbat), G::THR_PLANE, G::SMEM_PLANE, s>>>(
-        g, X, const_cast<C*>(static_cast<const C*>(W)), band0);
-    k_col_full<T, N, -1><<<dim3(N, nbat), G::THR_COLF, G::SMEM_COLF, s>>>(g, X);
-    k_gather_k<T><<<dim3((npw + 255) / 256, nbat), 256, 0, s>>>(npw, gidx, g.ntot, g.out_scale, X, 0, vpsiG);
+    k_orb_plane_fwd<T, N, true><<<dim3(N, nbat), G::THR_PLANE, G::SMEM_PLANE, s>>>(g, orb, W, X, band0, nbat, nbat);
+    k_orb_col_fwd<T, N, true><<<dim3(orb.ncta, nbat), G::THR_COL, G::SMEM_COL, s>>>(g, orb, X, g.out_scale, npw, nbat,
+                                                                                  0, nbat, vpsiG);
     return cudaGetLastError();
   }
 
   static constexpr KOps ops() {
-    return KOps{configure, to_real, pair_fwd, pair_col, pair_inv, to_sphere};
+    return KOps{G::NL, configure, to_real, pair_fwd, pair_col, pair_inv, to_sphere};
   }
 };
 

@@ -12,6 +12,7 @@
 #include <vector>
 
 #include "fock.h"
+#include "fock_columns.h"
 #include "fock_internal.h"
 #include "fock_lattice.h"
 
@@ -40,7 +41,9 @@ struct fock_kplan {
   std::vector<double> kfrac, wk;
   std::vector<std::vector<int32_t>> miller;
   std::vector<int> npw;
-  std::vector<int*> d_gidx;
+  int* d_cols = nullptr;  // DevPlan::cols
+  std::vector<int*> d_orb;  // the columns of each k point's sphere, and the set on the device
+  std::vector<fockx::ColumnSet> orb;
   int nq = 0;
   std::vector<int> qidx;  // [ka * nk + kb] -> distinct q = k_b - k_a
   void* d_vq = nullptr;
@@ -209,9 +212,6 @@ fock_status fock_kplan_create(fock_kplan_t* out, const int grid[3], const double
 
   // one sphere per k point (host only: a grid is refused before any CUDA call)
   const int64_t ntot = (int64_t)n * n * n;
-  auto off = [n](int m1, int m2, int m3) {
-    return ((((m1 % n) + n) % n) * n + (((m2 % n) + n) % n)) * n + (((m3 % n) + n) % n);
-  };
   std::vector<fockx::lattice::GEntry> sph;
   std::vector<int> mlo((size_t)3 * nk), mhi((size_t)3 * nk);
   for (int k = 0; k < nk; ++k) {
@@ -250,16 +250,48 @@ fock_status fock_kplan_create(fock_kplan_t* out, const int grid[3], const double
                               "(need N > 2 (max m - min m') over every pair of spheres)"));
   cudaError_t e = cudaGetDevice(&p->device);
   if (e != cudaSuccess) return bail(kcuda(p, e, "cudaGetDevice"));
+  // the columns of each sphere, and those the pair densities reach: |G + q| <= 2
+  // Gmax for some q = k_b - k_a, inside the ball |G| <= 2 Gmax + max |q|
+  const auto wrap = [n](int m) { return ((m % n) + n) % n; };
+  std::vector<unsigned char> mark((size_t)n * n, 0);
+  int64_t bytes = 0;
   for (int k = 0; k < nk; ++k) {
     const std::vector<int32_t>& mill = p->miller[k];
-    std::vector<int> gidx(mill.size() / 3);
-    for (size_t g = 0; g < gidx.size(); ++g) gidx[g] = off(mill[3 * g], mill[3 * g + 1], mill[3 * g + 2]);
-    int* d = nullptr;
-    if ((e = cudaMalloc((void**)&d, sizeof(int) * std::max<size_t>(1, gidx.size()))) != cudaSuccess)
-      return bail(kcuda(p, e, "cudaMalloc"));
-    p->d_gidx.push_back(d);
-    if ((e = cudaMemcpy(d, gidx.data(), sizeof(int) * gidx.size(), cudaMemcpyHostToDevice)) != cudaSuccess)
-      return bail(kcuda(p, e, "cudaMemcpy"));
+    std::fill(mark.begin(), mark.end(), 0);
+    for (size_t g = 0; 3 * g < mill.size(); ++g) mark[(size_t)wrap(mill[3 * g + 1]) * n + wrap(mill[3 * g + 2])] = 1;
+    fockx::columns::HostColumns c;
+    fockx::columns::build(n, mark, false, kops->col_lines, ops->row_place, c);
+    p->d_orb.push_back(nullptr);
+    p->orb.emplace_back();
+    e = fockx::columns::upload(
+        c, fockx::columns::coefficient_map(n, c, kops->col_lines, false, mill.data(), mill.size() / 3), &p->d_orb[k],
+        &p->orb[k], &bytes);
+    if (e != cudaSuccess) return bail(kcuda(p, e, "uploading a sphere's columns"));
+  }
+  {
+    double q2max = 0.0;
+    for (int ka = 0; ka < nk; ++ka)
+      for (int kb = 0; kb < nk; ++kb) {
+        double q[3];
+        for (int a = 0; a < 3; ++a) q[a] = p->kfrac[3 * kb + a] - p->kfrac[3 * ka + a];
+        q2max = std::max(q2max, fockx::lattice::g2_of(p->recip, 0, 0, 0, q));
+      }
+    const double r = (2.0 * std::sqrt(2.0 * ecut_ha) + std::sqrt(q2max)) * (1.0 + 1e-9);
+    int mb[3];
+    for (int a = 0; a < 3; ++a) {
+      const double len = std::sqrt(cell[3 * a] * cell[3 * a] + cell[3 * a + 1] * cell[3 * a + 1] +
+                                   cell[3 * a + 2] * cell[3 * a + 2]);
+      mb[a] = (int)std::floor(r * len / fockx::lattice::kTwoPi) + 1;
+    }
+    std::fill(mark.begin(), mark.end(), 0);
+    for (int m1 = -mb[0]; m1 <= mb[0]; ++m1)
+      for (int m2 = -mb[1]; m2 <= mb[1]; ++m2)
+        for (int m3 = -mb[2]; m3 <= mb[2]; ++m3)
+          if (fockx::lattice::g2_of(p->recip, m1, m2, m3) <= r * r) mark[(size_t)wrap(m2) * n + wrap(m3)] = 1;
+    fockx::columns::HostColumns c;
+    fockx::columns::build(n, mark, false, kops->col_lines, ops->row_place, c);
+    e = fockx::columns::upload(c, {}, &p->d_cols, &p->dp.cols, &bytes);
+    if (e != cudaSuccess) return bail(kcuda(p, e, "uploading the column sets"));
   }
 
   // distinct q = k_b - k_a and their kernel tables on the full grid
@@ -485,7 +517,7 @@ fock_status fock_kplan_apply(fock_kplan_t p, const void* const* psi_G, int nb, c
     for (int b0 = 0; b0 < nb; b0 += nbat) {
       const int cnt = std::min(nbat, nb - b0);
       const double2* src = static_cast<const double2*>(psi_G[k]) + (size_t)b0 * p->npw[k];
-      FOCK_KCUDA(p, p->kops->to_real(p->dp, src, p->npw[k], p->d_gidx[k], k * nb + b0, cnt, p->d_h, p->d_u, s));
+      FOCK_KCUDA(p, p->kops->to_real(p->dp, p->orb[k], src, p->npw[k], k * nb + b0, cnt, p->d_h, p->d_u, s));
     }
   DevPlan dp = p->dp;
   if (p->ops->real_bytes == 4 && dp.q0 >= 0) {
@@ -521,7 +553,7 @@ fock_status fock_kplan_apply(fock_kplan_t p, const void* const* psi_G, int nb, c
     for (int b0 = 0; b0 < nb; b0 += nbat) {
       const int cnt = std::min(nbat, nb - b0);
       double2* dst = static_cast<double2*>(vpsi_G[k]) + (size_t)b0 * p->npw[k];
-      FOCK_KCUDA(p, p->kops->to_sphere(p->dp, p->d_w, k * nb + b0, cnt, p->npw[k], p->d_gidx[k], p->d_h, dst, s));
+      FOCK_KCUDA(p, p->kops->to_sphere(p->dp, p->orb[k], p->d_w, k * nb + b0, cnt, p->npw[k], p->d_h, dst, s));
     }
   const double scale = -0.5 * p->vol / ((double)p->dp.ntot * (double)p->dp.ntot);
   FOCK_KCUDA(p, fockx::launch_energy_reduce(p->d_pairs, npairs, p->d_occw, p->d_epair, nullptr, scale,
@@ -539,7 +571,8 @@ const char* fock_kplan_last_error(fock_kplan_t p) { return p ? p->err.c_str() : 
 fock_status fock_kplan_destroy(fock_kplan_t p) {
   if (!p) return FOCK_OK;
   kfree_ws(p);
-  for (int* d : p->d_gidx) cudaFree(d);
+  for (int* d : p->d_orb) cudaFree(d);
+  cudaFree(p->d_cols);
   cudaFree(p->d_vq);
   cudaFree(p->d_vq64);
   cudaFree(p->d_qfrac);

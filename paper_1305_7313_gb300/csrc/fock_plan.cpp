@@ -15,6 +15,7 @@
 #include <string>
 #include <vector>
 
+#include "fock_columns.h"
 #include "fock_internal.h"
 #include "fock_lattice.h"
 
@@ -79,23 +80,19 @@ struct fock_plan {
   int chain_batch = 1;
   int band_block = kBandBlock;
   // device tables
-  int* d_gidx = nullptr;
-  int* d_gidxneg = nullptr;
   void* d_tw = nullptr;
   void* d_vtab = nullptr;
   void* d_dvtab = nullptr;
   double* d_vtab64 = nullptr;
   double* d_dvtab64 = nullptr;
-  int* d_ncol = nullptr;
-  int* d_colmap = nullptr;
-  int* d_kept = nullptr;
-  int* d_rowpos = nullptr;
+  int* d_cols = nullptr;  // DevPlan::cols and orb
+  int* d_orb = nullptr;
   // deterministic accumulation (fock_plan_set_deterministic)
   bool det = false;
   double vnorm = 0.0;          // ||v||_2 over the whole grid
   double* d_stats = nullptr;   // [2 * det_nb_cap] per-band max |psi| and sum psi^2
   double* d_scale = nullptr;   // [2] fixed-point scale 2^s and 2^-s
-  double* d_epart = nullptr;   // [det_npair_cap * ncta_col] per-CTA energy partials
+  double* d_epart = nullptr;   // [det_npair_cap * cols.ncta] per-CTA energy partials
   double* d_dpart = nullptr;
   int det_nb_cap = 0;
   int det_npair_cap = 0;
@@ -105,6 +102,9 @@ struct fock_plan {
   int64_t ovl_cap = 0;
   int* d_half = nullptr;  // G = 0, then one of each pair G, -G of the sphere (positions)
   int nhalf_g = 0;
+  // arrays of the Sternheimer solves
+  void* d_st = nullptr;
+  size_t st_cap = 0;
   // FP64: the kernel table scaled by -f0 (DevPlan::vtab_f)
   void* d_vtab_f = nullptr;
   double vtab_f_f0 = 0.0;
@@ -448,90 +448,6 @@ fock_status prepare_prescaled(fock_plan* p, const double* occ, int nb, DevPlan* 
   return FOCK_OK;
 }
 
-// The columns (k2, k3) of the pair densities' spectra that the pair passes keep.
-struct PairColumns {
-  std::vector<int> ncol;   // [N] per k3: k2 < (ncol & 0xffff) or k2 >= N - (ncol >> 16)
-  std::vector<int> kept;   // (k2 << 16) | k3, rows outer
-  std::vector<int> rowpos;  // [2][N] places of the kept rows in a transformed plane, ascending, per tiling
-  std::vector<int> pairs;  // (k2 << 16) | (self << 15) | k3 of one line of each mirror pair, rows outer
-  int64_t half_lines = 0;  // lines of the two densities' half spectra (k3 <= N/2) the ball marks
-  int row_lo = 0, row_hi = 0, col_max = 1;
-};
-
-void pair_columns(const fock_plan* p, PairColumns& out) {
-  const int n = p->n, kh = n / 2 + 1;
-  std::vector<unsigned char> mark((size_t)n * n, 0);
-  {
-    const double r2 = 8.0 * p->ecut * (1.0 + 1e-9);
-    int mb[3];
-    for (int a = 0; a < 3; ++a) {
-      const double* c = p->cell + 3 * a;
-      const double len = std::sqrt(c[0] * c[0] + c[1] * c[1] + c[2] * c[2]);
-      mb[a] = (int)std::floor(std::sqrt(r2) * len / (2.0 * kPi)) + 1;
-    }
-    for (int m1 = -mb[0]; m1 <= mb[0]; ++m1)
-      for (int m2 = -mb[1]; m2 <= mb[1]; ++m2)
-        for (int m3 = -mb[2]; m3 <= mb[2]; ++m3)
-          if (g2_of(p->recip, m1, m2, m3) <= r2)
-            mark[(size_t)(((m2 % n) + n) % n) * n + (((m3 % n) + n) % n)] = 1;
-  }
-  for (int k2 = 0; k2 < n; ++k2) {
-    int c = 0;
-    for (int k3 = 0; k3 < kh; ++k3)
-      if (mark[(size_t)k2 * n + k3]) c = k3 + 1;
-    out.half_lines += 2 * c;
-  }
-  // per column k3 <= N/2 the smallest runs k2 < up and k2 >= n - dn that cover
-  // the marked k2; the mirror column n - k3 keeps the mirror images.  Columns
-  // 0 and N/2 are their own mirror images: up = dn + 1 (k2 = 0 has no partner)
-  out.ncol.assign(n, 0);
-  for (int k3 = 0; k3 < kh; ++k3) {
-    int up = 0, dn = 0;
-    for (int k2 = 0; k2 < n; ++k2)
-      if (mark[(size_t)k2 * n + k3]) {
-        if (2 * k2 <= n) up = std::max(up, k2 + 1);
-        else dn = std::max(dn, n - k2);
-      }
-    if (up == 0 && dn == 0) continue;
-    up = std::max(up, 1);
-    if (k3 == 0 || 2 * k3 == n) {
-      up = std::max(up, dn + 1);
-      dn = up - 1;
-    }
-    out.ncol[k3] = up | (dn << 16);
-    if (k3 > 0 && 2 * k3 < n) out.ncol[n - k3] = (dn + 1) | ((up - 1) << 16);
-    out.col_max = std::max(out.col_max, k3 + 1);
-  }
-  const auto keeps = [&](int k2, int k3) {
-    return k2 < (out.ncol[k3] & 0xffff) || k2 >= n - (out.ncol[k3] >> 16);
-  };
-  for (int k3 = 0; k3 < n; ++k3) {
-    out.row_lo = std::max(out.row_lo, out.ncol[k3] & 0xffff);
-    out.row_hi = std::max(out.row_hi, out.ncol[k3] >> 16);
-  }
-  if (out.row_lo + out.row_hi >= n) {
-    out.row_lo = n;
-    out.row_hi = 0;
-  }
-  for (int t = 0; t < 2; ++t) {
-    std::vector<int> rows;
-    for (int k2 = 0; k2 < n; ++k2)
-      if (k2 < out.row_lo || k2 >= n - out.row_hi) rows.push_back(p->ops->row_place(t, k2));
-    std::sort(rows.begin(), rows.end());
-    rows.resize(n, 0);
-    out.rowpos.insert(out.rowpos.end(), rows.begin(), rows.end());
-  }
-  for (int k2 = 0; k2 < n; ++k2)
-    for (int k3 = 0; k3 < n; ++k3) {
-      if (!keeps(k2, k3)) continue;
-      out.kept.push_back((k2 << 16) | k3);
-      const int m2 = (n - k2) % n, m3 = (n - k3) % n;
-      const bool self = m2 == k2 && m3 == k3;
-      // the line with 0 < k3 < N/2, or of the two with k3 = 0 (N/2) the one with k2 <= N/2
-      if (k3 < m3 || (k3 == m3 && k2 <= m2)) out.pairs.push_back((k2 << 16) | (self ? 1 << 15 : 0) | k3);
-    }
-}
-
 int bands_per_grid_batch(const fock_plan* p) {
   const size_t grid_bytes = (size_t)p->dp.ntot * 2 * (size_t)p->ops->real_bytes;
   const int q = (int)std::max<size_t>(1, p->ws.h_bytes / grid_bytes);
@@ -543,7 +459,7 @@ fock_status orbitals_to_real(fock_plan* p, const void* psiG, int nb, cudaStream_
   p->stats.band_batch = nbat;
   for (int b0 = 0; b0 < nb; b0 += nbat) {
     const int cnt = std::min(nbat, nb - b0);
-    PhaseScope ps(p, FOCK_PHASE_TO_REAL, 3, s);
+    PhaseScope ps(p, FOCK_PHASE_TO_REAL, 2, s);
     FOCK_CUDA(p, p->ops->to_real(p->dp, static_cast<const double2*>(psiG), nb, b0, cnt, p->ws.h,
                                  p->ws.psi, s));
   }
@@ -573,7 +489,7 @@ fock_status det_buffers(fock_plan* p, int nbands, int npairs) {
     cudaFree(p->d_dpart);
     p->d_epart = p->d_dpart = nullptr;
     p->det_npair_cap = 0;
-    const size_t n = (size_t)npairs * (size_t)p->dp.ncta_col;
+    const size_t n = (size_t)npairs * (size_t)p->dp.cols.ncta;
     FOCK_CUDA(p, dev_alloc(&p->d_epart, sizeof(double) * n));
     FOCK_CUDA(p, dev_alloc(&p->d_dpart, sizeof(double) * n));
     p->det_npair_cap = npairs;
@@ -704,7 +620,7 @@ fock_status apply_impl(fock_plan* p, const void* psiG, int nb, const double* occ
   const int p0 = std::min(npairs, 2 * c0), p1 = std::min(npairs, 2 * c1);
   if (p->det) {
     FOCK_CUDA(p, fockx::launch_det_to_double(p->ws.w, (int64_t)nb * p->dp.ntot, p->d_scale, s));
-    const int nc = p->dp.ncta_col;
+    const int nc = p->dp.cols.ncta;
     FOCK_CUDA(p, fockx::launch_det_pair_sums(p->d_epart + (size_t)p0 * nc, p1 - p0, nc, p->ws.epair + p0, s));
     if (dp.dvtab64)
       FOCK_CUDA(p, fockx::launch_det_pair_sums(p->d_dpart + (size_t)p0 * nc, p1 - p0, nc, p->ws.dpair + p0, s));
@@ -713,7 +629,7 @@ fock_status apply_impl(fock_plan* p, const void* psiG, int nb, const double* occ
   const int nbat = bands_per_grid_batch(p);
   for (int b0 = 0; b0 < nb; b0 += nbat) {
     const int cnt = std::min(nbat, nb - b0);
-    PhaseScope ps(p, FOCK_PHASE_TO_SPHERE, 3, s);
+    PhaseScope ps(p, FOCK_PHASE_TO_SPHERE, 2, s);
     FOCK_CUDA(p, p->ops->to_sphere(p->dp, p->ws.w, nb, b0, cnt, p->ws.h,
                                    static_cast<double2*>(vpsiG), s));
   }
@@ -762,26 +678,6 @@ void plan_set_error(fock_plan* plan, const char* msg) {
 }
 
 }  // namespace fockx
-
-namespace {
-
-// Device buffers of one Sternheimer solve, freed on every exit path.
-struct StBuffers {
-  std::vector<void*> ptrs;
-  ~StBuffers() {
-    for (void* q : ptrs) cudaFree(q);
-  }
-  template <class P>
-  cudaError_t alloc(P** out, size_t bytes) {
-    void* q = nullptr;
-    const cudaError_t e = cudaMalloc(&q, bytes < 16 ? 16 : bytes);
-    if (e == cudaSuccess) ptrs.push_back(q);
-    *out = static_cast<P*>(q);
-    return e;
-  }
-};
-
-}  // namespace
 
 extern "C" {
 
@@ -862,19 +758,12 @@ fock_status fock_plan_create(fock_plan_t* out, const int grid[3], const double c
   }
   p->npw = (int)sph.size();
   p->miller.resize(3 * sph.size());
-  std::vector<int> gidx(sph.size()), gneg(sph.size());
-  auto off = [n](int m1, int m2, int m3) {
-    const int i1 = ((m1 % n) + n) % n, i2 = ((m2 % n) + n) % n, i3 = ((m3 % n) + n) % n;
-    return (i1 * n + i2) * n + i3;
-  };
   // half of the sphere for the Gamma-point overlaps: G = 0 first, then the G
   // whose first nonzero Miller index is positive
   std::vector<int> half;
   half.reserve(sph.size() / 2 + 1);
   for (size_t k = 0; k < sph.size(); ++k) {
     for (int a = 0; a < 3; ++a) p->miller[3 * k + a] = sph[k].m[a];
-    gidx[k] = off(sph[k].m[0], sph[k].m[1], sph[k].m[2]);
-    gneg[k] = off(-sph[k].m[0], -sph[k].m[1], -sph[k].m[2]);
     const int* m = sph[k].m;
     const int lead = m[0] != 0 ? m[0] : (m[1] != 0 ? m[1] : m[2]);
     if (lead == 0) half.insert(half.begin(), (int)k);
@@ -909,14 +798,35 @@ fock_status fock_plan_create(fock_plan_t* out, const int grid[3], const double c
   // |G|^2 <= 8 Ecut hits (indices modulo N, so a grid that aliases the pair
   // densities keeps what the aliases reach) are kept; the others hold rounding
   // noise only and are never stored, transformed or read.
-  PairColumns cols;
-  pair_columns(p, cols);
-  p->kept_columns = cols.half_lines;
-  const std::vector<int>&ncol = cols.ncol, &kept = cols.kept;
-  std::vector<int>& colmap = cols.pairs;
-  const int nlines = ops->col_lines;
-  const int ncta_col = std::max(1, (int)((colmap.size() + nlines - 1) / nlines));
-  colmap.resize((size_t)ncta_col * nlines, -1);
+  const auto wrap = [n](int m) { return ((m % n) + n) % n; };
+  std::vector<unsigned char> mark((size_t)n * n, 0);
+  {
+    const double r2 = 8.0 * ecut_ha * (1.0 + 1e-9);
+    int mb[3];
+    for (int a = 0; a < 3; ++a) {
+      const double len = std::sqrt(cell[3 * a] * cell[3 * a] + cell[3 * a + 1] * cell[3 * a + 1] +
+                                   cell[3 * a + 2] * cell[3 * a + 2]);
+      mb[a] = (int)std::floor(std::sqrt(r2) * len / (2.0 * kPi)) + 1;
+    }
+    for (int m1 = -mb[0]; m1 <= mb[0]; ++m1)
+      for (int m2 = -mb[1]; m2 <= mb[1]; ++m2)
+        for (int m3 = -mb[2]; m3 <= mb[2]; ++m3)
+          if (g2_of(p->recip, m1, m2, m3) <= r2) mark[(size_t)wrap(m2) * n + wrap(m3)] = 1;
+  }
+  for (int k2 = 0; k2 < n; ++k2) {
+    int c = 0;
+    for (int k3 = 0; k3 < kh; ++k3)
+      if (mark[(size_t)k2 * n + k3]) c = k3 + 1;
+    p->kept_columns += 2 * c;
+  }
+  fockx::columns::HostColumns cols, orb;
+  fockx::columns::build(n, mark, true, ops->col_pairs, ops->row_place, cols);
+  // and those of the sphere itself
+  std::fill(mark.begin(), mark.end(), 0);
+  for (const GEntry& e : sph) mark[(size_t)wrap(e.m[1]) * n + wrap(e.m[2])] = 1;
+  fockx::columns::build(n, mark, true, ops->col_pairs, ops->row_place, orb);
+  const std::vector<int> coef =
+      fockx::columns::coefficient_map(n, orb, ops->col_pairs, true, p->miller.data(), sph.size());
 
   const bool fp64 = prec == FOCK_PREC_FP64;
   // twiddles w[t] = exp(-2 pi i t / N)
@@ -943,16 +853,17 @@ fock_status fock_plan_create(fock_plan_t* out, const int grid[3], const double c
     delete p;
     return cuda_fail(nullptr, ge, "cudaGetDevice");
   }
-  bool ok = upload((void**)&p->d_gidx, gidx.data(), sizeof(int) * gidx.size()) &&
-            upload((void**)&p->d_gidxneg, gneg.data(), sizeof(int) * gneg.size()) &&
-            upload((void**)&p->d_half, half.data(), sizeof(int) * half.size()) &&
+  bool ok = upload((void**)&p->d_half, half.data(), sizeof(int) * half.size()) &&
             upload((void**)&p->d_vtab64, v64.data(), sizeof(double) * nhalf);
   if (ok && kind == FOCK_KERNEL_ERFC) ok = upload((void**)&p->d_dvtab64, dv64.data(), sizeof(double) * nhalf);
-  if (ok)
-    ok = upload((void**)&p->d_ncol, ncol.data(), sizeof(int) * ncol.size()) &&
-         upload((void**)&p->d_colmap, colmap.data(), sizeof(int) * colmap.size()) &&
-         upload((void**)&p->d_rowpos, cols.rowpos.data(), sizeof(int) * cols.rowpos.size()) &&
-         upload((void**)&p->d_kept, kept.data(), sizeof(int) * kept.size());
+  if (ok) {
+    cudaError_t e = fockx::columns::upload(cols, {}, &p->d_cols, &p->dp.cols, &p->table_bytes);
+    if (e == cudaSuccess) e = fockx::columns::upload(orb, coef, &p->d_orb, &p->dp.orb, &p->table_bytes);
+    if (e != cudaSuccess) {
+      st = cuda_fail(nullptr, e, "uploading the column sets");
+      ok = false;
+    }
+  }
   if (ok) {
     if (fp64) {
       std::vector<double> vs(nhalf);
@@ -1002,8 +913,6 @@ fock_status fock_plan_create(fock_plan_t* out, const int grid[3], const double c
   d.ntot = ntot;
   d.hsize = (int64_t)n * n * 2 * kh;
   d.npw = p->npw;
-  d.gidx = p->d_gidx;
-  d.gidxneg = p->d_gidxneg;
   d.tw = p->d_tw;
   d.vtab = p->d_vtab;
   d.vtab64 = p->d_vtab64;
@@ -1013,15 +922,6 @@ fock_status fock_plan_create(fock_plan_t* out, const int grid[3], const double c
   d.psi_scale = 1.0 / std::sqrt(p->vol);
   d.out_scale = std::sqrt(p->vol) / (double)ntot;
   d.msmall2 = prec == FOCK_PREC_MIXED32 ? kMsmall2 : -1;
-  d.ncol = p->d_ncol;
-  d.colmap = p->d_colmap;
-  d.ncta_col = ncta_col;
-  d.kept = p->d_kept;
-  d.rowpos = p->d_rowpos;
-  d.nkept = (int)kept.size();
-  d.row_lo = cols.row_lo;
-  d.row_hi = cols.row_hi;
-  d.col_max = cols.col_max;
   d.det = 0;  // set per call on a copy when the plan is deterministic
   d.tile[0] = d.tile[1] = d.tile[2] = 0;
   d.det_scale = nullptr;
@@ -1179,28 +1079,39 @@ fock_status fock_sternheimer_solve(fock_plan_t p, const double* vloc, const void
   fock_status st = check_device(p);
   if (st != FOCK_OK) return st;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  st = ensure_workspace(p, nrhs, 1);
+  st = ensure_workspace(p, 1, 1);  // the transform buffer is all that is used
   if (st != FOCK_OK) return st;
-  p->fixed_nb = 0;  // the real-space workspace is overwritten
+  p->fixed_nb = 0;
   const double2* u = static_cast<const double2*>(u_G);
-  StBuffers buf;
-  double2 *x, *r, *pk, *ap, *tmp;
-  double *kin, *d_eps, *c, *rr, *rrn, *pap, *sc;
-  int* perm;
   const size_t nb8 = sizeof(double) * nrhs;
-  FOCK_CUDA(p, buf.alloc(&x, kb));
-  FOCK_CUDA(p, buf.alloc(&r, kb));
-  FOCK_CUDA(p, buf.alloc(&pk, kb));
-  FOCK_CUDA(p, buf.alloc(&ap, kb));
-  FOCK_CUDA(p, buf.alloc(&tmp, kb));
-  FOCK_CUDA(p, buf.alloc(&kin, sizeof(double) * npw));
-  FOCK_CUDA(p, buf.alloc(&d_eps, nb8));
-  FOCK_CUDA(p, buf.alloc(&c, sizeof(double) * nocc * nrhs));
-  FOCK_CUDA(p, buf.alloc(&rr, nb8));
-  FOCK_CUDA(p, buf.alloc(&rrn, nb8));
-  FOCK_CUDA(p, buf.alloc(&pap, nb8));
-  FOCK_CUDA(p, buf.alloc(&sc, nb8));
-  FOCK_CUDA(p, buf.alloc(&perm, sizeof(int) * nrhs));
+  // one plan-owned buffer for the solve's arrays, grown on demand: an
+  // allocation a call for each of them cost as much as several CG updates
+  double2 *x, *r, *pk, *ap, *tmp;
+  double *kin, *d_eps, *c, *rr, *rrn, *part_a, *part_b, *sc;
+  int* perm;
+  {
+    const size_t bytes[] = {kb, kb, kb, kb, kb, sizeof(double) * npw, nb8,
+                            nb8 * nocc, nb8, nb8,
+                            nb8 * (size_t)fockx::st_chunks((int)npw), nb8 * (size_t)fockx::st_chunks((int)npw), nb8,
+                            sizeof(int) * (size_t)nrhs};
+    void** const ptrs[] = {(void**)&x, (void**)&r, (void**)&pk, (void**)&ap, (void**)&tmp, (void**)&kin,
+                           (void**)&d_eps, (void**)&c, (void**)&rr, (void**)&rrn, (void**)&part_a, (void**)&part_b,
+                           (void**)&sc, (void**)&perm};
+    size_t total = 0;
+    for (size_t n : bytes) total += (n + 255) / 256 * 256;
+    if (total > p->st_cap) {
+      cudaFree(p->d_st);
+      p->d_st = nullptr;
+      p->st_cap = 0;
+      FOCK_CUDA(p, dev_alloc(&p->d_st, total));
+      p->st_cap = total;
+    }
+    char* at = static_cast<char*>(p->d_st);
+    for (size_t k = 0; k < sizeof(bytes) / sizeof(bytes[0]); ++k) {
+      *ptrs[k] = at;
+      at += (bytes[k] + 255) / 256 * 256;
+    }
+  }
   // |G|^2 / 2 on the sphere, in the plan's canonical order
   std::vector<double> kin_h(npw);
   for (size_t g = 0; g < npw; ++g)
@@ -1211,42 +1122,32 @@ fock_status fock_sternheimer_solve(fock_plan_t p, const double* vloc, const void
 
   const int ip = (int)npw;
   const int nbat = bands_per_grid_batch(p);
-  // (H - eps_n + alpha P) on the kets q at positions [0, m) into out
-  auto apply_a = [&](const double2* q, int m, double2* out) -> fock_status {
-    for (int b0 = 0; b0 < m; b0 += nbat)
-      FOCK_CUDA(p, p->ops->to_real(p->dp, q, m, b0, std::min(nbat, m - b0), p->ws.h, p->ws.psi, s));
-    FOCK_CUDA(p, fockx::st_vmul(vloc, static_cast<const double*>(p->ws.psi), static_cast<double*>(p->ws.w), m,
-                                p->dp.ntot, s));
-    for (int b0 = 0; b0 < m; b0 += nbat)
-      FOCK_CUDA(p, p->ops->to_sphere(p->dp, p->ws.w, m, b0, std::min(nbat, m - b0), p->ws.h, out, s));
-    FOCK_CUDA(p, fockx::st_proj_coef(u, nocc, q, m, ip, c, s));
-    FOCK_CUDA(p, fockx::st_finish(out, q, kin, d_eps, u, c, nocc, alpha, m, ip, s));
-    return FOCK_OK;
-  };
-
   // b = -Q w into r; x = 0; p = r; rr = <r|r>
   FOCK_CUDA(p, fockx::st_proj_coef(u, nocc, static_cast<const double2*>(w_G), nrhs, ip, c, s));
-  FOCK_CUDA(p, fockx::st_rhs(static_cast<const double2*>(w_G), u, c, nocc, nrhs, ip, r, s));
+  FOCK_CUDA(p, fockx::st_rhs(static_cast<const double2*>(w_G), u, c, nocc, nrhs, ip, r, part_a, rr, s));
   FOCK_CUDA(p, cudaMemsetAsync(x, 0, kb, s));
   FOCK_CUDA(p, cudaMemcpyAsync(pk, r, kb, cudaMemcpyDeviceToDevice, s));
-  FOCK_CUDA(p, fockx::st_dots(r, r, nrhs, ip, rr, s));
 
   // order[k]: the band at position k; positions [0, m) are not converged
   std::vector<int> order(nrhs), it_h(nrhs, 0), keep;
   for (int n = 0; n < nrhs; ++n) order[n] = n;
-  std::vector<double> rr_h(nrhs);
+  std::vector<double> rr_h(nrhs), rr_last(nrhs, 0.0);  // this update's, and every band's latest
   int m = nrhs;
   for (int it = 0; it < maxiter && m > 0; ++it) {
-    st = apply_a(pk, m, ap);
-    if (st != FOCK_OK) return st;
-    FOCK_CUDA(p, fockx::st_dots(pk, ap, m, ip, pap, s));
-    FOCK_CUDA(p, fockx::st_step(x, r, pk, ap, rr, pap, m, ip, s));
-    FOCK_CUDA(p, fockx::st_dots(r, r, m, ip, rrn, s));
-    FOCK_CUDA(p, fockx::st_dir(pk, r, rrn, rr, m, ip, s));
-    FOCK_CUDA(p, cudaMemcpyAsync(rr, rrn, sizeof(double) * m, cudaMemcpyDeviceToDevice, s));
-    FOCK_CUDA(p, cudaMemcpyAsync(rr_h.data(), rrn, sizeof(double) * m, cudaMemcpyDeviceToHost, s));
+    // ap = (H - eps_n + alpha P) p for the kets at positions [0, m)
+    for (int b0 = 0; b0 < m; b0 += nbat)
+      FOCK_CUDA(p, p->ops->vloc(p->dp, pk, m, b0, std::min(nbat, m - b0), vloc, p->ws.h, ap, s));
+    FOCK_CUDA(p, fockx::st_proj_coef(u, nocc, pk, m, ip, c, s));
+    FOCK_CUDA(p, fockx::st_finish(ap, pk, kin, d_eps, u, c, nocc, alpha, m, ip, part_a, s));
+    FOCK_CUDA(p, fockx::st_step(x, r, pk, ap, rr, part_a, m, ip, part_b, s));
+    FOCK_CUDA(p, fockx::st_dir(pk, r, part_b, rr, m, ip, rrn, s));
+    std::swap(rr, rrn);
+    FOCK_CUDA(p, cudaMemcpyAsync(rr_h.data(), rr, sizeof(double) * m, cudaMemcpyDeviceToHost, s));
     FOCK_CUDA(p, cudaStreamSynchronize(s));
-    for (int k = 0; k < m; ++k) ++it_h[order[k]];
+    for (int k = 0; k < m; ++k) {
+      ++it_h[order[k]];
+      rr_last[order[k]] = rr_h[k];
+    }
     // regroup: not converged first, then converged, each in their order
     keep.clear();
     for (int k = 0; k < m; ++k)
@@ -1269,13 +1170,8 @@ fock_status fock_sternheimer_solve(fock_plan_t p, const double* vloc, const void
         FOCK_CUDA(p, cudaMemcpyAsync(a, sc, sizeof(double) * m, cudaMemcpyDeviceToDevice, s));
       }
       std::vector<int> o2(order);
-      std::vector<double> r2(rr_h);
-      for (int k = 0; k < m; ++k) {
-        o2[k] = order[keep[k]];
-        r2[k] = rr_h[keep[k]];
-      }
+      for (int k = 0; k < m; ++k) o2[k] = order[keep[k]];
       order.swap(o2);
-      rr_h.swap(r2);
     }
     m = m_new;
   }
@@ -1284,11 +1180,10 @@ fock_status fock_sternheimer_solve(fock_plan_t p, const double* vloc, const void
   for (int k = 0; k < nrhs; ++k) inv[order[k]] = k;
   FOCK_CUDA(p, cudaMemcpyAsync(perm, inv.data(), sizeof(int) * nrhs, cudaMemcpyHostToDevice, s));
   FOCK_CUDA(p, fockx::st_gather_rows(x, static_cast<double2*>(g_G), perm, nrhs, ip, s));
-  FOCK_CUDA(p, cudaMemcpyAsync(rr_h.data(), rr, nb8, cudaMemcpyDeviceToHost, s));
   FOCK_CUDA(p, cudaStreamSynchronize(s));
-  for (int k = 0; k < nrhs; ++k) {
-    if (iters) iters[order[k]] = it_h[order[k]];
-    if (resid) resid[order[k]] = std::sqrt(rr_h[k]);
+  for (int n = 0; n < nrhs; ++n) {
+    if (iters) iters[n] = it_h[n];
+    if (resid) resid[n] = std::sqrt(rr_last[n]);
   }
   return FOCK_OK;
 }
@@ -1370,7 +1265,7 @@ fock_status fock_plan_device_bytes(fock_plan_t plan, int64_t* bytes) {
   int64_t b = plan->table_bytes + 2 * (int64_t)w.psi_bytes + (int64_t)w.h_bytes;
   b += (int64_t)w.npair_cap * (2 * sizeof(double) + sizeof(int2)) +
        (int64_t)((w.npair_cap + 1) / 2) * sizeof(Chain);
-  b += (int64_t)w.nb_cap * (sizeof(double) + plan->ops->real_bytes);
+  b += (int64_t)w.nb_cap * (sizeof(double) + plan->ops->real_bytes) + (int64_t)plan->st_cap;
   *bytes = b;
   return FOCK_OK;
 }
@@ -1468,7 +1363,7 @@ fock_status fock_apply_fixed(fock_plan_t plan, const void* phi_G, int nt, void* 
   const int nbat = bands_per_grid_batch(p);
   p->stats.band_batch = nbat;
   for (int b0 = 0; b0 < nt; b0 += nbat) {
-    PhaseScope ps(p, FOCK_PHASE_TO_REAL, 3, s);
+    PhaseScope ps(p, FOCK_PHASE_TO_REAL, 2, s);
     FOCK_CUDA(p, p->ops->to_real(p->dp, static_cast<const double2*>(phi_G), nt, b0, std::min(nbat, nt - b0),
                                  p->ws.h, psi_trial, s));
   }
@@ -1510,7 +1405,7 @@ fock_status fock_apply_fixed(fock_plan_t plan, const void* phi_G, int nt, void* 
   }
   if (p->det) FOCK_CUDA(p, fockx::launch_det_to_double(w_trial, (int64_t)nt * p->dp.ntot, p->d_scale, s));
   for (int b0 = 0; b0 < nt; b0 += nbat) {
-    PhaseScope ps(p, FOCK_PHASE_TO_SPHERE, 3, s);
+    PhaseScope ps(p, FOCK_PHASE_TO_SPHERE, 2, s);
     FOCK_CUDA(p, p->ops->to_sphere(p->dp, w_trial, nt, b0, std::min(nbat, nt - b0), p->ws.h,
                                    static_cast<double2*>(vphi_G), s));
   }
@@ -1586,17 +1481,13 @@ fock_status fock_destroy(fock_plan_t plan) {
     if (plan->aux[k]) cudaStreamDestroy(plan->aux[k]);
   }
   free_ws(plan->ws);
-  cudaFree(plan->d_gidx);
-  cudaFree(plan->d_gidxneg);
   cudaFree(plan->d_tw);
   cudaFree(plan->d_vtab);
   cudaFree(plan->d_vtab64);
   cudaFree(plan->d_dvtab);
   cudaFree(plan->d_dvtab64);
-  cudaFree(plan->d_ncol);
-  cudaFree(plan->d_colmap);
-  cudaFree(plan->d_kept);
-  cudaFree(plan->d_rowpos);
+  cudaFree(plan->d_cols);
+  cudaFree(plan->d_orb);
   cudaFree(plan->d_stats);
   cudaFree(plan->d_scale);
   cudaFree(plan->d_epart);
@@ -1605,6 +1496,7 @@ fock_status fock_destroy(fock_plan_t plan) {
   cudaFree(plan->d_half);
   cudaFree(plan->d_cocc);
   cudaFree(plan->d_vtab_f);
+  cudaFree(plan->d_st);
   cudaFree(plan->d_result);
   if (plan->h_result) cudaFreeHost(plan->h_result);
   delete plan;
@@ -1700,7 +1592,7 @@ fock_status batch_enqueue(fock_batch* b, cudaStream_t s) {
     for (int b0 = 0; b0 < nb; b0 += nbat) {
       FOCK_BCUDA(b, p->ops->to_real(p->dp, static_cast<const double2*>(b->psi[k]), nb, b0,
                                     std::min(nbat, nb - b0), p->ws.h, p->ws.psi, s));
-      b->launches += 3;
+      b->launches += 2;
     }
     if (p->ops->prec == 1) {
       FOCK_BCUDA(b, fockx::launch_overlap(static_cast<const double2*>(b->psi[k]), nb,
@@ -1761,7 +1653,7 @@ fock_status batch_enqueue(fock_batch* b, cudaStream_t s) {
     for (int b0 = 0; b0 < nb; b0 += nbat) {
       FOCK_BCUDA(b, p->ops->to_sphere(p->dp, p->ws.w, nb, b0, std::min(nbat, nb - b0), p->ws.h,
                                       static_cast<double2*>(b->vpsi[k]), s));
-      b->launches += 3;
+      b->launches += 2;
     }
     const double scale = -0.5 * p->vol / ((double)p->dp.ntot * (double)p->dp.ntot);
     FOCK_BCUDA(b, fockx::launch_energy_reduce(p->ws.pairs, npairs, p->ws.occ, p->ws.epair,
@@ -1905,7 +1797,7 @@ fock_status fock_batch_create(fock_batch_t* out, int nsys, const fock_plan_t* pl
     sg.slot = t % D;
     sg.dep = dep;
     sg.dep2 = dep2;
-    sg.ntasks = (sg.kind == 1 ? b->plans[sg.sys]->dp.ncta_col : b->plans[sg.sys]->n) * sg.nch;
+    sg.ntasks = (sg.kind == 1 ? b->plans[sg.sys]->dp.cols.ncta : b->plans[sg.sys]->n) * sg.nch;
     b->segs.push_back(sg);
     return (int)b->segs.size() - 1;
   };

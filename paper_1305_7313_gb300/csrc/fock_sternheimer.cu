@@ -1,9 +1,13 @@
-// fock_sternheimer.cu — kernels of the Sternheimer CG (§3.1): the local
-// potential in real space, per-band inner products on the plane-wave sphere,
-// the occupied-manifold projector, the CG vector updates and the regrouping
-// gathers.  All in FP64 on complex128 kets [m][npw] (Gamma-point real
+// fock_sternheimer.cu — kernels of the Sternheimer CG (§3.1): per-band inner
+// products on the plane-wave sphere, the occupied-manifold projector, the CG
+// vector updates and the regrouping gathers.  All in FP64 on complex128 kets [m][npw] (Gamma-point real
 // functions, so every inner product <a|b> = sum_G conj(a(G)) b(G) is real).
-// The transforms of the kets to real space and back are the plan's own.
+// The local potential is the plan's KernelOps::vloc.
+//
+// One CG update is four launches after it: the projector's coefficients,
+// (H - eps + alpha P) p with the partial sums of <p|Ap>, the x and r updates with
+// those of <r|r>, and the new directions.  Each kernel that needs an inner
+// product adds the partial sums of the one before it in a fixed order.
 #include "fock_internal.h"
 
 namespace fockx {
@@ -12,110 +16,194 @@ namespace {
 constexpr int kThreads = 256;
 
 // Sum of one double over the CTA; the result is valid in thread 0.
-__device__ double block_sum(double v) {
-  __shared__ double red[kThreads / 32];
+template <int THR = kThreads> __device__ double block_sum(double v) {
+  __shared__ double red[THR / 32];
   for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
   __syncthreads();
   double s = 0.0;
   if (threadIdx.x == 0)
-    for (int w = 0; w < kThreads / 32; ++w) s += red[w];
+    for (int w = 0; w < THR / 32; ++w) s += red[w];
   return s;
 }
 
-// w[n][r] = v[r] psi[n][r] for the first m bands (grid-stride over all points).
-__global__ void k_vmul(const double* __restrict__ v, const double* __restrict__ psi, double* __restrict__ w,
-                       int m, int64_t ntot) {
-  const int64_t total = (int64_t)m * ntot;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x)
-    w[i] = v[i % ntot] * psi[i];
-}
+// Coefficients G a CTA of the vector kernels takes of one band, and of the
+// kernels with the projector's sums, whose FP64 work has to spread evenly over
+// the SMs (64: 624 CTAs for 32 bands of 4,945 coefficients; 256 would be 160, two
+// on a few SMs and one on the others).
+constexpr int kChunk = kThreads, kSumChunk = 64;
 
-// out[n] = Re sum_G conj(a_n(G)) b_n(G), one CTA per band.
-__global__ void k_dots(const double2* __restrict__ a, const double2* __restrict__ b, int npw, double* __restrict__ out) {
-  const double2* an = a + (int64_t)blockIdx.x * npw;
-  const double2* bn = b + (int64_t)blockIdx.x * npw;
-  double s = 0.0;
-  for (int g = threadIdx.x; g < npw; g += blockDim.x) s += an[g].x * bn[g].x + an[g].y * bn[g].y;
-  s = block_sum(s);
-  if (threadIdx.x == 0) out[blockIdx.x] = s;
-}
-
-// c[n * nocc + i] = Re sum_G conj(u_i(G)) x_n(G); CTA (i, n).
-__global__ void k_proj_coef(const double2* __restrict__ u, int nocc, const double2* __restrict__ x, int npw,
-                            double* __restrict__ c) {
-  const int i = blockIdx.x, n = blockIdx.y;
-  const double2* ui = u + (int64_t)i * npw;
-  const double2* xn = x + (int64_t)n * npw;
-  double s = 0.0;
-  for (int g = threadIdx.x; g < npw; g += blockDim.x) s += ui[g].x * xn[g].x + ui[g].y * xn[g].y;
-  s = block_sum(s);
-  if (threadIdx.x == 0) c[n * nocc + i] = s;
-}
-
-// b_n = -(w_n - sum_i c_ni u_i) = -Q w_n.
-__global__ void k_rhs(const double2* __restrict__ w, const double2* __restrict__ u, const double* __restrict__ c,
-                      int nocc, int m, int npw, double2* __restrict__ b) {
-  const int64_t total = (int64_t)m * npw;
-  for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < total; k += (int64_t)gridDim.x * blockDim.x) {
-    const int n = (int)(k / npw), g = (int)(k - (int64_t)n * npw);
-    double2 s = w[k];
-    for (int i = 0; i < nocc; ++i) {
-      const double ci = c[n * nocc + i];
-      const double2 ui = u[(int64_t)i * npw + g];
-      s.x -= ci * ui.x;
-      s.y -= ci * ui.y;
-    }
-    b[k] = make_double2(-s.x, -s.y);
+// Sum of the n partial sums part[0 .. n) in a fixed order, in every thread.
+__device__ double sum_partials(const double* __restrict__ part, int n) {
+  __shared__ double total;
+  if (threadIdx.x < 32) {
+    double s = 0.0;
+    for (int k = threadIdx.x; k < n; k += 32) s += part[k];
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+    if (threadIdx.x == 0) total = s;
   }
+  __syncthreads();
+  return total;
+}
+
+// Projector coefficients c[n nocc + i] = Re sum_G conj(u_i(G)) x_n(G): a CTA
+// takes 2 x 2 of them, so a row read serves two sums and the loads of four
+// coefficients are in flight together.  (Larger tiles leave too few warps to hide
+// the reads and spend the FP64 pipe on the reductions of their sums: 4 x 4 took
+// 30 to 63 us on average where one CTA per coefficient took 26.)
+constexpr int kProjTile = 2;
+__global__ void __launch_bounds__(kThreads)
+    k_proj_coef(const double2* __restrict__ u, int nocc, const double2* __restrict__ x, int m, int npw,
+                double* __restrict__ c) {
+  constexpr int TL = kProjTile;
+  const int i0 = blockIdx.x * TL, n0 = blockIdx.y * TL;
+  // rows past the end repeat the last one; their sums are not stored
+  const double2 *a[TL], *b[TL];
+#pragma unroll
+  for (int k = 0; k < TL; ++k) {
+    a[k] = u + (int64_t)(i0 + k < nocc ? i0 + k : nocc - 1) * npw;
+    b[k] = x + (int64_t)(n0 + k < m ? n0 + k : m - 1) * npw;
+  }
+  double acc[TL][TL] = {};
+#pragma unroll 4
+  for (int g = threadIdx.x; g < npw; g += kThreads) {
+#pragma unroll
+    for (int k = 0; k < TL; ++k) {
+      const double2 ak = a[k][g];
+#pragma unroll
+      for (int n = 0; n < TL; ++n) {
+        const double2 bn = b[n][g];
+        acc[k][n] = fma(ak.x, bn.x, fma(ak.y, bn.y, acc[k][n]));
+      }
+    }
+  }
+#pragma unroll
+  for (int k = 0; k < TL; ++k)
+#pragma unroll
+    for (int n = 0; n < TL; ++n) {
+      __syncthreads();
+      const double v = block_sum(acc[k][n]);
+      if (threadIdx.x == 0 && i0 + k < nocc && n0 + n < m) c[(int64_t)(n0 + n) * nocc + i0 + k] = v;
+    }
+}
+
+// scale sum_i c(n, i) u_i(G) of bands n0 .. n0 + 3 at one G per thread: the
+// coefficients are staged in shared memory, each u_i(G) is read once for the
+// four bands.
+constexpr int kBands = 4, kStage = 128;
+__device__ void project(const double2* __restrict__ u, const double* __restrict__ c, int nocc, int n0, int m, int npw,
+                        int g, double scale, double2 s[kBands]) {
+  __shared__ double cs[kStage][kBands];
+  for (int i0 = 0; i0 < nocc; i0 += kStage) {
+    const int cnt = nocc - i0 < kStage ? nocc - i0 : kStage;
+    __syncthreads();
+    for (int e = threadIdx.x; e < cnt * kBands; e += kSumChunk) {
+      const int i = e / kBands, n = n0 + e % kBands;
+      cs[i][e % kBands] = n < m ? scale * c[(int64_t)n * nocc + i0 + i] : 0.0;
+    }
+    __syncthreads();
+    if (g < npw) {
+#pragma unroll 4
+      for (int i = 0; i < cnt; ++i) {
+        const double2 ui = u[(int64_t)(i0 + i) * npw + g];
+#pragma unroll
+        for (int n = 0; n < kBands; ++n) {
+          s[n].x = fma(cs[i][n], ui.x, s[n].x);
+          s[n].y = fma(cs[i][n], ui.y, s[n].y);
+        }
+      }
+    }
+  }
+}
+
+// b_n = -(w_n - sum_i c_ni u_i) = -Q w_n; part[n][chunk]: partial sums of <b_n|b_n>.
+__global__ void __launch_bounds__(kSumChunk)
+    k_rhs(const double2* __restrict__ w, const double2* __restrict__ u, const double* __restrict__ c, int nocc, int m,
+          int npw, double2* __restrict__ b, double* __restrict__ part) {
+  const int g = blockIdx.x * kSumChunk + threadIdx.x, n0 = blockIdx.y * kBands;
+  double2 s[kBands] = {};
+  project(u, c, nocc, n0, m, npw, g, 1.0, s);
+  for (int n = 0; n < kBands && n0 + n < m; ++n) {
+    double d = 0.0;
+    if (g < npw) {
+      const int64_t k = (int64_t)(n0 + n) * npw + g;
+      const double2 wk = w[k], r = make_double2(s[n].x - wk.x, s[n].y - wk.y);
+      b[k] = r;
+      d = r.x * r.x + r.y * r.y;
+    }
+    __syncthreads();
+    d = block_sum<kSumChunk>(d);
+    if (threadIdx.x == 0) part[(int64_t)(n0 + n) * gridDim.x + blockIdx.x] = d;
+  }
+}
+
+// rr[n] = sum of part[n][0 .. nchunk).
+__global__ void k_sum_parts(const double* __restrict__ part, int nchunk, double* __restrict__ rr) {
+  const double s = sum_partials(part + (int64_t)blockIdx.x * nchunk, nchunk);
+  if (threadIdx.x == 0) rr[blockIdx.x] = s;
 }
 
 // ap_n = ap_n + (|G|^2/2 - eps_n) p_n + alpha sum_i c_ni u_i, where ap holds
 // the local-potential part of H p on entry: ap = (H - eps_n + alpha P) p.
-__global__ void k_finish(double2* __restrict__ ap, const double2* __restrict__ p, const double* __restrict__ kin,
-                         const double* __restrict__ eps, const double2* __restrict__ u, const double* __restrict__ c,
-                         int nocc, double alpha, int m, int npw) {
-  const int64_t total = (int64_t)m * npw;
-  for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < total; k += (int64_t)gridDim.x * blockDim.x) {
-    const int n = (int)(k / npw), g = (int)(k - (int64_t)n * npw);
-    const double d = kin[g] - eps[n];
-    double2 s = ap[k];
-    const double2 pk = p[k];
-    s.x += d * pk.x;
-    s.y += d * pk.y;
-    for (int i = 0; i < nocc; ++i) {
-      const double ci = alpha * c[n * nocc + i];
-      const double2 ui = u[(int64_t)i * npw + g];
-      s.x += ci * ui.x;
-      s.y += ci * ui.y;
+// part[n][chunk]: partial sums of <p_n|ap_n>.
+__global__ void __launch_bounds__(kSumChunk)
+    k_finish(double2* __restrict__ ap, const double2* __restrict__ p, const double* __restrict__ kin,
+             const double* __restrict__ eps, const double2* __restrict__ u, const double* __restrict__ c, int nocc,
+             double alpha, int m, int npw, double* __restrict__ part) {
+  const int g = blockIdx.x * kSumChunk + threadIdx.x, n0 = blockIdx.y * kBands;
+  double2 s[kBands] = {};
+  project(u, c, nocc, n0, m, npw, g, alpha, s);
+  for (int n = 0; n < kBands && n0 + n < m; ++n) {
+    double d = 0.0;
+    if (g < npw) {
+      const int64_t k = (int64_t)(n0 + n) * npw + g;
+      const double t = kin[g] - eps[n0 + n];
+      const double2 pk = p[k], ak = ap[k];
+      const double2 a = make_double2(fma(t, pk.x, ak.x + s[n].x), fma(t, pk.y, ak.y + s[n].y));
+      ap[k] = a;
+      d = pk.x * a.x + pk.y * a.y;
     }
-    ap[k] = s;
+    __syncthreads();
+    d = block_sum<kSumChunk>(d);
+    if (threadIdx.x == 0) part[(int64_t)(n0 + n) * gridDim.x + blockIdx.x] = d;
   }
 }
 
-// x_n += a_n p_n, r_n -= a_n ap_n with a_n = rr_n / pap_n.
-__global__ void k_step(double2* __restrict__ x, double2* __restrict__ r, const double2* __restrict__ p,
-                       const double2* __restrict__ ap, const double* __restrict__ rr, const double* __restrict__ pap,
-                       int m, int npw) {
-  const int64_t total = (int64_t)m * npw;
-  for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < total; k += (int64_t)gridDim.x * blockDim.x) {
-    const int n = (int)(k / npw);
-    const double a = rr[n] / pap[n];
+// x_n += a_n p_n, r_n -= a_n ap_n with a_n = rr_n / <p_n|ap_n>; part_rr[n][chunk]:
+// partial sums of the new <r_n|r_n>.  CTA (chunk, n).
+__global__ void __launch_bounds__(kThreads)
+    k_step(double2* __restrict__ x, double2* __restrict__ r, const double2* __restrict__ p,
+           const double2* __restrict__ ap, const double* __restrict__ rr, const double* __restrict__ part_pap, int nsum,
+           int npw, double* __restrict__ part_rr) {
+  const int n = blockIdx.y, g = blockIdx.x * kChunk + threadIdx.x;
+  const double a = rr[n] / sum_partials(part_pap + (int64_t)n * nsum, nsum);
+  double d = 0.0;
+  if (g < npw) {
+    const int64_t k = (int64_t)n * npw + g;
     const double2 pk = p[k], ak = ap[k];
-    x[k].x += a * pk.x;
-    x[k].y += a * pk.y;
-    r[k].x -= a * ak.x;
-    r[k].y -= a * ak.y;
+    double2 xk = x[k], rk = r[k];
+    xk.x += a * pk.x;
+    xk.y += a * pk.y;
+    rk.x -= a * ak.x;
+    rk.y -= a * ak.y;
+    x[k] = xk;
+    r[k] = rk;
+    d = rk.x * rk.x + rk.y * rk.y;
   }
+  d = block_sum(d);
+  if (threadIdx.x == 0) part_rr[(int64_t)n * gridDim.x + blockIdx.x] = d;
 }
 
-// p_n = r_n + (rr_new_n / rr_n) p_n.
-__global__ void k_dir(double2* __restrict__ p, const double2* __restrict__ r, const double* __restrict__ rr_new,
-                      const double* __restrict__ rr, int m, int npw) {
-  const int64_t total = (int64_t)m * npw;
-  for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < total; k += (int64_t)gridDim.x * blockDim.x) {
-    const int n = (int)(k / npw);
-    const double beta = rr_new[n] / rr[n];
+// p_n = r_n + (rr_new_n / rr_n) p_n, rr_new_n the sum of part_rr[n]; CTA (chunk, n).
+__global__ void __launch_bounds__(kThreads)
+    k_dir(double2* __restrict__ p, const double2* __restrict__ r, const double* __restrict__ part_rr,
+          const double* __restrict__ rr, int npw, double* __restrict__ rr_new) {
+  const int n = blockIdx.y, g = blockIdx.x * kChunk + threadIdx.x;
+  const double now = sum_partials(part_rr + (int64_t)n * gridDim.x, gridDim.x);
+  if (blockIdx.x == 0 && threadIdx.x == 0) rr_new[n] = now;
+  const double beta = now / rr[n];
+  if (g < npw) {
+    const int64_t k = (int64_t)n * npw + g;
     const double2 rk = r[k], pk = p[k];
     p[k] = make_double2(rk.x + beta * pk.x, rk.y + beta * pk.y);
   }
@@ -142,36 +230,37 @@ int grid_for(int64_t total) {
 
 }  // namespace
 
-cudaError_t st_vmul(const double* v, const double* psi, double* w, int m, int64_t ntot, cudaStream_t s) {
-  k_vmul<<<grid_for((int64_t)m * ntot), kThreads, 0, s>>>(v, psi, w, m, ntot);
-  return cudaGetLastError();
-}
-cudaError_t st_dots(const double2* a, const double2* b, int m, int npw, double* out, cudaStream_t s) {
-  k_dots<<<m, kThreads, 0, s>>>(a, b, npw, out);
-  return cudaGetLastError();
-}
+namespace {
+int chunks(int npw, int chunk) { return (npw + chunk - 1) / chunk; }
+}  // namespace
+int st_chunks(int npw) { return chunks(npw, kSumChunk); }
+
 cudaError_t st_proj_coef(const double2* u, int nocc, const double2* x, int m, int npw, double* c, cudaStream_t s) {
-  k_proj_coef<<<dim3(nocc, m), kThreads, 0, s>>>(u, nocc, x, npw, c);
+  k_proj_coef<<<dim3(chunks(nocc, kProjTile), chunks(m, kProjTile)), kThreads, 0, s>>>(u, nocc, x, m, npw, c);
   return cudaGetLastError();
 }
 cudaError_t st_rhs(const double2* w, const double2* u, const double* c, int nocc, int m, int npw, double2* b,
-                   cudaStream_t s) {
-  k_rhs<<<grid_for((int64_t)m * npw), kThreads, 0, s>>>(w, u, c, nocc, m, npw, b);
+                   double* part, double* rr, cudaStream_t s) {
+  const int nsum = chunks(npw, kSumChunk);
+  k_rhs<<<dim3(nsum, chunks(m, kBands)), kSumChunk, 0, s>>>(w, u, c, nocc, m, npw, b, part);
+  k_sum_parts<<<m, 32, 0, s>>>(part, nsum, rr);
   return cudaGetLastError();
 }
 cudaError_t st_finish(double2* ap, const double2* p, const double* kin, const double* eps, const double2* u,
-                      const double* c, int nocc, double alpha, int m, int npw, cudaStream_t s) {
-  k_finish<<<grid_for((int64_t)m * npw), kThreads, 0, s>>>(ap, p, kin, eps, u, c, nocc, alpha, m, npw);
+                      const double* c, int nocc, double alpha, int m, int npw, double* part, cudaStream_t s) {
+  k_finish<<<dim3(chunks(npw, kSumChunk), chunks(m, kBands)), kSumChunk, 0, s>>>(ap, p, kin, eps, u, c, nocc, alpha, m,
+                                                                               npw, part);
   return cudaGetLastError();
 }
-cudaError_t st_step(double2* x, double2* r, const double2* p, const double2* ap, const double* rr, const double* pap,
-                    int m, int npw, cudaStream_t s) {
-  k_step<<<grid_for((int64_t)m * npw), kThreads, 0, s>>>(x, r, p, ap, rr, pap, m, npw);
+cudaError_t st_step(double2* x, double2* r, const double2* p, const double2* ap, const double* rr,
+                    const double* part_pap, int m, int npw, double* part_rr, cudaStream_t s) {
+  k_step<<<dim3(chunks(npw, kChunk), m), kThreads, 0, s>>>(x, r, p, ap, rr, part_pap, chunks(npw, kSumChunk), npw,
+                                                         part_rr);
   return cudaGetLastError();
 }
-cudaError_t st_dir(double2* p, const double2* r, const double* rr_new, const double* rr, int m, int npw,
-                   cudaStream_t s) {
-  k_dir<<<grid_for((int64_t)m * npw), kThreads, 0, s>>>(p, r, rr_new, rr, m, npw);
+cudaError_t st_dir(double2* p, const double2* r, const double* part_rr, const double* rr, int m, int npw,
+                   double* rr_new, cudaStream_t s) {
+  k_dir<<<dim3(chunks(npw, kChunk), m), kThreads, 0, s>>>(p, r, part_rr, rr, npw, rr_new);
   return cudaGetLastError();
 }
 cudaError_t st_gather_rows(const double2* src, double2* dst, const int* perm, int m, int npw, cudaStream_t s) {
