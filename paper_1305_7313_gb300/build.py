@@ -35,9 +35,10 @@ def _cuda_home():
 
 
 def grid_sizes():
+    """The users' grid sizes and the further ones of the plans' working grids."""
     text = open(os.path.join(CSRC, "fock_sizes.h")).read()
-    m = re.search(r"#define FOCK_GRID_SIZES\(X\)(.*)", text)
-    return [int(x) for x in re.findall(r"X\((\d+)\)", m.group(1))]
+    lists = re.findall(r"#define FOCK_(?:GRID|PAIR)_SIZES\(X\)(.*)", text)
+    return sorted(int(x) for line in lists for x in re.findall(r"X\((\d+)\)", line))
 
 
 def _newest_dependency():
@@ -77,6 +78,8 @@ def _jobs():
         jobs.append(("fock_df_%d.o" % n,
                      nv + ["-DFOCK_T=fockx::df64", "-DFOCK_N=%d" % n, "-DFOCK_OPS_NAME=kOps_df_%d" % n,
                            "-c", os.path.join(CSRC, "fock_kernels_inst.cu")]))
+    # the longest compilations first, so that none is left running alone at the end
+    jobs.sort(key=lambda j: ("persist" not in j[0], -int((re.findall(r"_(\d+)\.o", j[0]) or [0])[0])))
     return nvcc, jobs
 
 

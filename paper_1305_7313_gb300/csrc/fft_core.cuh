@@ -1,5 +1,5 @@
 // fft_core.cuh — the transforms of the Fock apply: in-register DFTs of radix 2,
-// 3, 4 and 8 and of the composites 6, 9, 12, 16, 18 and 24, and the stages that
+// 3, 4, 5, 7 and 8 and of their composites up to 24, and the stages that
 // put them together on lines and planes held in shared memory, specialised at
 // compile time for one line length N.
 //
@@ -348,6 +348,45 @@ template <int SIGN, class T> struct Dft {
     x[3] = cmake<T>(fmadd(-c, q.x, e3.x), fmadd(c, q.y, e3.y));
     x[7] = cmake<T>(fmadd(c, q.x, e3.x), fmadd(-c, q.y, e3.y));
   }
+  // a + c b for a compile-time real c
+  static FFT_HD T axpy(T c, T b, T a) {
+    if constexpr (FftTraits<T>::fused) return fmadd(c, b, a);
+    else return a + c * b;
+  }
+  // DFT of odd prime length: with s_j = x_j + x_R-j and d_j = x_j - x_R-j (j = 1 ..
+  // (R-1)/2), y_q = a_q +- SIGN i u_q, a_q = x_0 + sum_j cos(2 pi j q / R) s_j, u_q =
+  // sum_j sin(2 pi j q / R) d_j.
+  template <int R, int Q, int J = 1> static FFT_HD void odd_sums(const C* s, const C* d, C& a, C& u) {
+    if constexpr (2 * J < R) {
+      constexpr T c = T(ct_trig(J * Q, R, false)), h = T(ct_trig(J * Q, R, true));
+      a = cmake<T>(axpy(c, s[J].x, a.x), axpy(c, s[J].y, a.y));
+      if constexpr (J == 1) u = cmake<T>(h * d[1].x, h * d[1].y);
+      else u = cmake<T>(axpy(h, d[J].x, u.x), axpy(h, d[J].y, u.y));
+      odd_sums<R, Q, J + 1>(s, d, a, u);
+    }
+  }
+  template <int R, int Q = 1> static FFT_HD void odd_outputs(const C* s, const C* d, C x0, C* y) {
+    if constexpr (2 * Q < R) {
+      C a = x0, u = x0;
+      odd_sums<R, Q>(s, d, a, u);
+      const C v = cmul_si<SIGN>(u);
+      y[Q] = cadd(a, v);
+      y[R - Q] = csub(a, v);
+      odd_outputs<R, Q + 1>(s, d, x0, y);
+    }
+  }
+  template <int R> static FFT_HD void odd_prime(C* x) {
+    constexpr int H = (R + 1) / 2;
+    C s[H], d[H], sum = x[0];
+#pragma unroll
+    for (int j = 1; j < H; ++j) {
+      s[j] = cadd(x[j], x[R - j]);
+      d[j] = csub(x[j], x[R - j]);
+      sum = cadd(sum, s[j]);
+    }
+    odd_outputs<R>(s, d, x[0], x);
+    x[0] = sum;
+  }
   // W0: x_0 carries a twiddle w_0 too
   template <int R, bool W0> static FFT_HD void run_tw(C* x, const C* w) {
     if constexpr (W0) x[0] = cmul(x[0], w[0]);
@@ -358,6 +397,15 @@ template <int SIGN, class T> struct Dft {
     else if constexpr (R == 6) prime_factor<2, 3, true>(x, w);
     else if constexpr (R == 9) composite<3, 3, true>(x, w);
     else if constexpr (R == 12) prime_factor<4, 3, true>(x, w);
+    else if constexpr (R == 5 || R == 7) {
+#pragma unroll
+      for (int r = 1; r < R; ++r) x[r] = cmul(x[r], w[r]);
+      odd_prime<R>(x);
+    }
+    else if constexpr (R == 10) prime_factor<2, 5, true>(x, w);
+    else if constexpr (R == 14) prime_factor<2, 7, true>(x, w);
+    else if constexpr (R == 15) prime_factor<3, 5, true>(x, w);
+    else if constexpr (R == 20) prime_factor<4, 5, true>(x, w);
     else if constexpr (R == 18) prime_factor<9, 2, true>(x, w);
     else if constexpr (R == 24) prime_factor<8, 3, true>(x, w);
     else composite<4, 4, true>(x, w);  // R == 16
@@ -485,6 +533,11 @@ template <int SIGN, class T> struct Dft {
     else if constexpr (R == 6) prime_factor<2, 3>(x);
     else if constexpr (R == 9) composite<3, 3>(x);
     else if constexpr (R == 12) prime_factor<4, 3>(x);
+    else if constexpr (R == 5 || R == 7) odd_prime<R>(x);
+    else if constexpr (R == 10) prime_factor<2, 5>(x);
+    else if constexpr (R == 14) prime_factor<2, 7>(x);
+    else if constexpr (R == 15) prime_factor<3, 5>(x);
+    else if constexpr (R == 20) prime_factor<4, 5>(x);
     else if constexpr (R == 18) prime_factor<9, 2>(x);
     else if constexpr (R == 24) prime_factor<8, 3>(x);
     else composite<4, 4>(x);  // R == 16
@@ -518,13 +571,19 @@ struct TwoFactor {
   int a, b;
 };
 template <int N, int TILE = 0> constexpr TwoFactor two_factor() {
-  static_assert(N == 8 || N == 12 || N == 16 || N == 24 || N == 32 || N == 36 || N == 48 || N == 64 || N == 72 ||
-                    N == 96,
+  static_assert(N == 8 || N == 12 || N == 16 || N == 20 || N == 24 || N == 28 || N == 32 || N == 36 || N == 40 ||
+                    N == 48 || N == 56 || N == 60 || N == 64 || N == 72 || N == 80 || N == 96,
                 "no factors chosen for this line length");
   return N == 8    ? TwoFactor{4, 2}
          : N == 12 ? TwoFactor{4, 3}
          : N == 16 ? TwoFactor{4, 4}
+         : N == 20 ? TwoFactor{4, 5}
          : N == 24 ? TwoFactor{4, 6}
+         : N == 28 ? TwoFactor{4, 7}
+         : N == 40 ? TwoFactor{8, 5}
+         : N == 56 ? TwoFactor{8, 7}
+         : N == 60 ? TwoFactor{12, 5}
+         : N == 80 ? TwoFactor{16, 5}
          : N == 32 ? TwoFactor{8, 4}
          : N == 36 ? TwoFactor{12, 3}
          : N == 48 ? TwoFactor{4, 12}

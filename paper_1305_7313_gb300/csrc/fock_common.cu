@@ -1,5 +1,7 @@
 // Size-independent device code: the energy reduction and the table of the
 // compiled (precision, grid size) kernel sets.
+#include <algorithm>
+
 #include "fock_kernels.cuh"
 #include "fock_sizes.h"
 
@@ -12,22 +14,45 @@ namespace fockx {
   extern const KOps kKOps_f64_##N;     \
   extern const KOps kKOps_f32_##N;
 FOCK_GRID_SIZES(FOCK_DECLARE)
+FOCK_PAIR_SIZES(FOCK_DECLARE)
 #undef FOCK_DECLARE
 
 const KernelOps* find_kernel_ops(int prec, int n) {
 #define FOCK_FIND(N) \
   if (n == N) return prec == 0 ? &kOps_f64_##N : prec == 1 ? &kOps_f32_##N : prec == 2 ? &kOps_df_##N : nullptr;
   FOCK_GRID_SIZES(FOCK_FIND)
-#undef FOCK_FIND
   return nullptr;
+}
+
+const KernelOps* find_pair_ops(int prec, int n) {
+  FOCK_PAIR_SIZES(FOCK_FIND)
+#undef FOCK_FIND
+  return find_kernel_ops(prec, n);
 }
 
 const KOps* find_kops(int prec, int n) {
 #define FOCK_FINDK(N) \
   if (n == N) return prec == 0 ? &kKOps_f64_##N : prec == 1 ? &kKOps_f32_##N : nullptr;
   FOCK_GRID_SIZES(FOCK_FINDK)
-#undef FOCK_FINDK
   return nullptr;
+}
+
+const KOps* find_pair_kops(int prec, int n) {
+  FOCK_PAIR_SIZES(FOCK_FINDK)
+#undef FOCK_FINDK
+  return find_kops(prec, n);
+}
+
+std::vector<int> pair_grid_sizes(int n) {
+  std::vector<int> all;
+#define FOCK_SIZE(N) all.push_back(N);
+  FOCK_GRID_SIZES(FOCK_SIZE)
+  FOCK_PAIR_SIZES(FOCK_SIZE)
+#undef FOCK_SIZE
+  std::sort(all.begin(), all.end());
+  if (persist_supports(n))  // such plans may join a batch
+    all.erase(std::remove_if(all.begin(), all.end(), [](int s) { return !persist_runs(s); }), all.end());
+  return all;
 }
 
 extern const PersistOps kPersist_f64;
@@ -37,6 +62,9 @@ const PersistOps* find_persist_ops(int prec) { return prec == 0 ? &kPersist_f64 
 
 bool persist_supports(int n) {
   return n == 24 || n == 32 || n == 48 || n == 64 || n == 72 || n == 96;
+}
+bool persist_runs(int n) {
+  return persist_supports(n) || n == 20 || n == 28 || n == 40 || n == 56 || n == 60 || n == 80;
 }
 
 // E_x = scale * sum over the unique pairs of f_i f_j (2 if i != j) e_ij, with

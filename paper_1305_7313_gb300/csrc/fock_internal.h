@@ -5,6 +5,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <vector>
+
 
 struct fock_plan;
 
@@ -51,7 +53,7 @@ struct ColumnSet {
 
 // Everything a kernel needs to know about a plan (device pointers included).
 struct DevPlan {
-  int n;            // cubic grid N
+  int n;            // cubic grid N the kernels work on (lattice::pair_grid of the caller's)
   int k3h;          // N/2 + 1: stored half of the last axis
   int64_t ntot;     // N^3
   int64_t hsize;    // elements reserved per pair-transform buffer (at least N^3: [i1][k2][k3])
@@ -137,8 +139,13 @@ struct KernelOps {
                       double2* out, cudaStream_t);
 };
 
-// Kernels for grid size n and precision (0: FP64, 1: mixed); NULL if not built.
+// Kernels for grid size n and precision (0: FP64, 1: mixed, 2: double-float);
+// NULL if not built.  find_pair_ops: also the sizes that only serve as a plan's
+// working grid.
 const KernelOps* find_kernel_ops(int prec, int n);
+const KernelOps* find_pair_ops(int prec, int n);
+// Working grids a plan on an n^3 grid may take (lattice::pair_grid), ascending.
+std::vector<int> pair_grid_sizes(int n);
 
 // Kernels of the Brillouin-zone-sampled apply (complex periodic parts, one pair
 // per transform; band0 is a global state index, psiG / vpsiG point at the
@@ -157,6 +164,7 @@ struct KOps {
                            double2* vpsiG, cudaStream_t);
 };
 const KOps* find_kops(int prec, int n);
+const KOps* find_pair_kops(int prec, int n);
 
 // One system of a batch as the persistent kernel sees it.
 struct SysDesc {
@@ -199,12 +207,14 @@ struct PersistOps {
 
 // Persistent pair kernel of a precision (0: FP64, 1: mixed).
 const PersistOps* find_persist_ops(int prec);
-// Grid sizes the persistent kernel runs.
+// Grid sizes of the plans a batch takes, and the working grids its kernels run.
 bool persist_supports(int n);
+bool persist_runs(int n);
 
 // What code outside fock_plan.cpp may read of a plan.
 struct PlanView {
   int device;
+  int n;  // the caller's grid
   const KernelOps* ops;
   DevPlan dp;
 };

@@ -183,10 +183,9 @@ fock_status fock_kplan_create(fock_kplan_t* out, const int grid[3], const double
     if (!std::isfinite(wk[i])) return kfail(nullptr, FOCK_ERR_INVALID_ARG, "weights are not finite");
   if (grid[0] != grid[1] || grid[1] != grid[2])
     return kfail(nullptr, FOCK_ERR_UNSUPPORTED_SIZE, "the FFT grid must be cubic (N1 = N2 = N3)");
-  const int n = grid[0];
-  const fockx::KernelOps* ops = fockx::find_kernel_ops(prec == FOCK_PREC_FP64 ? 0 : 1, n);
-  const fockx::KOps* kops = fockx::find_kops(prec == FOCK_PREC_FP64 ? 0 : 1, n);
-  if (!ops || !kops) return kfail(nullptr, FOCK_ERR_UNSUPPORTED_SIZE, "no kernels compiled for this N");
+  const int n_grid = grid[0], iprec = prec == FOCK_PREC_FP64 ? 0 : 1;
+  if (!fockx::find_kernel_ops(iprec, n_grid) || !fockx::find_kops(iprec, n_grid))
+    return kfail(nullptr, FOCK_ERR_UNSUPPORTED_SIZE, "no kernels compiled for this N");
 
   fock_kplan* p = new (std::nothrow) fock_kplan();
   if (!p) return kfail(nullptr, FOCK_ERR_OOM, "host allocation failed");
@@ -196,13 +195,10 @@ fock_status fock_kplan_create(fock_kplan_t* out, const int grid[3], const double
     return st;
   };
   std::memcpy(p->cell, cell, sizeof(p->cell));
-  p->n = n;
   p->ecut = ecut_ha;
   p->kind = kind;
   p->omega = omega;
   p->prec = prec;
-  p->ops = ops;
-  p->kops = kops;
   p->nk = nk;
   p->kfrac.assign(kpts, kpts + 3 * nk);
   p->wk.assign(wk, wk + nk);
@@ -211,11 +207,10 @@ fock_status fock_kplan_create(fock_kplan_t* out, const int grid[3], const double
   p->vol = std::fabs(vs);
 
   // one sphere per k point (host only: a grid is refused before any CUDA call)
-  const int64_t ntot = (int64_t)n * n * n;
   std::vector<fockx::lattice::GEntry> sph;
   std::vector<int> mlo((size_t)3 * nk), mhi((size_t)3 * nk);
   for (int k = 0; k < nk; ++k) {
-    if (!fockx::lattice::build_sphere(cell, p->recip, ecut_ha, n, sph, &p->kfrac[3 * k]))
+    if (!fockx::lattice::build_sphere(cell, p->recip, ecut_ha, n_grid, sph, &p->kfrac[3 * k]))
       return bail(kfail(p, FOCK_ERR_GRID_TOO_SMALL, "a G-sphere does not fit on the grid"));
     std::vector<int32_t> mill(3 * sph.size());
     for (int a = 0; a < 3; ++a) {
@@ -240,14 +235,22 @@ fock_status fock_kplan_create(fock_kplan_t* out, const int grid[3], const double
   // see the kernel at another |G + q|.  The frequencies of u_a* u_b are the
   // differences m_b - m_a of the two spheres, so every pair of k points
   // (k = k' included) must keep max m_b - min m_a below N/2 on every axis.
-  if (n % 2 == 0)
-    for (int ka = 0; ka < nk; ++ka)
-      for (int kb = 0; kb < nk; ++kb)
-        for (int a = 0; a < 3; ++a)
-          if (2 * (mhi[3 * kb + a] - mlo[3 * ka + a]) >= n)
-            return bail(kfail(p, FOCK_ERR_GRID_TOO_SMALL,
-                              "the pair densities reach the Nyquist frequency -N/2 of the grid "
-                              "(need N > 2 (max m - min m') over every pair of spheres)"));
+  int reach = 0;
+  for (int ka = 0; ka < nk; ++ka)
+    for (int kb = 0; kb < nk; ++kb)
+      for (int a = 0; a < 3; ++a) reach = std::max(reach, mhi[3 * kb + a] - mlo[3 * ka + a]);
+  if (n_grid % 2 == 0 && 2 * reach >= n_grid)
+    return bail(kfail(p, FOCK_ERR_GRID_TOO_SMALL,
+                      "the pair densities reach the Nyquist frequency -N/2 of the grid "
+                      "(need N > 2 (max m - min m') over every pair of spheres)"));
+  // the working grid
+  const int n = fockx::lattice::pair_grid(n_grid, reach, fockx::pair_grid_sizes(n_grid));
+  const int64_t ntot = (int64_t)n * n * n;
+  const fockx::KernelOps* ops = fockx::find_pair_ops(iprec, n);
+  const fockx::KOps* kops = fockx::find_pair_kops(iprec, n);
+  p->n = n;
+  p->ops = ops;
+  p->kops = kops;
   cudaError_t e = cudaGetDevice(&p->device);
   if (e != cudaSuccess) return bail(kcuda(p, e, "cudaGetDevice"));
   // the columns of each sphere, and those the pair densities reach: |G + q| <= 2

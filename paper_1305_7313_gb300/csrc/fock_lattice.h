@@ -88,6 +88,21 @@ inline bool build_sphere(const double* cell, const double* recip, double ecut, i
   return true;
 }
 
+// The grid a plan works on.  Pair densities of sphere orbitals have frequencies
+// at most `reach` on each axis; on a grid of s > 2 reach points they do not
+// alias, the kernel acts on their true frequencies, and no product psi phi folds
+// into the sphere (it reaches at most 3/2 reach, and 3/2 reach - s < -reach / 2).
+// Every such grid therefore gives the same operator, energies and derivatives up
+// to rounding, and the smallest one is the cheapest: the smallest of `sizes`
+// (ascending) with s > 2 reach that is smaller than the caller's n, else n.  A
+// grid that aliases its pair densities (n <= 2 reach) is its own operator and is
+// always worked on itself.
+inline int pair_grid(int n, int reach, const std::vector<int>& sizes) {
+  for (int s : sizes)
+    if (s > 2 * reach && s < n) return s;
+  return n;
+}
+
 inline int freq_of(int k, int n) { return k < (n + 1) / 2 ? k : k - n; }
 
 // v(G) and dv/domega for |G|^2 = g2 (Spencer-Alavi: Rc = (3 Omega / 4 pi)^(1/3)).

@@ -133,11 +133,17 @@ __global__ void __launch_bounds__(kPersistMaxT<T>, PersistGeo<T>::MIN_CTAS)
     const int n = sys[sg.sys].g.n;
     const int64_t hsize = sys[sg.sys].g.hsize;
     switch (n) {
+      case 20: run_task<T, 20>(sys, sg, local, hslot, hsize); break;
       case 24: run_task<T, 24>(sys, sg, local, hslot, hsize); break;
+      case 28: run_task<T, 28>(sys, sg, local, hslot, hsize); break;
       case 32: run_task<T, 32>(sys, sg, local, hslot, hsize); break;
+      case 40: run_task<T, 40>(sys, sg, local, hslot, hsize); break;
       case 48: run_task<T, 48>(sys, sg, local, hslot, hsize); break;
+      case 56: run_task<T, 56>(sys, sg, local, hslot, hsize); break;
+      case 60: run_task<T, 60>(sys, sg, local, hslot, hsize); break;
       case 64: run_task<T, 64>(sys, sg, local, hslot, hsize); break;
       case 72: run_task<T, 72>(sys, sg, local, hslot, hsize); break;
+      case 80: run_task<T, 80>(sys, sg, local, hslot, hsize); break;
       case 96: run_task<T, 96>(sys, sg, local, hslot, hsize); break;
       default: break;  // the host admits only the sizes above
     }
@@ -219,11 +225,17 @@ __global__ void __launch_bounds__(kPersistMaxT<T>, PersistGeo<T>::MIN_CTAS)
   cplx<T>* hslot = reinterpret_cast<cplx<T>*>(hring + (size_t)sg.slot * slot_bytes);
   const int local = t - sg.task0;
   switch (sys[sg.sys].g.n) {
+    case 20: dataflow_task<T, 20>(sys, sg, local, hslot, smem_raw); break;
     case 24: dataflow_task<T, 24>(sys, sg, local, hslot, smem_raw); break;
+    case 28: dataflow_task<T, 28>(sys, sg, local, hslot, smem_raw); break;
     case 32: dataflow_task<T, 32>(sys, sg, local, hslot, smem_raw); break;
+    case 40: dataflow_task<T, 40>(sys, sg, local, hslot, smem_raw); break;
     case 48: dataflow_task<T, 48>(sys, sg, local, hslot, smem_raw); break;
+    case 56: dataflow_task<T, 56>(sys, sg, local, hslot, smem_raw); break;
+    case 60: dataflow_task<T, 60>(sys, sg, local, hslot, smem_raw); break;
     case 64: dataflow_task<T, 64>(sys, sg, local, hslot, smem_raw); break;
     case 72: dataflow_task<T, 72>(sys, sg, local, hslot, smem_raw); break;
+    case 80: dataflow_task<T, 80>(sys, sg, local, hslot, smem_raw); break;
     case 96: dataflow_task<T, 96>(sys, sg, local, hslot, smem_raw); break;
     default: break;  // the host admits only the sizes above
   }

@@ -65,7 +65,7 @@ struct Workspace {
 
 struct fock_plan {
   int device = 0;
-  int n = 0;
+  int n = 0;  // the caller's grid; ops and dp are those of the working grid
   double cell[9];
   double recip[9];
   double vol = 0.0;
@@ -77,6 +77,10 @@ struct fock_plan {
   int npw = 0;
   const KernelOps* ops = nullptr;
   DevPlan dp{};
+  // kernels of the caller's grid: its FFT tilings, and (FP64, with the columns
+  // and twiddles in dp_full) the local potential of the Sternheimer solves
+  const KernelOps* ops_full = nullptr;
+  DevPlan dp_full{};
   int chain_batch = 1;
   int band_block = kBandBlock;
   // device tables
@@ -87,6 +91,8 @@ struct fock_plan {
   double* d_dvtab64 = nullptr;
   int* d_cols = nullptr;  // DevPlan::cols and orb
   int* d_orb = nullptr;
+  int* d_orb_full = nullptr;  // dp_full.orb and tw where the working grid is smaller
+  void* d_tw_full = nullptr;
   // deterministic accumulation (fock_plan_set_deterministic)
   bool det = false;
   double vnorm = 0.0;          // ||v||_2 over the whole grid
@@ -668,6 +674,7 @@ namespace fockx {
 bool plan_view(fock_plan* plan, PlanView* out) {
   if (!plan || !out) return false;
   out->device = plan->device;
+  out->n = plan->n;
   out->ops = plan->ops;
   out->dp = plan->dp;
   return true;
@@ -724,23 +731,23 @@ fock_status fock_plan_create(fock_plan_t* out, const int grid[3], const double c
     if (!std::isfinite(cell[i])) return fail(nullptr, FOCK_ERR_INVALID_ARG, "cell is not finite");
   if (grid[0] != grid[1] || grid[1] != grid[2])
     return fail(nullptr, FOCK_ERR_UNSUPPORTED_SIZE, "the FFT grid must be cubic (N1 = N2 = N3)");
-  const int n = grid[0];
-  if (n < 2 || !supported_n(n)) return fail(nullptr, FOCK_ERR_UNSUPPORTED_SIZE, "N must be 2^a 3^b");
-  const KernelOps* ops = fockx::find_kernel_ops((int)prec, n);
-  if (!ops) {
+  const int n_grid = grid[0];
+  if (n_grid < 2 || !supported_n(n_grid)) return fail(nullptr, FOCK_ERR_UNSUPPORTED_SIZE, "N must be 2^a 3^b");
+  const KernelOps* ops_full = fockx::find_kernel_ops((int)prec, n_grid);
+  if (!ops_full) {
     return fail(nullptr, FOCK_ERR_UNSUPPORTED_SIZE,
-                "no kernels compiled for N = " + std::to_string(n));
+                "no kernels compiled for N = " + std::to_string(n_grid));
   }
 
   fock_plan* p = new (std::nothrow) fock_plan();
   if (!p) return fail(nullptr, FOCK_ERR_OOM, "host allocation failed");
   std::memcpy(p->cell, cell, sizeof(p->cell));
-  p->n = n;
+  p->n = n_grid;
   p->ecut = ecut_ha;
   p->kind = kind;
   p->omega = omega;
   p->prec = prec;
-  p->ops = ops;
+  p->ops_full = ops_full;
 
   // cell volume and reciprocal lattice, b_i = (2 pi / Omega) (a_j x a_k)
   reciprocal(cell, p->recip, &p->vol);
@@ -752,11 +759,18 @@ fock_status fock_plan_create(fock_plan_t* out, const int grid[3], const double c
 
   // the sphere |G|^2 <= 2 Ecut in canonical order
   std::vector<GEntry> sph;
-  if (!build_sphere(cell, p->recip, ecut_ha, n, sph)) {
+  if (!build_sphere(cell, p->recip, ecut_ha, n_grid, sph)) {
     delete p;
     return fail(nullptr, FOCK_ERR_GRID_TOO_SMALL, "the G-sphere does not fit on the grid");
   }
   p->npw = (int)sph.size();
+  // the working grid: pair densities reach twice the sphere's largest index
+  int reach = 0;
+  for (const GEntry& e : sph)
+    for (int a = 0; a < 3; ++a) reach = std::max(reach, 2 * std::abs(e.m[a]));
+  const int n = fockx::lattice::pair_grid(n_grid, reach, fockx::pair_grid_sizes(n_grid));
+  const KernelOps* ops = n == n_grid ? ops_full : fockx::find_pair_ops((int)prec, n);
+  p->ops = ops;
   p->miller.resize(3 * sph.size());
   // half of the sphere for the Gamma-point overlaps: G = 0 first, then the G
   // whose first nonzero Miller index is positive
@@ -830,12 +844,16 @@ fock_status fock_plan_create(fock_plan_t* out, const int grid[3], const double c
 
   const bool fp64 = prec == FOCK_PREC_FP64;
   // twiddles w[t] = exp(-2 pi i t / N)
-  std::vector<double> tw64(2 * n);
-  for (int t = 0; t < n; ++t) {
-    const long double ang = 2.0L * 3.141592653589793238462643383279502884L * t / n;
-    tw64[2 * t] = (double)std::cos(ang);
-    tw64[2 * t + 1] = -(double)std::sin(ang);
-  }
+  const auto twiddles = [](int m) {
+    std::vector<double> w(2 * m);
+    for (int t = 0; t < m; ++t) {
+      const long double ang = 2.0L * 3.141592653589793238462643383279502884L * t / m;
+      w[2 * t] = (double)std::cos(ang);
+      w[2 * t + 1] = -(double)std::sin(ang);
+    }
+    return w;
+  };
+  const std::vector<double> tw64 = twiddles(n);
 
   fock_status st = FOCK_OK;
   auto upload = [&](void** dst, const void* src, size_t bytes) -> bool {
@@ -894,6 +912,23 @@ fock_status fock_plan_create(fock_plan_t* out, const int grid[3], const double c
       }
     }
   }
+  if (ok && fp64 && n != n_grid) {
+    // the sphere's columns on the caller's grid, for the local potential
+    const auto wrap_full = [n_grid](int m) { return ((m % n_grid) + n_grid) % n_grid; };
+    std::vector<unsigned char> full((size_t)n_grid * n_grid, 0);
+    for (const GEntry& e : sph) full[(size_t)wrap_full(e.m[1]) * n_grid + wrap_full(e.m[2])] = 1;
+    fockx::columns::HostColumns c;
+    fockx::columns::build(n_grid, full, true, ops_full->col_pairs, ops_full->row_place, c);
+    const cudaError_t e = fockx::columns::upload(
+        c, fockx::columns::coefficient_map(n_grid, c, ops_full->col_pairs, true, p->miller.data(), sph.size()),
+        &p->d_orb_full, &p->dp_full.orb, &p->table_bytes);
+    if (e != cudaSuccess) {
+      st = cuda_fail(nullptr, e, "uploading the column sets");
+      ok = false;
+    }
+    const std::vector<double> w = twiddles(n_grid);
+    ok = ok && upload(&p->d_tw_full, w.data(), sizeof(double) * w.size());
+  }
   if (ok) ok = upload((void**)&p->d_result, std::vector<double>(4, 0.0).data(), 4 * sizeof(double));
   if (ok) {
     cudaError_t e = cudaMallocHost((void**)&p->h_result, 4 * sizeof(double));
@@ -922,6 +957,16 @@ fock_status fock_plan_create(fock_plan_t* out, const int grid[3], const double c
   d.psi_scale = 1.0 / std::sqrt(p->vol);
   d.out_scale = std::sqrt(p->vol) / (double)ntot;
   d.msmall2 = prec == FOCK_PREC_MIXED32 ? kMsmall2 : -1;
+  if (n == n_grid) {
+    p->dp_full = d;
+  } else {
+    DevPlan& f = p->dp_full;
+    f.n = n_grid;
+    f.ntot = (int64_t)n_grid * n_grid * n_grid;
+    f.npw = p->npw;
+    f.tw = p->d_tw_full;
+    f.inv_ntot = 1.0 / (double)f.ntot;
+  }
   d.det = 0;  // set per call on a copy when the plan is deterministic
   d.tile[0] = d.tile[1] = d.tile[2] = 0;
   d.det_scale = nullptr;
@@ -953,6 +998,7 @@ fock_status fock_plan_create(fock_plan_t* out, const int grid[3], const double c
     return fail(nullptr, FOCK_ERR_UNSUPPORTED_SIZE, "the grid needs more shared memory than a CTA has");
   }
   e = ops->configure(d);
+  if (e == cudaSuccess && fp64 && n != n_grid) e = ops_full->configure(p->dp_full);
   if (e != cudaSuccess) {
     fock_destroy(p);
     return cuda_fail(nullptr, e, "configuring kernels");
@@ -1031,7 +1077,7 @@ fock_status fock_plan_tiling_info(fock_plan_t plan, int pass, int tile, int* rad
     return fail(plan, FOCK_ERR_INVALID_ARG, "NULL output");
   if (pass < 0 || pass > 2 || tile < 0 || tile > 1) return fail(plan, FOCK_ERR_INVALID_ARG, "pass or tile out of range");
   int r[8], nst = 0, tl = 0, thr = 0;
-  const int nt = plan->ops->tile_plan(pass, tile, r, &nst, &tl, &thr);
+  const int nt = plan->ops_full->tile_plan(pass, tile, r, &nst, &tl, &thr);
   if (tile >= nt) return fail(plan, FOCK_ERR_INVALID_ARG, "this plan has one tiling for that pass");
   for (int k = 0; k < nst; ++k) radices[k] = r[k];
   *nstages = nst;
@@ -1046,7 +1092,7 @@ fock_status fock_plan_set_tiling(fock_plan_t plan, const int tiles[3]) {
   if (!tiles) return fail(plan, FOCK_ERR_INVALID_ARG, "tiles is NULL");
   for (int pass = 0; pass < 3; ++pass) {
     int r[8], nst = 0, tl = 0, thr = 0;
-    const int nt = plan->ops->tile_plan(pass, 0, r, &nst, &tl, &thr);
+    const int nt = plan->ops_full->tile_plan(pass, 0, r, &nst, &tl, &thr);
     if (tiles[pass] < 0 || tiles[pass] >= nt)
       return fail(plan, FOCK_ERR_INVALID_ARG, "a tile index is not below the pass's number of tilings");
   }
@@ -1089,12 +1135,19 @@ fock_status fock_sternheimer_solve(fock_plan_t p, const double* vloc, const void
   double2 *x, *r, *pk, *ap, *tmp;
   double *kin, *d_eps, *c, *rr, *rrn, *part_a, *part_b, *sc;
   int* perm;
+  void* xgrid;
+  int nbat;
   {
-    const size_t bytes[] = {kb, kb, kb, kb, kb, sizeof(double) * npw, nb8,
+    // transform blocks for the local potential, on the caller's grid: the plan's
+    // transform buffer, or of their own where the working grid is smaller
+    const size_t grid_bytes = (size_t)p->dp_full.ntot * sizeof(double2);
+    const size_t own = p->n == p->dp.n ? 0 : std::min<size_t>(((size_t)nrhs + 1) / 2, 32);
+    nbat = p->n == p->dp.n ? bands_per_grid_batch(p) : 2 * (int)own;
+    const size_t bytes[] = {own * grid_bytes, kb, kb, kb, kb, kb, sizeof(double) * npw, nb8,
                             nb8 * nocc, nb8, nb8,
                             nb8 * (size_t)fockx::st_chunks((int)npw), nb8 * (size_t)fockx::st_chunks((int)npw), nb8,
                             sizeof(int) * (size_t)nrhs};
-    void** const ptrs[] = {(void**)&x, (void**)&r, (void**)&pk, (void**)&ap, (void**)&tmp, (void**)&kin,
+    void** const ptrs[] = {&xgrid, (void**)&x, (void**)&r, (void**)&pk, (void**)&ap, (void**)&tmp, (void**)&kin,
                            (void**)&d_eps, (void**)&c, (void**)&rr, (void**)&rrn, (void**)&part_a, (void**)&part_b,
                            (void**)&sc, (void**)&perm};
     size_t total = 0;
@@ -1111,6 +1164,7 @@ fock_status fock_sternheimer_solve(fock_plan_t p, const double* vloc, const void
       *ptrs[k] = at;
       at += (bytes[k] + 255) / 256 * 256;
     }
+    if (own == 0) xgrid = p->ws.h;
   }
   // |G|^2 / 2 on the sphere, in the plan's canonical order
   std::vector<double> kin_h(npw);
@@ -1121,7 +1175,6 @@ fock_status fock_sternheimer_solve(fock_plan_t p, const double* vloc, const void
   FOCK_CUDA(p, cudaMemcpyAsync(d_eps, eps_h.data(), nb8, cudaMemcpyHostToDevice, s));
 
   const int ip = (int)npw;
-  const int nbat = bands_per_grid_batch(p);
   // b = -Q w into r; x = 0; p = r; rr = <r|r>
   FOCK_CUDA(p, fockx::st_proj_coef(u, nocc, static_cast<const double2*>(w_G), nrhs, ip, c, s));
   FOCK_CUDA(p, fockx::st_rhs(static_cast<const double2*>(w_G), u, c, nocc, nrhs, ip, r, part_a, rr, s));
@@ -1136,7 +1189,7 @@ fock_status fock_sternheimer_solve(fock_plan_t p, const double* vloc, const void
   for (int it = 0; it < maxiter && m > 0; ++it) {
     // ap = (H - eps_n + alpha P) p for the kets at positions [0, m)
     for (int b0 = 0; b0 < m; b0 += nbat)
-      FOCK_CUDA(p, p->ops->vloc(p->dp, pk, m, b0, std::min(nbat, m - b0), vloc, p->ws.h, ap, s));
+      FOCK_CUDA(p, p->ops_full->vloc(p->dp_full, pk, m, b0, std::min(nbat, m - b0), vloc, xgrid, ap, s));
     FOCK_CUDA(p, fockx::st_proj_coef(u, nocc, pk, m, ip, c, s));
     FOCK_CUDA(p, fockx::st_finish(ap, pk, kin, d_eps, u, c, nocc, alpha, m, ip, part_a, s));
     FOCK_CUDA(p, fockx::st_step(x, r, pk, ap, rr, part_a, m, ip, part_b, s));
@@ -1255,7 +1308,7 @@ fock_status fock_plan_set_deterministic(fock_plan_t plan, int enable) {
 fock_status fock_plan_columns(fock_plan_t plan, int64_t* kept, int64_t* total) {
   if (!plan) return fail(nullptr, FOCK_ERR_INVALID_ARG, "plan is NULL");
   if (kept) *kept = plan->kept_columns;
-  if (total) *total = (int64_t)plan->n * 2 * (plan->n / 2 + 1);
+  if (total) *total = (int64_t)plan->n * 2 * (plan->n / 2 + 1);  // of the caller's grid
   return FOCK_OK;
 }
 
@@ -1488,6 +1541,8 @@ fock_status fock_destroy(fock_plan_t plan) {
   cudaFree(plan->d_dvtab64);
   cudaFree(plan->d_cols);
   cudaFree(plan->d_orb);
+  cudaFree(plan->d_orb_full);
+  cudaFree(plan->d_tw_full);
   cudaFree(plan->d_stats);
   cudaFree(plan->d_scale);
   cudaFree(plan->d_epart);
@@ -1797,7 +1852,7 @@ fock_status fock_batch_create(fock_batch_t* out, int nsys, const fock_plan_t* pl
     sg.slot = t % D;
     sg.dep = dep;
     sg.dep2 = dep2;
-    sg.ntasks = (sg.kind == 1 ? b->plans[sg.sys]->dp.cols.ncta : b->plans[sg.sys]->n) * sg.nch;
+    sg.ntasks = (sg.kind == 1 ? b->plans[sg.sys]->dp.cols.ncta : b->plans[sg.sys]->dp.n) * sg.nch;
     b->segs.push_back(sg);
     return (int)b->segs.size() - 1;
   };

@@ -155,7 +155,10 @@ extern "C" fock_status fock_pair_energies_static(fock_plan_t plan, const void* p
   const size_t off_e = align256(off_chains + sizeof(fockx::Chain) * (size_t)nch);
   const size_t off_d = align256(off_e + sizeof(double) * (size_t)npairs);
   const size_t off_h = align256(off_d + sizeof(double) * (size_t)npairs);
-  if (off_h + chain_bytes > kStaticScratchBytes) {
+  // refused by the size on the caller's grid (the working grid is no larger)
+  const size_t n = (size_t)v.n;
+  const size_t want = off_h - off_pairs + align256((size_t)nb * n * n * n * rb) + n * n * (n + 2) * 2 * rb;
+  if (std::max(want, off_h + chain_bytes) > kStaticScratchBytes) {
     return fail(plan, FOCK_ERR_INVALID_ARG,
                 "the request needs more than the 32 MiB static scratch "
                 "(real-space orbitals nb*N^3 reals + one N^2(N+2) complex transform buffer)");
