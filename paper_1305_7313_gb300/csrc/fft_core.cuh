@@ -22,6 +22,7 @@
 #include <cuda_runtime.h>
 
 #include <cmath>
+#include <type_traits>
 
 #include "df64.cuh"
 
@@ -211,12 +212,120 @@ FFT_HD cplx<T> cmake(T x, T y) {
   r.y = y;
   return r;
 }
-template <class C> FFT_HD C cadd(C a, C b) { a.x += b.x; a.y += b.y; return a; }
-template <class C> FFT_HD C csub(C a, C b) { a.x -= b.x; a.y -= b.y; return a; }
+// x y and x + S y rounded once, in any type.
+template <class T> FFT_HD T rmul(T x, T y) { return x * y; }
+// a compile-time factor as the multiplications take it
+template <class T> FFT_HD T factor(T c) { return c; }
+template <int S, class T> FFT_HD T radd(T x, T y) { return S > 0 ? x + y : x - y; }
+#ifdef __CUDA_ARCH__
+// FP64: as fused multiply-adds, x y + (-0) and x + y 1, which round the same, with
+// every operand in a register.  A DADD, a DMUL or a DFMA with an immediate or
+// constant operand occupies the FP64 unit of an SM for 20 clocks a warp, a DFMA of
+// registers for 16.8 (measured with independent operations: 504 against 598 G a
+// second over the chip).  The factors come from a register the compiler cannot see
+// through (%smid < 2^24), or it would turn them back.  FP64 pair passes at 96^3:
+// 165 -> 151 us a chain, the FP64 unit 92-97% busy.
+__device__ __forceinline__ double opaque_one() {
+  double o;
+  asm("{.reg .u32 t; mov.u32 t, %%smid; shr.u32 t, t, 24; add.u32 t, t, 1; cvt.rn.f64.u32 %0, t;}" : "=d"(o));
+  return o;
+}
+__device__ __forceinline__ double opaque_minus_zero() {
+  double o;
+  asm("{.reg .u32 t; mov.u32 t, %%smid; shr.u32 t, t, 24; cvt.rn.f64.u32 %0, t; neg.f64 %0, %0;}" : "=d"(o));
+  return o;
+}
+template <> __device__ __forceinline__ double rmul<double>(double x, double y) {
+  return __fma_rn(x, y, opaque_minus_zero());
+}
+template <> __device__ __forceinline__ double factor<double>(double c) { return __dmul_rn(c, opaque_one()); }
+template <> __device__ __forceinline__ double radd<1, double>(double x, double y) { return __fma_rn(y, opaque_one(), x); }
+template <> __device__ __forceinline__ double radd<-1, double>(double x, double y) {
+  return __fma_rn(-y, opaque_one(), x);
+}
+#endif
+
+template <class C> FFT_HD C cadd(C a, C b) {
+  a.x = radd<1>(a.x, b.x);
+  a.y = radd<1>(a.y, b.y);
+  return a;
+}
+template <class C> FFT_HD C csub(C a, C b) {
+  a.x = radd<-1>(a.x, b.x);
+  a.y = radd<-1>(a.y, b.y);
+  return a;
+}
+// c b and a + c b for a real c (one rounding per component where T has a fused
+// multiply-add).
+template <class T, class C> FFT_HD C cscale(T c, C b) {
+  const T f = factor(c);
+  b.x = rmul(f, b.x);
+  b.y = rmul(f, b.y);
+  return b;
+}
+template <class T, class C> FFT_HD C caxpy(T c, C b, C a) {
+  if constexpr (FftTraits<T>::fused) {
+    const T f = factor(c);
+    a.x = fmadd(f, b.x, a.x);
+    a.y = fmadd(f, b.y, a.y);
+  } else {
+    a.x = a.x + c * b.x;
+    a.y = a.y + c * b.y;
+  }
+  return a;
+}
+#ifdef __CUDA_ARCH__
+// FP32: both components in one instruction, with the same roundings.  The FP32
+// pipe runs the two-wide forms at the rate of two scalar ones, but an instruction
+// takes one issue slot: the forward plane pass at 96^3 went from 3.01 to 2.83 us a
+// chain, the apply (256 bands) from 136.8 to 134.4 ms.
+template <> __device__ __forceinline__ float2 cadd<float2>(float2 a, float2 b) {
+  float2 r;
+  asm("{.reg .b64 a, b, c; mov.b64 a, {%2, %3}; mov.b64 b, {%4, %5}; add.rn.f32x2 c, a, b; mov.b64 {%0, %1}, c;}"
+      : "=f"(r.x), "=f"(r.y)
+      : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+  return r;
+}
+template <> __device__ __forceinline__ float2 csub<float2>(float2 a, float2 b) {
+  float2 r;
+  asm("{.reg .b64 a, b, c; mov.b64 a, {%2, %3}; mov.b64 b, {%4, %5}; sub.rn.f32x2 c, a, b; mov.b64 {%0, %1}, c;}"
+      : "=f"(r.x), "=f"(r.y)
+      : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+  return r;
+}
+template <> __device__ __forceinline__ float2 cscale<float, float2>(float c, float2 b) {
+  float2 r;
+  asm("{.reg .b64 a, b, c; mov.b64 a, {%2, %2}; mov.b64 b, {%3, %4}; mul.rn.f32x2 c, a, b; mov.b64 {%0, %1}, c;}"
+      : "=f"(r.x), "=f"(r.y)
+      : "f"(c), "f"(b.x), "f"(b.y));
+  return r;
+}
+template <> __device__ __forceinline__ float2 caxpy<float, float2>(float c, float2 b, float2 a) {
+  float2 r;
+  asm("{.reg .b64 a, b, c, d; mov.b64 a, {%2, %2}; mov.b64 b, {%3, %4}; mov.b64 c, {%5, %6}; fma.rn.f32x2 d, a, b, c; "
+      "mov.b64 {%0, %1}, d;}"
+      : "=f"(r.x), "=f"(r.y)
+      : "f"(c), "f"(b.x), "f"(b.y), "f"(a.x), "f"(a.y));
+  return r;
+}
+#endif
+// a + S i b and a - S i b for S = +1 or -1
+template <int S, class C> FFT_HD C cadd_si(C a, C b) {
+  C r;
+  r.x = radd<-S>(a.x, b.y);
+  r.y = radd<S>(a.y, b.x);
+  return r;
+}
+template <int S, class C> FFT_HD C csub_si(C a, C b) { return cadd_si<-S>(a, b); }
 template <class C> FFT_HD C cmul(C a, C b) {
   C r;
-  r.x = a.x * b.x - a.y * b.y;
-  r.y = a.x * b.y + a.y * b.x;
+  if constexpr (std::is_same<decltype(a.x), double>::value) {
+    r.x = fmadd(-a.y, b.y, rmul(a.x, b.x));
+    r.y = fmadd(a.y, b.x, rmul(a.x, b.y));
+  } else {
+    r.x = a.x * b.x - a.y * b.y;
+    r.y = a.x * b.y + a.y * b.x;
+  }
   return r;
 }
 // S * i * a for S = +1 or -1
@@ -239,19 +348,26 @@ template <int SIGN, class T> struct Dft {
   // the length-3 DFT from x0, s = x1 + x2 and d = x1 - x2
   static FFT_HD void r3_sd(C* x, C s, C d) {
     constexpr T h0 = T(0.86602540378443864676372317075293618);  // sin(2 pi / 3)
-    const T h = sgn<SIGN>(h0);
-    C m = cmake<T>(x[0].x - half_of(s.x), x[0].y - half_of(s.y));
-    C u = cmake<T>(-h * d.y, h * d.x);
-    x[0] = cadd(x[0], s);
-    x[1] = cadd(m, u);
-    x[2] = csub(m, u);
+    if constexpr (FftTraits<T>::fused) {
+      const T h = factor(SIGN > 0 ? h0 : -h0);
+      const C m = caxpy(T(-0.5), s, x[0]);
+      x[0] = cadd(x[0], s);
+      x[1] = cmake<T>(fmadd(-h, d.y, m.x), fmadd(h, d.x, m.y));
+      x[2] = cmake<T>(fmadd(h, d.y, m.x), fmadd(-h, d.x, m.y));
+    } else {
+      const C m = cmake<T>(x[0].x - half_of(s.x), x[0].y - half_of(s.y));
+      const C u = cscale(h0, d);
+      x[0] = cadd(x[0], s);
+      x[1] = cadd_si<SIGN>(m, u);
+      x[2] = csub_si<SIGN>(m, u);
+    }
   }
   static FFT_HD void r4v(C& x0, C& x1, C& x2, C& x3) {
-    C a = cadd(x0, x2), b = csub(x0, x2), c = cadd(x1, x3), d = cmul_si<SIGN>(csub(x1, x3));
+    C a = cadd(x0, x2), b = csub(x0, x2), c = cadd(x1, x3), d = csub(x1, x3);
     x0 = cadd(a, c);
     x2 = csub(a, c);
-    x1 = cadd(b, d);
-    x3 = csub(b, d);
+    x1 = cadd_si<SIGN>(b, d);
+    x3 = csub_si<SIGN>(b, d);
   }
   static FFT_HD void r4(C* x) { r4v(x[0], x[1], x[2], x[3]); }
   static FFT_HD void r8(C* x) {
@@ -260,18 +376,16 @@ template <int SIGN, class T> struct Dft {
     C o0 = x[1], o1 = x[3], o2 = x[5], o3 = x[7];
     r4v(e0, e1, e2, e3);
     r4v(o0, o1, o2, o3);
-    // o_q *= exp(SIGN 2 pi i q / 8)
-    C t1 = cmake<T>(c * (o1.x - sgn<SIGN>(o1.y)), c * (o1.y + sgn<SIGN>(o1.x)));
-    C t2 = cmul_si<SIGN>(o2);
-    C t3 = cmake<T>(-(c * (o3.x + sgn<SIGN>(o3.y))), c * (sgn<SIGN>(o3.x) - o3.y));
+    // x_q = e_q +- exp(SIGN 2 pi i q / 8) o_q, the pi/4 rotations as c * p
+    const C p = cadd_si<SIGN>(o1, o1), q = csub_si<SIGN>(o3, o3);
     x[0] = cadd(e0, o0);
     x[4] = csub(e0, o0);
-    x[1] = cadd(e1, t1);
-    x[5] = csub(e1, t1);
-    x[2] = cadd(e2, t2);
-    x[6] = csub(e2, t2);
-    x[3] = cadd(e3, t3);
-    x[7] = csub(e3, t3);
+    x[1] = caxpy(c, p, e1);
+    x[5] = caxpy(-c, p, e1);
+    x[2] = cadd_si<SIGN>(e2, o2);
+    x[6] = csub_si<SIGN>(e2, o2);
+    x[3] = caxpy(-c, q, e3);
+    x[7] = caxpy(c, q, e3);
   }
   // x *= exp(SIGN 2 pi i M / R) with compile-time M, R (exact for the quarter turns)
   template <int M, int R> static FFT_HD C twiddle(C x) {
@@ -285,9 +399,8 @@ template <int SIGN, class T> struct Dft {
     } else if constexpr (4 * m == 3 * R) {
       return cmul_si<-SIGN>(x);
     } else {
-      constexpr T c = T(ct_trig(m, R, false));
-      constexpr T s = T(SIGN * ct_trig(m, R, true));
-      return cmake<T>(c * x.x - s * x.y, c * x.y + s * x.x);
+      const T c = factor(T(ct_trig(m, R, false))), s = factor(T(SIGN * ct_trig(m, R, true)));
+      return cmul(x, cmake<T>(c, s));
     }
   }
   // ---- twiddled inputs, for types with a fused multiply-add (FftTraits::fused).
@@ -302,11 +415,12 @@ template <int SIGN, class T> struct Dft {
   }
   // 2 a - b
   static FFT_HD C ctwice_sub(C a, C b) {
-    return cmake<T>(fmadd(T(2), a.x, -b.x), fmadd(T(2), a.y, -b.y));
+    const T two = factor(T(2));
+    return cmake<T>(fmadd(two, a.x, -b.x), fmadd(two, a.y, -b.y));
   }
   // a - 2 b
   static FFT_HD C csub_twice(C a, C b) {
-    return cmake<T>(fmadd(T(-2), b.x, a.x), fmadd(T(-2), b.y, a.y));
+    return caxpy(T(-2), b, a);
   }
   static FFT_HD void r2_tw(C& x0, C& x1, C w1) {
     const C a = cfma(x0, w1, x1);
@@ -323,11 +437,11 @@ template <int SIGN, class T> struct Dft {
     const C b = ctwice_sub(x0, a);     // x0 - w2 x2
     const C x3w = cmul(x3, w3);
     const C c = cfma(x3w, w1, x1);     // w1 x1 + w3 x3
-    const C d = cmul_si<SIGN>(csub_twice(c, x3w));  // S i (w1 x1 - w3 x3)
+    const C d = csub_twice(c, x3w);  // w1 x1 - w3 x3
     x0 = cadd(a, c);
     x2 = csub(a, c);
-    x1 = cadd(b, d);
-    x3 = csub(b, d);
+    x1 = cadd_si<SIGN>(b, d);
+    x3 = csub_si<SIGN>(b, d);
   }
   static FFT_HD void r8_tw(C* x, const C* w) {
     constexpr T c = T(0.70710678118654752440084436210484904);  // cos(pi / 4)
@@ -336,22 +450,15 @@ template <int SIGN, class T> struct Dft {
     r4v_tw(e0, e1, e2, e3, w[2], w[4], w[6]);
     r4v_tw(o0, o1, o2, o3, w[3], w[5], w[7]);
     // x_q = e_q +- exp(SIGN 2 pi i q / 8) o_q, the pi/4 rotations as c * p
-    const C p = cmake<T>(o1.x - sgn<SIGN>(o1.y), o1.y + sgn<SIGN>(o1.x));
-    const C q = cmake<T>(o3.x + sgn<SIGN>(o3.y), sgn<SIGN>(o3.x) - o3.y);
-    const C t2 = cmul_si<SIGN>(o2);
+    const C p = cadd_si<SIGN>(o1, o1), q = csub_si<SIGN>(o3, o3);
     x[0] = cadd(e0, o0);
     x[4] = csub(e0, o0);
-    x[1] = cmake<T>(fmadd(c, p.x, e1.x), fmadd(c, p.y, e1.y));
-    x[5] = cmake<T>(fmadd(-c, p.x, e1.x), fmadd(-c, p.y, e1.y));
-    x[2] = cadd(e2, t2);
-    x[6] = csub(e2, t2);
-    x[3] = cmake<T>(fmadd(-c, q.x, e3.x), fmadd(c, q.y, e3.y));
-    x[7] = cmake<T>(fmadd(c, q.x, e3.x), fmadd(-c, q.y, e3.y));
-  }
-  // a + c b for a compile-time real c
-  static FFT_HD T axpy(T c, T b, T a) {
-    if constexpr (FftTraits<T>::fused) return fmadd(c, b, a);
-    else return a + c * b;
+    x[1] = caxpy(c, p, e1);
+    x[5] = caxpy(-c, p, e1);
+    x[2] = cadd_si<SIGN>(e2, o2);
+    x[6] = csub_si<SIGN>(e2, o2);
+    x[3] = caxpy(-c, q, e3);
+    x[7] = caxpy(c, q, e3);
   }
   // DFT of odd prime length: with s_j = x_j + x_R-j and d_j = x_j - x_R-j (j = 1 ..
   // (R-1)/2), y_q = a_q +- SIGN i u_q, a_q = x_0 + sum_j cos(2 pi j q / R) s_j, u_q =
@@ -359,9 +466,9 @@ template <int SIGN, class T> struct Dft {
   template <int R, int Q, int J = 1> static FFT_HD void odd_sums(const C* s, const C* d, C& a, C& u) {
     if constexpr (2 * J < R) {
       constexpr T c = T(ct_trig(J * Q, R, false)), h = T(ct_trig(J * Q, R, true));
-      a = cmake<T>(axpy(c, s[J].x, a.x), axpy(c, s[J].y, a.y));
-      if constexpr (J == 1) u = cmake<T>(h * d[1].x, h * d[1].y);
-      else u = cmake<T>(axpy(h, d[J].x, u.x), axpy(h, d[J].y, u.y));
+      a = caxpy(c, s[J], a);
+      if constexpr (J == 1) u = cscale(h, d[1]);
+      else u = caxpy(h, d[J], u);
       odd_sums<R, Q, J + 1>(s, d, a, u);
     }
   }
@@ -369,9 +476,8 @@ template <int SIGN, class T> struct Dft {
     if constexpr (2 * Q < R) {
       C a = x0, u = x0;
       odd_sums<R, Q>(s, d, a, u);
-      const C v = cmul_si<SIGN>(u);
-      y[Q] = cadd(a, v);
-      y[R - Q] = csub(a, v);
+      y[Q] = cadd_si<SIGN>(a, u);
+      y[R - Q] = csub_si<SIGN>(a, u);
       odd_outputs<R, Q + 1>(s, d, x0, y);
     }
   }
@@ -501,7 +607,7 @@ template <int SIGN, class T> struct Dft {
         C wc[R2];
 #pragma unroll
         for (int n2 = 0; n2 < R2; ++n2)
-          wc[n2] = cmake<T>(T(ct_trig(n2 * K1, R1 * R2, false)), T(SIGN * ct_trig(n2 * K1, R1 * R2, true)));
+          wc[n2] = cmake<T>(factor(T(ct_trig(n2 * K1, R1 * R2, false))), factor(T(SIGN * ct_trig(n2 * K1, R1 * R2, true))));
         run_tw<R2, false>(t, wc);
       } else {
         twiddle_col<R1, R2, K1, 1>(t);
@@ -563,42 +669,31 @@ template <int SIGN, class T> struct Dft {
 // DFT over s, twiddles on the A-stage's inputs, A-point DFT over q) and leaves
 // natural order.
 //
-// Factors: A is a multiple of 4, so that four consecutive points 4c .. 4c + 3
-// of a spectrum-ordered line sit B apart (the accumulator updates read them as
-// one group), and consecutive k fall on distinct shared-memory banks except at
-// N = 64 (at 96, 12 x 8 would put them 8 values apart: six-way conflicts).
+// Factors: the larger one first, its DFTs without twiddles; N / 4 and 4 need the
+// fewest operations (96: 24 x 4 takes 1,584 additions and multiply-adds, 8 x 12
+// 1,648; FP64 forward pass at 96^3 58.9 -> 57.4 us a chain, at 60^3 15 x 4 against
+// 12 x 5 15.9 -> 15.5) except at 72 and 36, and in double-float at 96, whose
+// 24-point DFT is too long for the instruction cache (17.7 us against 17.2 with
+// 12 x 8).
 struct TwoFactor {
   int a, b;
 };
-template <int N, int TILE = 0> constexpr TwoFactor two_factor() {
+template <class T, int N, int TILE = 0> constexpr TwoFactor two_factor() {
   static_assert(N == 8 || N == 12 || N == 16 || N == 20 || N == 24 || N == 28 || N == 32 || N == 36 || N == 40 ||
                     N == 48 || N == 56 || N == 60 || N == 64 || N == 72 || N == 80 || N == 96,
                 "no factors chosen for this line length");
-  return N == 8    ? TwoFactor{4, 2}
-         : N == 12 ? TwoFactor{4, 3}
-         : N == 16 ? TwoFactor{4, 4}
-         : N == 20 ? TwoFactor{4, 5}
-         : N == 24 ? TwoFactor{4, 6}
-         : N == 28 ? TwoFactor{4, 7}
-         : N == 40 ? TwoFactor{8, 5}
-         : N == 56 ? TwoFactor{8, 7}
-         : N == 60 ? TwoFactor{12, 5}
-         : N == 80 ? TwoFactor{16, 5}
-         : N == 32 ? TwoFactor{8, 4}
-         : N == 36 ? TwoFactor{12, 3}
-         : N == 48 ? TwoFactor{4, 12}
-         : N == 64 ? TwoFactor{8, 8}
-         : N == 72 ? TwoFactor{12, 6}
-         : TILE == 1 ? TwoFactor{12, 8}
-                     : TwoFactor{8, 12};
+  if (TILE == 1) return TwoFactor{12, 8};
+  if (N == 96 && !FftTraits<T>::fused) return TwoFactor{12, 8};
+  if (N == 72) return TwoFactor{12, 6};
+  if (N == 36) return TwoFactor{12, 3};
+  if (N == 8 || N == 12) return TwoFactor{4, N / 4};
+  return TwoFactor{N / 4, 4};
 }
 template <int A, int B> FFT_HD constexpr int spec_pos(int k) { return k / A + B * (k % A); }
 
-// DFT of x_0, w[1] x_1, ..., w[R-1] x_{R-1} (w: R consecutive twiddles in shared
-// memory, two to a 16-byte load in FP32).
-template <class T, int R, int SIGN>
-__device__ __forceinline__ void dft_twiddled(cplx<T>* x, const cplx<T>* wp) {
-  cplx<T> w[R];
+// R consecutive twiddles in shared memory, two to a 16-byte load in FP32 (w_0 is
+// not used: x_0 carries no twiddle).
+template <class T, int R> __device__ __forceinline__ void load_twiddle_row(cplx<T>* w, const cplx<T>* wp) {
   if constexpr (sizeof(cplx<T>) == 8 && R % 2 == 0) {
     const float4* w4 = reinterpret_cast<const float4*>(wp);
 #pragma unroll
@@ -610,8 +705,15 @@ __device__ __forceinline__ void dft_twiddled(cplx<T>* x, const cplx<T>* wp) {
   } else {
 #pragma unroll
     for (int r = 1; r < R; ++r) w[r] = wp[r];
-    w[0] = w[1];  // not read: x_0 carries no twiddle
+    w[0] = w[1];
   }
+}
+
+// DFT of x_0, w[1] x_1, ..., w[R-1] x_{R-1} (wp: the R twiddles in shared memory).
+template <class T, int R, int SIGN>
+__device__ __forceinline__ void dft_twiddled(cplx<T>* x, const cplx<T>* wp) {
+  cplx<T> w[R];
+  load_twiddle_row<T, R>(w, wp);
   if constexpr (FftTraits<T>::fused) {
     Dft<SIGN, T>::template run_tw<R, false>(x, w);
   } else {

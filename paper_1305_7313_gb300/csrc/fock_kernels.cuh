@@ -94,6 +94,12 @@ __device__ __forceinline__ float4 ld_f4_hint(const float* p, unsigned long long 
   return v;
 }
 
+// Four floats added at p in one reduction, with an L2 eviction policy.
+__device__ __forceinline__ void red_f4_hint(float* p, float4 v, unsigned long long pol) {
+  asm volatile("red.global.add.L2::cache_hint.v4.f32 [%0], {%1, %2, %3, %4}, %5;" ::"l"(p), "f"(v.x), "f"(v.y),
+               "f"(v.z), "f"(v.w), "l"(pol)
+               : "memory");
+}
 template <class T> __device__ __forceinline__ void atomic_add_real(T* p, T v) { atomicAdd(p, v); }
 // df64 into an FP64 accumulator: both parts become doubles by integer
 // instructions, one FP64 add joins them (exact to the rounding of that add).
@@ -289,9 +295,9 @@ __device__ inline void block_sum4_ff(const float v[4], float hi[4], float lo[4],
 template <class T, int N, int TILE = 0>
 struct PairGeo {
   using C = cplx<T>;
-  static constexpr TwoFactor f = two_factor<N, TILE>();
+  static constexpr TwoFactor f = two_factor<T, N, TILE>();
   static constexpr int A = f.a, B = f.b;
-  static_assert(A * B == N && A % 4 == 0, "factors of the line length, the first a multiple of 4");
+  static_assert(A * B == N, "factors of the line length");
   static constexpr int RP = N + 1;  // odd row stride of a plane: rows on distinct banks
   // FP32 plane passes transform all N rows or columns in shared memory, kept
   // or not (85 of 96 at 96^3, L 27): packing the kept ones leaves gaps and
@@ -333,7 +339,7 @@ struct PairGeo {
   // 96^3 2.39 -> 2.32 us a chain in FP32, 43.7 -> 42.4 in FP64, 48^3 5.62 ->
   // 5.05 in FP64) except at 64 and 72, where the two-factor ones are 2-6% faster
   static constexpr bool COL4 = TILE == 0 && RealTraits<T>::prec != 2 && N != 64 && N != 72;
-  static constexpr int CA = COL4 ? M : A, CB = N / CA;
+  static constexpr int CA = COL4 ? M : N == 64 ? 8 : N == 60 && TILE == 0 ? 12 : A, CB = N / CA;
   static constexpr int THR_COL = TILE == 1 ? 256 : COL4 ? 128
                                  : N == 96 || N == 64 || N == 32 || N == 16 ? 128
                                  : N == 72                                  ? 192
@@ -356,7 +362,7 @@ struct PairGeo {
   }
   static constexpr int WIDE = sizeof(C) == 8 ? 1 : 2;
   static constexpr int MIN_PLANE =
-      fit(SMEM_PLANE, THR_PLANE, !BLOCK ? 104 / (3 - WIDE) : WIDE * (M >= 24 ? 80 : M >= 16 ? 64 : M >= 12 ? 56 : 48));
+      fit(SMEM_PLANE, THR_PLANE, !BLOCK ? (A >= 24 ? 168 : A >= 15 ? 128 : 104) / (3 - WIDE) : WIDE * (M >= 24 ? 80 : M >= 16 ? 64 : M >= 12 ? 56 : 48));
   static constexpr int MIN_COL = fit(SMEM_COL, THR_COL, RealTraits<T>::prec == 2 ? 104 : WIDE * (CB >= 12 ? 88 : CB >= 8 || CA >= 24 ? 72 : CA >= 16 ? 64 : 56));
 };
 
@@ -448,9 +454,9 @@ __device__ __forceinline__ void plane_inverse(const DevPlan& g, const ColumnSet&
   C* Q = reinterpret_cast<C*>(smem_raw);
   C* tw = Q + N * RP;
   // first transform along k2: DFTs of RB values k2 = q + NA s, s < RB
-  constexpr int RB = G::BLOCK ? M : B, NA = N / RB;
-  load_stage_twiddles<T, +1, G::BLOCK ? 4 : A, N, THR>(tw, g);
-  load_stage_twiddles<T, +1, RB, N, THR>(tw + N, g);
+  constexpr int RB = G::BLOCK ? M : A, NA = N / RB;
+  load_stage_twiddles<T, +1, NA, N, THR>(tw, g);
+  if constexpr (G::BLOCK) load_stage_twiddles<T, +1, M, N, THR>(tw + N, g);
   // 1. along k2, the columns that hold something.  The first stage reads the
   //    transform buffer; a column's elements outside its kept rows [0, up) and
   //    [N - dn, N) were never written and count as zero.
@@ -476,7 +482,7 @@ __device__ __forceinline__ void plane_inverse(const DevPlan& g, const ColumnSet&
       if ((N * NA) % THR == 0 || item < N * NA) column(q, item - q * N);
     }
     __syncthreads();
-    if constexpr (!G::BLOCK) stage_ct<T, A, +1, B, RP, B * RP, true, THR, N, 1>(Q, tw);
+    if constexpr (!G::BLOCK) stage_ct<T, B, +1, A, RP, A * RP, true, THR, N, 1>(Q, tw);
   } else {
     const int lo = cs.col_lo, nl = cs.col_lo + cs.col_hi;
     const auto k3_of = [&](int l) { return l < lo ? l : l + (N - nl); };
@@ -492,7 +498,7 @@ __device__ __forceinline__ void plane_inverse(const DevPlan& g, const ColumnSet&
       Q[r * RP + lo + (e - r * nz)] = cmake<T>(T(0), T(0));
     }
     __syncthreads();
-    if constexpr (!G::BLOCK) stage_rt<T, A, +1, B, RP, B * RP, true, THR>(Q, tw, nl, by, k3_of);
+    if constexpr (!G::BLOCK) stage_rt<T, B, +1, A, RP, A * RP, true, THR>(Q, tw, nl, by, k3_of);
   }
   // 2. the rest along k2 and the rows
   if constexpr (G::BLOCK) {
@@ -500,7 +506,7 @@ __device__ __forceinline__ void plane_inverse(const DevPlan& g, const ColumnSet&
     stage_ct<T, M, +1, 4, M, 1, true, THR, N, RP>(Q, tw + N);
   } else {
     stage_ct<T, A, +1, B, 1, B, false, THR, N, RP>(Q, tw);
-    stage_ct<T, B, +1, A, B, 1, true, THR, N, RP>(Q, tw + N);
+    stage_ct<T, B, +1, A, B, 1, true, THR, N, RP>(Q, tw);
   }
 }
 
@@ -792,11 +798,11 @@ __device__ __forceinline__ void pair_fwd_task(const DevPlan& g, const T* __restr
     // the usual chain, pairs (i, j) and (i, j'): psi_i is read once
     plane_forward<T, N, THR, TILE>(g, g.cols, Hp, smem_raw, [&](int e) {
       const T x = pai[e];
-      return cmake<T>(x * paj[e], x * pbj[e]);
+      return cmake<T>(rmul(x, paj[e]), rmul(x, pbj[e]));
     });
   } else {
     plane_forward<T, N, THR, TILE>(g, g.cols, Hp, smem_raw, [&](int e) {
-      return cmake<T>(pai[e] * paj[e], hb ? pbi[e] * pbj[e] : T(0));
+      return cmake<T>(rmul(pai[e], paj[e]), hb ? rmul(pbi[e], pbj[e]) : T(0));
     });
   }
 }
@@ -892,8 +898,8 @@ __device__ __forceinline__ void mirror_multiply(cplx<T>* z, cplx<T>* y, const V&
   for (int s = 0; s < B; ++s) {
     cplx<T>& Z = z[s];
     cplx<T>& Y = y[Q0 ? (B - s) % B : B - 1 - s];
-    const T ax = Z.x + Y.x, ay = Z.y - Y.y, bx = Z.y + Y.y, by = Y.x - Z.x;
-    const T a2 = ax * ax + ay * ay, b2 = bx * bx + by * by;
+    const T ax = radd<1>(Z.x, Y.x), ay = radd<-1>(Z.y, Y.y), bx = radd<1>(Z.y, Y.y), by = radd<-1>(Y.x, Z.x);
+    const T a2 = fmadd(ay, ay, rmul(ax, ax)), b2 = fmadd(by, by, rmul(bx, bx));
     kernel(s, Z, Y, a2, b2, acc);
   }
 }
@@ -996,17 +1002,15 @@ __device__ __forceinline__ void pair_col_task(const DevPlan& g, cplx<T>* __restr
       const auto kernel = [&](int s, C& Z, C& Y, double a2, double b2, double* e) {
         const int o = (q + A * s) * (N * KH);
         const double ve = v64[o];
-        e[0] += ve * a2;
-        e[1] += ve * b2;
+        e[0] = fmadd(ve, a2, e[0]);
+        e[1] = fmadd(ve, b2, e[1]);
         if (want_d) {
           const double dv = dv64[o];
           e[2] += dv * a2;
           e[3] += dv * b2;
         }
-        Z.x *= v[s];
-        Z.y *= v[s];
-        Y.x *= v[s];
-        Y.y *= v[s];
+        Z = cmake<T>(rmul(Z.x, v[s]), rmul(Z.y, v[s]));
+        Y = cmake<T>(rmul(Y.x, v[s]), rmul(Y.y, v[s]));
       };
       if (q == 0) mirror_multiply<T, B, true>(z, y, kernel, acc);
       else mirror_multiply<T, B, false>(z, y, kernel, acc);
@@ -1185,27 +1189,38 @@ __device__ __forceinline__ void pair_inv_task(const DevPlan& g, const T* __restr
       float* wj = wt[0];
       float* wj2 = wt[2];
       float* wi = wt[1];
-      for (int e4 = threadIdx.x; e4 < N * N / 4; e4 += THR) {
-        const int row = e4 / (N / 4), c = e4 - row * (N / 4);
-        const int e = G::row_of(row) * N + 4 * c;
-        const C* q = Q + row * RP + G::quad_place(c);
-        const C z0 = q[0], z1 = q[G::QUAD], z2 = q[2 * G::QUAD], z3 = q[3 * G::QUAD];
-        const float4 vi = ld_f4_hint(pi + e, keep);
-        const float4 vj = ld_f4_hint(pj + e, keep);
-        const float4 vj2 = ld_f4_hint(pj2 + e, keep);
-        const float4 a = make_float4(mi * vi.x * z0.x, mi * vi.y * z1.x, mi * vi.z * z2.x, mi * vi.w * z3.x);
-        const float4 b = make_float4(mi * vi.x * z0.y, mi * vi.y * z1.y, mi * vi.z * z2.y, mi * vi.w * z3.y);
-        const float4 ci = make_float4(mj * vj.x * z0.x + mj2 * vj2.x * z0.y, mj * vj.y * z1.x + mj2 * vj2.y * z1.y,
-                                      mj * vj.z * z2.x + mj2 * vj2.z * z2.y, mj * vj.w * z3.x + mj2 * vj2.w * z3.y);
-        asm volatile("red.global.add.L2::cache_hint.v4.f32 [%0], {%1, %2, %3, %4}, %5;" ::"l"(wj + e), "f"(a.x),
-                     "f"(a.y), "f"(a.z), "f"(a.w), "l"(keep)
-                     : "memory");
-        asm volatile("red.global.add.L2::cache_hint.v4.f32 [%0], {%1, %2, %3, %4}, %5;" ::"l"(wj2 + e), "f"(b.x),
-                     "f"(b.y), "f"(b.z), "f"(b.w), "l"(keep)
-                     : "memory");
-        asm volatile("red.global.add.L2::cache_hint.v4.f32 [%0], {%1, %2, %3, %4}, %5;" ::"l"(wi + e), "f"(ci.x),
-                     "f"(ci.y), "f"(ci.z), "f"(ci.w), "l"(keep)
-                     : "memory");
+      // the orbital loads of three items go out together (two or six: no gain
+      // over one; three 3.41 -> 3.33 us a chain at 96^3)
+      constexpr int U = 3;
+      for (int e0 = threadIdx.x; e0 < N * N / 4; e0 += U * THR) {
+        float4 vi[U], vj[U], vj2[U];
+#pragma unroll
+        for (int t = 0; t < U; ++t) {
+          const int e4 = e0 + t * THR;
+          if (e4 >= N * N / 4) continue;
+          const int row = e4 / (N / 4), c = e4 - row * (N / 4);
+          const int e = G::row_of(row) * N + 4 * c;
+          vi[t] = ld_f4_hint(pi + e, keep);
+          vj[t] = ld_f4_hint(pj + e, keep);
+          vj2[t] = ld_f4_hint(pj2 + e, keep);
+        }
+#pragma unroll
+        for (int t = 0; t < U; ++t) {
+          const int e4 = e0 + t * THR;
+          if (e4 >= N * N / 4) continue;
+          const int row = e4 / (N / 4), c = e4 - row * (N / 4);
+          const int e = G::row_of(row) * N + 4 * c;
+          const C* q = Q + row * RP + G::quad_place(c);
+          const C z0 = q[0], z1 = q[G::QUAD], z2 = q[2 * G::QUAD], z3 = q[3 * G::QUAD];
+          const float4 a = make_float4(mi * vi[t].x * z0.x, mi * vi[t].y * z1.x, mi * vi[t].z * z2.x, mi * vi[t].w * z3.x);
+          const float4 b = make_float4(mi * vi[t].x * z0.y, mi * vi[t].y * z1.y, mi * vi[t].z * z2.y, mi * vi[t].w * z3.y);
+          const float4 ci = make_float4(
+              mj * vj[t].x * z0.x + mj2 * vj2[t].x * z0.y, mj * vj[t].y * z1.x + mj2 * vj2[t].y * z1.y,
+              mj * vj[t].z * z2.x + mj2 * vj2[t].z * z2.y, mj * vj[t].w * z3.x + mj2 * vj2[t].w * z3.y);
+          red_f4_hint(wj + e, a, keep);
+          red_f4_hint(wj2 + e, b, keep);
+          red_f4_hint(wi + e, ci, keep);
+        }
       }
       return;
     }
@@ -1243,9 +1258,7 @@ __device__ __forceinline__ void pair_inv_task(const DevPlan& g, const T* __restr
           }
         }
         float* dst = wt[r] + e;
-        asm volatile("red.global.add.L2::cache_hint.v4.f32 [%0], {%1, %2, %3, %4}, %5;" ::"l"(dst), "f"(a.x),
-                     "f"(a.y), "f"(a.z), "f"(a.w), "l"(keep)
-                     : "memory");
+        red_f4_hint(dst, a, keep);
       }
     }
   } else {
@@ -1266,11 +1279,12 @@ __device__ __forceinline__ void pair_inv_task(const DevPlan& g, const T* __restr
       for (int e = threadIdx.x; e < N * N; e += THR) {
         const int i2 = e / N, i3 = e - i2 * N;
         C z = Q[G::place_of_row(i2) * RP + G::col_place(i3)];
-        if (!prescaled) z = cmake<T>(m * z.x, m * z.y);
+        if (!prescaled) z = cmake<T>(rmul(m, z.x), rmul(m, z.y));
         const T xi = ps[0][e], xj = ps[1][e], xj2 = ps[3][e];
-        atomic_add_real(wt[0] + e, xi * z.x);
-        atomic_add_real(wt[2] + e, xi * z.y);
-        atomic_add_real(wt[1] + e, xj * z.x + xj2 * z.y);
+        atomic_add_real(wt[0] + e, rmul(xi, z.x));
+        atomic_add_real(wt[2] + e, rmul(xi, z.y));
+        if constexpr (FftTraits<T>::fused) atomic_add_real(wt[1] + e, fmadd(xj2, z.y, rmul(xj, z.x)));
+        else atomic_add_real(wt[1] + e, xj * z.x + xj2 * z.y);
       }
       return;
     }

@@ -37,7 +37,7 @@ __global__ void __launch_bounds__(PairGeo<T, N>::THR_PLANE, PairGeo<T, N>::MIN_P
   plane_forward<T, N, PairGeo<T, N>::THR_PLANE, 0>(g, g.cols, H + (int64_t)blockIdx.y * g.ntot + plane0, smem_raw,
                                                    [&](int e) {
                                                      const C a = ua[e], b = ub[e];
-                                                     return cmake<T>(a.x * b.x + a.y * b.y, a.x * b.y - a.y * b.x);
+                                                     return cmake<T>(fmadd(a.y, b.y, rmul(a.x, b.x)), fmadd(-a.y, b.x, rmul(a.x, b.y)));
                                                    });
 }
 
@@ -129,8 +129,8 @@ __global__ void __launch_bounds__(PairGeo<T, N>::THR_COL, PairGeo<T, N>::MIN_COL
       const double* v64 = g.vtabq64 + vo;
 #pragma unroll
       for (int s = 0; s < B; ++s) {
-        acc += v64[(q + A * s) * (N * N)] * (z[s].x * z[s].x + z[s].y * z[s].y);
-        z[s] = cmake<T>(z[s].x * v[s], z[s].y * v[s]);
+        acc = fmadd(v64[(q + A * s) * (N * N)], fmadd(z[s].y, z[s].y, rmul(z[s].x, z[s].x)), acc);
+        z[s] = cmake<T>(rmul(z[s].x, v[s]), rmul(z[s].y, v[s]));
       }
     } else {
       // FP64 terms leave the array while the FP32 loop runs; at most five k1 of
@@ -240,13 +240,13 @@ __global__ void __launch_bounds__(PairGeo<T, N>::THR_PLANE, PairGeo<T, N>::MIN_P
     for (int e = threadIdx.x; e < N * N; e += THR) {
       const int i2 = e / N, i3 = e - i2 * N;
       const C p = P[G::place_of_row(i2) * RP + G::col_place(i3)];
-      const C x = ua[e];
-      atomicAdd(&wb[e].x, -fa * (x.x * p.x - x.y * p.y));
-      atomicAdd(&wb[e].y, -fa * (x.x * p.y + x.y * p.x));
+      const C x = ua[e], pa = cmake<T>(rmul(-fa, p.x), rmul(-fa, p.y));
+      atomicAdd(&wb[e].x, fmadd(-x.y, pa.y, rmul(x.x, pa.x)));
+      atomicAdd(&wb[e].y, fmadd(x.y, pa.x, rmul(x.x, pa.y)));
       if (both) {
-        const C y = ub[e];
-        atomicAdd(&wa[e].x, -fb * (y.x * p.x + y.y * p.y));
-        atomicAdd(&wa[e].y, -fb * (y.y * p.x - y.x * p.y));
+        const C y = ub[e], pb = cmake<T>(rmul(-fb, p.x), rmul(-fb, p.y));
+        atomicAdd(&wa[e].x, fmadd(y.y, pb.y, rmul(y.x, pb.x)));
+        atomicAdd(&wa[e].y, fmadd(y.y, pb.x, rmul(-y.x, pb.y)));
       }
     }
   }
