@@ -315,8 +315,10 @@ struct PairGeo {
   // against 1.05 us, 48^3 6.39 against 6.49, 96^3 even)
   static constexpr bool BLOCK = RealTraits<T>::prec == 1 && TILE == 0;
   static constexpr int M = N / 4;
-  // threads per line: an M-point item each, or whole two-factor items
-  static constexpr int TPL = TILE == 1 ? 8 : (!BLOCK && (N == 72 || N == 36) ? 3 : 4);
+  // threads per line: an M-point item each, or whole two-factor items; in
+  // double-float at 96, one CTA an SM, eight (four: 17.1 and 22.2 us a chain
+  // forward and inverse, eight: 16.8 and 20.3)
+  static constexpr int TPL = TILE == 1 ? 8 : (!BLOCK && (N == 72 || N == 36) ? 3 : RealTraits<T>::prec == 2 && N == 96 ? 8 : 4);
   static constexpr int THR_PLANE = (N * TPL + 31) / 32 * 32;
   // where a plane's passes leave frequency k of the columns and of the rows
   static __host__ __device__ constexpr int row_place(int k) {
@@ -362,7 +364,7 @@ struct PairGeo {
   }
   static constexpr int WIDE = sizeof(C) == 8 ? 1 : 2;
   static constexpr int MIN_PLANE =
-      fit(SMEM_PLANE, THR_PLANE, !BLOCK ? (A >= 24 ? 168 : A >= 15 ? 128 : 104) / (3 - WIDE) : WIDE * (M >= 24 ? 80 : M >= 16 ? 64 : M >= 12 ? 56 : 48));
+      fit(SMEM_PLANE, THR_PLANE, RealTraits<T>::prec == 2 ? 80 : !BLOCK ? (A >= 24 ? 168 : A >= 15 ? 128 : 104) / (3 - WIDE) : WIDE * (M >= 24 ? 80 : M >= 16 ? 64 : M >= 12 ? 56 : 48));
   static constexpr int MIN_COL = fit(SMEM_COL, THR_COL, RealTraits<T>::prec == 2 ? 104 : WIDE * (CB >= 12 ? 88 : CB >= 8 || CA >= 24 ? 72 : CA >= 16 ? 64 : 56));
 };
 
