@@ -189,8 +189,8 @@ cudaError_t launch_det_pair_sums(const double* part, int npairs, int ncta, doubl
 namespace {
 
 // Overlap tiles: TB x TB entries of S per CTA (16 x 16 threads, each
-// TB/16 x TB/16 entries 16 apart; TB = 64, or 32 for matrices of at most 32
-// rows), the sum over the real views of the rows split into chunks over
+// TB/16 x TB/16 entries 16 apart; TB = 64, 32 or 16, whichever pads the matrix
+// least), the sum over the real views of the rows split into chunks over
 // gridDim.y and reduced with FP64 atomics.
 constexpr int kOvK = 16, kOvThreads = 256;
 
@@ -364,8 +364,13 @@ __global__ void __launch_bounds__(kOvThreads)
 cudaError_t launch_overlap_sets(const double2* const* rows, const int* npw, int npw_max, int nsets, int nb,
                                 double* Sre, double* Sim, cudaStream_t s) {
   if (nsets < 1 || nb < 1) return cudaSuccess;
-  FOCK_OV_CHECK(cudaMemsetAsync(Sre, 0, sizeof(double) * (size_t)nsets * nb * nb, s));
-  FOCK_OV_CHECK(cudaMemsetAsync(Sim, 0, sizeof(double) * (size_t)nsets * nb * nb, s));
+  const size_t bytes = sizeof(double) * (size_t)nsets * nb * nb;
+  if (Sim == Sre + (size_t)nsets * nb * nb) {
+    FOCK_OV_CHECK(cudaMemsetAsync(Sre, 0, 2 * bytes, s));
+  } else {
+    FOCK_OV_CHECK(cudaMemsetAsync(Sre, 0, bytes, s));
+    FOCK_OV_CHECK(cudaMemsetAsync(Sim, 0, bytes, s));
+  }
   const int tj = (nb + 31) / 32, tiles = tj * (tj + 1) / 2;
   // chunks: two CTAs per SM over all sets, each chunk at least 4 k-blocks,
   // at most 64 chunks adding into one entry
@@ -393,7 +398,18 @@ cudaError_t overlap_impl(const double2* a, int na, const double2* b, int nbb, in
   if (na < 1 || nbb < 1) return cudaSuccess;
   const int64_t RS = 2 * (int64_t)npw;                        // the real view of a row
   const int64_t K = half != nullptr ? 2 * (int64_t)nhalf : RS;  // terms of the sum
-  const int TB = (na <= 32 && nbb <= 32) ? 32 : 64;
+  // The FP64 unit is the bound and computes the padding too: take the tile with
+  // the fewest entries (37 bands, upper triangle: 703 entries; 6 tiles of 16 hold
+  // 1,536, one of 64 holds 4,096: 20 us against 76 for the sphere of a 48^3 grid),
+  // a larger one where it costs at most an eighth more, for its fewer
+  // shared-memory reads and atomics.
+  const auto tile_count = [&](int tb) {
+    const int a_ = (na + tb - 1) / tb, b_ = (nbb + tb - 1) / tb;
+    return sym ? b_ * (b_ + 1) / 2 : a_ * b_;
+  };
+  int TB = 64;
+  for (int tb : {32, 16})
+    if (8LL * TB * TB * tile_count(TB) > 9LL * tb * tb * tile_count(tb)) TB = tb;
   const int ti = (na + TB - 1) / TB, tj = (nbb + TB - 1) / TB;
   const int tiles = sym ? tj * (tj + 1) / 2 : ti * tj;
   // chunks of the sum: at least two CTAs per SM (152 SMs) and among up to
@@ -426,7 +442,10 @@ cudaError_t overlap_impl(const double2* a, int na, const double2* b, int nbb, in
                                                                                                 sym ? 1 : 0, ld);
   const double* A = reinterpret_cast<const double*>(a);
   const double* B = reinterpret_cast<const double*>(b);
-  if (TB == 32)
+  if (TB == 16)
+    k_overlap<16><<<dim3(tiles, splits), kOvThreads, 0, s>>>(A, na, B, nbb, K, RS, half, sym ? 1 : 0, tj, kchunk,
+                                                            S, ld);
+  else if (TB == 32)
     k_overlap<32><<<dim3(tiles, splits), kOvThreads, 0, s>>>(A, na, B, nbb, K, RS, half, sym ? 1 : 0, tj, kchunk,
                                                             S, ld);
   else
@@ -439,7 +458,8 @@ cudaError_t overlap_impl(const double2* a, int na, const double2* b, int nbb, in
 cudaError_t launch_energy_reduce(const int2* pairs, int npairs, const double* occ,
                                  const double* epair, const double* dpair, double scale,
                                  double* out, cudaStream_t s) {
-  k_energy<<<1, 1024, 0, s>>>(pairs, npairs, occ, epair, dpair, scale, out);
+  const int threads = npairs >= 1024 ? 1024 : (npairs + 31) / 32 * 32;
+  k_energy<<<1, threads, 0, s>>>(pairs, npairs, occ, epair, dpair, scale, out);
   return cudaGetLastError();
 }
 

@@ -105,6 +105,15 @@ struct DevPlan {
   double vtab_f_factor;
 };
 
+// What a transform of the orbitals to real space clears on the way (any may be
+// NULL): the accumulators of the same bands, and n doubles at each of e and d.
+struct ClearOnWay {
+  void* w;
+  double* e;
+  double* d;
+  int n;
+};
+
 struct KernelOps {
   int real_bytes;  // sizeof of the working real type
   int prec;        // 0 FP64, 1 mixed FP32, 2 double-float (fock_precision)
@@ -114,7 +123,7 @@ struct KernelOps {
   cudaError_t (*configure)(const DevPlan&);
   // c(G) of bands [band0, band0 + nbat) to psi(r); X is scratch of >= ceil(nbat/2) grids.
   cudaError_t (*to_real)(const DevPlan&, const double2* psiG, int nb, int band0, int nbat, void* X,
-                         void* psi, cudaStream_t);
+                         void* psi, const ClearOnWay&, cudaStream_t);
   // Forward plane pass of the pair densities of `nch` chains into H.
   cudaError_t (*pair_fwd)(const DevPlan&, const void* psi, const Chain* ch, int nch, void* H,
                           cudaStream_t);
@@ -155,7 +164,7 @@ struct KOps {
   cudaError_t (*configure)();
   // orb, npw: the columns and the size of one k point's sphere
   cudaError_t (*to_real)(const DevPlan&, const ColumnSet& orb, const double2* psiG, int npw, int band0, int nbat,
-                         void* X, void* u, cudaStream_t);
+                         void* X, void* u, const ClearOnWay&, cudaStream_t);
   cudaError_t (*pair_fwd)(const DevPlan&, const void* u, const Chain* ch, int nch, void* H, cudaStream_t);
   cudaError_t (*pair_col)(const DevPlan&, void* H, const Chain* ch, int nch, double* epair, cudaStream_t);
   cudaError_t (*pair_inv)(const DevPlan&, const void* u, void* W, const void* occw, const Chain* ch, int nch,

@@ -318,7 +318,7 @@ struct PairGeo {
   // threads per line: an M-point item each, or whole two-factor items; in
   // double-float at 96, one CTA an SM, eight (four: 17.1 and 22.2 us a chain
   // forward and inverse, eight: 16.8 and 20.3)
-  static constexpr int TPL = TILE == 1 ? 8 : (!BLOCK && (N == 72 || N == 36) ? 3 : RealTraits<T>::prec == 2 && N == 96 ? 8 : 4);
+    static constexpr int TPL = TILE == 1 ? 8 : (!BLOCK && (N == 72 || N == 36) ? 3 : RealTraits<T>::prec == 2 && N == 96 ? 8 : 4);
   static constexpr int THR_PLANE = (N * TPL + 31) / 32 * 32;
   // where a plane's passes leave frequency k of the columns and of the rows
   static __host__ __device__ constexpr int row_place(int k) {
@@ -536,7 +536,7 @@ __device__ __forceinline__ C* line_ptr(C* H, const int* lines, int cta, int l) {
 template <class T, int N, bool KP>
 __global__ void __launch_bounds__(PairGeo<T, N>::THR_COL)
     k_orb_col_inv(DevPlan g, ColumnSet cs, const double2* __restrict__ psiG, int npw, int nb, int band0, int nbat,
-                  cplx<T>* __restrict__ X) {
+                  cplx<T>* __restrict__ X, ClearOnWay clr) {
   using C = cplx<T>;
   using G = PairGeo<T, N>;
   constexpr int A = G::CA, B = G::CB, NL = G::NL, NP = KP ? NL : G::NP, THR = G::THR_COL;
@@ -545,6 +545,10 @@ __global__ void __launch_bounds__(PairGeo<T, N>::THR_COL)
   C* tw = S + N * NL;
   load_stage_twiddles<T, +1, B, N, THR>(tw, g);
   const int q0 = blockIdx.y, cta = blockIdx.x;
+  for (int e = (q0 * gridDim.x + cta) * THR + threadIdx.x; e < clr.n; e += gridDim.x * gridDim.y * THR) {
+    if (clr.e != nullptr) clr.e[e] = 0.0;
+    if (clr.d != nullptr) clr.d[e] = 0.0;
+  }
   const int b0 = band0 + (KP ? q0 : 2 * q0);
   const bool has1 = !KP && (2 * q0 + 1 < nbat) && (b0 + 1 < nb);
   const double2* c0 = psiG + (int64_t)b0 * npw;
@@ -687,8 +691,8 @@ __global__ void __launch_bounds__(PairGeo<T, N>::THR_COL)
 // = z psi_scale, complex).
 template <class T, int N, bool KP>
 __global__ void __launch_bounds__(PairGeo<T, N>::THR_PLANE, PairGeo<T, N>::MIN_PLANE)
-    k_orb_plane_inv(DevPlan g, ColumnSet cs, const cplx<T>* __restrict__ X, void* __restrict__ psiv, int band0, int nb,
-                    int nbat) {
+    k_orb_plane_inv(DevPlan g, ColumnSet cs, const cplx<T>* __restrict__ X, void* __restrict__ psiv,
+                    void* __restrict__ wv, int band0, int nb, int nbat) {
   using C = cplx<T>;
   using G = PairGeo<T, N>;
   constexpr int THR = G::THR_PLANE, RP = G::RP;
@@ -703,12 +707,19 @@ __global__ void __launch_bounds__(PairGeo<T, N>::THR_PLANE, PairGeo<T, N>::MIN_P
   for (int e = threadIdx.x; e < N * N; e += THR) {
     const int i2 = e / N, i3 = e - i2 * N;
     const C z = Q[G::place_of_row(i2) * RP + G::col_place(i3)];
+    const int64_t at = (int64_t)b0 * g.ntot + plane0 + e;
     if constexpr (KP) {
-      static_cast<C*>(psiv)[(int64_t)b0 * g.ntot + plane0 + e] = cmake<T>(z.x * s, z.y * s);
+      static_cast<C*>(psiv)[at] = cmake<T>(z.x * s, z.y * s);
+      if (wv != nullptr) static_cast<C*>(wv)[at] = cmake<T>(T(0), T(0));
     } else {
-      T* psi = static_cast<T*>(psiv) + (int64_t)b0 * g.ntot + plane0 + e;
+      T* psi = static_cast<T*>(psiv) + at;
       *psi = z.x * s;
       if (has1) psi[g.ntot] = z.y * s;
+      if (wv != nullptr) {
+        acc_t<T>* w = static_cast<acc_t<T>*>(wv) + at;
+        *w = acc_t<T>(0);
+        if (has1) w[g.ntot] = acc_t<T>(0);
+      }
     }
   }
 }
@@ -1403,12 +1414,12 @@ struct Launch {
   static int row_place(int tile, int k2) { return tile == 1 ? P1::row_place(k2) : P0::row_place(k2); }
 
   static cudaError_t to_real(const DevPlan& g, const double2* psiG, int nb, int band0, int nbat,
-                             void* Xv, void* psiv, cudaStream_t s) {
+                             void* Xv, void* psiv, const ClearOnWay& clr, cudaStream_t s) {
     C* X = static_cast<C*>(Xv);
     const int nq = (nbat + 1) / 2;
     k_orb_col_inv<T, N, false><<<dim3(g.orb.ncta, nq), P0::THR_COL, P0::SMEM_COL, s>>>(g, g.orb, psiG, g.npw, nb, band0,
-                                                                                     nbat, X);
-    k_orb_plane_inv<T, N, false><<<dim3(N, nq), P0::THR_PLANE, P0::SMEM_PLANE, s>>>(g, g.orb, X, psiv, band0, nb,
+                                                                                     nbat, X, clr);
+    k_orb_plane_inv<T, N, false><<<dim3(N, nq), P0::THR_PLANE, P0::SMEM_PLANE, s>>>(g, g.orb, X, psiv, clr.w, band0, nb,
                                                                                     nbat);
     return cudaGetLastError();
   }
@@ -1419,7 +1430,7 @@ struct Launch {
       C* X = static_cast<C*>(Xv);
       const int nq = (nbat + 1) / 2;
       k_orb_col_inv<T, N, false><<<dim3(g.orb.ncta, nq), P0::THR_COL, P0::SMEM_COL, s>>>(g, g.orb, psiG, g.npw, nb,
-                                                                                       band0, nbat, X);
+                                                                                       band0, nbat, X, ClearOnWay{});
       k_orb_plane_vloc<T, N><<<dim3(N, nq), P0::THR_PLANE, P0::SMEM_PLANE, s>>>(g, g.orb, vloc, X);
       k_orb_col_fwd<T, N, false><<<dim3(g.orb.ncta, nq), P0::THR_COL, P0::SMEM_COL, s>>>(
           g, g.orb, X, g.inv_ntot, g.npw, nb, band0, nbat, out);

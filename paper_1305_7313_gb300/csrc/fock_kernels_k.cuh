@@ -272,10 +272,11 @@ struct LaunchK {
   }
 
   static cudaError_t to_real(const DevPlan& g, const ColumnSet& orb, const double2* psiG, int npw, int band0, int nbat,
-                             void* Xv, void* u, cudaStream_t s) {
+                             void* Xv, void* u, const ClearOnWay& clr, cudaStream_t s) {
     C* X = static_cast<C*>(Xv);
-    k_orb_col_inv<T, N, true><<<dim3(orb.ncta, nbat), G::THR_COL, G::SMEM_COL, s>>>(g, orb, psiG, npw, nbat, 0, nbat, X);
-    k_orb_plane_inv<T, N, true><<<dim3(N, nbat), G::THR_PLANE, G::SMEM_PLANE, s>>>(g, orb, X, u, band0, nbat, nbat);
+    k_orb_col_inv<T, N, true><<<dim3(orb.ncta, nbat), G::THR_COL, G::SMEM_COL, s>>>(g, orb, psiG, npw, nbat, 0, nbat, X, clr);
+    k_orb_plane_inv<T, N, true><<<dim3(N, nbat), G::THR_PLANE, G::SMEM_PLANE, s>>>(g, orb, X, u, clr.w, band0, nbat,
+                                                                                       nbat);
     return cudaGetLastError();
   }
 

@@ -70,8 +70,7 @@ struct fock_kplan {
   int2* d_pairs = nullptr;
   Chain* d_chains = nullptr;
   double* d_occw = nullptr;
-  void* d_occwT = nullptr;
-  double* d_result = nullptr;
+  std::vector<unsigned char> occ_stage;  // occupations, FP64 and FP32
   double* h_result = nullptr;
   int sched_ns = -1;
   int sched_nb = -1;
@@ -110,8 +109,7 @@ void kfree_ws(fock_kplan* p) {
   cudaFree(p->d_pairs);
   cudaFree(p->d_chains);
   cudaFree(p->d_occw);
-  cudaFree(p->d_occwT);
-  p->d_u = p->d_w = p->d_h = p->d_occwT = nullptr;
+  p->d_u = p->d_w = p->d_h = nullptr;
   p->d_epair = p->d_occw = nullptr;
   p->d_pairs = nullptr;
   p->d_chains = nullptr;
@@ -124,14 +122,12 @@ fock_status kensure(fock_kplan* p, int ns, int npairs) {
     cudaFree(p->d_u);
     cudaFree(p->d_w);
     cudaFree(p->d_occw);
-    cudaFree(p->d_occwT);
-    p->d_u = p->d_w = p->d_occwT = nullptr;
+    p->d_u = p->d_w = nullptr;
     p->d_occw = nullptr;
     p->ns_cap = 0;
     FOCK_KCUDA(p, cudaMalloc(&p->d_u, grid_bytes * ns));
     FOCK_KCUDA(p, cudaMalloc(&p->d_w, grid_bytes * ns));
-    FOCK_KCUDA(p, cudaMalloc((void**)&p->d_occw, sizeof(double) * ns));
-    FOCK_KCUDA(p, cudaMalloc(&p->d_occwT, (size_t)p->ops->real_bytes * ns));
+    FOCK_KCUDA(p, cudaMalloc((void**)&p->d_occw, 2 * sizeof(double) * ns));
     p->ns_cap = ns;
   }
   if (!p->d_h) FOCK_KCUDA(p, cudaMalloc(&p->d_h, grid_bytes * p->chain_batch));
@@ -353,8 +349,7 @@ fock_status fock_kplan_create(fock_kplan_t* out, const int grid[3], const double
         (e = cudaMemcpy(p->d_tw, tw32.data(), sizeof(float) * tw32.size(), cudaMemcpyHostToDevice)) != cudaSuccess)
       return bail(kcuda(p, e, "uploading tables"));
   }
-  if ((e = cudaMalloc((void**)&p->d_result, 4 * sizeof(double))) != cudaSuccess ||
-      (e = cudaMallocHost((void**)&p->h_result, 4 * sizeof(double))) != cudaSuccess)
+  if ((e = cudaMallocHost((void**)&p->h_result, 4 * sizeof(double))) != cudaSuccess)
     return bail(kcuda(p, e, "allocating results"));
 
   DevPlan& d = p->dp;
@@ -500,27 +495,28 @@ fock_status fock_kplan_apply(fock_kplan_t p, const void* const* psi_G, int nb, c
     p->sched_ns = ns;
     p->sched_nb = nb;
   }
-  // occupation times k weight, per state
-  std::vector<double> ow(ns);
+  // occupation times k weight, per state, in FP64 and in the working type, in one
+  // copy from the plan's own buffer; it is over before the next call may change it
+  const bool wide = p->ops->real_bytes == 8;
+  p->occ_stage.resize((size_t)ns * (wide ? 8 : 12));
+  double* ow = reinterpret_cast<double*>(p->occ_stage.data());
+  float* of = reinterpret_cast<float*>(p->occ_stage.data() + (size_t)ns * 8);
   for (int k = 0; k < nk; ++k)
-    for (int b = 0; b < nb; ++b) ow[(size_t)k * nb + b] = p->wk[k] * occ[(size_t)k * nb + b];
-  FOCK_KCUDA(p, cudaMemcpyAsync(p->d_occw, ow.data(), sizeof(double) * ns, cudaMemcpyHostToDevice, s));
-  if (p->ops->real_bytes == 8) {
-    FOCK_KCUDA(p, cudaMemcpyAsync(p->d_occwT, ow.data(), sizeof(double) * ns, cudaMemcpyHostToDevice, s));
-  } else {
-    std::vector<float> f(ow.begin(), ow.end());
-    FOCK_KCUDA(p, cudaMemcpyAsync(p->d_occwT, f.data(), sizeof(float) * ns, cudaMemcpyHostToDevice, s));
-  }
-  FOCK_KCUDA(p, cudaStreamSynchronize(s));  // the host vectors above are locals
-  const size_t grid_bytes = (size_t)p->dp.ntot * csz(p);
-  FOCK_KCUDA(p, cudaMemsetAsync(p->d_w, 0, grid_bytes * ns, s));
-  FOCK_KCUDA(p, cudaMemsetAsync(p->d_epair, 0, sizeof(double) * npairs, s));
+    for (int b = 0; b < nb; ++b) {
+      const size_t i = (size_t)k * nb + b;
+      ow[i] = p->wk[k] * occ[i];
+      if (!wide) of[i] = (float)ow[i];
+    }
+  FOCK_KCUDA(p, cudaMemcpyAsync(p->d_occw, p->occ_stage.data(), p->occ_stage.size(), cudaMemcpyHostToDevice, s));
+  if (!ex) FOCK_KCUDA(p, cudaStreamSynchronize(s));  // else at the end
+  const void* occwT = wide ? (const void*)p->d_occw : (const void*)(p->d_occw + ns);
   const int nbat = p->chain_batch;  // bands per O(nb) launch: the transform buffer holds chain_batch grids
   for (int k = 0; k < nk; ++k)
     for (int b0 = 0; b0 < nb; b0 += nbat) {
       const int cnt = std::min(nbat, nb - b0);
       const double2* src = static_cast<const double2*>(psi_G[k]) + (size_t)b0 * p->npw[k];
-      FOCK_KCUDA(p, p->kops->to_real(p->dp, p->orb[k], src, p->npw[k], k * nb + b0, cnt, p->d_h, p->d_u, s));
+      const fockx::ClearOnWay clr{p->d_w, p->d_epair, nullptr, k == 0 && b0 == 0 ? npairs : 0};
+      FOCK_KCUDA(p, p->kops->to_real(p->dp, p->orb[k], src, p->npw[k], k * nb + b0, cnt, p->d_h, p->d_u, clr, s));
     }
   DevPlan dp = p->dp;
   if (p->ops->real_bytes == 4 && dp.q0 >= 0) {
@@ -550,7 +546,7 @@ fock_status fock_kplan_apply(fock_kplan_t p, const void* const* psi_G, int nb, c
     const Chain* ch = p->d_chains + c;
     FOCK_KCUDA(p, p->kops->pair_fwd(dp, p->d_u, ch, cnt, p->d_h, s));
     FOCK_KCUDA(p, p->kops->pair_col(dp, p->d_h, ch, cnt, p->d_epair, s));
-    FOCK_KCUDA(p, p->kops->pair_inv(dp, p->d_u, p->d_w, p->d_occwT, ch, cnt, p->d_h, s));
+    FOCK_KCUDA(p, p->kops->pair_inv(dp, p->d_u, p->d_w, occwT, ch, cnt, p->d_h, s));
   }
   for (int k = 0; k < nk; ++k)
     for (int b0 = 0; b0 < nb; b0 += nbat) {
@@ -560,9 +556,8 @@ fock_status fock_kplan_apply(fock_kplan_t p, const void* const* psi_G, int nb, c
     }
   const double scale = -0.5 * p->vol / ((double)p->dp.ntot * (double)p->dp.ntot);
   FOCK_KCUDA(p, fockx::launch_energy_reduce(p->d_pairs, npairs, p->d_occw, p->d_epair, nullptr, scale,
-                                            p->d_result, s));
+                                            p->h_result, s));  // pinned, written by the kernel
   if (ex) {
-    FOCK_KCUDA(p, cudaMemcpyAsync(p->h_result, p->d_result, 2 * sizeof(double), cudaMemcpyDeviceToHost, s));
     FOCK_KCUDA(p, cudaStreamSynchronize(s));
     *ex = p->h_result[0];
   }
@@ -583,7 +578,6 @@ fock_status fock_kplan_destroy(fock_kplan_t p) {
   cudaFree(p->d_krows);
   cudaFree(p->d_knpw);
   cudaFree(p->d_tw);
-  cudaFree(p->d_result);
   if (p->h_result) cudaFreeHost(p->h_result);
   delete p;
   return FOCK_OK;

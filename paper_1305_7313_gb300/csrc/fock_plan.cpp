@@ -54,11 +54,11 @@ struct Workspace {
   size_t h_bytes = 0;
   int npair_cap = 0;
   double* epair = nullptr;
-  double* dpair = nullptr;
+  double* dpair = nullptr;  // inside epair's allocation
   int2* pairs = nullptr;
   Chain* chains = nullptr;
   double* occ = nullptr;
-  void* occT = nullptr;
+  void* occT = nullptr;  // in the working type; inside occ's allocation (FP64: occ itself)
 };
 
 }  // namespace
@@ -117,7 +117,6 @@ struct fock_plan {
   double2* d_cocc = nullptr;
   int64_t cocc_cap = 0;
   int64_t kept_columns = 0;  // lines of the column map (both pairs)
-  double* d_result = nullptr;
   double* h_result = nullptr;  // pinned
   int64_t table_bytes = 0;
   Workspace ws;
@@ -126,6 +125,7 @@ struct fock_plan {
   std::vector<int2> pairs;
   std::vector<Chain> chains;
   std::vector<double> occ_host;
+  std::vector<float> occ_stage;  // in the working type
   // fixed operator (fock_set_occupied): the first fixed_nb bands of the
   // real-space workspace hold the occupied orbitals that define V_x
   int fixed_nb = 0;
@@ -177,11 +177,9 @@ void free_ws(Workspace& w) {
   cudaFree(w.h);
   for (void* x : w.hx) cudaFree(x);
   cudaFree(w.epair);
-  cudaFree(w.dpair);
   cudaFree(w.pairs);
   cudaFree(w.chains);
   cudaFree(w.occ);
-  cudaFree(w.occT);
   w = Workspace{};
 }
 
@@ -305,15 +303,14 @@ fock_status ensure_workspace(fock_plan* p, int nb, int npairs) {
     cudaFree(w.psi);
     cudaFree(w.w);
     cudaFree(w.occ);
-    cudaFree(w.occT);
     w.psi = w.w = w.occT = nullptr;
     w.occ = nullptr;
     w.nb_cap = 0;
     w.psi_bytes = (size_t)nb * (size_t)p->dp.ntot * rb;
     FOCK_CUDA(p, dev_alloc(&w.psi, w.psi_bytes));
     FOCK_CUDA(p, dev_alloc(&w.w, w.psi_bytes));
-    FOCK_CUDA(p, dev_alloc(&w.occ, sizeof(double) * nb));
-    FOCK_CUDA(p, dev_alloc(&w.occT, rb * nb));
+    FOCK_CUDA(p, dev_alloc(&w.occ, (sizeof(double) + rb) * nb));
+    w.occT = p->prec == FOCK_PREC_FP64 ? w.occ : w.occ + nb;
     w.nb_cap = nb;
   }
   if (w.h == nullptr) {
@@ -323,7 +320,6 @@ fock_status ensure_workspace(fock_plan* p, int nb, int npairs) {
   }
   if (npairs > w.npair_cap) {
     cudaFree(w.epair);
-    cudaFree(w.dpair);
     cudaFree(w.pairs);
     cudaFree(w.chains);
     w.epair = w.dpair = nullptr;
@@ -332,8 +328,8 @@ fock_status ensure_workspace(fock_plan* p, int nb, int npairs) {
     w.npair_cap = 0;
     p->sched_nb = -1;
     p->fixed_sched_nt = -1;
-    FOCK_CUDA(p, dev_alloc(&w.epair, sizeof(double) * npairs));
-    FOCK_CUDA(p, dev_alloc(&w.dpair, sizeof(double) * npairs));
+    FOCK_CUDA(p, dev_alloc(&w.epair, 2 * sizeof(double) * npairs));
+    w.dpair = w.epair + npairs;
     FOCK_CUDA(p, dev_alloc(&w.pairs, sizeof(int2) * npairs));
     FOCK_CUDA(p, dev_alloc(&w.chains, sizeof(Chain) * ((npairs + 1) / 2)));
     w.npair_cap = npairs;
@@ -348,57 +344,59 @@ fock_status grow_keeping(fock_plan* p, int nb, int keep) {
   if (nb <= w.nb_cap) return FOCK_OK;
   const size_t rb = (size_t)p->ops->real_bytes;
   const size_t bytes = (size_t)nb * (size_t)p->dp.ntot * rb;
-  void *psi = nullptr, *wacc = nullptr, *occT = nullptr;
+  void *psi = nullptr, *wacc = nullptr;
   double* occ = nullptr;
   cudaError_t e;
   if ((e = dev_alloc(&psi, bytes)) != cudaSuccess || (e = dev_alloc(&wacc, bytes)) != cudaSuccess ||
-      (e = dev_alloc(&occ, sizeof(double) * nb)) != cudaSuccess || (e = dev_alloc(&occT, rb * nb)) != cudaSuccess) {
+      (e = dev_alloc(&occ, (sizeof(double) + rb) * nb)) != cudaSuccess) {
     cudaFree(psi);
     cudaFree(wacc);
     cudaFree(occ);
-    cudaFree(occT);
     return cuda_fail(p, e, "growing the workspace");
   }
   if (keep > 0 && w.psi) {
     e = cudaMemcpy(psi, w.psi, (size_t)keep * (size_t)p->dp.ntot * rb, cudaMemcpyDeviceToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(occ, w.occ, sizeof(double) * keep, cudaMemcpyDeviceToDevice);
-    if (e == cudaSuccess) e = cudaMemcpy(occT, w.occT, rb * keep, cudaMemcpyDeviceToDevice);
+    if (e == cudaSuccess && p->prec != FOCK_PREC_FP64)
+      e = cudaMemcpy(occ + nb, w.occT, rb * keep, cudaMemcpyDeviceToDevice);
     if (e != cudaSuccess) {
       cudaFree(psi);
       cudaFree(wacc);
       cudaFree(occ);
-      cudaFree(occT);
       return cuda_fail(p, e, "copying the occupied orbitals");
     }
   }
   cudaFree(w.psi);
   cudaFree(w.w);
   cudaFree(w.occ);
-  cudaFree(w.occT);
   w.psi = psi;
   w.w = wacc;
   w.occ = occ;
-  w.occT = occT;
+  w.occT = p->prec == FOCK_PREC_FP64 ? occ : occ + nb;
   w.psi_bytes = bytes;
   w.nb_cap = nb;
   return FOCK_OK;
 }
 
-fock_status upload_occ(fock_plan* p, const double* occ, int nb, cudaStream_t s) {
+// Occupations to the device, in FP64 and in the working type.  The copies from the
+// plan's own buffers are over before the next call may change them: `synced` says
+// that the caller synchronises the stream before it returns, otherwise it is done
+// here.
+fock_status upload_occ(fock_plan* p, const double* occ, int nb, bool synced, cudaStream_t s) {
   p->occ_host.assign(occ, occ + nb);
-  FOCK_CUDA(p, cudaMemcpyAsync(p->ws.occ, occ, sizeof(double) * nb, cudaMemcpyHostToDevice, s));
-  if (p->prec == FOCK_PREC_FP64) {
-    FOCK_CUDA(p, cudaMemcpyAsync(p->ws.occT, occ, sizeof(double) * nb, cudaMemcpyHostToDevice, s));
-  } else if (p->prec == FOCK_PREC_DF64) {
-    std::vector<float> f(2 * (size_t)nb);
-    for (int k = 0; k < nb; ++k) split_df64(occ[k], &f[2 * k]);
-    FOCK_CUDA(p, cudaMemcpyAsync(p->ws.occT, f.data(), sizeof(float) * f.size(), cudaMemcpyHostToDevice, s));
-    FOCK_CUDA(p, cudaStreamSynchronize(s));  // f is a local buffer
-  } else {
-    std::vector<float> f(occ, occ + nb);
-    FOCK_CUDA(p, cudaMemcpyAsync(p->ws.occT, f.data(), sizeof(float) * nb, cudaMemcpyHostToDevice, s));
-    FOCK_CUDA(p, cudaStreamSynchronize(s));  // f is a local buffer
+  const bool wide = p->prec == FOCK_PREC_FP64;  // ws.occT is ws.occ
+  FOCK_CUDA(p, cudaMemcpyAsync(p->ws.occ, wide ? occ : p->occ_host.data(), sizeof(double) * nb,
+                               cudaMemcpyHostToDevice, s));
+  if (wide) return FOCK_OK;
+  const bool df = p->prec == FOCK_PREC_DF64;
+  p->occ_stage.resize((size_t)nb * (df ? 2 : 1));
+  for (int k = 0; k < nb; ++k) {
+    if (df) split_df64(occ[k], &p->occ_stage[2 * k]);
+    else p->occ_stage[k] = (float)occ[k];
   }
+  FOCK_CUDA(p, cudaMemcpyAsync(p->ws.occT, p->occ_stage.data(), sizeof(float) * p->occ_stage.size(),
+                               cudaMemcpyHostToDevice, s));
+  if (!synced) FOCK_CUDA(p, cudaStreamSynchronize(s));
   return FOCK_OK;
 }
 
@@ -460,14 +458,16 @@ int bands_per_grid_batch(const fock_plan* p) {
   return 2 * q;
 }
 
-fock_status orbitals_to_real(fock_plan* p, const void* psiG, int nb, cudaStream_t s) {
+fock_status orbitals_to_real(fock_plan* p, const void* psiG, int nb, const fockx::ClearOnWay& clear, cudaStream_t s) {
   const int nbat = bands_per_grid_batch(p);
   p->stats.band_batch = nbat;
   for (int b0 = 0; b0 < nb; b0 += nbat) {
     const int cnt = std::min(nbat, nb - b0);
     PhaseScope ps(p, FOCK_PHASE_TO_REAL, 2, s);
+    fockx::ClearOnWay c = clear;
+    if (b0 > 0) c.n = 0;
     FOCK_CUDA(p, p->ops->to_real(p->dp, static_cast<const double2*>(psiG), nb, b0, cnt, p->ws.h,
-                                 p->ws.psi, s));
+                                 p->ws.psi, c, s));
   }
   return FOCK_OK;
 }
@@ -555,13 +555,9 @@ fock_status apply_impl(fock_plan* p, const void* psiG, int nb, const double* occ
     FOCK_CUDA(p, cudaStreamSynchronize(s));  // the host vectors may change on the next call
     p->sched_nb = nb;
   }
-  st = upload_occ(p, occ, nb, s);
+  st = upload_occ(p, occ, nb, ex || dex, s);
   if (st != FOCK_OK) return st;
-  const size_t rb = (size_t)p->ops->real_bytes;
-  FOCK_CUDA(p, cudaMemsetAsync(p->ws.w, 0, (size_t)nb * (size_t)p->dp.ntot * rb, s));
-  FOCK_CUDA(p, cudaMemsetAsync(p->ws.epair, 0, sizeof(double) * npairs, s));
-  FOCK_CUDA(p, cudaMemsetAsync(p->ws.dpair, 0, sizeof(double) * npairs, s));
-  st = orbitals_to_real(p, psiG, nb, s);
+  st = orbitals_to_real(p, psiG, nb, fockx::ClearOnWay{p->ws.w, p->ws.epair, p->ws.dpair, npairs}, s);
   if (st != FOCK_OK) return st;
 
   DevPlan dp = p->dp;
@@ -646,13 +642,11 @@ fock_status apply_impl(fock_plan* p, const void* psiG, int nb, const double* occ
     FOCK_CUDA(p, fockx::launch_energy_reduce(p->ws.pairs + p0, p1 - p0, p->ws.occ,
                                              p->ws.epair + p0,
                                              dp.dvtab64 ? p->ws.dpair + p0 : nullptr, scale,
-                                             p->d_result, s));
+                                             p->h_result, s));  // pinned, written by the kernel
   }
   st = collect_timing(p, s);
   if (st != FOCK_OK) return st;
   if (ex || dex) {
-    FOCK_CUDA(p, cudaMemcpyAsync(p->h_result, p->d_result, 2 * sizeof(double),
-                                 cudaMemcpyDeviceToHost, s));
     FOCK_CUDA(p, cudaStreamSynchronize(s));
     if (ex) *ex = p->h_result[0];
     if (dex) *dex = p->h_result[1];
@@ -929,7 +923,6 @@ fock_status fock_plan_create(fock_plan_t* out, const int grid[3], const double c
     const std::vector<double> w = twiddles(n_grid);
     ok = ok && upload(&p->d_tw_full, w.data(), sizeof(double) * w.size());
   }
-  if (ok) ok = upload((void**)&p->d_result, std::vector<double>(4, 0.0).data(), 4 * sizeof(double));
   if (ok) {
     cudaError_t e = cudaMallocHost((void**)&p->h_result, 4 * sizeof(double));
     if (e != cudaSuccess) {
@@ -1346,9 +1339,9 @@ fock_status fock_set_occupied(fock_plan_t plan, const void* psi_G, int nb, const
   plan->fixed_nb = 0;
   st = ensure_workspace(plan, nb, 1);
   if (st != FOCK_OK) return st;
-  st = upload_occ(plan, occ, nb, s);
+  st = upload_occ(plan, occ, nb, false, s);
   if (st != FOCK_OK) return st;
-  st = orbitals_to_real(plan, psi_G, nb, s);
+  st = orbitals_to_real(plan, psi_G, nb, fockx::ClearOnWay{}, s);
   if (st != FOCK_OK) return st;
   if (plan->ops->prec == 1) {
     // the coefficients of the occupied set, for the FP64 overlaps of the
@@ -1412,13 +1405,12 @@ fock_status fock_apply_fixed(fock_plan_t plan, const void* phi_G, int nt, void* 
   const size_t off = (size_t)nb * (size_t)p->dp.ntot * rb;
   char* psi_trial = static_cast<char*>(p->ws.psi) + off;
   char* w_trial = static_cast<char*>(p->ws.w) + off;
-  FOCK_CUDA(p, cudaMemsetAsync(w_trial, 0, (size_t)nt * (size_t)p->dp.ntot * rb, s));
   const int nbat = bands_per_grid_batch(p);
   p->stats.band_batch = nbat;
   for (int b0 = 0; b0 < nt; b0 += nbat) {
     PhaseScope ps(p, FOCK_PHASE_TO_REAL, 2, s);
     FOCK_CUDA(p, p->ops->to_real(p->dp, static_cast<const double2*>(phi_G), nt, b0, std::min(nbat, nt - b0),
-                                 p->ws.h, psi_trial, s));
+                                 p->ws.h, psi_trial, fockx::ClearOnWay{w_trial, nullptr, nullptr, 0}, s));
   }
   DevPlan dp = p->dp;
   dp.dvtab64 = nullptr;
@@ -1488,9 +1480,7 @@ fock_status fock_pair_energies(fock_plan_t plan, const void* psi_G, int nb, cons
   stats_reset(plan);
   FOCK_CUDA(plan, cudaMemcpyAsync(plan->ws.chains, chains.data(), sizeof(Chain) * chains.size(),
                                   cudaMemcpyHostToDevice, s));
-  FOCK_CUDA(plan, cudaMemsetAsync(plan->ws.epair, 0, sizeof(double) * npairs, s));
-  FOCK_CUDA(plan, cudaMemsetAsync(plan->ws.dpair, 0, sizeof(double) * npairs, s));
-  st = orbitals_to_real(plan, psi_G, nb, s);
+  st = orbitals_to_real(plan, psi_G, nb, fockx::ClearOnWay{nullptr, plan->ws.epair, plan->ws.dpair, npairs}, s);
   if (st != FOCK_OK) return st;
   const int nch = (int)chains.size();
   for (int c = 0; c < nch; c += plan->chain_batch) {
@@ -1552,7 +1542,6 @@ fock_status fock_destroy(fock_plan_t plan) {
   cudaFree(plan->d_cocc);
   cudaFree(plan->d_vtab_f);
   cudaFree(plan->d_st);
-  cudaFree(plan->d_result);
   if (plan->h_result) cudaFreeHost(plan->h_result);
   delete plan;
   return FOCK_OK;
@@ -1639,14 +1628,11 @@ fock_status batch_enqueue(fock_batch* b, cudaStream_t s) {
     fock_plan* p = b->plans[k];
     const int nb = b->nb[k];
     const int npairs = nb * (nb + 1) / 2;
-    const size_t rb = (size_t)p->ops->real_bytes;
-    FOCK_BCUDA(b, cudaMemsetAsync(p->ws.w, 0, (size_t)nb * (size_t)p->dp.ntot * rb, s));
-    FOCK_BCUDA(b, cudaMemsetAsync(p->ws.epair, 0, sizeof(double) * npairs, s));
-    FOCK_BCUDA(b, cudaMemsetAsync(p->ws.dpair, 0, sizeof(double) * npairs, s));
     const int nbat = bands_per_grid_batch(p);
     for (int b0 = 0; b0 < nb; b0 += nbat) {
       FOCK_BCUDA(b, p->ops->to_real(p->dp, static_cast<const double2*>(b->psi[k]), nb, b0,
-                                    std::min(nbat, nb - b0), p->ws.h, p->ws.psi, s));
+                                    std::min(nbat, nb - b0), p->ws.h, p->ws.psi,
+                                    fockx::ClearOnWay{p->ws.w, p->ws.epair, p->ws.dpair, b0 == 0 ? npairs : 0}, s));
       b->launches += 2;
     }
     if (p->ops->prec == 1) {
@@ -1821,7 +1807,7 @@ fock_status fock_batch_create(fock_batch_t* out, int nsys, const fock_plan_t* pl
                              cudaMemcpyHostToDevice, b->cap_stream)) != cudaSuccess)
       return fail_create(bcuda(b, e, "uploading a schedule"));
     p->sched_nb = nb[k];
-    st = upload_occ(p, occ[k], nb[k], b->cap_stream);
+    st = upload_occ(p, occ[k], nb[k], false, b->cap_stream);
     if (st != FOCK_OK) return fail_create(bfail(b, st, p->err));
     if ((e = cudaStreamSynchronize(b->cap_stream)) != cudaSuccess) return fail_create(bcuda(b, e, "sync"));
     nmax = std::max(nmax, p->n);

@@ -186,7 +186,7 @@ extern "C" fock_status fock_pair_energies_static(fock_plan_t plan, const void* p
   if ((err = cudaMemsetAsync(dp, 0, sizeof(double) * (size_t)npairs, s)) != cudaSuccess) return cuda_fail(plan, err);
   // orbitals to real space one band pair at a time (one grid of the transform buffer)
   for (int b0 = 0; b0 < nb; b0 += 2) {
-    err = v.ops->to_real(g, static_cast<const double2*>(psi_G), nb, b0, std::min(2, nb - b0), hbuf, psi, s);
+    err = v.ops->to_real(g, static_cast<const double2*>(psi_G), nb, b0, std::min(2, nb - b0), hbuf, psi, fockx::ClearOnWay{}, s);
     if (err != cudaSuccess) return cuda_fail(plan, err);
   }
   for (int c = 0; c < nch; c += cb) {
