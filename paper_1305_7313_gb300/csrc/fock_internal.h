@@ -243,8 +243,10 @@ cudaError_t launch_det_to_double(void* w, int64_t n, const double* scale, cudaSt
 cudaError_t launch_det_pair_sums(const double* part, int npairs, int ncta, double* out, cudaStream_t s);
 
 // Sternheimer CG (fock_sternheimer.cu): kets are complex128 [m][npw], FP64.
-// part buffers: partial sums, at most st_chunks(npw) a band; c: [m][nocc].
+// part buffers: partial sums, at most st_chunks(npw) a band; c:
+// [st_proj_parts()][m][nocc]; rr_host: pinned [m], the new <r|r>.
 int st_chunks(int npw);
+int st_proj_parts();
 cudaError_t st_proj_coef(const double2* u, int nocc, const double2* x, int m, int npw, double* c, cudaStream_t s);
 // b = -Q w, rr[n] = <b_n|b_n>
 cudaError_t st_rhs(const double2* w, const double2* u, const double* c, int nocc, int m, int npw, double2* b,
@@ -254,7 +256,7 @@ cudaError_t st_finish(double2* ap, const double2* p, const double* kin, const do
 cudaError_t st_step(double2* x, double2* r, const double2* p, const double2* ap, const double* rr,
                     const double* part_pap, int m, int npw, double* part_rr, cudaStream_t s);
 cudaError_t st_dir(double2* p, const double2* r, const double* part_rr, const double* rr, int m, int npw,
-                   double* rr_new, cudaStream_t s);
+                   double* rr_new, double* rr_host, cudaStream_t s);
 cudaError_t st_gather_rows(const double2* src, double2* dst, const int* perm, int m, int npw, cudaStream_t s);
 cudaError_t st_gather_scalars(const double* src, double* dst, const int* perm, int m, cudaStream_t s);
 

@@ -111,6 +111,8 @@ struct fock_plan {
   // arrays of the Sternheimer solves
   void* d_st = nullptr;
   size_t st_cap = 0;
+  double* h_st = nullptr;  // pinned residual norms
+  int h_st_cap = 0;
   // FP64: the kernel table scaled by -f0 (DevPlan::vtab_f)
   void* d_vtab_f = nullptr;
   double vtab_f_f0 = 0.0;
@@ -1137,7 +1139,7 @@ fock_status fock_sternheimer_solve(fock_plan_t p, const double* vloc, const void
     const size_t own = p->n == p->dp.n ? 0 : std::min<size_t>(((size_t)nrhs + 1) / 2, 32);
     nbat = p->n == p->dp.n ? bands_per_grid_batch(p) : 2 * (int)own;
     const size_t bytes[] = {own * grid_bytes, kb, kb, kb, kb, kb, sizeof(double) * npw, nb8,
-                            nb8 * nocc, nb8, nb8,
+                            nb8 * nocc * (size_t)fockx::st_proj_parts(), nb8, nb8,
                             nb8 * (size_t)fockx::st_chunks((int)npw), nb8 * (size_t)fockx::st_chunks((int)npw), nb8,
                             sizeof(int) * (size_t)nrhs};
     void** const ptrs[] = {&xgrid, (void**)&x, (void**)&r, (void**)&pk, (void**)&ap, (void**)&tmp, (void**)&kin,
@@ -1151,6 +1153,13 @@ fock_status fock_sternheimer_solve(fock_plan_t p, const double* vloc, const void
       p->st_cap = 0;
       FOCK_CUDA(p, dev_alloc(&p->d_st, total));
       p->st_cap = total;
+    }
+    if (nrhs > p->h_st_cap) {
+      if (p->h_st) cudaFreeHost(p->h_st);
+      p->h_st = nullptr;
+      p->h_st_cap = 0;
+      FOCK_CUDA(p, cudaMallocHost((void**)&p->h_st, nb8));
+      p->h_st_cap = nrhs;
     }
     char* at = static_cast<char*>(p->d_st);
     for (size_t k = 0; k < sizeof(bytes) / sizeof(bytes[0]); ++k) {
@@ -1186,10 +1195,10 @@ fock_status fock_sternheimer_solve(fock_plan_t p, const double* vloc, const void
     FOCK_CUDA(p, fockx::st_proj_coef(u, nocc, pk, m, ip, c, s));
     FOCK_CUDA(p, fockx::st_finish(ap, pk, kin, d_eps, u, c, nocc, alpha, m, ip, part_a, s));
     FOCK_CUDA(p, fockx::st_step(x, r, pk, ap, rr, part_a, m, ip, part_b, s));
-    FOCK_CUDA(p, fockx::st_dir(pk, r, part_b, rr, m, ip, rrn, s));
+    FOCK_CUDA(p, fockx::st_dir(pk, r, part_b, rr, m, ip, rrn, p->h_st, s));
     std::swap(rr, rrn);
-    FOCK_CUDA(p, cudaMemcpyAsync(rr_h.data(), rr, sizeof(double) * m, cudaMemcpyDeviceToHost, s));
     FOCK_CUDA(p, cudaStreamSynchronize(s));
+    std::copy(p->h_st, p->h_st + m, rr_h.begin());
     for (int k = 0; k < m; ++k) {
       ++it_h[order[k]];
       rr_last[order[k]] = rr_h[k];
@@ -1542,6 +1551,7 @@ fock_status fock_destroy(fock_plan_t plan) {
   cudaFree(plan->d_cocc);
   cudaFree(plan->d_vtab_f);
   cudaFree(plan->d_st);
+  if (plan->h_st) cudaFreeHost(plan->h_st);
   if (plan->h_result) cudaFreeHost(plan->h_result);
   delete plan;
   return FOCK_OK;

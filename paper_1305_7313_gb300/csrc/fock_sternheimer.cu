@@ -46,17 +46,19 @@ __device__ double sum_partials(const double* __restrict__ part, int n) {
   return total;
 }
 
-// Projector coefficients c[n nocc + i] = Re sum_G conj(u_i(G)) x_n(G): a CTA
-// takes 2 x 2 of them, so a row read serves two sums and the loads of four
-// coefficients are in flight together.  (Larger tiles leave too few warps to hide
-// the reads and spend the FP64 pipe on the reductions of their sums: 4 x 4 took
-// 30 to 63 us on average where one CTA per coefficient took 26.)
-constexpr int kProjTile = 2;
+// Projector coefficients Re sum_G conj(u_i(G)) x_n(G): a CTA takes 2 x 2 of them
+// over 1 / kProjParts of the sphere, c[(part m + n) nocc + i] its share, so a row
+// read serves two sums and enough CTAs run to hide the reads.  (Larger tiles leave
+// too few warps and spend the FP64 unit on the reductions of their sums: 4 x 4
+// took 30 to 63 us on average where one CTA per coefficient took 26.)
+constexpr int kProjTile = 2, kProjParts = 2;
 __global__ void __launch_bounds__(kThreads)
     k_proj_coef(const double2* __restrict__ u, int nocc, const double2* __restrict__ x, int m, int npw,
                 double* __restrict__ c) {
   constexpr int TL = kProjTile;
-  const int i0 = blockIdx.x * TL, n0 = blockIdx.y * TL;
+  const int i0 = blockIdx.x * TL, n0 = blockIdx.y * TL, part = blockIdx.z;
+  const int len = (npw + kProjParts - 1) / kProjParts;
+  const int g1 = (part + 1) * len < npw ? (part + 1) * len : npw;
   // rows past the end repeat the last one; their sums are not stored
   const double2 *a[TL], *b[TL];
 #pragma unroll
@@ -66,7 +68,7 @@ __global__ void __launch_bounds__(kThreads)
   }
   double acc[TL][TL] = {};
 #pragma unroll 4
-  for (int g = threadIdx.x; g < npw; g += kThreads) {
+  for (int g = part * len + threadIdx.x; g < g1; g += kThreads) {
 #pragma unroll
     for (int k = 0; k < TL; ++k) {
       const double2 ak = a[k][g];
@@ -83,7 +85,7 @@ __global__ void __launch_bounds__(kThreads)
     for (int n = 0; n < TL; ++n) {
       __syncthreads();
       const double v = block_sum(acc[k][n]);
-      if (threadIdx.x == 0 && i0 + k < nocc && n0 + n < m) c[(int64_t)(n0 + n) * nocc + i0 + k] = v;
+      if (threadIdx.x == 0 && i0 + k < nocc && n0 + n < m) c[((int64_t)part * m + n0 + n) * nocc + i0 + k] = v;
     }
 }
 
@@ -99,7 +101,10 @@ __device__ void project(const double2* __restrict__ u, const double* __restrict_
     __syncthreads();
     for (int e = threadIdx.x; e < cnt * kBands; e += kSumChunk) {
       const int i = e / kBands, n = n0 + e % kBands;
-      cs[i][e % kBands] = n < m ? scale * c[(int64_t)n * nocc + i0 + i] : 0.0;
+      double v = 0.0;
+      if (n < m)
+        for (int part = 0; part < kProjParts; ++part) v += c[((int64_t)part * m + n) * nocc + i0 + i];
+      cs[i][e % kBands] = scale * v;
     }
     __syncthreads();
     if (g < npw) {
@@ -197,10 +202,13 @@ __global__ void __launch_bounds__(kThreads)
 // p_n = r_n + (rr_new_n / rr_n) p_n, rr_new_n the sum of part_rr[n]; CTA (chunk, n).
 __global__ void __launch_bounds__(kThreads)
     k_dir(double2* __restrict__ p, const double2* __restrict__ r, const double* __restrict__ part_rr,
-          const double* __restrict__ rr, int npw, double* __restrict__ rr_new) {
+          const double* __restrict__ rr, int npw, double* __restrict__ rr_new, double* __restrict__ rr_host) {
   const int n = blockIdx.y, g = blockIdx.x * kChunk + threadIdx.x;
   const double now = sum_partials(part_rr + (int64_t)n * gridDim.x, gridDim.x);
-  if (blockIdx.x == 0 && threadIdx.x == 0) rr_new[n] = now;
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    rr_new[n] = now;
+    rr_host[n] = now;  // pinned: the host decides on it which bands go on
+  }
   const double beta = now / rr[n];
   if (g < npw) {
     const int64_t k = (int64_t)n * npw + g;
@@ -234,9 +242,10 @@ namespace {
 int chunks(int npw, int chunk) { return (npw + chunk - 1) / chunk; }
 }  // namespace
 int st_chunks(int npw) { return chunks(npw, kSumChunk); }
+int st_proj_parts() { return kProjParts; }
 
 cudaError_t st_proj_coef(const double2* u, int nocc, const double2* x, int m, int npw, double* c, cudaStream_t s) {
-  k_proj_coef<<<dim3(chunks(nocc, kProjTile), chunks(m, kProjTile)), kThreads, 0, s>>>(u, nocc, x, m, npw, c);
+  k_proj_coef<<<dim3(chunks(nocc, kProjTile), chunks(m, kProjTile), kProjParts), kThreads, 0, s>>>(u, nocc, x, m, npw, c);
   return cudaGetLastError();
 }
 cudaError_t st_rhs(const double2* w, const double2* u, const double* c, int nocc, int m, int npw, double2* b,
@@ -259,8 +268,8 @@ cudaError_t st_step(double2* x, double2* r, const double2* p, const double2* ap,
   return cudaGetLastError();
 }
 cudaError_t st_dir(double2* p, const double2* r, const double* part_rr, const double* rr, int m, int npw,
-                   double* rr_new, cudaStream_t s) {
-  k_dir<<<dim3(chunks(npw, kChunk), m), kThreads, 0, s>>>(p, r, part_rr, rr, npw, rr_new);
+                   double* rr_new, double* rr_host, cudaStream_t s) {
+  k_dir<<<dim3(chunks(npw, kChunk), m), kThreads, 0, s>>>(p, r, part_rr, rr, npw, rr_new, rr_host);
   return cudaGetLastError();
 }
 cudaError_t st_gather_rows(const double2* src, double2* dst, const int* perm, int m, int npw, cudaStream_t s) {
