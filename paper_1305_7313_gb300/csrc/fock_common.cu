@@ -73,6 +73,7 @@ bool persist_runs(int n) {
 __global__ void k_energy(const int2* __restrict__ pairs, int npairs, const double* __restrict__ occ,
                          const double* __restrict__ ep, const double* __restrict__ dp,
                          double scale, double* __restrict__ out) {
+  after_previous();
   __shared__ double red[32 * 4];
   double v[4] = {0.0, 0.0, 0.0, 0.0};
   for (int p = threadIdx.x; p < npairs; p += blockDim.x) {
@@ -201,6 +202,7 @@ template <int TB>
 __global__ void __launch_bounds__(kOvThreads)
     k_overlap(const double* __restrict__ A, int na, const double* __restrict__ B, int nbb, int64_t K, int64_t RS,
               const int* __restrict__ half, int sym, int tiles_j, int64_t kchunk, double* __restrict__ S, int ld) {
+  after_previous();
   constexpr int MT = TB / 16;
   int ti, tj;
   if (sym) {  // blockIdx.x enumerates the tiles ti <= tj row by row
@@ -269,6 +271,7 @@ __global__ void __launch_bounds__(kOvThreads)
 }
 
 __global__ void k_overlap_zero(double* S, int na, int nbb, int sym, int ld) {
+  after_previous();
   const int64_t total = (int64_t)na * nbb;
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
     const int i = (int)(e / nbb), j = (int)(e - (int64_t)i * nbb);
@@ -438,20 +441,14 @@ cudaError_t overlap_impl(const double2* a, int na, const double2* b, int nbb, in
   kchunk = (kchunk + kOvK - 1) / kOvK * kOvK;
   splits = (int)((K + kchunk - 1) / kchunk);
   const int64_t entries = (int64_t)na * nbb;
-  k_overlap_zero<<<(int)((entries + 255) / 256 < 1216 ? (entries + 255) / 256 : 1216), 256, 0, s>>>(S, na, nbb,
-                                                                                                sym ? 1 : 0, ld);
+  const int64_t zb = (entries + 255) / 256;
+  const cudaError_t e = launch_after(k_overlap_zero, dim3((int)(zb < 1216 ? zb : 1216)), 256, 0, s, S, na, nbb,
+      sym ? 1 : 0, ld);
+  if (e != cudaSuccess) return e;
   const double* A = reinterpret_cast<const double*>(a);
   const double* B = reinterpret_cast<const double*>(b);
-  if (TB == 16)
-    k_overlap<16><<<dim3(tiles, splits), kOvThreads, 0, s>>>(A, na, B, nbb, K, RS, half, sym ? 1 : 0, tj, kchunk,
-                                                            S, ld);
-  else if (TB == 32)
-    k_overlap<32><<<dim3(tiles, splits), kOvThreads, 0, s>>>(A, na, B, nbb, K, RS, half, sym ? 1 : 0, tj, kchunk,
-                                                            S, ld);
-  else
-    k_overlap<64><<<dim3(tiles, splits), kOvThreads, 0, s>>>(A, na, B, nbb, K, RS, half, sym ? 1 : 0, tj, kchunk,
-                                                            S, ld);
-  return cudaGetLastError();
+  return launch_after(TB == 16 ? k_overlap<16> : TB == 32 ? k_overlap<32> : k_overlap<64>, dim3(tiles, splits),
+      kOvThreads, 0, s, A, na, B, nbb, K, RS, half, sym ? 1 : 0, tj, kchunk, S, ld);
 }
 }  // namespace
 
@@ -459,8 +456,7 @@ cudaError_t launch_energy_reduce(const int2* pairs, int npairs, const double* oc
                                  const double* epair, const double* dpair, double scale,
                                  double* out, cudaStream_t s) {
   const int threads = npairs >= 1024 ? 1024 : (npairs + 31) / 32 * 32;
-  k_energy<<<1, threads, 0, s>>>(pairs, npairs, occ, epair, dpair, scale, out);
-  return cudaGetLastError();
+  return launch_after(k_energy, dim3(1), threads, 0, s, pairs, npairs, occ, epair, dpair, scale, out);
 }
 
 }  // namespace fockx

@@ -27,6 +27,7 @@
 
 #include "fft_core.cuh"
 #include "fock_internal.h"
+#include "fock_launch.cuh"
 
 namespace fockx {
 
@@ -537,6 +538,7 @@ template <class T, int N, bool KP>
 __global__ void __launch_bounds__(PairGeo<T, N>::THR_COL)
     k_orb_col_inv(DevPlan g, ColumnSet cs, const double2* __restrict__ psiG, int npw, int nb, int band0, int nbat,
                   cplx<T>* __restrict__ X, ClearOnWay clr) {
+  after_previous();
   using C = cplx<T>;
   using G = PairGeo<T, N>;
   constexpr int A = G::CA, B = G::CB, NL = G::NL, NP = KP ? NL : G::NP, THR = G::THR_COL;
@@ -607,6 +609,7 @@ template <class T, int N, bool KP>
 __global__ void __launch_bounds__(PairGeo<T, N>::THR_COL)
     k_orb_col_fwd(DevPlan g, ColumnSet cs, const cplx<T>* __restrict__ X, double scale, int npw, int nb, int band0,
                   int nbat, double2* __restrict__ out) {
+  after_previous();
   using C = cplx<T>;
   using G = PairGeo<T, N>;
   constexpr int A = G::CA, B = G::CB, NL = G::NL, NP = KP ? NL : G::NP, THR = G::THR_COL;
@@ -693,6 +696,7 @@ template <class T, int N, bool KP>
 __global__ void __launch_bounds__(PairGeo<T, N>::THR_PLANE, PairGeo<T, N>::MIN_PLANE)
     k_orb_plane_inv(DevPlan g, ColumnSet cs, const cplx<T>* __restrict__ X, void* __restrict__ psiv,
                     void* __restrict__ wv, int band0, int nb, int nbat) {
+  after_previous();
   using C = cplx<T>;
   using G = PairGeo<T, N>;
   constexpr int THR = G::THR_PLANE, RP = G::RP;
@@ -729,6 +733,7 @@ template <class T, int N, bool KP>
 __global__ void __launch_bounds__(PairGeo<T, N>::THR_PLANE, PairGeo<T, N>::MIN_PLANE)
     k_orb_plane_fwd(DevPlan g, ColumnSet cs, const void* __restrict__ Wv, cplx<T>* __restrict__ X, int band0, int nb,
                     int nbat) {
+  after_previous();
   using C = cplx<T>;
   using G = PairGeo<T, N>;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -756,6 +761,7 @@ __global__ void __launch_bounds__(PairGeo<T, N>::THR_PLANE, PairGeo<T, N>::MIN_P
 template <class T, int N>
 __global__ void __launch_bounds__(PairGeo<T, N>::THR_PLANE, PairGeo<T, N>::MIN_PLANE)
     k_orb_plane_vloc(DevPlan g, ColumnSet cs, const T* __restrict__ vloc, cplx<T>* __restrict__ X) {
+  after_previous();
   using C = cplx<T>;
   using G = PairGeo<T, N>;
   static_assert(!G::BLOCK && !G::ALL_LINES, "written for the two-factor stages");
@@ -824,6 +830,7 @@ template <class T, int N, int TILE = 0>
 __global__ void __launch_bounds__(PairGeo<T, N, TILE>::THR_PLANE, PairGeo<T, N, TILE>::MIN_PLANE)
     k_pair_fwd(DevPlan g, const T* __restrict__ psi, const Chain* __restrict__ chains,
                cplx<T>* __restrict__ H) {
+  after_previous();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const Chain ch = chains[blockIdx.y];
   pair_fwd_task<T, N, PairGeo<T, N, TILE>::THR_PLANE, TILE>(g, psi, ch, H + (int64_t)blockIdx.y * g.hsize,
@@ -1140,6 +1147,7 @@ template <class T, int N, int TILE = 0>
 __global__ void __launch_bounds__(PairGeo<T, N, TILE>::THR_COL, PairGeo<T, N, TILE>::MIN_COL)
     k_pair_col(DevPlan g, cplx<T>* __restrict__ H, const Chain* __restrict__ chains,
                double* __restrict__ epair, double* __restrict__ dpair) {
+  after_previous();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const Chain ch = chains[blockIdx.y];
   pair_col_task<T, N, PairGeo<T, N, TILE>::THR_COL, TILE>(g, H + (int64_t)blockIdx.y * g.hsize, ch, blockIdx.x,
@@ -1334,6 +1342,7 @@ template <class T, int N, int TILE = 0>
 __global__ void __launch_bounds__(PairGeo<T, N, TILE>::THR_PLANE, PairGeo<T, N, TILE>::MIN_PLANE)
     k_pair_inv(DevPlan g, const T* __restrict__ psi, acc_t<T>* __restrict__ W, const T* __restrict__ occ,
                const Chain* __restrict__ chains, const cplx<T>* __restrict__ H) {
+  after_previous();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const Chain ch = chains[blockIdx.y];
   pair_inv_task<T, N, PairGeo<T, N, TILE>::THR_PLANE, TILE>(g, psi, W, occ, ch, H + (int64_t)blockIdx.y * g.hsize,
@@ -1417,11 +1426,10 @@ struct Launch {
                              void* Xv, void* psiv, const ClearOnWay& clr, cudaStream_t s) {
     C* X = static_cast<C*>(Xv);
     const int nq = (nbat + 1) / 2;
-    k_orb_col_inv<T, N, false><<<dim3(g.orb.ncta, nq), P0::THR_COL, P0::SMEM_COL, s>>>(g, g.orb, psiG, g.npw, nb, band0,
-                                                                                     nbat, X, clr);
-    k_orb_plane_inv<T, N, false><<<dim3(N, nq), P0::THR_PLANE, P0::SMEM_PLANE, s>>>(g, g.orb, X, psiv, clr.w, band0, nb,
-                                                                                    nbat);
-    return cudaGetLastError();
+    cudaError_t e = launch_after(k_orb_col_inv<T, N, false>, dim3(g.orb.ncta, nq), P0::THR_COL, P0::SMEM_COL, s, g,
+        g.orb, psiG, g.npw, nb, band0, nbat, X, clr);
+    return e != cudaSuccess ? e : launch_after(k_orb_plane_inv<T, N, false>, dim3(N, nq), P0::THR_PLANE,
+        P0::SMEM_PLANE, s, g, g.orb, X, psiv, clr.w, band0, nb, nbat);
   }
 
   static cudaError_t apply_vloc(const DevPlan& g, const double2* psiG, int nb, int band0, int nbat, const double* vloc,
@@ -1429,12 +1437,12 @@ struct Launch {
     if constexpr (RealTraits<T>::prec == 0) {
       C* X = static_cast<C*>(Xv);
       const int nq = (nbat + 1) / 2;
-      k_orb_col_inv<T, N, false><<<dim3(g.orb.ncta, nq), P0::THR_COL, P0::SMEM_COL, s>>>(g, g.orb, psiG, g.npw, nb,
-                                                                                       band0, nbat, X, ClearOnWay{});
-      k_orb_plane_vloc<T, N><<<dim3(N, nq), P0::THR_PLANE, P0::SMEM_PLANE, s>>>(g, g.orb, vloc, X);
-      k_orb_col_fwd<T, N, false><<<dim3(g.orb.ncta, nq), P0::THR_COL, P0::SMEM_COL, s>>>(
-          g, g.orb, X, g.inv_ntot, g.npw, nb, band0, nbat, out);
-      return cudaGetLastError();
+      cudaError_t e = launch_after(k_orb_col_inv<T, N, false>, dim3(g.orb.ncta, nq), P0::THR_COL, P0::SMEM_COL, s,
+          g, g.orb, psiG, g.npw, nb, band0, nbat, X, ClearOnWay{});
+      if (e == cudaSuccess) e = launch_after(k_orb_plane_vloc<T, N>, dim3(N, nq), P0::THR_PLANE, P0::SMEM_PLANE, s,
+          g, g.orb, vloc, X);
+      return e != cudaSuccess ? e : launch_after(k_orb_col_fwd<T, N, false>, dim3(g.orb.ncta, nq), P0::THR_COL,
+          P0::SMEM_COL, s, g, g.orb, X, g.inv_ntot, g.npw, nb, band0, nbat, out);
     } else {
       return cudaErrorNotSupported;
     }
@@ -1443,9 +1451,8 @@ struct Launch {
   template <int TILE>
   static cudaError_t fwd_tile(const DevPlan& g, const void* psi, const Chain* ch, int nch, void* H, cudaStream_t s) {
     using P = PairGeo<T, N, TILE>;
-    k_pair_fwd<T, N, TILE><<<dim3(N, nch), P::THR_PLANE, P::SMEM_PLANE, s>>>(g, static_cast<const T*>(psi), ch,
-                                                                             static_cast<C*>(H));
-    return cudaGetLastError();
+    return launch_after(k_pair_fwd<T, N, TILE>, dim3(N, nch), P::THR_PLANE, P::SMEM_PLANE, s, g,
+        static_cast<const T*>(psi), ch, static_cast<C*>(H));
   }
   static cudaError_t pair_fwd(const DevPlan& g, const void* psi, const Chain* ch, int nch, void* H,
                               cudaStream_t s) {
@@ -1456,8 +1463,8 @@ struct Launch {
   static cudaError_t col_tile(const DevPlan& g, void* H, const Chain* ch, int nch, double* ep, double* dp,
                               cudaStream_t s) {
     using P = PairGeo<T, N, TILE>;
-    k_pair_col<T, N, TILE><<<dim3(g.cols.ncta, nch), P::THR_COL, P::SMEM_COL, s>>>(g, static_cast<C*>(H), ch, ep, dp);
-    return cudaGetLastError();
+    return launch_after(k_pair_col<T, N, TILE>, dim3(g.cols.ncta, nch), P::THR_COL, P::SMEM_COL, s, g,
+        static_cast<C*>(H), ch, ep, dp);
   }
   static cudaError_t pair_col(const DevPlan& g, void* H, const Chain* ch, int nch, double* ep,
                               double* dp, cudaStream_t s) {
@@ -1468,10 +1475,9 @@ struct Launch {
   static cudaError_t inv_tile(const DevPlan& g, const void* psi, void* W, const void* occ, const Chain* ch, int nch,
                               const void* H, cudaStream_t s) {
     using P = PairGeo<T, N, TILE>;
-    k_pair_inv<T, N, TILE><<<dim3(N, nch), P::THR_PLANE, P::SMEM_PLANE, s>>>(
-        g, static_cast<const T*>(psi), static_cast<acc_t<T>*>(W), static_cast<const T*>(occ), ch,
+    return launch_after(k_pair_inv<T, N, TILE>, dim3(N, nch), P::THR_PLANE, P::SMEM_PLANE, s, g,
+        static_cast<const T*>(psi), static_cast<acc_t<T>*>(W), static_cast<const T*>(occ), ch,
         static_cast<const C*>(H));
-    return cudaGetLastError();
   }
   static cudaError_t pair_inv(const DevPlan& g, const void* psi, void* W, const void* occ,
                               const Chain* ch, int nch, const void* H, cudaStream_t s) {
@@ -1483,10 +1489,10 @@ struct Launch {
                                void* Xv, double2* vpsiG, cudaStream_t s) {
     C* X = static_cast<C*>(Xv);
     const int nq = (nbat + 1) / 2;
-    k_orb_plane_fwd<T, N, false><<<dim3(N, nq), P0::THR_PLANE, P0::SMEM_PLANE, s>>>(g, g.orb, W, X, band0, nb, nbat);
-    k_orb_col_fwd<T, N, false><<<dim3(g.orb.ncta, nq), P0::THR_COL, P0::SMEM_COL, s>>>(
-        g, g.orb, X, g.out_scale, g.npw, nb, band0, nbat, vpsiG);
-    return cudaGetLastError();
+    cudaError_t e = launch_after(k_orb_plane_fwd<T, N, false>, dim3(N, nq), P0::THR_PLANE, P0::SMEM_PLANE, s, g,
+        g.orb, W, X, band0, nb, nbat);
+    return e != cudaSuccess ? e : launch_after(k_orb_col_fwd<T, N, false>, dim3(g.orb.ncta, nq), P0::THR_COL,
+        P0::SMEM_COL, s, g, g.orb, X, g.out_scale, g.npw, nb, band0, nbat, vpsiG);
   }
 
   static constexpr KernelOps ops() {

@@ -27,6 +27,7 @@ template <class T, int N>
 __global__ void __launch_bounds__(PairGeo<T, N>::THR_PLANE, PairGeo<T, N>::MIN_PLANE)
     k_kpair_fwd(DevPlan g, const cplx<T>* __restrict__ u, const Chain* __restrict__ chains,
                 cplx<T>* __restrict__ H) {
+  after_previous();
   using C = cplx<T>;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int i1 = blockIdx.x;
@@ -71,6 +72,7 @@ template <class T, int N>
 __global__ void __launch_bounds__(PairGeo<T, N>::THR_COL, PairGeo<T, N>::MIN_COL)
     k_kpair_col(DevPlan g, cplx<T>* __restrict__ H, const Chain* __restrict__ chains,
                 double* __restrict__ epair) {
+  after_previous();
   using C = cplx<T>;
   using G = PairGeo<T, N>;
   constexpr int A = G::CA, B = G::CB, NL = G::NL, THR = G::THR_COL;
@@ -192,6 +194,7 @@ template <class T, int N>
 __global__ void __launch_bounds__(PairGeo<T, N>::THR_PLANE, PairGeo<T, N>::MIN_PLANE)
     k_kpair_inv(DevPlan g, const cplx<T>* __restrict__ u, cplx<T>* __restrict__ W,
                 const T* __restrict__ occw, const Chain* __restrict__ chains, const cplx<T>* __restrict__ H) {
+  after_previous();
   using C = cplx<T>;
   using G = PairGeo<T, N>;
   constexpr int RP = G::RP, THR = G::THR_PLANE;
@@ -274,40 +277,37 @@ struct LaunchK {
   static cudaError_t to_real(const DevPlan& g, const ColumnSet& orb, const double2* psiG, int npw, int band0, int nbat,
                              void* Xv, void* u, const ClearOnWay& clr, cudaStream_t s) {
     C* X = static_cast<C*>(Xv);
-    k_orb_col_inv<T, N, true><<<dim3(orb.ncta, nbat), G::THR_COL, G::SMEM_COL, s>>>(g, orb, psiG, npw, nbat, 0, nbat, X, clr);
-    k_orb_plane_inv<T, N, true><<<dim3(N, nbat), G::THR_PLANE, G::SMEM_PLANE, s>>>(g, orb, X, u, clr.w, band0, nbat,
-                                                                                       nbat);
-    return cudaGetLastError();
+    cudaError_t e = launch_after(k_orb_col_inv<T, N, true>, dim3(orb.ncta, nbat), G::THR_COL, G::SMEM_COL, s, g,
+        orb, psiG, npw, nbat, 0, nbat, X, clr);
+    return e != cudaSuccess ? e : launch_after(k_orb_plane_inv<T, N, true>, dim3(N, nbat), G::THR_PLANE,
+        G::SMEM_PLANE, s, g, orb, X, u, clr.w, band0, nbat, nbat);
   }
 
   static cudaError_t pair_fwd(const DevPlan& g, const void* u, const Chain* ch, int nch, void* H,
                               cudaStream_t s) {
-    k_kpair_fwd<T, N><<<dim3(N, nch), G::THR_PLANE, G::SMEM_PLANE, s>>>(g, static_cast<const C*>(u), ch,
-                                                                      static_cast<C*>(H));
-    return cudaGetLastError();
+    return launch_after(k_kpair_fwd<T, N>, dim3(N, nch), G::THR_PLANE, G::SMEM_PLANE, s, g,
+        static_cast<const C*>(u), ch, static_cast<C*>(H));
   }
 
   static cudaError_t pair_col(const DevPlan& g, void* H, const Chain* ch, int nch, double* ep,
                               cudaStream_t s) {
-    k_kpair_col<T, N><<<dim3(g.cols.ncta, nch), G::THR_COL, G::SMEM_COL, s>>>(g, static_cast<C*>(H), ch, ep);
-    return cudaGetLastError();
+    return launch_after(k_kpair_col<T, N>, dim3(g.cols.ncta, nch), G::THR_COL, G::SMEM_COL, s, g,
+        static_cast<C*>(H), ch, ep);
   }
 
   static cudaError_t pair_inv(const DevPlan& g, const void* u, void* W, const void* occw, const Chain* ch,
                               int nch, const void* H, cudaStream_t s) {
-    k_kpair_inv<T, N><<<dim3(N, nch), G::THR_PLANE, G::SMEM_PLANE, s>>>(
-        g, static_cast<const C*>(u), static_cast<C*>(W), static_cast<const T*>(occw), ch,
-        static_cast<const C*>(H));
-    return cudaGetLastError();
+    return launch_after(k_kpair_inv<T, N>, dim3(N, nch), G::THR_PLANE, G::SMEM_PLANE, s, g,
+        static_cast<const C*>(u), static_cast<C*>(W), static_cast<const T*>(occw), ch, static_cast<const C*>(H));
   }
 
   static cudaError_t to_sphere(const DevPlan& g, const ColumnSet& orb, const void* W, int band0, int nbat, int npw,
                                void* Xv, double2* vpsiG, cudaStream_t s) {
     C* X = static_cast<C*>(Xv);
-    k_orb_plane_fwd<T, N, true><<<dim3(N, nbat), G::THR_PLANE, G::SMEM_PLANE, s>>>(g, orb, W, X, band0, nbat, nbat);
-    k_orb_col_fwd<T, N, true><<<dim3(orb.ncta, nbat), G::THR_COL, G::SMEM_COL, s>>>(g, orb, X, g.out_scale, npw, nbat,
-                                                                                  0, nbat, vpsiG);
-    return cudaGetLastError();
+    cudaError_t e = launch_after(k_orb_plane_fwd<T, N, true>, dim3(N, nbat), G::THR_PLANE, G::SMEM_PLANE, s, g, orb,
+        W, X, band0, nbat, nbat);
+    return e != cudaSuccess ? e : launch_after(k_orb_col_fwd<T, N, true>, dim3(orb.ncta, nbat), G::THR_COL,
+        G::SMEM_COL, s, g, orb, X, g.out_scale, npw, nbat, 0, nbat, vpsiG);
   }
 
   static constexpr KOps ops() {

@@ -9,6 +9,7 @@
 // those of <r|r>, and the new directions.  Each kernel that needs an inner
 // product adds the partial sums of the one before it in a fixed order.
 #include "fock_internal.h"
+#include "fock_launch.cuh"
 
 namespace fockx {
 namespace {
@@ -55,6 +56,7 @@ constexpr int kProjTile = 2, kProjParts = 2;
 __global__ void __launch_bounds__(kThreads)
     k_proj_coef(const double2* __restrict__ u, int nocc, const double2* __restrict__ x, int m, int npw,
                 double* __restrict__ c) {
+  after_previous();
   constexpr int TL = kProjTile;
   const int i0 = blockIdx.x * TL, n0 = blockIdx.y * TL, part = blockIdx.z;
   const int len = (npw + kProjParts - 1) / kProjParts;
@@ -125,6 +127,7 @@ __device__ void project(const double2* __restrict__ u, const double* __restrict_
 __global__ void __launch_bounds__(kSumChunk)
     k_rhs(const double2* __restrict__ w, const double2* __restrict__ u, const double* __restrict__ c, int nocc, int m,
           int npw, double2* __restrict__ b, double* __restrict__ part) {
+  after_previous();
   const int g = blockIdx.x * kSumChunk + threadIdx.x, n0 = blockIdx.y * kBands;
   double2 s[kBands] = {};
   project(u, c, nocc, n0, m, npw, g, 1.0, s);
@@ -144,6 +147,7 @@ __global__ void __launch_bounds__(kSumChunk)
 
 // rr[n] = sum of part[n][0 .. nchunk).
 __global__ void k_sum_parts(const double* __restrict__ part, int nchunk, double* __restrict__ rr) {
+  after_previous();
   const double s = sum_partials(part + (int64_t)blockIdx.x * nchunk, nchunk);
   if (threadIdx.x == 0) rr[blockIdx.x] = s;
 }
@@ -155,6 +159,7 @@ __global__ void __launch_bounds__(kSumChunk)
     k_finish(double2* __restrict__ ap, const double2* __restrict__ p, const double* __restrict__ kin,
              const double* __restrict__ eps, const double2* __restrict__ u, const double* __restrict__ c, int nocc,
              double alpha, int m, int npw, double* __restrict__ part) {
+  after_previous();
   const int g = blockIdx.x * kSumChunk + threadIdx.x, n0 = blockIdx.y * kBands;
   double2 s[kBands] = {};
   project(u, c, nocc, n0, m, npw, g, alpha, s);
@@ -180,6 +185,7 @@ __global__ void __launch_bounds__(kThreads)
     k_step(double2* __restrict__ x, double2* __restrict__ r, const double2* __restrict__ p,
            const double2* __restrict__ ap, const double* __restrict__ rr, const double* __restrict__ part_pap, int nsum,
            int npw, double* __restrict__ part_rr) {
+  after_previous();
   const int n = blockIdx.y, g = blockIdx.x * kChunk + threadIdx.x;
   const double a = rr[n] / sum_partials(part_pap + (int64_t)n * nsum, nsum);
   double d = 0.0;
@@ -203,6 +209,7 @@ __global__ void __launch_bounds__(kThreads)
 __global__ void __launch_bounds__(kThreads)
     k_dir(double2* __restrict__ p, const double2* __restrict__ r, const double* __restrict__ part_rr,
           const double* __restrict__ rr, int npw, double* __restrict__ rr_new, double* __restrict__ rr_host) {
+  after_previous();
   const int n = blockIdx.y, g = blockIdx.x * kChunk + threadIdx.x;
   const double now = sum_partials(part_rr + (int64_t)n * gridDim.x, gridDim.x);
   if (blockIdx.x == 0 && threadIdx.x == 0) {
@@ -220,6 +227,7 @@ __global__ void __launch_bounds__(kThreads)
 // dst[k] = src[perm[k]] for ket arrays (rows of npw) and for per-band scalars.
 __global__ void k_gather_rows(const double2* __restrict__ src, double2* __restrict__ dst, const int* __restrict__ perm,
                               int m, int npw) {
+  after_previous();
   const int64_t total = (int64_t)m * npw;
   for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < total; k += (int64_t)gridDim.x * blockDim.x) {
     const int n = (int)(k / npw), g = (int)(k - (int64_t)n * npw);
@@ -228,6 +236,7 @@ __global__ void k_gather_rows(const double2* __restrict__ src, double2* __restri
 }
 __global__ void k_gather_scalars(const double* __restrict__ src, double* __restrict__ dst,
                                  const int* __restrict__ perm, int m) {
+  after_previous();
   for (int n = blockIdx.x * blockDim.x + threadIdx.x; n < m; n += gridDim.x * blockDim.x) dst[n] = src[perm[n]];
 }
 
@@ -245,40 +254,35 @@ int st_chunks(int npw) { return chunks(npw, kSumChunk); }
 int st_proj_parts() { return kProjParts; }
 
 cudaError_t st_proj_coef(const double2* u, int nocc, const double2* x, int m, int npw, double* c, cudaStream_t s) {
-  k_proj_coef<<<dim3(chunks(nocc, kProjTile), chunks(m, kProjTile), kProjParts), kThreads, 0, s>>>(u, nocc, x, m, npw, c);
-  return cudaGetLastError();
+  return launch_after(k_proj_coef, dim3(chunks(nocc, kProjTile), chunks(m, kProjTile), kProjParts), kThreads, 0, s,
+      u, nocc, x, m, npw, c);
 }
 cudaError_t st_rhs(const double2* w, const double2* u, const double* c, int nocc, int m, int npw, double2* b,
                    double* part, double* rr, cudaStream_t s) {
   const int nsum = chunks(npw, kSumChunk);
-  k_rhs<<<dim3(nsum, chunks(m, kBands)), kSumChunk, 0, s>>>(w, u, c, nocc, m, npw, b, part);
-  k_sum_parts<<<m, 32, 0, s>>>(part, nsum, rr);
-  return cudaGetLastError();
+  const cudaError_t e = launch_after(k_rhs, dim3(nsum, chunks(m, kBands)), kSumChunk, 0, s, w, u, c, nocc, m, npw,
+      b, part);
+  return e != cudaSuccess ? e : launch_after(k_sum_parts, dim3(m), 32, 0, s, part, nsum, rr);
 }
 cudaError_t st_finish(double2* ap, const double2* p, const double* kin, const double* eps, const double2* u,
                       const double* c, int nocc, double alpha, int m, int npw, double* part, cudaStream_t s) {
-  k_finish<<<dim3(chunks(npw, kSumChunk), chunks(m, kBands)), kSumChunk, 0, s>>>(ap, p, kin, eps, u, c, nocc, alpha, m,
-                                                                               npw, part);
-  return cudaGetLastError();
+  return launch_after(k_finish, dim3(chunks(npw, kSumChunk), chunks(m, kBands)), kSumChunk, 0, s, ap, p, kin, eps,
+      u, c, nocc, alpha, m, npw, part);
 }
 cudaError_t st_step(double2* x, double2* r, const double2* p, const double2* ap, const double* rr,
                     const double* part_pap, int m, int npw, double* part_rr, cudaStream_t s) {
-  k_step<<<dim3(chunks(npw, kChunk), m), kThreads, 0, s>>>(x, r, p, ap, rr, part_pap, chunks(npw, kSumChunk), npw,
-                                                         part_rr);
-  return cudaGetLastError();
+  return launch_after(k_step, dim3(chunks(npw, kChunk), m), kThreads, 0, s, x, r, p, ap, rr, part_pap, chunks(npw,
+      kSumChunk), npw, part_rr);
 }
 cudaError_t st_dir(double2* p, const double2* r, const double* part_rr, const double* rr, int m, int npw,
                    double* rr_new, double* rr_host, cudaStream_t s) {
-  k_dir<<<dim3(chunks(npw, kChunk), m), kThreads, 0, s>>>(p, r, part_rr, rr, npw, rr_new, rr_host);
-  return cudaGetLastError();
+  return launch_after(k_dir, dim3(chunks(npw, kChunk), m), kThreads, 0, s, p, r, part_rr, rr, npw, rr_new, rr_host);
 }
 cudaError_t st_gather_rows(const double2* src, double2* dst, const int* perm, int m, int npw, cudaStream_t s) {
-  k_gather_rows<<<grid_for((int64_t)m * npw), kThreads, 0, s>>>(src, dst, perm, m, npw);
-  return cudaGetLastError();
+  return launch_after(k_gather_rows, dim3(grid_for((int64_t)m * npw)), kThreads, 0, s, src, dst, perm, m, npw);
 }
 cudaError_t st_gather_scalars(const double* src, double* dst, const int* perm, int m, cudaStream_t s) {
-  k_gather_scalars<<<1, kThreads, 0, s>>>(src, dst, perm, m);
-  return cudaGetLastError();
+  return launch_after(k_gather_scalars, dim3(1), kThreads, 0, s, src, dst, perm, m);
 }
 
 }  // namespace fockx
