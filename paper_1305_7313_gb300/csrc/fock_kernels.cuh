@@ -309,9 +309,9 @@ struct PairGeo {
   // ones only.
   static constexpr bool ALL_LINES = sizeof(C) == 8;
   // FP32 plane passes take three trips through registers (N = 4 M): shared
-  // memory bounds them, and a trip fewer takes 20.5 -> 15.1 M wavefronts a
-  // 38-chain launch at 96^3 (forward; 3.44 -> 3.06 us a chain, inverse 4.29 ->
-  // 3.65).  FP64 and double-float are bound by arithmetic: the two-factor
+  // memory bounds them, and a trip fewer takes the inverse pass at 96^3 from 4.29
+  // to 3.65 us a chain, the forward pass, whose result then goes out from
+  // registers, from 3.44 to 2.37.  FP64 and double-float are bound by arithmetic: the two-factor
   // stages' items are smaller and share out more evenly (FP64 24^3 forward 0.85
   // against 1.05 us, 48^3 6.39 against 6.49, 96^3 even)
   static constexpr bool BLOCK = RealTraits<T>::prec == 1 && TILE == 0;
@@ -399,7 +399,6 @@ __device__ __forceinline__ void plane_forward(const DevPlan& g, const ColumnSet&
   C* P = reinterpret_cast<C*>(smem_raw);
   C* tw = P + N * RP;
   load_stage_twiddles<T, -1, G::BLOCK ? 4 : B, N, THR>(tw, g);
-  if constexpr (G::BLOCK) load_stage_twiddles<T, -1, M, N, THR>(tw + N, g);
   // Columns (along i2) first: the first stage reads its input through load (a
   // warp's items are consecutive columns i3, so the loads coalesce); only its
   // outputs enter shared memory.
@@ -418,14 +417,27 @@ __device__ __forceinline__ void plane_forward(const DevPlan& g, const ColumnSet&
     }
   }
   __syncthreads();
-  if constexpr (G::BLOCK) plane_block_pass<T, M, -1, THR, RP>(P, tw);
-  else stage_ct<T, B, -1, A, B * RP, RP, true, THR, N, 1>(P, tw);
+  if constexpr (G::BLOCK) {
+    plane_row_stage<T, M, -1, THR, RP>(P);
+    plane_block_out<T, M, -1, THR, RP>(P, tw, [&](const C(&v)[4][4], int x, int y) {
+#pragma unroll
+      for (int t = 0; t < 4; ++t) {
+        const int k3 = y + M * t, ud = __ldg(cs.ncol + k3);
+        const int up = ud & 0xffff, dn = N - (ud >> 16);
+#pragma unroll
+        for (int s = 0; s < 4; ++s) {
+          const int k2 = x + M * s;
+          if (k2 < up || k2 >= dn) Hp[k2 * N + k3] = v[s][t];
+        }
+      }
+    });
+    return;
+  }
+  stage_ct<T, B, -1, A, B * RP, RP, true, THR, N, 1>(P, tw);
   // k2 is now at row G::row_place(k2); the rest of the transforms along i3
-  constexpr int R1 = G::BLOCK ? M : B;
-  const C* tw1 = G::BLOCK ? tw + N : tw;
   if constexpr (G::ALL_LINES) {
-    if constexpr (!G::BLOCK) stage_ct<T, A, -1, B, 1, B, false, THR, N, RP>(P, tw);
-    stage_ct<T, R1, -1, N / R1, R1, 1, true, THR, N, RP>(P, tw1);
+    stage_ct<T, A, -1, B, 1, B, false, THR, N, RP>(P, tw);
+    stage_ct<T, B, -1, A, B, 1, true, THR, N, RP>(P, tw);
   } else {
     // only the rows k2 that hold kept columns, in order of their places
     int* rows = reinterpret_cast<int*>(tw + 2 * N);
@@ -434,8 +446,8 @@ __device__ __forceinline__ void plane_forward(const DevPlan& g, const ColumnSet&
     for (int r = threadIdx.x; r < nrows; r += THR) rows[r] = __ldg(cs.rowpos + TILE * N + r) * RP;
     __syncthreads();
     const auto row_off = [&](int l) { return rows[l]; };
-    if constexpr (!G::BLOCK) stage_rt<T, A, -1, B, 1, B, false, THR>(P, tw, nrows, by, row_off);
-    stage_rt<T, R1, -1, N / R1, R1, 1, true, THR>(P, tw1, nrows, by, row_off);
+    stage_rt<T, A, -1, B, 1, B, false, THR>(P, tw, nrows, by, row_off);
+    stage_rt<T, B, -1, A, B, 1, true, THR>(P, tw, nrows, by, row_off);
   }
   // the kept columns (k2, k3), consecutive threads on consecutive k3 of a row
   for (int e = threadIdx.x; e < cs.nkept; e += THR) {
