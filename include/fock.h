@@ -209,12 +209,11 @@ fock_status fock_plan_set_band_block(fock_plan_t plan, int band_block);
 /*
  * FFT tilings of the pair passes.  Each of the three pair passes (pass 0: the
  * forward plane pass, 1: the column pass, 2: the inverse plane pass) has one
- * or two compiled radix plans ("tilings"): tile 0 holds FftTraits' element
- * budget per thread (24 complex values in the mixed form, 12 in FP64 and
- * double-float), tile 1 the plan found with the other budget (12 in the mixed
- * form, 24 in FP64; none in double-float).  When both budgets give the same
- * plan for N, the pass has one tiling.  The results do not depend on the
- * tiling beyond rounding; the speed does (the tuner in autotune.py times them).
+ * or two compiled forms ("tilings") for the plan's working grid (the smallest
+ * compiled grid that holds its pair densities): tile 0 the fastest measured, tile
+ * 1, in FP64 and the mixed form where that grid is 96^3, 12 x 8 with eight threads
+ * a line.  The results do not depend on the tiling beyond rounding; the speed
+ * does (the tuner in autotune.py times them).
  *
  * fock_plan_tiling_info: the plan of tile `tile` of pass `pass`: radices
  *   (host int[8], stage order), nstages, threads per transformed line,
@@ -244,8 +243,9 @@ fock_status fock_plan_device_bytes(fock_plan_t plan, int64_t* bytes);
  * plans). */
 fock_status fock_plan_set_deterministic(fock_plan_t plan, int enable);
 
-/* Columns of the stored half spectrum (N x 2(N/2+1) per plane, both pairs of a
- * chain) that the pair-density ball |G| <= 2 Gmax reaches and the column pass
+/* Columns of the pair densities' half spectra (n x 2(n/2+1) per plane of the
+ * working grid, both pairs of a chain; stored as the columns of one complex
+ * spectrum) that the pair-density ball |G| <= 2 Gmax reaches and the column pass
  * transforms (`kept`), out of `total`: the overlap densities of §4 are products
  * of two orbitals on the sphere, so their spectra live in that ball.  Host
  * outputs; either may be NULL.  Errors: INVALID_ARG (plan NULL). */
