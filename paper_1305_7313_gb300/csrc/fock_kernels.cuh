@@ -319,7 +319,7 @@ struct PairGeo {
   // threads per line: an M-point item each, or whole two-factor items; in
   // double-float at 96, one CTA an SM, eight (four: 17.1 and 22.2 us a chain
   // forward and inverse, eight: 16.8 and 20.3)
-    static constexpr int TPL = TILE == 1 ? 8 : (!BLOCK && (N == 72 || N == 36) ? 3 : RealTraits<T>::prec == 2 && N == 96 ? 8 : 4);
+  static constexpr int TPL = TILE == 1 ? 8 : (!BLOCK && (N == 72 || N == 36) ? 3 : RealTraits<T>::prec == 2 && N == 96 ? 8 : 4);
   static constexpr int THR_PLANE = (N * TPL + 31) / 32 * 32;
   // where a plane's passes leave frequency k of the columns and of the rows
   static __host__ __device__ constexpr int row_place(int k) {
