@@ -171,12 +171,17 @@ def time_form(plan, psi, occ, steps, warmup, want_dex=False, rank=0, world=1):
 # of the 96^3 pair passes of the 64-band case at 38 chains per launch, one
 # stream (profiles/pair_traffic_96.md); scaled
 # to a launch by its chains, reported only for a captured band block (the
-# orbital re-reads depend on it).
+# orbital re-reads depend on it).  The captures are of earlier kernels; the present
+# ones move 53.2 MB (FP64, double-float) and 12.5 MB (mixed) a chain in the
+# inverse pass at band block 8 (profiles/pair_passes_96.md), TRAFFIC_SRC says so.
 MEASURED_TRAFFIC_PER_CHAIN = {
     ("fp64", 96, "pair_inv", 8): 54.04e6, ("fp64", 96, "pair_inv", 16): 47.18e6, ("fp64", 96, "pair_inv", 32): 52.54e6,
     ("df64", 96, "pair_inv", 8): 57.45e6, ("df64", 96, "pair_inv", 16): 50.67e6, ("df64", 96, "pair_inv", 32): 53.20e6,
     ("mixed32", 96, "pair_inv", 8): 12.61e6, ("mixed32", 96, "pair_inv", 16): 19.28e6,
 }
+
+
+TRAFFIC_SRC = "ncu captures of earlier kernels"
 
 
 def pair_loop_ms(res, steps):
@@ -229,7 +234,7 @@ def roofline(form, plan, res, steps, peaks, peak_src, band_block=16, streams=1):
                "measured FP32 FMA loop / 9.4 FP32 instructions per double-float flop, 2070 MHz")
         return {"bound": "alu", "kernel": dom, "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
                 "frac": achieved / peak,
-                "traffic": measured_traffic(form, n, dom, band_block, chains_per_launch),
+                "traffic": measured_traffic(form, n, dom, band_block, chains_per_launch), "traffic_src": TRAFFIC_SRC,
                 "peak_src": src, "frac_at_sampled_clock": achieved / (per_clk * mhz * 1e6 / 1e12),
                 "ms_per_launch": ms_per_launch, "chains_per_launch": chains_per_launch}
     # Algorithmic bytes per chain (two pairs): the kept columns of the complex64
@@ -245,7 +250,7 @@ def roofline(form, plan, res, steps, peaks, peak_src, band_block=16, streams=1):
     peak = float(peaks["hbm_gbs"])
     return {"bound": "hbm", "kernel": dom, "achieved": achieved, "peak": peak, "unit": "GB/s",
             "frac": achieved / peak,
-            "traffic": measured_traffic(form, n, dom, band_block, chains_per_launch),
+            "traffic": measured_traffic(form, n, dom, band_block, chains_per_launch), "traffic_src": TRAFFIC_SRC,
             "peak_src": peak_src + " (hbm copy)", "bytes_per_chain": per_chain,
             "ms_per_launch": ms_per_launch, "chains_per_launch": chains_per_launch}
 
@@ -326,7 +331,7 @@ def loop_roofline(form, plan, res, steps, peaks, peak_src, band_block, streams):
                "frac": achieved / peak, "peak_src": peak_src + " (hbm copy)", "bytes_per_chain": per_chain}
     per = MEASURED_LOOP_TRAFFIC_PER_CHAIN.get((form, n, band_block))
     out.update({"traffic": per * chains if per else None, "traffic_unit": "DRAM bytes per step (ncu, all three kernels)",
-                "ms_pair_loop": ms, "chains_per_step": chains})
+                "traffic_src": TRAFFIC_SRC, "ms_pair_loop": ms, "chains_per_step": chains})
     return out
 
 
@@ -518,7 +523,7 @@ def run_kpoints(args, peaks, peak_src):
                          "peak": float(peaks["hbm_gbs"]), "unit": "GB/s",
                          "frac": achieved / float(peaks["hbm_gbs"]), "traffic": traffic,
                          "traffic_unit": "DRAM bytes per step (ncu, all three kernels)",
-                         "peak_src": peak_src + " (hbm copy)"}}
+                         "traffic_src": TRAFFIC_SRC, "peak_src": peak_src + " (hbm copy)"}}
 
 
 KPOINT_DRAM_PER_PAIR = 3.351e6
