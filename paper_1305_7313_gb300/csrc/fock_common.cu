@@ -455,7 +455,8 @@ cudaError_t overlap_impl(const double2* a, int na, const double2* b, int nbb, in
 cudaError_t launch_energy_reduce(const int2* pairs, int npairs, const double* occ,
                                  const double* epair, const double* dpair, double scale,
                                  double* out, cudaStream_t s) {
-  const int threads = npairs >= 1024 ? 1024 : (npairs + 31) / 32 * 32;
+  // whole warps; one for no pairs (a shard without any: E = dE = 0)
+  const int threads = npairs >= 1024 ? 1024 : npairs > 0 ? (npairs + 31) / 32 * 32 : 32;
   return launch_after(k_energy, dim3(1), threads, 0, s, pairs, npairs, occ, epair, dpair, scale, out);
 }
 
