@@ -123,5 +123,27 @@ inline void kernel_value(fock_kernel kind, double vol, double omega, double g2, 
   }
 }
 
+// v and dv/domega of the Gamma-point kernel table at point (k1, k2, k3) of an n^3
+// grid: the means of their values at k and at -k (indices modulo n).  Pair densities
+// of real orbitals have |rho(k)| = |rho(-k)| and a real potential, so the mean is the
+// operator that the sum over the full grid gives, whatever the two values are.  They
+// differ on the Nyquist planes of cells whose reciprocal vectors are not orthogonal
+// only: -n/2 is its own negative there, so -k stands for a G of another length.
+// Pair densities reach those planes on grids that alias them.  Everywhere else the
+// mean is the value itself, bit for bit.
+inline void grid_kernel(fock_kernel kind, double vol, double omega, const double* recip, int n, int k1, int k2,
+                        int k3, double* v, double* dv) {
+  const int m[3] = {freq_of(k1, n), freq_of(k2, n), freq_of(k3, n)};
+  const auto minus = [n](int f) { return 2 * f == -n ? f : -f; };
+  const double g2 = g2_of(recip, m[0], m[1], m[2]);
+  const double g2_minus = g2_of(recip, minus(m[0]), minus(m[1]), minus(m[2]));
+  kernel_value(kind, vol, omega, g2, v, dv);
+  if (g2_minus == g2) return;
+  double v_minus, dv_minus;
+  kernel_value(kind, vol, omega, g2_minus, &v_minus, &dv_minus);
+  *v = 0.5 * (*v + v_minus);
+  *dv = 0.5 * (*dv + dv_minus);
+}
+
 }  // namespace lattice
 }  // namespace fockx

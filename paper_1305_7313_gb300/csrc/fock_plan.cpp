@@ -40,7 +40,6 @@ thread_local std::string g_create_error;
 
 using fockx::lattice::GEntry;
 using fockx::lattice::build_sphere;
-using fockx::lattice::freq_of;
 using fockx::lattice::g2_of;
 using fockx::lattice::kPi;
 
@@ -187,10 +186,6 @@ void free_ws(Workspace& w) {
 
 void reciprocal(const double* cell, double* recip, double* vol_signed) {
   *vol_signed = fockx::lattice::reciprocal(cell, recip);
-}
-
-void kernel_value(const fock_plan* p, double g2, double* v, double* dv) {
-  fockx::lattice::kernel_value(p->kind, p->vol, p->omega, g2, v, dv);
 }
 
 // Unique pairs i <= j in band blocks of kBandBlock (block rows outer), i outer and j
@@ -789,9 +784,8 @@ fock_status fock_plan_create(fock_plan_t* out, const int grid[3], const double c
   for (int k1 = 0; k1 < n; ++k1)
     for (int k2 = 0; k2 < n; ++k2)
       for (int k3 = 0; k3 < kh; ++k3) {
-        const double g2 = g2_of(p->recip, freq_of(k1, n), freq_of(k2, n), freq_of(k3, n));
         const int64_t i = ((int64_t)k1 * n + k2) * kh + k3;
-        kernel_value(p, g2, &v64[i], &dv64[i]);
+        fockx::lattice::grid_kernel(kind, p->vol, omega, p->recip, n, k1, k2, k3, &v64[i], &dv64[i]);
       }
   {
     double s2 = 0.0;  // ||v||_2^2 over the full grid from the stored half
