@@ -12,6 +12,7 @@ instead, on a bounded sample of the same workload.
 
 import argparse
 import json
+import math
 import os
 import statistics
 import subprocess
@@ -426,10 +427,10 @@ def run_batched(args, peaks, peak_src):
     bb = tuned.get("band_block", 16)
     nbytes = 0.0
     for sy, p in zip(systems, plans):
-        n = sy["N"]
-        kept, total = p.columns()
+        kept, total = p.columns()  # n x 2(n/2+1) columns of the plan's working grid n^3
+        n = math.isqrt(total + 1) - 1
         chains = (sy["nb"] * (sy["nb"] + 1) // 2 + 1) // 2
-        hbytes = n * n * 2 * (n // 2 + 1) * 8.0 * kept / total
+        hbytes = n * kept * 8.0
         nbytes += chains * (4 * hbytes + 16 * n ** 3 * 4.0 / max(1, min(bb, sy["nb"])))
     pm = statistics.median(pms)
     achieved = nbytes / (pm * 1e-3) / 1e9

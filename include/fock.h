@@ -245,10 +245,11 @@ fock_status fock_plan_set_deterministic(fock_plan_t plan, int enable);
 
 /* Columns of the pair densities' half spectra (n x 2(n/2+1) per plane of the
  * working grid, both pairs of a chain; stored as the columns of one complex
- * spectrum) that the pair-density ball |G| <= 2 Gmax reaches and the column pass
- * transforms (`kept`), out of `total`: the overlap densities of §4 are products
- * of two orbitals on the sphere, so their spectra live in that ball.  Host
- * outputs; either may be NULL.  Errors: INVALID_ARG (plan NULL). */
+ * spectrum) that the pair-density ball |G| <= 2 Gmax reaches (`kept`; of each row
+ * k2 up to the last one reached), out of `total`: the overlap densities of §4 are
+ * products of two orbitals on the sphere, so their spectra live in that ball, and
+ * only the columns it reaches are transformed.  Host outputs; either may be NULL.
+ * Errors: INVALID_ARG (plan NULL). */
 fock_status fock_plan_columns(fock_plan_t plan, int64_t* kept, int64_t* total);
 
 /*

@@ -311,7 +311,7 @@ def fock_plan_set_deterministic(plan, enable=True):
 
 
 def fock_plan_columns(plan):
-    """(kept, total) columns of the stored half spectrum the column pass transforms."""
+    """(kept, total) half-spectrum columns of the working grid: those the pair densities reach, all."""
     k = ctypes.c_int64()
     t = ctypes.c_int64()
     _check(load().fock_plan_columns(plan, ctypes.byref(k), ctypes.byref(t)), plan)

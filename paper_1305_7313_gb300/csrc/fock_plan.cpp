@@ -117,7 +117,7 @@ struct fock_plan {
   double vtab_f_f0 = 0.0;
   double2* d_cocc = nullptr;
   int64_t cocc_cap = 0;
-  int64_t kept_columns = 0;  // lines of the column map (both pairs)
+  int64_t kept_columns = 0;  // half-spectrum columns of both pairs that the ball reaches
   double* h_result = nullptr;  // pinned
   int64_t table_bytes = 0;
   Workspace ws;
@@ -1304,7 +1304,7 @@ fock_status fock_plan_set_deterministic(fock_plan_t plan, int enable) {
 fock_status fock_plan_columns(fock_plan_t plan, int64_t* kept, int64_t* total) {
   if (!plan) return fail(nullptr, FOCK_ERR_INVALID_ARG, "plan is NULL");
   if (kept) *kept = plan->kept_columns;
-  if (total) *total = (int64_t)plan->n * 2 * (plan->n / 2 + 1);  // of the caller's grid
+  if (total) *total = (int64_t)plan->dp.n * 2 * plan->dp.k3h;  // of the working grid, as kept
   return FOCK_OK;
 }
 

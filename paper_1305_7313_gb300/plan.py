@@ -77,7 +77,7 @@ class FockPlan:
         _lib.fock_plan_set_deterministic(self.handle, enable)
 
     def columns(self):
-        """(kept, total) half-spectrum columns the column pass transforms."""
+        """(kept, total) half-spectrum columns of the working grid: those the pair densities reach, all."""
         return _lib.fock_plan_columns(self.handle)
 
     def apply(self, psi_G, occ, vpsi_G=None, want_ex=True, want_dex=False, stream=None):
