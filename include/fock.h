@@ -211,9 +211,9 @@ fock_status fock_plan_set_band_block(fock_plan_t plan, int band_block);
  * forward plane pass, 1: the column pass, 2: the inverse plane pass) has one
  * or two compiled forms ("tilings") for the plan's working grid (the smallest
  * compiled grid that holds its pair densities): tile 0 the fastest measured, tile
- * 1, in FP64 and the mixed form where that grid is 96^3, 12 x 8 with eight threads
- * a line.  The results do not depend on the tiling beyond rounding; the speed
- * does (the tuner in autotune.py times them).
+ * 1, in FP64 and the mixed form where that grid is 96^3 (12 x 8) or 16^3 (8 x 2),
+ * two-factor stages with eight threads a line.  The results do not depend on the
+ * tiling beyond rounding; the speed does (the tuner in autotune.py times them).
  *
  * fock_plan_tiling_info: the plan of tile `tile` of pass `pass`: radices
  *   (host int[8], stage order), nstages, threads per transformed line,

@@ -770,7 +770,7 @@ template <class T, int N, int TILE = 0> constexpr TwoFactor two_factor() {
   static_assert(N == 8 || N == 12 || N == 16 || N == 20 || N == 24 || N == 28 || N == 32 || N == 36 || N == 40 ||
                     N == 48 || N == 56 || N == 60 || N == 64 || N == 72 || N == 80 || N == 96,
                 "no factors chosen for this line length");
-  if (TILE == 1) return TwoFactor{12, 8};
+  if (TILE == 1) return N == 16 ? TwoFactor{8, 2} : TwoFactor{12, 8};
   if (N == 96 && !FftTraits<T>::fused) return TwoFactor{12, 8};
   if (N == 72) return TwoFactor{12, 6};
   if (N == 36) return TwoFactor{12, 3};

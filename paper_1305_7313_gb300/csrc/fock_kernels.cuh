@@ -1392,8 +1392,11 @@ template <class T, int N>
 struct Launch {
   using C = cplx<T>;
   using P0 = PairGeo<T, N, 0>;
-  // the second tiling of the pair passes, where one is compiled
-  static constexpr int T1 = (N == 96 && RealTraits<T>::prec != 2) ? 1 : 0;
+  // the second tiling of the pair passes, where one is compiled: the sizes that have
+  // taken index 1 all along keep it.  It is the slower one in every pass measured
+  // (12 bands at 96^3, one pass on it: FP64 6.74 -> 7.06, 7.07, 6.88 ms, mixed 470 ->
+  // 534, 477, 515 us).
+  static constexpr int T1 = ((N == 96 || N == 16) && RealTraits<T>::prec != 2) ? 1 : 0;
   using P1 = PairGeo<T, N, T1>;
 
   static cudaError_t configure(const DevPlan&) {
