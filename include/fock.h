@@ -215,14 +215,15 @@ fock_status fock_plan_set_band_block(fock_plan_t plan, int band_block);
  * two-factor stages with eight threads a line.  The results do not depend on the
  * tiling beyond rounding; the speed does (the tuner in autotune.py times them).
  *
- * fock_plan_tiling_info: the plan of tile `tile` of pass `pass`: radices
- *   (host int[8], stage order), nstages, threads per transformed line,
- *   threads per CTA, and ntiles (1 or 2) for that pass.  INVALID_ARG for a
+ * fock_plan_tiling_info: the plan of tile `tile` of pass `pass` on the working
+ *   grid: radices (host int[8], stage order), nstages, threads per transformed
+ *   line, threads per CTA, and ntiles (1 or 2) for that pass.  INVALID_ARG for a
  *   tile the pass does not have.
- * fock_plan_set_tiling: tiles host int[3], the tile of each pass (each below
- *   that pass's ntiles); takes effect at the next call (fock_apply,
- *   fock_apply_shard, fock_apply_fixed, fock_pair_energies).  Default 0, 0, 0.
- *   Errors: INVALID_ARG.
+ * fock_plan_set_tiling: tiles host int[3], the tile of each pass; takes effect at
+ *   the next call (fock_apply, fock_apply_shard, fock_apply_fixed,
+ *   fock_pair_energies).  Tile 1 is taken where the working grid or the caller's
+ *   grid has it; a pass that has one tiling on the working grid runs that one.
+ *   Default 0, 0, 0.  Errors: INVALID_ARG.
  */
 fock_status fock_plan_tiling_info(fock_plan_t plan, int pass, int tile, int* radices, int* nstages,
                                   int* threads_per_line, int* threads, int* ntiles);

@@ -76,8 +76,8 @@ struct fock_plan {
   int npw = 0;
   const KernelOps* ops = nullptr;
   DevPlan dp{};
-  // kernels of the caller's grid: its FFT tilings, and (FP64, with the columns
-  // and twiddles in dp_full) the local potential of the Sternheimer solves
+  // kernels of the caller's grid: the tiling indices a plan takes, and (FP64, with
+  // the columns and twiddles in dp_full) the local potential of the Sternheimer solves
   const KernelOps* ops_full = nullptr;
   DevPlan dp_full{};
   int chain_batch = 1;
@@ -1066,7 +1066,7 @@ fock_status fock_plan_tiling_info(fock_plan_t plan, int pass, int tile, int* rad
     return fail(plan, FOCK_ERR_INVALID_ARG, "NULL output");
   if (pass < 0 || pass > 2 || tile < 0 || tile > 1) return fail(plan, FOCK_ERR_INVALID_ARG, "pass or tile out of range");
   int r[8], nst = 0, tl = 0, thr = 0;
-  const int nt = plan->ops_full->tile_plan(pass, tile, r, &nst, &tl, &thr);
+  const int nt = plan->ops->tile_plan(pass, tile, r, &nst, &tl, &thr);
   if (tile >= nt) return fail(plan, FOCK_ERR_INVALID_ARG, "this plan has one tiling for that pass");
   for (int k = 0; k < nst; ++k) radices[k] = r[k];
   *nstages = nst;
@@ -1081,7 +1081,9 @@ fock_status fock_plan_set_tiling(fock_plan_t plan, const int tiles[3]) {
   if (!tiles) return fail(plan, FOCK_ERR_INVALID_ARG, "tiles is NULL");
   for (int pass = 0; pass < 3; ++pass) {
     int r[8], nst = 0, tl = 0, thr = 0;
-    const int nt = plan->ops_full->tile_plan(pass, 0, r, &nst, &tl, &thr);
+    // of the working grid, or of the caller's: a pass without tiling 1 runs tiling 0
+    const int nt = std::max(plan->ops->tile_plan(pass, 0, r, &nst, &tl, &thr),
+                            plan->ops_full->tile_plan(pass, 0, r, &nst, &tl, &thr));
     if (tiles[pass] < 0 || tiles[pass] >= nt)
       return fail(plan, FOCK_ERR_INVALID_ARG, "a tile index is not below the pass's number of tilings");
   }

@@ -39,3 +39,31 @@ def test_both_tilings_of_16_give_the_oracles_results(prec):
             v, e, d = plan.apply(torch.from_numpy(c).cuda(), occ, want_dex=True)
             assert rel_inf(v.cpu().numpy(), vr) <= tv
             assert abs(e - er) <= te * abs(er) and abs(d - dr) <= te * abs(dr)
+
+
+@FORMS
+def test_a_plan_on_a_smaller_grid_reports_the_tilings_it_runs(prec):
+    # 96^3 at L 24: the pair passes run on 80^3, which has one tiling; index 1, which
+    # 96^3 has, is still taken, and those passes run the one there is
+    torch = require_gpu()
+    n, cell = 96, cubic(24.0)
+    with FockPlan(n, cell, 12.0, precision=prec) as plan:
+        assert plan.columns()[1] == 80 * 2 * 41
+        for p, name in enumerate(_lib.PASSES):
+            (tiling,) = plan.tilings()[name]
+            assert product(tiling) == 80
+            with pytest.raises(_lib.FockError):
+                _lib.fock_plan_tiling_info(plan.handle, p, 1)
+        psi = torch.from_numpy(synth.orbitals(plan.miller, cell, 2, 5)).cuda()
+        occ = np.array([2.0, 1.0])
+        v0, e0, _ = plan.apply(psi, occ)
+        plan.set_tiling([1, 1, 1])
+        v1, e1, _ = plan.apply(psi, occ)
+        tv, te = TOL[prec]
+        assert rel_inf(v1.cpu().numpy(), v0.cpu().numpy()) <= tv and abs(e1 - e0) <= te * abs(e0)
+        for bad in ([2, 0, 0], [0, -1, 0]):
+            with pytest.raises(_lib.FockError):
+                plan.set_tiling(bad)
+    with FockPlan(48, cubic(13.5), 12.0, precision=prec) as plan:  # 48 has one
+        with pytest.raises(_lib.FockError):
+            plan.set_tiling([1, 0, 0])
