@@ -22,10 +22,15 @@ The knobs are the ones that decide how pair work maps onto the GPU:
 
 Each candidate is timed on the caller's own inputs with CUDA events (one
 warm-up, then the median of ``reps`` runs) and the fastest is returned.  Results
-are cached in a JSON file keyed by the workload's shape (``FOCK_TUNE_CACHE``,
-default ``~/.cache/fockx/tune.json``) so a second process skips the search.
+are cached in a JSON file (``FOCK_TUNE_CACHE``, default
+``~/.cache/fockx/tune.json``) so a second process skips the search.  Its keys hold
+what a time depends on: the GPU, the library's kernels, the grid, the form and the
+band counts, and how many columns of which working grid the pair densities reach
+(the cell and the cutoff decide that).
 """
 
+import functools
+import hashlib
 import itertools
 import json
 import os
@@ -66,6 +71,28 @@ def _gpu_name():
     return torch.cuda.get_device_name(torch.cuda.current_device())
 
 
+@functools.lru_cache(maxsize=None)
+def _kernels():
+    """Digest of the library's sources: times of other kernels are not reused."""
+    src = os.path.join(os.path.dirname(os.path.abspath(__file__)), "csrc")
+    h = hashlib.sha256()
+    for name in sorted(n for n in os.listdir(src) if n.endswith((".cu", ".cuh", ".cpp", ".h"))):
+        with open(os.path.join(src, name), "rb") as f:
+            h.update(name.encode() + b"\0" + f.read())
+    return h.hexdigest()[:12]
+
+
+def _work(plan):
+    """The pair passes' size: kept and all columns of the plan's working grid."""
+    return "%d/%d" % tuple(plan.columns()) if hasattr(plan, "columns") else ""
+
+
+def _set_tiles(plan, tiles):
+    """Set the tiling of each pass, 0 where the plan has no other."""
+    t = plan.tilings()
+    plan.set_tiling([tiles[j] if tiles[j] < len(t.get(name, ())) else 0 for j, name in enumerate(PASSES)])
+
+
 def _time_ms(fn, reps):
     import torch
     fn()
@@ -99,7 +126,8 @@ def tune_apply(plan, psi, occ, chain_batches=(8, 17, 19, 32, 38), band_blocks=(8
     "table"}``; ``tiling`` names each pass's chosen radix plan and threads per
     line.
     """
-    key = "apply|%s|N%d|prec%d|nb%d" % (_gpu_name(), plan.grid[0], plan.precision, psi.shape[0])
+    key = "apply|%s|%s|N%d|%s|prec%d|nb%d" % (_gpu_name(), _kernels(), plan.grid[0], _work(plan), plan.precision,
+                                            psi.shape[0])
     has_tiling = tiling and hasattr(plan, "tilings")
     has_streams = bool(streams) and hasattr(plan, "set_streams")
     if use_cache:
@@ -108,7 +136,7 @@ def tune_apply(plan, psi, occ, chain_batches=(8, 17, 19, 32, 38), band_blocks=(8
             plan.set_batch(hit["chain_batch"])
             plan.set_band_block(hit["band_block"])
             if has_tiling:
-                plan.set_tiling(hit["tiles"])
+                _set_tiles(plan, hit["tiles"])
             if has_streams:
                 plan.set_streams(hit["streams"])
             return dict(hit, cached=True)
@@ -170,17 +198,16 @@ def tune_batch(plans, psi, occ, slot_chains=(4, 8, 16), rings=(3, 4), ctas_per_s
     batch with ``FockBatch(plans, psi, occ, **result["options"])``.
     """
     import torch
-    shape = ",".join("%dx%d" % (p.grid[0], x.shape[0]) for p, x in zip(plans, psi))
-    key = "batch|%s|prec%d|%s|%s" % (_gpu_name(), plans[0].precision, shape,
-                                     json.dumps(fixed, sort_keys=True))
+    shape = ",".join("%dx%d:%s" % (p.grid[0], x.shape[0], _work(p)) for p, x in zip(plans, psi))
+    key = "batch|%s|%s|prec%d|%s|%s" % (_gpu_name(), _kernels(), plans[0].precision, shape,
+                                        json.dumps(fixed, sort_keys=True))
     if use_cache:
         hit = _load_cache().get(key)
         if hit:
             for p in plans:
                 p.set_band_block(hit["band_block"])
                 if hit.get("tiles") and hasattr(p, "tilings"):
-                    t = p.tilings()
-                    p.set_tiling([hit["tiles"][j] if len(t[name]) > 1 else 0 for j, name in enumerate(PASSES)])
+                    _set_tiles(p, hit["tiles"])
             return dict(hit, cached=True)
     table = []
     combos = []
