@@ -335,8 +335,9 @@ fock_status ensure_workspace(fock_plan* p, int nb, int npairs) {
 }
 
 // Grow the real-space workspace to `nb` bands, keeping the first `keep` bands
-// of the orbitals (the fixed occupied set).
-fock_status grow_keeping(fock_plan* p, int nb, int keep) {
+// of the orbitals (the fixed occupied set), which work queued on s may still be
+// writing: the copies are ordered after it in s.
+fock_status grow_keeping(fock_plan* p, int nb, int keep, cudaStream_t s) {
   Workspace& w = p->ws;
   if (nb <= w.nb_cap) return FOCK_OK;
   const size_t rb = (size_t)p->ops->real_bytes;
@@ -352,10 +353,11 @@ fock_status grow_keeping(fock_plan* p, int nb, int keep) {
     return cuda_fail(p, e, "growing the workspace");
   }
   if (keep > 0 && w.psi) {
-    e = cudaMemcpy(psi, w.psi, (size_t)keep * (size_t)p->dp.ntot * rb, cudaMemcpyDeviceToDevice);
-    if (e == cudaSuccess) e = cudaMemcpy(occ, w.occ, sizeof(double) * keep, cudaMemcpyDeviceToDevice);
+    e = cudaMemcpyAsync(psi, w.psi, (size_t)keep * (size_t)p->dp.ntot * rb, cudaMemcpyDeviceToDevice, s);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(occ, w.occ, sizeof(double) * keep, cudaMemcpyDeviceToDevice, s);
     if (e == cudaSuccess && p->prec != FOCK_PREC_FP64)
-      e = cudaMemcpy(occ + nb, w.occT, rb * keep, cudaMemcpyDeviceToDevice);
+      e = cudaMemcpyAsync(occ + nb, w.occT, rb * keep, cudaMemcpyDeviceToDevice, s);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);  // the old buffers are freed below
     if (e != cudaSuccess) {
       cudaFree(psi);
       cudaFree(wacc);
@@ -1380,7 +1382,7 @@ fock_status fock_apply_fixed(fock_plan_t plan, const void* phi_G, int nt, void* 
   if ((int64_t)nb * nt > (int64_t)1 << 30) return fail(p, FOCK_ERR_INVALID_ARG, "too many pairs");
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   stats_reset(p);
-  st = grow_keeping(p, nb + nt, nb);
+  st = grow_keeping(p, nb + nt, nb, s);
   if (st != FOCK_OK) return st;
   const int npairs = nb * nt;
   st = ensure_workspace(p, nb + nt, npairs);
