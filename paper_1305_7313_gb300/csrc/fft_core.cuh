@@ -37,6 +37,9 @@ constexpr int kTwiddleTable = 2;  // forward and inverse twiddles
 constexpr int kMaxThreads = 1024;
 constexpr int kEmax = 24;  // elements a thread may hold across a stage
 
+// Radix plans: factorisations of a line into stages with whole lines shared by
+// tl threads.  No kernel is laid out by them (the passes' factors are two_factor's
+// and their geometry PairGeo's); the host checks of the radices and of Geo are.
 struct RadixPlan {
   int nst;                 // number of stages
   int r[kMaxStages];       // radices, in stage order
@@ -134,8 +137,7 @@ __host__ __device__ constexpr void radix_search(int n, int rem, int first, Radix
 }
 
 // Fewest stages first, then the most threads per line, with CTAs of at most
-// maxt threads.  Radices 6, 9, 12 and 16 are done in registers as two small
-// DFTs, so a plan such as 96 = 12 x 8 needs two shared-memory stages.
+// maxt threads.
 __host__ __device__ constexpr RadixPlan make_radix_plan(int n, int maxt = kMaxThreads, int emax = kEmax) {
   RadixPlan best{};
   best.nst = 0;
@@ -146,12 +148,10 @@ __host__ __device__ constexpr RadixPlan make_radix_plan(int n, int maxt = kMaxTh
   return best;
 }
 
-// Per working type.  emax: elements a thread may hold across a stage (24 in
-// FP32; 12 in FP64 and double-float, whose values take twice the registers of
-// a float, so their plans use more threads per line: 96 = 12 x 4 x 2 with 8
-// threads per line instead of 12 x 8 with 4).  fused: the type has a hardware
-// fused multiply-add, so twiddle products are folded into the butterfly sums
-// (Dft::run_tw) instead of being rounded on their own.
+// Per working type.  fused: the type has a hardware fused multiply-add, so twiddle
+// products are folded into the butterfly sums (Dft::run_tw) instead of being
+// rounded on their own.  emax: elements a thread may hold across a stage of a radix
+// plan (RadixPlan).
 template <class T> struct FftTraits {
   static constexpr int emax = kEmax;
   static constexpr bool fused = true;
@@ -161,8 +161,6 @@ template <class T> struct CplxOf;
 template <> struct CplxOf<float> { using type = float2; };
 template <> struct CplxOf<double> { using type = double2; };
 template <> struct CplxOf<df64> { using type = cdf64; };
-// FP64: the 12-element plans keep twice the warps of the 24-element ones in
-// flight on the FP64 pipe at the same instruction count
 template <> struct FftTraits<double> {
   static constexpr int emax = 12;
   static constexpr bool fused = true;
@@ -173,8 +171,8 @@ template <> struct FftTraits<df64> {
 };
 template <class T> using cplx = typename CplxOf<T>::type;
 
-// Elements a thread may hold across a stage for radix-plan variant EMAX (0:
-// the type's own, FftTraits<T>::emax).  A plan is named by (N, MAXT, EMAX).
+// Elements a thread may hold across a stage of radix plan (N, MAXT, EMAX) (0:
+// FftTraits<T>::emax).
 template <class T, int EMAX> __host__ __device__ constexpr int plan_emax() {
   return EMAX > 0 ? EMAX : FftTraits<T>::emax;
 }

@@ -169,10 +169,10 @@ __device__ inline void block_sum4_df(df64 v[4], float* red) {
 // Shared memory of one SM on sm_103 (228 KB; each resident CTA also reserves 1 KB).
 constexpr size_t kSmemPerSM = 233472;
 
-// Compile-time geometry of line transforms by radix plans (make_radix_plan; the
-// host checks print it; the passes' own geometry is PairGeo below) for grid size
-// N and radix-plan variant
-// EMAX (elements a thread holds across a stage; 0: the type's own).
+// Compile-time geometry of line transforms by radix plans (make_radix_plan) for grid
+// size N and element budget EMAX (0: the type's own): the layout of the passes
+// before the two-factor and block stages, kept for the host checks that print it.
+// No kernel is launched with it: that is PairGeo below.
 template <class T, int N, int MAXT = kMaxThreads, int EMAX = 0>
 struct Geo {
   using C = cplx<T>;
@@ -189,7 +189,6 @@ struct Geo {
   // NC lines at the column tiling: the inverse plane pass's CTA (its k2
   // transform of up to NC stored columns); the column pass sizes its own below
   static constexpr int THR_COLH = (NC * TLC + 31) / 32 * 32;
-  static constexpr int THR_COLF = (N * TLP + 31) / 32 * 32;
   // lines per CTA of the column pass: the NC columns of a row's width, or
   // about half as many, rounded up to 8 lines (whole warps at 4 and 8 threads
   // a line), where two CTAs of that width do not fit the SM's shared memory
@@ -216,18 +215,11 @@ struct Geo {
   // no bound below (two 224-thread CTAs fit the 142 registers FP64 takes)
   static constexpr int MIN_CTAS_COL =
       NLC < NC ? (sizeof(C) == 8 ? 65536 / (72 * THR_COL) : (THR_COL > 256 ? 2 : MIN_CTAS)) : MIN_CTAS;
-  // CTAs per SM the k-point inverse plane pass is register-budgeted for: in
-  // FP32, eight where eight CTAs of 40 registers a thread fit the register file
-  // (its shared memory allows that many up to N = 48); 0 leaves the choice to
-  // the compiler, as a bound without a minimum does (a minimum of 1 changes
-  // its register allocation: 89 instead of 78 registers at 96^3 in FP32)
-  static constexpr int MIN_CTAS_KINV = (sizeof(T) == 4 && 8 * 40 * THR_PLANE <= 65536) ? 8 : 0;
   // twiddle table in shared memory: e^{-2 pi i t/N} and its conjugate (2N values)
   static constexpr int TWN = kTwiddleTable * N;
   static constexpr size_t SMEM_PLANE = sizeof(C) * (size_t)(N * RP + TWN);
   static constexpr size_t SMEM_COLH =
       sizeof(C) * (size_t)(N * NLC + TWN) + 32 * 4 * sizeof(double) + NLC * sizeof(int);
-  static constexpr size_t SMEM_COLF = sizeof(C) * (size_t)(N * N + TWN);
   // inverse plane pass: the stored half plane with an odd row stride NC + 1,
   // the twiddles and the column map's row lengths
   static constexpr int NCP = NC + 1;
@@ -1361,13 +1353,8 @@ __global__ void __launch_bounds__(PairGeo<T, N, TILE>::THR_PLANE, PairGeo<T, N, 
                                                             blockIdx.x, smem_raw);
 }
 
-// ------------------------------------------------------------ FFT tilings
-//
-// Each pair pass can run one of two radix plans ("tilings"): tile 0 is the
-// type's own (FftTraits::emax elements per thread), tile 1 the plan found
-// with the other element budget (12 for FP32, 24 for FP64; none for the
-// double-float form).  When both budgets give the same plan for N, tile 1 is
-// tile 0 and no second kernel is compiled.
+// The element budget whose radix plan differs from the type's own (Geo; 0: none).
+// The tilings of the passes are Launch::T1's.
 template <class T> constexpr int alt_emax() {
   return RealTraits<T>::prec == 1 ? 12 : (RealTraits<T>::prec == 0 ? 24 : 0);
 }
