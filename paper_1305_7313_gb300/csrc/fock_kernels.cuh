@@ -1006,102 +1006,103 @@ __device__ __forceinline__ void pair_col_task(const DevPlan& g, cplx<T>* __restr
     }
     __syncthreads();
     stage_ct<T, B, +1, A, B * NL, NL, false, THR, NL, 1>(S, tw);
-  } else
-  for (int item = threadIdx.x; item < NP * A; item += THR) {
-    const int q = item / NP, qm = q == 0 ? 0 : A - q;
-    C z[B], y[B];
-    T v[B];
+  } else {
+    for (int item = threadIdx.x; item < NP * A; item += THR) {
+      const int q = item / NP, qm = q == 0 ? 0 : A - q;
+      C z[B], y[B];
+      T v[B];
 #pragma unroll
-    for (int s = 0; s < B; ++s) v[s] = vt[(q + A * s) * (N * KH)];
+      for (int s = 0; s < B; ++s) v[s] = vt[(q + A * s) * (N * KH)];
 #pragma unroll
-    for (int b = 0; b < B; ++b) {
-      z[b] = S[(B * q + b) * NL + p];
-      y[b] = S[(B * qm + b) * NL + NP + p];
-    }
-    dft_twiddled<T, B, -1>(z, tw + q * B);
-    dft_twiddled<T, B, -1>(y, tw + qm * B);
-    if constexpr (PREC == 0) {
-      const double* v64 = g.vtab64 + vo;
-      const double* dv64 = want_d ? g.dvtab64 + vo : nullptr;
-      const auto kernel = [&](int s, C& Z, C& Y, double a2, double b2, double* e) {
-        const int o = (q + A * s) * (N * KH);
-        const double ve = v64[o];
-        e[0] = fmadd(ve, a2, e[0]);
-        e[1] = fmadd(ve, b2, e[1]);
-        if (want_d) {
-          const double dv = dv64[o];
-          e[2] += dv * a2;
-          e[3] += dv * b2;
-        }
-        Z = cmake<T>(rmul(Z.x, v[s]), rmul(Z.y, v[s]));
-        Y = cmake<T>(rmul(Y.x, v[s]), rmul(Y.y, v[s]));
-      };
-      if (q == 0) mirror_multiply<T, B, true>(z, y, kernel, acc);
-      else mirror_multiply<T, B, false>(z, y, kernel, acc);
-    } else {
-      // the table holds v / Ntot, undone in FP64 after the CTA reduction
-      const auto kernel = [&](int s, C& Z, C& Y, T a2, T b2, T* e) {
-        e[0] += v[s] * a2;
-        e[1] += v[s] * b2;
-        if (want_d) {
-          const T dv = dvt[(q + A * s) * (N * KH)];
-          e[2] += dv * a2;
-          e[3] += dv * b2;
-        }
-        Z.x *= v[s];
-        Z.y *= v[s];
-        Y.x *= v[s];
-        Y.y *= v[s];
-      };
-      const int m2 = freq_of(k2, N), m3 = freq_of(k3, N);
-      const int r23 = m2 * m2 + m3 * m3;
-      bool small = false;
-      {
-        // terms with |m|^2 <= msmall2 (at most 3, so |m1| <= 1: k1 = 0 and 1
-        // in element 0 of blocks 0 and 1, N - 1 in the last of block A - 1) in FP64
-        small = code >= 0 && r23 <= g.msmall2 && (q <= 1 || q == A - 1);
-        if (small) {
-          const double wgt = line_self(code) ? 1.0 : 2.0;
-          const bool first = q <= 1 && q * q + r23 <= g.msmall2;
-          const bool last = q == A - 1 && 1 + r23 <= g.msmall2;
-          const C zero = cmake<T>(T(0), T(0));
-          // the FP64 terms' values leave the arrays while the FP32 loop runs
-          C z0 = z[0], y0 = q == 0 ? y[0] : y[B - 1], z1 = z[B - 1], y1 = q == 0 ? y[1 % B] : y[0];
-          if (first) {
-            small_g_term_fp64<T, N>(g, &z0, &y0, q, k2, k3, wgt, ch, epair, dpair);
-            z[0] = zero;
-            if (q == 0) y[0] = zero;
-            else y[B - 1] = zero;
-          }
-          if (last) {  // q = A - 1 > 0
-            small_g_term_fp64<T, N>(g, &z1, &y1, N - 1, k2, k3, wgt, ch, epair, dpair);
-            z[B - 1] = zero;
-            y[0] = zero;
-          }
-          if (q == 0) mirror_multiply<T, B, true>(z, y, kernel, acc);
-          else mirror_multiply<T, B, false>(z, y, kernel, acc);
-          if (first) {
-            z[0] = z0;
-            if (q == 0) y[0] = y0;
-            else y[B - 1] = y0;
-          }
-          if (last) {
-            z[B - 1] = z1;
-            y[0] = y1;
-          }
-        }
+      for (int b = 0; b < B; ++b) {
+        z[b] = S[(B * q + b) * NL + p];
+        y[b] = S[(B * qm + b) * NL + NP + p];
       }
-      if (!small) {
+      dft_twiddled<T, B, -1>(z, tw + q * B);
+      dft_twiddled<T, B, -1>(y, tw + qm * B);
+      if constexpr (PREC == 0) {
+        const double* v64 = g.vtab64 + vo;
+        const double* dv64 = want_d ? g.dvtab64 + vo : nullptr;
+        const auto kernel = [&](int s, C& Z, C& Y, double a2, double b2, double* e) {
+          const int o = (q + A * s) * (N * KH);
+          const double ve = v64[o];
+          e[0] = fmadd(ve, a2, e[0]);
+          e[1] = fmadd(ve, b2, e[1]);
+          if (want_d) {
+            const double dv = dv64[o];
+            e[2] += dv * a2;
+            e[3] += dv * b2;
+          }
+          Z = cmake<T>(rmul(Z.x, v[s]), rmul(Z.y, v[s]));
+          Y = cmake<T>(rmul(Y.x, v[s]), rmul(Y.y, v[s]));
+        };
         if (q == 0) mirror_multiply<T, B, true>(z, y, kernel, acc);
         else mirror_multiply<T, B, false>(z, y, kernel, acc);
+      } else {
+        // the table holds v / Ntot, undone in FP64 after the CTA reduction
+        const auto kernel = [&](int s, C& Z, C& Y, T a2, T b2, T* e) {
+          e[0] += v[s] * a2;
+          e[1] += v[s] * b2;
+          if (want_d) {
+            const T dv = dvt[(q + A * s) * (N * KH)];
+            e[2] += dv * a2;
+            e[3] += dv * b2;
+          }
+          Z.x *= v[s];
+          Z.y *= v[s];
+          Y.x *= v[s];
+          Y.y *= v[s];
+        };
+        const int m2 = freq_of(k2, N), m3 = freq_of(k3, N);
+        const int r23 = m2 * m2 + m3 * m3;
+        bool small = false;
+        {
+          // terms with |m|^2 <= msmall2 (at most 3, so |m1| <= 1: k1 = 0 and 1
+          // in element 0 of blocks 0 and 1, N - 1 in the last of block A - 1) in FP64
+          small = code >= 0 && r23 <= g.msmall2 && (q <= 1 || q == A - 1);
+          if (small) {
+            const double wgt = line_self(code) ? 1.0 : 2.0;
+            const bool first = q <= 1 && q * q + r23 <= g.msmall2;
+            const bool last = q == A - 1 && 1 + r23 <= g.msmall2;
+            const C zero = cmake<T>(T(0), T(0));
+            // the FP64 terms' values leave the arrays while the FP32 loop runs
+            C z0 = z[0], y0 = q == 0 ? y[0] : y[B - 1], z1 = z[B - 1], y1 = q == 0 ? y[1 % B] : y[0];
+            if (first) {
+              small_g_term_fp64<T, N>(g, &z0, &y0, q, k2, k3, wgt, ch, epair, dpair);
+              z[0] = zero;
+              if (q == 0) y[0] = zero;
+              else y[B - 1] = zero;
+            }
+            if (last) {  // q = A - 1 > 0
+              small_g_term_fp64<T, N>(g, &z1, &y1, N - 1, k2, k3, wgt, ch, epair, dpair);
+              z[B - 1] = zero;
+              y[0] = zero;
+            }
+            if (q == 0) mirror_multiply<T, B, true>(z, y, kernel, acc);
+            else mirror_multiply<T, B, false>(z, y, kernel, acc);
+            if (first) {
+              z[0] = z0;
+              if (q == 0) y[0] = y0;
+              else y[B - 1] = y0;
+            }
+            if (last) {
+              z[B - 1] = z1;
+              y[0] = y1;
+            }
+          }
+        }
+        if (!small) {
+          if (q == 0) mirror_multiply<T, B, true>(z, y, kernel, acc);
+          else mirror_multiply<T, B, false>(z, y, kernel, acc);
+        }
       }
-    }
-    Dft<+1, T>::template run<B>(z);
-    Dft<+1, T>::template run<B>(y);
+      Dft<+1, T>::template run<B>(z);
+      Dft<+1, T>::template run<B>(y);
 #pragma unroll
-    for (int b = 0; b < B; ++b) {
-      S[(B * q + b) * NL + p] = z[b];
-      S[(B * qm + b) * NL + NP + p] = y[b];
+      for (int b = 0; b < B; ++b) {
+        S[(B * q + b) * NL + p] = z[b];
+        S[(B * qm + b) * NL + NP + p] = y[b];
+      }
     }
   }
   // energies: each point and its mirror image counted once here (weight 2, a
