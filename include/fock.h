@@ -299,9 +299,11 @@ fock_status fock_apply_shard(fock_plan_t plan, const void* psi_G, int nb, const 
  * nb*nt pairs, two per complex transform, the occupied orbitals are not
  * transformed again.  With phi = psi it equals fock_apply's V_x psi.
  * Any other apply on the plan (fock_apply, fock_apply_shard,
- * fock_pair_energies) replaces the occupied set; fock_apply_fixed then
- * fails with INVALID_ARG until fock_set_occupied is called again.
- * Both are stream-ordered and return without synchronising.
+ * fock_pair_energies, fock_sternheimer_solve, a batch it joins) replaces the
+ * occupied set; fock_apply_fixed then fails with INVALID_ARG until
+ * fock_set_occupied is called again.
+ * Both are stream-ordered; they wait for the stream only to upload occupations
+ * (not in FP64) or a new pair schedule and to grow the workspace.
  * Errors: INVALID_ARG, OOM, CUDA.
  */
 fock_status fock_set_occupied(fock_plan_t plan, const void* psi_G, int nb, const double* occ,
@@ -425,7 +427,7 @@ fock_status fock_batch_default_options(fock_batch_options* opt);
  *   plans    host [nsys] distinct plans of one precision on the current device,
  *            each on a grid of 24, 32, 48, 64, 72 or 96 points per axis.  While
  *            the batch exists it owns the plans' workspaces: do not call other
- *            entry points on them.
+ *            entry points on them.  Occupied sets fixed on them are dropped.
  *   nb       host [nsys] band counts.
  *   psi_G    host [nsys] device pointers, complex128 [nb_s][npw_s] each.
  *   occ      host [nsys] host pointers, double [nb_s] each (copied now).

@@ -1809,6 +1809,8 @@ fock_status fock_batch_create(fock_batch_t* out, int nsys, const fock_plan_t* pl
     if (st != FOCK_OK) return fail_create(bfail(b, st, p->err));
     build_schedule(p, nb[k]);
     chains_from_pairs(p->pairs, p->chains);
+    p->fixed_nb = 0;  // the batch overwrites the real-space workspace and the chain list
+    p->fixed_sched_nt = -1;
     if ((e = cudaMemcpyAsync(p->ws.pairs, p->pairs.data(), sizeof(int2) * npairs, cudaMemcpyHostToDevice,
                              b->cap_stream)) != cudaSuccess ||
         (e = cudaMemcpyAsync(p->ws.chains, p->chains.data(), sizeof(Chain) * p->chains.size(),

@@ -5,7 +5,7 @@ import numpy as np
 import pytest
 
 import oracle
-from paper_1305_7313_gb300 import FockPlan, _lib, synth
+from paper_1305_7313_gb300 import FockBatch, FockPlan, _lib, synth
 from tests._common import cubic, rel_inf, require_gpu
 
 pytestmark = pytest.mark.gpu
@@ -29,3 +29,21 @@ def test_growing_waits_for_the_occupied_set(prec, tol):
         s.synchronize()
         vr = oracle.fock_apply_to(c, occ, t, plan.miller, (n,) * 3, cell, "erfc", 0.4)
         assert rel_inf(v.cpu().numpy(), vr) <= tol
+
+
+def test_a_batch_drops_the_occupied_set():
+    # a batch takes the plan's workspace over: the operator fixed before is gone
+    torch = require_gpu()
+    n, cell = 24, cubic(9.0)
+    with FockPlan(n, cell, 8.0, _lib.ERFC, 0.4) as plan:
+        psi = torch.from_numpy(synth.orbitals(plan.miller, cell, 5, 1)).cuda()
+        occ = np.full(5, 2.0)
+        plan.set_occupied(psi, occ)
+        before = plan.apply_fixed(psi)
+        b = FockBatch([plan], [psi[:3].contiguous()], [occ[:3]])
+        b.run()
+        b.close()
+        with pytest.raises(_lib.FockError):
+            plan.apply_fixed(psi)
+        plan.set_occupied(psi, occ)
+        assert rel_inf(plan.apply_fixed(psi).cpu().numpy(), before.cpu().numpy()) <= 1e-12
