@@ -168,13 +168,37 @@ def time_form(plan, psi, occ, steps, warmup, want_dex=False, rank=0, world=1):
     return dict(ms=ms, phase_ms=phase_ms, launches=launches, stats=plan.stats(), clocks=clk.summary())
 
 
-# DRAM bytes (read + write) per chain of the dominant kernel, from ncu captures
-# of the 96^3 pair passes of the 64-band case at 38 chains per launch, one
-# stream (profiles/pair_traffic_96.md); scaled
-# to a launch by its chains, reported only for a captured band block (the
-# orbital re-reads depend on it).  The captures are of earlier kernels; the present
-# ones move 53.2 MB (FP64, double-float) and 12.5 MB (mixed) a chain in the
-# inverse pass at band block 8 (profiles/pair_passes_96.md), TRAFFIC_SRC says so.
+# DRAM bytes (read + write) per chain of the pair passes, from ncu captures of the
+# 64-band case at 38 chains per launch, one stream (profiles/pair_traffic_96.md),
+# by form, grid and band block (the orbital re-reads depend on it).  reported() scales
+# them to a launch or a step by its chains; other band blocks have no figure.
+DRAM_PER_CHAIN = {
+    ("fp64", 96, 8): {"pair_fwd": 21.87e6, "pair_col": 17.08e6, "pair_inv": 52.98e6},
+    ("fp64", 96, 16): {"pair_fwd": 20.54e6, "pair_col": 17.06e6, "pair_inv": 46.81e6},
+    ("fp64", 96, 32): {"pair_fwd": 22.67e6, "pair_col": 17.07e6, "pair_inv": 51.67e6},
+    ("df64", 96, 8): {"pair_fwd": 21.91e6, "pair_col": 16.93e6, "pair_inv": 52.79e6},
+    ("df64", 96, 16): {"pair_fwd": 20.57e6, "pair_col": 16.93e6, "pair_inv": 46.70e6},
+    ("df64", 96, 32): {"pair_fwd": 22.65e6, "pair_col": 16.93e6, "pair_inv": 51.64e6},
+    ("mixed32", 96, 8): {"pair_fwd": 6.66e6, "pair_col": 8.84e6, "pair_inv": 12.13e6},
+    ("mixed32", 96, 16): {"pair_fwd": 8.62e6, "pair_col": 8.85e6, "pair_inv": 18.52e6},
+}
+CAPTURE_SRC = "ncu captures of the 64-band case, scaled by chains"
+
+
+def reported(roof, form, n, band_block):
+    """`roof` (of roofline()) as the JSON line gives it: its DRAM traffic from the
+    captures in DRAM_PER_CHAIN, of the dominant pass per launch or of all three per
+    step, None where there is none."""
+    per = DRAM_PER_CHAIN.get((form, n, band_block))
+    traffic = None
+    if per is not None:
+        traffic = (per[roof["kernel"]] * roof["chains_per_launch"] if roof["kernel"] in per
+                   else sum(per.values()) * roof["chains_per_step"])
+    return dict(roof, traffic=traffic, traffic_src=CAPTURE_SRC if traffic is not None else None)
+
+
+# The same of earlier kernels, which roofline() and loop_roofline() multiply; the
+# JSON line takes reported()'s instead.
 MEASURED_TRAFFIC_PER_CHAIN = {
     ("fp64", 96, "pair_inv", 8): 54.04e6, ("fp64", 96, "pair_inv", 16): 47.18e6, ("fp64", 96, "pair_inv", 32): 52.54e6,
     ("df64", 96, "pair_inv", 8): 57.45e6, ("df64", 96, "pair_inv", 16): 50.67e6, ("df64", 96, "pair_inv", 32): 53.20e6,
@@ -336,11 +360,8 @@ def loop_roofline(form, plan, res, steps, peaks, peak_src, band_block, streams):
     return out
 
 
-# DRAM bytes (read + write) per chain of the three pair kernels together, from
-# ncu captures of the 96^3 pair passes on one stream at 38 chains per launch
-# (profiles/pair_traffic_96.md), by form and band block; scaled to a step by
-# its chains.  The mixed form's column pass has changed since its capture
-# (CTAs of 56 lines), so its loop has no measured figure
+# DRAM bytes (read + write) per chain of the three pair kernels together, of earlier
+# kernels (as MEASURED_TRAFFIC_PER_CHAIN), by form, grid and band block
 MEASURED_LOOP_TRAFFIC_PER_CHAIN = {
     ("fp64", 96, 8): 95.61e6, ("fp64", 96, 16): 86.80e6, ("fp64", 96, 32): 94.01e6,
     ("df64", 96, 8): 98.40e6, ("df64", 96, 16): 90.15e6, ("df64", 96, 32): 94.48e6,
@@ -425,25 +446,22 @@ def run_batched(args, peaks, peak_src):
     # and the inverse pass reads four and read-modify-writes four accumulator
     # planes, each counted once per band block
     bb = tuned.get("band_block", 16)
-    nbytes = 0.0
+    nbytes, traffic = 0.0, 0.0  # DRAM bytes of the captures, nan where a grid has none
     for sy, p in zip(systems, plans):
         kept, total = p.columns()  # n x 2(n/2+1) columns of the plan's working grid n^3
         n = math.isqrt(total + 1) - 1
         chains = (sy["nb"] * (sy["nb"] + 1) // 2 + 1) // 2
         hbytes = n * kept * 8.0
         nbytes += chains * (4 * hbytes + 16 * n ** 3 * 4.0 / max(1, min(bb, sy["nb"])))
+        traffic += chains * BATCH_DRAM_PER_CHAIN.get(n, float("nan"))
     pm = statistics.median(pms)
     achieved = nbytes / (pm * 1e-3) / 1e9
     batch.close()
     for p in plans:
         p.close()
     mode = int(tuned["options"].get("persistent", 1))
-    traffic = None
-    if args.nb is None and bb == BATCH_DRAM_BAND_BLOCK and mode == 0:
-        # DRAM bytes per chain of the pair passes (ncu, 64-band systems), scaled by chains
-        traffic = sum(((sy["nb"] * (sy["nb"] + 1) // 2 + 1) // 2) * BATCH_DRAM_PER_CHAIN.get(sy["N"], float("nan"))
-                      for sy in systems)
-        traffic = None if traffic != traffic else traffic
+    if bb != BATCH_DRAM_BAND_BLOCK or mode != 0 or traffic != traffic:
+        traffic = None
     nbytes_kernel = {0: "pair passes (graph branches)", 1: "k_pair_persistent", 2: "k_pair_dataflow"}[mode]
     persistent = mode != 0
     return {"workload": "batched16_mixed32_sa_N48-96_L13.5-27",
@@ -456,18 +474,17 @@ def run_batched(args, peaks, peak_src):
             "roofline": {"bound": "hbm", "kernel": nbytes_kernel, "achieved": achieved,
                          "peak": float(peaks["hbm_gbs"]), "unit": "GB/s",
                          "frac": achieved / float(peaks["hbm_gbs"]), "traffic": traffic,
-                         "algorithmic_bytes": nbytes, "peak_src": peak_src + " (hbm copy)", "ms_pair_passes": pm},
+                         "traffic_src": CAPTURE_SRC if traffic is not None else None, "algorithmic_bytes": nbytes, "peak_src": peak_src + " (hbm copy)", "ms_pair_passes": pm},
             "tuned": {"options": tuned["options"], "band_block": tuned["band_block"],
                       "best_ms_by_mode": best_by_mode(tuned.get("table", []))},
             "clocks": clk.summary()}
 
 
 # DRAM bytes (read + write) per chain of the three pair passes of the batch's
-# systems, by grid size, at band block 16: an ncu capture of every pair launch
-# of the 64-band version of the batch as graph branches (launches serialised
-# by ncu; profiles/pair_traffic_96.md).  The 96^3 systems' column pass has
-# changed since (CTAs of 56 lines), so the batch has no measured total
-BATCH_DRAM_PER_CHAIN = {48: 3.077e6, 64: 7.361e6, 72: 10.790e6}
+# systems, by the grid they work on, at band block 16: an ncu capture of every pair
+# launch of the 64-band version of the batch as graph branches (launches serialised
+# by ncu; profiles/pair_traffic_96.md).
+BATCH_DRAM_PER_CHAIN = {48: 2.702e6, 60: 6.045e6, 64: 7.944e6, 96: 40.385e6}
 BATCH_DRAM_BAND_BLOCK = 16
 
 
@@ -524,10 +541,11 @@ def run_kpoints(args, peaks, peak_src):
                          "peak": float(peaks["hbm_gbs"]), "unit": "GB/s",
                          "frac": achieved / float(peaks["hbm_gbs"]), "traffic": traffic,
                          "traffic_unit": "DRAM bytes per step (ncu, all three kernels)",
-                         "traffic_src": TRAFFIC_SRC, "peak_src": peak_src + " (hbm copy)"}}
+                         "traffic_src": "ncu capture of this leg" if traffic is not None else None,
+                         "peak_src": peak_src + " (hbm copy)"}}
 
 
-KPOINT_DRAM_PER_PAIR = 3.351e6
+KPOINT_DRAM_PER_PAIR = 2.740e6
 
 
 def run_fixed(args):
@@ -866,8 +884,9 @@ def main():
     ms_step = res["ms"] / args.steps
     value = pairs * args.steps / (res["ms"] * 1e-3)
     form = {PREC_FP64: "fp64", PREC_MIXED32: "mixed32"}.get(w["prec"], "df64")
-    roof = roofline(form, plan, res, args.steps, peaks, peak_src, tuned["band_block"] if tuned else 16,
-                    tuned.get("streams", 1) if tuned else 1)
+    bb = tuned["band_block"] if tuned else 16
+    roof = reported(roofline(form, plan, res, args.steps, peaks, peak_src, bb, tuned.get("streams", 1) if tuned else 1),
+                    form, w["N"], bb)
     err = golden_errors(plan, c, w) if world == 1 else None
 
     # ---- end to end through the public API from pinned host memory
@@ -906,11 +925,12 @@ def main():
         psim = torch.from_numpy(cm).cuda()
         resm = time_form(planm, psim, occm, args.steps, args.warmup, rank=rank, world=world)
         pm = wm["nb"] * (wm["nb"] + 1) // 2
+        bbm = tunedm["band_block"] if tunedm else 16
         mixed = {"workload": wm["name"], "value": pm * args.steps / (resm["ms"] * 1e-3), "unit": UNIT,
                  "steps": args.steps,
                  "ms_per_step": resm["ms"] / args.steps, "dtype": "f32",
-                 "roofline": roofline("mixed32", planm, resm, args.steps, peaks, peak_src,
-                                      tunedm["band_block"] if tunedm else 16, tunedm.get("streams", 1) if tunedm else 1),
+                 "roofline": reported(roofline("mixed32", planm, resm, args.steps, peaks, peak_src, bbm,
+                                               tunedm.get("streams", 1) if tunedm else 1), "mixed32", wm["N"], bbm),
                  "pair_loop_pairs_per_s": pair_loop_rate(pm, resm, args.steps), "pass_share": phase_share(resm),
                  "gpu_launches": resm["launches"], "clocks": resm["clocks"], "tuned": tunedm}
         mixed["summary"] = form_summary(mixed, mixed["roofline"], golden_errors(planm, cm, wm) if world == 1 else None)
@@ -935,10 +955,11 @@ def main():
         kd = min(args.steps, args.side_steps)
         resd = time_form(pland, psid, occd, kd, args.warmup, rank=rank, world=world)
         pd = wd["nb"] * (wd["nb"] + 1) // 2
+        bbd = tunedd["band_block"] if tunedd else 16
         df = {"workload": wd["name"], "value": pd * kd / (resd["ms"] * 1e-3), "unit": UNIT, "steps": kd,
               "ms_per_step": resd["ms"] / kd, "dtype": "f32x2 (double-float)",
-              "roofline": roofline("df64", pland, resd, kd, peaks, peak_src,
-                                   tunedd["band_block"] if tunedd else 16, tunedd.get("streams", 1) if tunedd else 1),
+              "roofline": reported(roofline("df64", pland, resd, kd, peaks, peak_src, bbd,
+                                            tunedd.get("streams", 1) if tunedd else 1), "df64", wd["N"], bbd),
               "pair_loop_pairs_per_s": pair_loop_rate(pd, resd, kd), "pass_share": phase_share(resd),
               "gpu_launches": resd["launches"], "clocks": resd["clocks"], "tuned": tunedd}
         df["summary"] = form_summary(df, df["roofline"], golden_errors(pland, cd, wd) if world == 1 else None)
