@@ -498,6 +498,12 @@ def best_by_mode(table):
     return out
 
 
+def columns_reached(radius, L):
+    """Columns (m2, m3) of a cubic cell's reciprocal lattice that the ball |G| <= radius reaches."""
+    m = np.arange(-int(radius * L / (2.0 * math.pi)) - 1, int(radius * L / (2.0 * math.pi)) + 2)
+    return int(np.count_nonzero((2.0 * math.pi / L) ** 2 * (m[:, None] ** 2 + m[None, :] ** 2) <= radius * radius))
+
+
 def run_kpoints(args, peaks, peak_src):
     """2x2x2 Monkhorst-Pack mesh (k in {0, 1/2}^3, weights 1/8), 48^3 grid,
     L = 13.5 bohr, Ecut = 12 Ha, 32 bands per k, erfc kernel, mixed form."""
@@ -528,7 +534,10 @@ def run_kpoints(args, peaks, peak_src):
     ms = start.elapsed_time(end)
     ns = len(kpts) * nb
     pairs = ns * (ns + 1) // 2
-    nbytes = pairs * 4.0 * n**3 * 8.0  # complex64 full spectrum: written, read + written, read
+    # complex64 spectrum: written, read + written, read; of its n^2 columns those that
+    # the pair densities' ball |G| <= 2 Gmax + max |q| reaches
+    kept = columns_reached(2.0 * math.sqrt(2.0 * ecut) + math.pi * math.sqrt(3.0) / L, L)
+    nbytes = pairs * 4.0 * kept * n * 8.0
     achieved = nbytes * args.steps / (ms * 1e-3) / 1e9
     # DRAM bytes (read + write) per pair of the three k-point pair kernels, from
     # an ncu capture of every pair launch of this leg (profiles/kpair_traffic_48.md)
