@@ -277,7 +277,8 @@ fock_status fock_apply(fock_plan_t plan, const void* psi_G, int nb, const double
  * results are summed at the end).  The unique pairs are cut, in the library's
  * fixed schedule, into nshards contiguous parts of near-equal size; this call
  * evaluates part `shard` (0 <= shard < nshards) and returns the partial
- * V_x psi and partial E_x, dE_x/domega.  Summing the results of all shards
+ * V_x psi and partial E_x, dE_x/domega (zeros for a part without pairs: there may
+ * be more parts than chains of two pairs).  Summing the results of all shards
  * reproduces fock_apply up to rounding.  Arguments as in fock_apply.
  */
 fock_status fock_apply_shard(fock_plan_t plan, const void* psi_G, int nb, const double* occ,
@@ -377,9 +378,12 @@ fock_status fock_pair_energies_static(fock_plan_t plan, const void* psi_G, int n
  *   iters    host int [nrhs] or NULL: CG updates each band received.
  *   resid    host double [nrhs] or NULL: final residual norms (a band that
  *            did not reach tol within maxiter keeps its last iterate).
- * Uses the plan's real-space workspace (any fixed operator set by
- * fock_set_occupied is dropped) and allocates its own CG vectors for the
- * call.  Synchronises the stream once per CG iteration.
+ * Uses the plan's transform buffer (any fixed operator set by fock_set_occupied
+ * is dropped).  The CG vectors (five ket arrays and the projector coefficients) and,
+ * on a plan that works on a smaller grid, transform blocks of its own (up to 32
+ * N^3 complex grids) live in one buffer of the plan, which grows with the largest
+ * call, counts in fock_plan_device_bytes and is freed with the plan.  Synchronises
+ * the stream once per CG iteration.
  * Errors: INVALID_ARG, OOM, CUDA.
  */
 fock_status fock_sternheimer_solve(fock_plan_t plan, const double* vloc, const void* u_G, int nocc,

@@ -1,5 +1,5 @@
 // fock_internal.h — what the host plan (fock_plan.cpp) and the kernel
-// translation units (fock_kernels_f64.cu, fock_kernels_f32.cu) share.
+// translation units (fock_kernels_inst.cu, once per form and grid size) share.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -69,7 +69,7 @@ struct DevPlan {
   int msmall2;         // |m|^2 at or below which kernel terms are done in FP64 (mixed form)
   ColumnSet cols;  // columns the pair densities reach
   ColumnSet orb;   // columns of the orbitals' sphere (Gamma point)
-  // radix-plan variant ("tiling", 0 or 1) of the forward plane, column and
+  // tiling (0 or 1) of the forward plane, column and
   // inverse plane passes
   int tile[3];
   // deterministic accumulation: W holds 64-bit fixed point scaled by det_scale[0]

@@ -301,9 +301,10 @@ struct PairGeo {
   // ones only.
   static constexpr bool ALL_LINES = sizeof(C) == 8;
   // FP32 plane passes take three trips through registers (N = 4 M): shared
-  // memory bounds them, and a trip fewer takes the inverse pass at 96^3 from 4.29
-  // to 3.65 us a chain, the forward pass, whose result then goes out from
-  // registers, from 3.44 to 2.37.  FP64 and double-float are bound by arithmetic: the two-factor
+  // memory bounds them, and a trip fewer took the inverse pass at 96^3 from 4.29
+  // to 3.65 us a chain and the forward pass from 3.44 to 3.06 (with packed additions
+  // 3.26 and 2.89 since, and 2.37 with the result going out from registers, see
+  // plane_row_stage).  FP64 and double-float are bound by arithmetic: the two-factor
   // stages' items are smaller and share out more evenly (FP64 24^3 forward 0.85
   // against 1.05 us, 48^3 6.39 against 6.49, 96^3 even)
   static constexpr bool BLOCK = RealTraits<T>::prec == 1 && TILE == 0;

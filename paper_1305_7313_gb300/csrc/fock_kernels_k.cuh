@@ -8,12 +8,14 @@
 //   rho_ab = u_a* u_b,   phi_ab = IFFT[v(G + q) FFT(rho_ab)],
 //   W_b -= w_a f_a u_a phi_ab,   W_a -= w_b f_b u_b conj(phi_ab)   (a != b)
 // (the reverse pair has rho_ba = rho_ab* and q -> -q, so phi_ba = phi_ab*).
-// One pair per chain and per complex transform; the whole spectrum is kept.
+// One pair per chain and per complex transform; the columns that the pair densities
+// reach are kept.
 //
 // Layout in HBM:
 //   u    [Ns][N][N][N] complex T     periodic parts in real space
 //   W    [Ns][N][N][N] complex T     periodic parts of V_x psi
-//   H    [chain][N][N][N] complex T  pair density after the plane pass
+//   H    [chain][N][N][N] complex T  per plane i1 the kept columns (k2, k3) of a pair
+//        density's 2D transform
 //   vq   [nq][N][N][N] T             v(G + q) / Ntot per distinct q
 //   vq64 [nq][N][N][N] double        v(G + q)
 #pragma once

@@ -970,8 +970,8 @@ fock_status fock_plan_create(fock_plan_t* out, const int grid[3], const double c
     return cuda_fail(nullptr, e, "cudaDeviceGetAttribute");
   }
   // Default chains per launch: a multiple of c0 = SMs / gcd(N, SMs), so the N
-  // CTAs per chain of the plane passes fill whole waves (19 on a 152-SM GPU for
-  // every compiled N), as many multiples as the buffer budget holds.
+  // CTAs per chain of the plane passes fill whole waves (on a 152-SM GPU 19 where N
+  // is a multiple of 8, else 38), as many multiples as the buffer budget holds.
   const size_t chain_bytes = (size_t)d.hsize * 2 * (size_t)ops->real_bytes;
   {
     int a = n, b = std::max(1, sms);

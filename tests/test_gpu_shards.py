@@ -14,13 +14,16 @@ pytestmark = pytest.mark.gpu
 TOL = {_lib.PREC_FP64: (1e-13, 1e-13), _lib.PREC_DF64: (1e-13, 1e-13), _lib.PREC_MIXED32: (2e-5, 5e-6)}
 
 
-@pytest.mark.parametrize("det", [False, True], ids=["plain", "deterministic"])
-@pytest.mark.parametrize("prec", sorted(TOL), ids=["fp64", "mixed32", "df64"])
+# (deterministic accumulation is not offered for the mixed form)
+FORMS = {"fp64": (_lib.PREC_FP64, False), "mixed32": (_lib.PREC_MIXED32, False), "df64": (_lib.PREC_DF64, False),
+         "fp64-det": (_lib.PREC_FP64, True), "df64-det": (_lib.PREC_DF64, True)}
+
+
+@pytest.mark.parametrize("form", FORMS)
 @pytest.mark.parametrize("nb", [1, 2, 3])
-def test_shards_without_pairs(nb, prec, det):
+def test_shards_without_pairs(nb, form):
     torch = require_gpu()
-    if det and prec == _lib.PREC_MIXED32:
-        pytest.skip("deterministic accumulation is not offered for the mixed form")
+    prec, det = FORMS[form]
     n, cell, nshards = 24, cubic(10.0), 8
     mill, _ = oracle.gsphere((n,) * 3, cell, 10.0)
     psi = torch.from_numpy(synth.orbitals(mill, cell, nb, nb)).cuda()
